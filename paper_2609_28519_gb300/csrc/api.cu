@@ -144,6 +144,30 @@ static int tg_plan_tables(bdct_plan *p)
     return BDCT_OK;
 }
 
+// The line engine's tables: one per axis and scale (the forward and the
+// inverse of a normalization share their scale of the indices above 0).
+static int lines_plan_tables(bdct_plan *p)
+{
+    const size_t ew = lines_table_elems(p->cols), eh = lines_table_elems(p->rows);
+    const bool plain = p->norm != BDCT_NORM_ORTHO && (p->kind & (BDCT_FORWARD | BDCT_INVERSE));
+    const size_t total = (plain ? 2 : 1) * (ew + eh);
+    cudaError_t e = cudaMalloc(&p->line_tw, total * sizeof(float4));
+    if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
+    p->line_w = p->line_w_ortho = 0;
+    p->line_h = p->line_h_ortho = ew;
+    e = lines_gen_table(p->line_tw, p->cols, std::sqrt(2.0 / p->cols), 0);
+    if (e == cudaSuccess) e = lines_gen_table(p->line_tw + ew, p->rows, std::sqrt(2.0 / p->rows), 0);
+    if (plain) {
+        p->line_w = ew + eh;
+        p->line_h = p->line_w + ew;
+        if (e == cudaSuccess) e = lines_gen_table(p->line_tw + p->line_w, p->cols, 2.0, 0);
+        if (e == cudaSuccess) e = lines_gen_table(p->line_tw + p->line_h, p->rows, 2.0, 0);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    p->table_bytes = total * sizeof(float4);
+    return BDCT_OK;
+}
+
 // The input-term buffer of the warp-specialized tensor-core passes (long
 // contractions): three BF16 terms of every element of a chunk, in whole
 // 128-row tiles, for either pass.  Only plans with such an axis get one.
@@ -265,13 +289,8 @@ extern "C" int bdct_plan_create(bdct_plan **plan, int rows, int cols, unsigned k
         p->work_bytes = (size_t)chunk * arr_bytes;
         e = cudaMalloc(&p->work, p->work_bytes);
         if (e != cudaSuccess) { plan_free(p); t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
-        p->line_tw_h = lines_table_elems(cols);
-        e = cudaMalloc(&p->line_tw, (lines_table_elems(cols) + lines_table_elems(rows)) * sizeof(float2));
-        if (e != cudaSuccess) { plan_free(p); t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
-        e = lines_gen_table(p->line_tw, cols, 0);
-        if (e == cudaSuccess) e = lines_gen_table(p->line_tw + p->line_tw_h, rows, 0);
-        if (e != cudaSuccess) { plan_free(p); return cuda_fail(e); }
-        p->table_bytes = (lines_table_elems(cols) + lines_table_elems(rows)) * sizeof(float2);
+        st = lines_plan_tables(p);
+        if (st != BDCT_OK) { plan_free(p); return st; }
     } else {
         p->variant = 2;
         // operator matrices: forward and inverse in the plan's norm, and the
@@ -355,22 +374,46 @@ static bool ranges_partially_overlap(const void *a, const void *b, size_t bytes)
     return x < y + bytes && y < x + bytes;
 }
 
-static int run_lines(const bdct_plan *p, Dir dir, const DirScales &sc, const float *in, const long long *in_off,
-                     float *out, const long long *out_off, long long count, cudaStream_t s,
-                     const float *lam = nullptr)
+static DirScales ortho_scales(const bdct_plan *p, Dir dir);
+
+// The line engine, chunk by chunk through the workspace.  Forward: along w,
+// then along h; inverse: along h, then along w; round trip: a row pair, then a
+// column pair; spectral: the forward along w, the pair along h with Lambda
+// between (in place in the workspace), the inverse along w.
+static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long long *in_off, float *out,
+                     const long long *out_off, long long count, cudaStream_t s)
 {
     const int h = p->rows, w = p->cols;
     const long long hw = (long long)h * w;
+    const bool ortho = dir == DIR_RT || dir == DIR_SPEC;
+    const DirScales sc = ortho ? ortho_scales(p, DIR_FWD) : p->scales[dir];
+    const float4 *tw = p->line_tw + (ortho ? p->line_w_ortho : p->line_w);
+    const float4 *th = p->line_tw + (ortho ? p->line_h_ortho : p->line_h);
     for (long long b0 = 0; b0 < count; b0 += p->chunk_arrays) {
         const long long nb = (count - b0) < p->chunk_arrays ? (count - b0) : p->chunk_arrays;
         const float *src = in_off ? in : in + b0 * hw;
         float *dst = out_off ? out : out + b0 * hw;
-        // rows of X (h lines of w) -> workspace (w x h), then rows of that (w lines of h) -> out (h x w)
-        cudaError_t e = lines_pass(src, p->work, h, w, nb, dir, sc.w, p->line_tw, p->status, s,
-                                   in_off ? in_off + b0 : nullptr, nullptr);
-        if (e == cudaSuccess)
-            e = lines_pass_lam(p->work, dst, w, h, nb, dir, sc.h, p->line_tw + p->line_tw_h, p->status, s,
-                               nullptr, out_off ? out_off + b0 : nullptr, true, lam);
+        const long long *so = in_off ? in_off + b0 : nullptr, *dof = out_off ? out_off + b0 : nullptr;
+        cudaError_t e;
+        if (dir == DIR_INV) {
+            e = lines_pass(src, p->work, w, h, nb, LINES_INVERSE, sc.h, th, nullptr, p->status, s, so, nullptr);
+            if (e == cudaSuccess)
+                e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE, sc.w, tw, nullptr, p->status, s, nullptr, dof, true);
+        } else if (dir == DIR_RT) {
+            e = lines_pass(src, p->work, h, w, nb, LINES_PAIR_ROWS, sc.w, tw, nullptr, p->status, s, so, nullptr);
+            if (e == cudaSuccess)
+                e = lines_pass(p->work, dst, w, h, nb, LINES_PAIR_COLS, sc.h, th, nullptr, p->status, s, nullptr, dof, true);
+        } else {
+            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, tw, nullptr, p->status, s, so, nullptr);
+            if (e == cudaSuccess && dir == DIR_FWD) {
+                e = lines_pass(p->work, dst, w, h, nb, LINES_FORWARD, sc.h, th, nullptr, p->status, s, nullptr, dof, true);
+            } else if (e == cudaSuccess) {
+                e = lines_pass(p->work, p->work, w, h, nb, LINES_PAIR_ROWS, sc.h, th, p->spec_plain, p->status, s, nullptr,
+                               nullptr, true);
+                if (e == cudaSuccess)
+                    e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE, sc.w, tw, nullptr, p->status, s, nullptr, dof);
+            }
+        }
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return BDCT_OK;
@@ -591,14 +634,7 @@ static int execute_dir(const bdct_plan *p, Dir dir, const float *in, const long 
         return run_onchip(p, dir, g, s);
     }
     if (p->variant == 4) return run_tg(p, dir, in, in_off, out, out_off, count, s);
-    if (p->lines) {
-        if (dir != DIR_SPEC) return run_lines(p, dir, p->scales[dir], in, in_off, out, out_off, count, s);
-        // the orthonormal forward, its second pass storing the spectrum times
-        // Lambda, then the orthonormal inverse in place
-        int st = run_lines(p, DIR_FWD, ortho_scales(p, DIR_FWD), in, in_off, out, out_off, count, s, p->spec_plain);
-        if (st == BDCT_OK) st = run_lines(p, DIR_INV, ortho_scales(p, DIR_INV), out, out_off, out, out_off, count, s);
-        return st;
-    }
+    if (p->lines) return run_lines(p, dir, in, in_off, out, out_off, count, s);
     return run_separable(p, dir, in, in_off, out, out_off, count, s);
 }
 

@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "bdct_internal.h"
+#include "fp32_lines.h"
 #include "dct_cores.cuh"
 #include "ptx.cuh"
 

@@ -1,32 +1,49 @@
 // FFT-based FP32 line engine: one separable pass of the 2D DCT for long
 // lines (64 .. 4096 points, powers of two, and 192, 384, 768, 1536 =
-// 3 * 2^6 .. 3 * 2^9: the half-length FFT takes one radix-3 stage).
+// 3 * 2^6 .. 3 * 2^9).
 //
 // What is computed: the 1D factor of Eq. 2 of the BRiDCT paper along every
-// row of a batch of arrays -- y_k = s_k sum_j x_j cos(pi (2j+1) k / (2N))
+// line of a batch of arrays -- y_k = s_k sum_j x_j cos(pi (2j+1) k / (2N))
 // (forward), its adjoint x_j = sum_k s_k y_k cos(...) (inverse), or the
-// forward, the E_n^2 correction and the adjoint (round trip, Prop. 1) -- with
-// the result written transposed, so that two passes (rows, then the rows of
-// the transposed intermediate) give the 2D transform in natural layout.
+// forward, a diagonal and the adjoint in one pass (round trip and spectral
+// composition, Prop. 1).  The forward reads rows and writes its result
+// transposed, the inverse reads transposed and writes rows, so two passes
+// give the 2D transform in natural layout.
 //
 // The length-N DCT-II of a real line is evaluated exactly through a complex
-// FFT of L = N/2 points (Makhoul's reordering):
-//   v_i = x_{2i} (i < L),  v_{N-1-i} = x_{2i+1};   z_m = v_{2m} + i v_{2m+1};
-//   Z = FFT_L(z) by the four-step method, L = L1 * L2: L2 FFTs of length L1
-//   on stride-L2 subsequences, twiddles exp(-2 pi i m2 k1 / L), L1 FFTs of
-//   length L2; then with E_k = (Z_k + conj Z_{L-k}) / 2,
-//   O_k = (Z_k - conj Z_{L-k}) / (2i), V_k = E_k + exp(-2 pi i k / N) O_k:
-//   y_k = Re(exp(-i pi k / (2N)) V_k), y_{N-k} = -Im(exp(-i pi k / (2N)) V_k).
-// The DCT-III runs the same steps backwards (its 1/L folded into a factor 2
-// on y_0).
+// FFT of L = N/2 points (Makhoul's reordering): z_m = (x_{4m}, x_{4m+2}) and
+// z_{L-1-m} = (x_{4m+3}, x_{4m+1}) for m < L/2, Z = FFT_L(z), then with
+// E = Z_k + conj Z_{L-k}, O = -i (Z_k - conj Z_{L-k}), P = exp(-2 pi i k/N) O,
+// V = E + P, V' = conj(E - P) and W_k = exp(-i pi k / (2N)) / 2:
+//   y_k = Re(W_k V),  y_{N-k} = -Im(W_k V),
+//   y_{L-k} = Re(W_{L-k} V'),  y_{L+k} = -Im(W_{L-k} V').
+// The FFT takes two or three steps, L = R1 R2 R3 (R2 = 1 for two), each a set
+// of short FFTs in registers with one exchange through shared memory between
+// steps.  The DCT-III is the exact transpose of those steps in reverse order.
 //
-// GPU organization: T threads share a line, T dividing L1 and L2, so that in
-// both FFT steps every thread runs whole register-resident sub-FFTs (radix 2
-// and 3, dct_cores.cuh); the step-C results stay in registers and the split
-// partner Z_{L-k}, held by thread T - t of the same line, arrives by warp
-// shuffle.  All twiddles come from per-plan tables generated in FP64 and
-// staged in shared memory.  The FFT stays within FP32 rounding of the exact
-// sums (error grows like log N).
+// Packed pairs.  A thread transforms two short FFTs ("a couple") at once in
+// the halves of float2 registers (one packed instruction serves both): column
+// cc and its mirror MC-1-cc, taken in reversed order with real and imaginary
+// parts swapped.  In that form one aligned float4 of the line, (x_{4q} ..
+// x_{4q+3}), is exactly one element of both halves, so nothing is shuffled to
+// form the pairs, and so is one float4 of every exchange (a "unit").  The
+// last step pairs column c with C-c, conjugated, which puts Z_k and
+// conj Z_{L-k} in the two halves of one register.  Phases that the mirrored
+// and the conjugated halves pick up are part of the twiddle tables: the
+// mirrored half of column cc takes exp(2 pi i k (cc+1) / (R MC)), and the
+// step before the last uses signed k in [-R/2, R/2).
+//
+// Shared memory.  A CTA holds a panel of PR lines, one line per lane: line l
+// at pitch N + 4 floats, which puts the lanes' float4 of one index on
+// distinct banks in every phase.  A step writes its results over the units it
+// read, so there is one panel buffer, and the only barriers are one between
+// steps.  The transposed side goes straight between registers and global
+// memory: at a fixed index the PR lanes hold PR consecutive elements.  The
+// row side moves by one bulk copy (TMA) per line.
+//
+// What bounds it: 16 bytes of shared-memory traffic per element, pass and
+// exchange (37 TB/s on the chip) and about 16 multiply-adds, against 8 bytes
+// of HBM traffic per element and pass.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -46,554 +63,628 @@ bool lines_supported(int n)
            n == 384 || n == 768 || n == 1536;
 }
 
-// Four-step split L = N/2 = L1 * L2 (step A: L2 FFTs of length L1, step C:
-// L1 FFTs of length L2) and the threads that share one line: T divides both
-// L1 and L2, so in both steps every thread has whole sub-FFTs.
+namespace {
+
+// Radices, lines per panel and threads per line of length N.
 template <int N>
 struct LineCfg {
     static constexpr int L = N / 2;
-    static constexpr int L1 = N == 64 ? 4 : N == 128 ? 8 : N == 256 ? 8 : N == 512 ? 16 : N == 1024 ? 16
-                            : (N == 192 || N == 384) ? 12 : N == 768 ? 24 : N == 1536 ? 48 : 32;
-    static constexpr int L2 = L / L1;
-    static constexpr int T = (N == 64 || N == 192 || N == 384) ? 4 : (N == 128 || N == 256 || N == 768) ? 8
-                           : (N == 512 || N == 1024 || N == 1536) ? 16 : 32;
-    static constexpr int JA = L2 / T;  // step-A sub-FFTs per thread
-    static constexpr int JC = L1 / T;  // step-C sub-FFTs per thread
-    static constexpr int LPW = 32 / T;  // lines per warp
-    static constexpr int NW = 8;  // warps per CTA
-    static constexpr int THREADS = 32 * NW;
-    static constexpr int LPR = NW * LPW;  // lines per round
-    // Rows per panel.  For T < 16 a half-warp holds several lines; they sit T
-    // rows apart (rows 32 b + w + T sub of a 32-row block, w < T), which with a
-    // row pitch of 2 mod 32 floats puts them 2T banks apart.  At least 8 rows,
-    // so that the transposed store writes whole 32-byte sectors (4096-point
-    // lines with 4-row panels wrote half sectors: 4 x 4096^2 forward 0.135 ->
-    // 0.203 of HBM with 8 rows, the same eight warps per SM).
-    static constexpr int PR = T < 16 ? (T == 4 ? 64 : 32) : (N <= 1536 ? 16 : 8);
-    static constexpr int ROUNDS = PR / LPR;
-    // With L2 >= 16 both FFT steps run in place in the line buffer: step A's
-    // results are held in registers across a warp barrier and written back
-    // with a 16-periodic XOR swizzle that keeps step C conflict-free, so no
-    // per-line scratch is needed.  Shorter lines use a padded scratch.
-    static constexpr bool INPLACE = L2 >= 16;
-    static constexpr int A_FLOATS = INPLACE ? N : 2 * L1 * (L2 + 1);  // step-A output
-    static constexpr int pitch(int need, int mod)
-    {
-        int p = need;
-        while (p % 32 != mod) ++p;
-        return p;
-    }
-    // line pitch: room for the step-A output of the inverse; 2 mod 32 floats so
-    // that the transposed store (16 rows x 2 columns per warp) is conflict-free
-    static constexpr int PP = pitch(A_FLOATS > N ? A_FLOATS : N, 2);
-    // per-line scratch: the lines of one warp 2T banks apart
-    static constexpr int SCR = INPLACE ? 0 : pitch(A_FLOATS > N ? A_FLOATS : N, (2 * T) % 32);
-    static constexpr int SEG = PR < 16 ? PR : 16;  // rows per transposed-store segment (a multiple of 4)
-    static constexpr int TAB_F2 = 3 * L;           // L step-A twiddles, then L float4 split twiddles
-    static constexpr size_t SMEM = (size_t)PR * PP * 4 + (size_t)LPR * SCR * 4 + (size_t)TAB_F2 * 8;
-    static_assert(L1 * L2 == L && L1 % T == 0 && L2 % T == 0 && 32 % T == 0, "split");
-    static_assert(ROUNDS >= 1 && ROUNDS * LPR == PR, "panel");
-    static_assert(T >= 16 || PR % 32 == 0, "line spacing");
-    static_assert(JC * L2 <= 64, "registers held through the split");
-    static_assert(SEG % 4 == 0 && THREADS % (SEG / 4) == 0 && N % (THREADS / (SEG / 4)) == 0, "store mapping");
+    static constexpr int R1 = N == 64 ? 4 : N == 128 ? 8 : N == 192 ? 8 : N == 256 ? 16 : N == 384 ? 16
+                            : N == 512 ? 16 : N == 2048 ? 16 : N == 4096 ? 16 : 8;
+    static constexpr int R3 = N == 64 ? 8 : N == 128 ? 8 : N == 192 ? 12 : N == 256 ? 8 : N == 384 ? 12
+                            : N == 512 ? 16 : N == 4096 ? 16 : 8;
+    static constexpr int R2 = L / (R1 * R3);
+    static constexpr int M1 = L / R1;  // columns of the first step
+    static constexpr int C = L / R3;   // columns of the last step
+    static constexpr int G = N == 64 || N == 192 ? 2 : N <= 256 ? 4 : N <= 512 ? 8 : N == 768 ? 12
+                           : N == 1024 || N == 1536 ? 16 : N == 2048 ? 32 : 64;  // threads per line
+    static constexpr int PR = N <= 256 ? 32 : N <= 1536 ? 16 : 8;  // lines per panel
+    static constexpr int THREADS = PR * G;
+    // resident CTAs per SM the registers are held to: as many as shared memory
+    // and spill-free code allow (one more measured slower from 384 points on,
+    // 1024 points forward 0.378 -> 0.349 of HBM)
+    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? 5 : N == 384 ? 4 : N == 512 ? 4
+                            : N == 768 ? 3 : N == 1024 ? 2 : N == 1536 ? 2 : N == 2048 ? 2 : 1;
+    static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
+    static constexpr int U1 = R1 * (M1 / 2);                // twiddle entries of the first step
+    static constexpr int U2 = R2 > 1 ? R2 * (R3 / 2) : 0;   // and of the middle step
+    static constexpr int US = L / 2 + L / 4;                // float4 entries of the split (L/2 slots of 24 bytes)
+    // float4 entries staged in shared memory (the split's read through L1
+    // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
+    static constexpr int TAB = U1 + U2 + US;
+    static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)TAB * 16 + 16;
+    static_assert(R1 * R2 * R3 == L && R1 % 2 == 0 && R3 % 2 == 0 && M1 % 2 == 0 && C % 2 == 0, "split");
+    static_assert(R2 == 1 || R2 % 2 == 0, "split");
+    static_assert(THREADS % 32 == 0 && PR <= 32 && PR % 4 == 0, "lanes");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// Panel row of line `sub` of warp-slot `slot` (slot = round * NW + warp).
-template <int N>
-__device__ __forceinline__ int line_row(int slot, int sub)
-{
-    using C = LineCfg<N>;
-    if constexpr (C::T < 16) return 32 * (slot / C::T) + (slot % C::T) + C::T * sub;
-    else return slot * C::LPW + sub;
-}
-
-size_t lines_table_elems(int n) { return (size_t)3 * (n / 2); }
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
-{
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-
-__device__ __forceinline__ float2 cmulc(float2 a, float2 b)  // a * conj(b)
-{
-    return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
-}
-
-// Step A for this thread: for m2 = t + T j, the length-L1 FFT of
-// src[L2 m1 + m2] (m1 < L1) times exp(-2 pi i m2 k1 / L), to A[k1][m2].
-template <int N>
-__device__ __forceinline__ void four_step_a(const float2 *src, float2 *A, const float2 *ta, int t)
-{
-    using C = LineCfg<N>;
-#pragma unroll
-    for (int j = 0; j < C::JA; ++j) {
-        const int m2 = t + C::T * j;
-        float re[C::L1], im[C::L1];
-#pragma unroll
-        for (int m1 = 0; m1 < C::L1; ++m1) {
-            const float2 v = src[C::L2 * m1 + m2];
-            re[m1] = v.x;
-            im[m1] = v.y;
-        }
-        FFT<C::L1>::run(re, im);
-        A[m2] = make_float2(re[0], im[0]);
-#pragma unroll
-        for (int k1 = 1; k1 < C::L1; ++k1)
-            A[k1 * (C::L2 + 1) + m2] = cmul(make_float2(re[k1], im[k1]), ta[k1 * C::L2 + m2]);
-    }
-}
-
-// Step C for this thread: for k1 = t + T j, the length-L2 FFT of A[k1][*];
-// Z_{k1 + L1 k2} lands in zr[j][k2], zi[j][k2].
-template <int N>
-__device__ __forceinline__ void four_step_c(const float2 *A, int t, float (&zr)[LineCfg<N>::JC][LineCfg<N>::L2],
-                                            float (&zi)[LineCfg<N>::JC][LineCfg<N>::L2])
-{
-    using C = LineCfg<N>;
-#pragma unroll
-    for (int j = 0; j < C::JC; ++j) {
-        const int k1 = t + C::T * j;
-#pragma unroll
-        for (int m2 = 0; m2 < C::L2; ++m2) {
-            const float2 v = A[k1 * (C::L2 + 1) + m2];
-            zr[j][m2] = v.x;
-            zi[j][m2] = v.y;
-        }
-        FFT<C::L2>::run(zr[j], zi[j]);
-    }
-}
-
-// In-place variants (L2 >= 16).  A[k1][m2] sits at k1 L2 + (m2 XOR (k1 mod 16)).
-template <int N>
-__device__ __forceinline__ void four_step_a_inplace(float2 *buf, const float2 *ta, int t)
-{
-    using C = LineCfg<N>;
-    float hr[C::JA][C::L1], hi[C::JA][C::L1];
-#pragma unroll
-    for (int j = 0; j < C::JA; ++j) {
-        const int m2 = t + C::T * j;
-#pragma unroll
-        for (int m1 = 0; m1 < C::L1; ++m1) {
-            const float2 v = buf[C::L2 * m1 + m2];
-            hr[j][m1] = v.x;
-            hi[j][m1] = v.y;
-        }
-        FFT<C::L1>::run(hr[j], hi[j]);
-#pragma unroll
-        for (int k1 = 1; k1 < C::L1; ++k1) {
-            const float2 w = cmul(make_float2(hr[j][k1], hi[j][k1]), ta[k1 * C::L2 + m2]);
-            hr[j][k1] = w.x;
-            hi[j][k1] = w.y;
-        }
-    }
-    __syncwarp();  // every read of the line done before A overwrites it
-#pragma unroll
-    for (int j = 0; j < C::JA; ++j) {
-        const int m2 = t + C::T * j;
-#pragma unroll
-        for (int k1 = 0; k1 < C::L1; ++k1) buf[k1 * C::L2 + (m2 ^ (k1 & 15))] = make_float2(hr[j][k1], hi[j][k1]);
-    }
-    __syncwarp();
-}
-
-template <int N>
-__device__ __forceinline__ void four_step_c_inplace(const float2 *buf, int t,
-                                                    float (&zr)[LineCfg<N>::JC][LineCfg<N>::L2],
-                                                    float (&zi)[LineCfg<N>::JC][LineCfg<N>::L2])
-{
-    using C = LineCfg<N>;
-#pragma unroll
-    for (int j = 0; j < C::JC; ++j) {
-        const int k1 = t + C::T * j;
-        const float2 *row = buf + k1 * C::L2;
-        const int x = k1 & 15;
-#pragma unroll
-        for (int m2 = 0; m2 < C::L2; ++m2) {
-            const float2 v = row[(m2 & ~15) + ((m2 & 15) ^ x)];
-            zr[j][m2] = v.x;
-            zi[j][m2] = v.y;
-        }
-        FFT<C::L2>::run(zr[j], zi[j]);
-    }
-    __syncwarp();  // every read of A done before the line is overwritten
-}
-
-// Forward DCT-II of one line.  On entry `line` holds z (Makhoul order, as
-// float2); on exit y_k * s_k in natural order.  Z_k and its split partner
-// Z_{L-k} sit in registers of threads t and T - t of the line (the same
-// warp), so the partner comes by shuffle.
-// With FOLD the table's exp(-i pi k / (2N)) carries the factor s_1 / 2
-// (folded in when the table is staged), saving the scalings below.
-template <int N, bool FOLD = false>
-__device__ __forceinline__ void line_forward(float *line, float *scr, const float2 *ta, const float4 *ts, int t,
-                                             int lane, AxisScale s)
-{
-    using C = LineCfg<N>;
-    float2 *z = reinterpret_cast<float2 *>(line);
-    float zr[C::JC][C::L2], zi[C::JC][C::L2];
-    if constexpr (C::INPLACE) {
-        four_step_a_inplace<N>(z, ta, t);
-        four_step_c_inplace<N>(z, t, zr, zi);
-    } else {
-        float2 *A = reinterpret_cast<float2 *>(scr);
-        four_step_a<N>(z, A, ta, t);
-        __syncwarp();
-        four_step_c<N>(A, t, zr, zi);
-    }
-    // the line buffer is free (its last reader passed a warp barrier).
-    // The outputs k and L-k both come from Z_k and Z_{L-k} (the latter's E and O
-    // are the former's with the imaginary parts negated), so one thread takes
-    // both: k runs over this thread's slots with k2 < L2/2 (k < L/2); thread 0
-    // also takes k = L/2, its own mirror.
-    const int src = lane - t + (C::T - t) % C::T;
-    // y_k and y_{N-k} of one index from its E and O and table entry
-    auto put = [&](int k, float2 E, float2 O, const float4 &w) {
-        const float2 P = cmul(make_float2(w.x, w.y), O);
-        const float2 WV = cmul(make_float2(w.z, w.w), make_float2(E.x + P.x, E.y + P.y));
-        if constexpr (FOLD) {
-            // the table's second factor carries s_1 / 2 (E and O are 2E, 2O)
-            line[k] = WV.x;
-            line[N - k] = -WV.y;
-        } else {
-            line[k] = WV.x * s.s1;
-            line[N - k] = -WV.y * s.s1;
-        }
-    };
-    // E, O of index k from Z_k = (ar, ai) and its partner Z_{L-k} = (cr, ci)
-    auto eo = [&](float ar, float ai, float cr, float ci, float2 &E, float2 &O) {
-        if constexpr (FOLD) {
-            E = make_float2(ar + cr, ai - ci);
-            O = make_float2(ai + ci, cr - ar);
-        } else {
-            E = make_float2(0.5f * (ar + cr), 0.5f * (ai - ci));
-            O = make_float2(0.5f * (ai + ci), 0.5f * (cr - ar));
-        }
-    };
-#pragma unroll
-    for (int j = 0; j < C::JC; ++j) {
-#pragma unroll
-        for (int k2 = 0; k2 < C::L2 / 2; ++k2) {
-            // partner Z_{L-k}: thread T - t, slot (JC - 1 - j, L2 - 1 - k2); for
-            // t = 0 the partner is this thread's own (JC - j) % JC or, for j = 0,
-            // slot (0, (L2 - k2) % L2)
-            float cr = __shfl_sync(0xffffffffu, zr[C::JC - 1 - j][C::L2 - 1 - k2], src);
-            float ci = __shfl_sync(0xffffffffu, zi[C::JC - 1 - j][C::L2 - 1 - k2], src);
-            constexpr int j0 = 0;
-            if (t == 0) {
-                if (j == 0) {
-                    cr = zr[j0][(C::L2 - k2) % C::L2];
-                    ci = zi[j0][(C::L2 - k2) % C::L2];
-                } else {
-                    cr = zr[(C::JC - j) % C::JC][C::L2 - 1 - k2];
-                    ci = zi[(C::JC - j) % C::JC][C::L2 - 1 - k2];
-                }
-            }
-            const int k = t + C::T * j + C::L1 * k2;
-            const float ar = zr[j][k2], ai = zi[j][k2];
-            if (k == 0) {
-                line[0] = (ar + ai) * s.s0;
-                line[C::L] = (ar - ai) * 0.70710678118654752f * s.s1;
-                // k = L/2: thread 0, slot (0, L2/2), partnered with itself
-                const float hr = zr[j0][C::L2 / 2], hi = zi[j0][C::L2 / 2];
-                float2 E, O;
-                eo(hr, hi, hr, hi, E, O);
-                put(C::L / 2, E, O, ts[C::L / 2]);
-            } else {
-                float2 E, O;
-                eo(ar, ai, cr, ci, E, O);
-                put(k, E, O, ts[k]);
-                put(C::L - k, make_float2(E.x, -E.y), make_float2(O.x, -O.y), ts[C::L - k]);
-            }
-        }
-    }
-    __syncwarp();
-}
-template <int N, bool FOLD = false>
-__device__ __forceinline__ void line_inverse(float *line, float *scr, const float2 *ta, const float4 *ts, int t,
-                                             AxisScale s)
-{
-    using C = LineCfg<N>;
-    // conj(Z) in natural order: a scratch buffer, or (in place) registers
-    // written over the line once every y has been read
-    float2 *Zc = reinterpret_cast<float2 *>(C::INPLACE ? line : scr);
-    float qr[C::JC][C::L2], qi[C::JC][C::L2];
-    // y -> conj(Z): Z_k needs y_k, y_{N-k}, y_{L-k}, y_{L+k} and the table
-    // entries k and L-k, and Z_{L-k} needs the same, so one thread takes both:
-    // k runs over this thread's slots with k2 < L2/2 (k < L/2), and the second
-    // half of the slot array holds Z_{L-k} (for k = 0: Z_{L/2}, its own mirror)
-    const float sy = FOLD ? 1.0f : s.s1;  // with FOLD the table carries s_1 / 2
-    const float hf = FOLD ? 1.0f : 0.5f;
-#pragma unroll
-    for (int j = 0; j < C::JC; ++j) {
-#pragma unroll
-        for (int k2 = 0; k2 < C::L2 / 2; ++k2) {
-            const int k = t + C::T * j + C::L1 * k2;
-            float2 za, zb;  // conj Z_k and conj Z_{L-k}
-            if (k == 0) {
-                const float v0 = 2.0f * line[0] * s.s0;  // factor 2 carries 1/L
-                const float vl = 1.41421356237309505f * line[C::L] * s.s1;
-                za = make_float2(0.5f * (v0 + vl), -0.5f * (v0 - vl));
-                constexpr int H = C::L / 2;
-                const float yh = line[H] * sy, ynh = line[N - H] * sy;
-                const float4 w = ts[H];
-                const float2 V = cmulc(make_float2(yh, -ynh), make_float2(w.z, w.w));
-                const float2 E = make_float2(hf * (V.x + V.x), hf * (V.y - V.y));
-                const float2 D = make_float2(hf * (V.x - V.x), hf * (V.y + V.y));
-                const float2 O = cmulc(D, make_float2(w.x, w.y));
-                zb = make_float2(E.x - O.y, -(E.y + O.x));
-            } else {
-                const float yk = line[k] * sy, ynk = line[N - k] * sy;
-                const float ylk = line[C::L - k] * sy, ylpk = line[C::L + k] * sy;
-                const float4 w = ts[k], wl = ts[C::L - k];
-                // V_k = conj(W_k) (y_k - i y_{N-k}), V_{L-k} likewise
-                const float2 Vk = cmulc(make_float2(yk, -ynk), make_float2(w.z, w.w));
-                const float2 Vl = cmulc(make_float2(ylk, -ylpk), make_float2(wl.z, wl.w));
-                const float2 E = make_float2(hf * (Vk.x + Vl.x), hf * (Vk.y - Vl.y));
-                const float2 D = make_float2(hf * (Vk.x - Vl.x), hf * (Vk.y + Vl.y));
-                const float2 O = cmulc(D, make_float2(w.x, w.y));  // / exp(-2 pi i k / N)
-                za = make_float2(E.x - O.y, -(E.y + O.x));         // conj(E + i O)
-                // for L-k the two V swap: E -> (E.x, -E.y), D -> (-D.x, D.y)
-                const float2 Ol = cmulc(make_float2(-D.x, D.y), make_float2(wl.x, wl.y));
-                zb = make_float2(E.x - Ol.y, -(Ol.x - E.y));
-            }
-            const int km = k == 0 ? C::L / 2 : C::L - k;
-            if constexpr (C::INPLACE) {
-                qr[j][k2] = za.x;
-                qi[j][k2] = za.y;
-                qr[j][k2 + C::L2 / 2] = zb.x;
-                qi[j][k2 + C::L2 / 2] = zb.y;
-            } else {
-                Zc[k] = za;
-                Zc[km] = zb;
-            }
-        }
-    }
-    __syncwarp();  // every read of y done before the line is overwritten
-    float rr[C::JC][C::L2], ri[C::JC][C::L2];
-    if constexpr (C::INPLACE) {
-#pragma unroll
-        for (int j = 0; j < C::JC; ++j) {
-#pragma unroll
-            for (int k2 = 0; k2 < C::L2 / 2; ++k2) {
-                const int k = t + C::T * j + C::L1 * k2;
-                Zc[k] = make_float2(qr[j][k2], qi[j][k2]);
-                Zc[k == 0 ? C::L / 2 : C::L - k] = make_float2(qr[j][k2 + C::L2 / 2], qi[j][k2 + C::L2 / 2]);
-            }
-        }
-        __syncwarp();
-        four_step_a_inplace<N>(Zc, ta, t);
-        four_step_c_inplace<N>(Zc, t, rr, ri);
-    } else {
-        float2 *A = reinterpret_cast<float2 *>(line);
-        four_step_a<N>(Zc, A, ta, t);
-        __syncwarp();
-        four_step_c<N>(A, t, rr, ri);
-    }
-    __syncwarp();  // all of A read before x overwrites the line
-    // z_m = conj(result): v_{2m} = Re z_m, v_{2m+1} = -Im z_m, and x_{2i} = v_i
-    // (i < L), x_{2i+1} = v_{N-1-i}.  For m < L/2 the four outputs x_{4m} ..
-    // x_{4m+3} are v_{2m}, v_{2m'+1}, v_{2m+1}, v_{2m'} with m' = L-1-m, whose
-    // z sits in thread T-1-t at slot (JC-1-j, L2-1-k2) (k2 < L2/2 exactly when
-    // m < L/2): the partner's values arrive by shuffle and the four outputs
-    // leave as two 8-byte stores, taken in opposite order by the two halves of
-    // each 16-lane group so that one store instruction covers distinct banks.
-    const int lane = (int)(threadIdx.x & 31);
-    const int src = lane - t + (C::T - 1 - t);
-    const int swap = (lane >> 3) & 1;
-    float2 *x2 = reinterpret_cast<float2 *>(line);
-#pragma unroll
-    for (int j = 0; j < C::JC; ++j) {
-#pragma unroll
-        for (int k2 = 0; k2 < C::L2 / 2; ++k2) {
-            // each lane sends its slot (JC-1-j, L2-1-k2) and receives the partner's
-            const float pe = __shfl_sync(0xffffffffu, rr[C::JC - 1 - j][C::L2 - 1 - k2], src);
-            const float po = __shfl_sync(0xffffffffu, ri[C::JC - 1 - j][C::L2 - 1 - k2], src);
-            const int m = t + C::T * j + C::L1 * k2;
-            const float2 lo = make_float2(rr[j][k2], -po);  // x_{4m}, x_{4m+1}
-            const float2 hi = make_float2(-ri[j][k2], pe);  // x_{4m+2}, x_{4m+3}
-            x2[2 * m + swap] = swap ? hi : lo;
-            x2[2 * m + 1 - swap] = swap ? lo : hi;
-        }
-    }
-    __syncwarp();
-}
+// rows -> transposed (forward), transposed -> rows (inverse), and forward,
+// diagonal, adjoint in one pass: rows -> rows or transposed -> transposed
+enum Mode { MODE_F = 0, MODE_I = 1, MODE_RR = 2, MODE_CC = 3 };
 
 struct LinesParams {
     const float *src;
     float *dst;
-    int rows;            // rows per array (lines per array)
-    long long nrows;     // total rows
+    int rows;                            // lines per array
     int npanels;
-    AxisScale sc;        // forward: output scales; inverse: input scales; round trip: E^2
+    AxisScale sc;                        // forward: output scales, inverse: input scales (both when both run)
     const long long *src_off, *dst_off;  // indexed arrays (element offsets), or null
-    const float2 *tw;    // the plan's tables for N (lines_gen_table), generated in FP64
-    int reverse;         // take panels last to first (the second pass reads the
-                         // intermediate the first pass wrote last, still in L2, first)
-    const float *lam;    // or null: every output element (k, r) of array b is
-                         // multiplied by lam[k * rows + r] as it is stored
+    const float4 *tw;                    // the plan's table for N (lines_gen_table)
+    const float *lam;                    // MODE_RR, or null: output k of line r times lam[k * rows + r]
+    unsigned int *status;
+    int reverse;                         // take panels last to first (the pass then starts with
+                                         // what the previous pass wrote last, still in L2)
 };
 
-template <int N, int DIR>
-__global__ void __launch_bounds__(LineCfg<N>::THREADS) k_lines(const LinesParams p)
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// (ar + i ai) exp(-2 pi i j / R) on both halves
+template <int R>
+__device__ __forceinline__ void rotr(float2 ar, float2 ai, int j, float2 &rr, float2 &ri)
+{
+    if constexpr (R % 3 == 0) rot3(ar, ai, j, R, rr, ri);
+    else rot(ar, ai, 2 * j, R, rr, ri);
+}
+
+// Second half of a decimation-in-frequency FFT of R points: u_j = a_j +
+// a_{j+R/2} and v_j = a_j - a_{j+R/2} give the even and odd outputs.
+template <int R>
+__device__ __forceinline__ void fft_from_uv(float2 (&ur)[R / 2], float2 (&ui)[R / 2], float2 (&vr)[R / 2],
+                                            float2 (&vi)[R / 2], float2 (&dr)[R], float2 (&di)[R])
+{
+#pragma unroll
+    for (int j = 1; j < R / 2; ++j) {
+        float2 a, b;
+        rotr<R>(vr[j], vi[j], j, a, b);
+        vr[j] = a;
+        vi[j] = b;
+    }
+    FFT<R / 2, float2>::run(ur, ui);
+    FFT<R / 2, float2>::run(vr, vi);
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+        dr[2 * k] = ur[k]; di[2 * k] = ui[k];
+        dr[2 * k + 1] = vr[k]; di[2 * k + 1] = vi[k];
+    }
+}
+
+// Its transpose up to the last sums and differences (called with the real and
+// imaginary arrays exchanged: the conjugate FFT).
+template <int R>
+__device__ __forceinline__ void uv_from_fft(const float2 (&dr)[R], const float2 (&di)[R], float2 (&ur)[R / 2],
+                                            float2 (&ui)[R / 2], float2 (&vr)[R / 2], float2 (&vi)[R / 2])
+{
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+        ur[k] = dr[2 * k]; ui[k] = di[2 * k];
+        vr[k] = dr[2 * k + 1]; vi[k] = di[2 * k + 1];
+    }
+    FFT<R / 2, float2>::run(ur, ui);
+    FFT<R / 2, float2>::run(vr, vi);
+#pragma unroll
+    for (int j = 1; j < R / 2; ++j) {
+        float2 a, b;
+        rotr<R>(vr[j], vi[j], j, a, b);
+        vr[j] = a;
+        vi[j] = b;
+    }
+}
+
+// ------------------------------------------------------- first and middle steps
+// The couple of columns cc and MC-1-cc: x holds units cc + MC j, y units
+// MC-1-cc + MC j (j < R/2).  Results k: into x (k < R/2) and y, the slots
+// they came from, times the twiddles tw[k * (MC/2)].
+template <int R, int MC>
+__device__ __forceinline__ void step_forward(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2], dr[R], di[R];
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const float4 a = x[j], b = y[R / 2 - 1 - j];
+        ur[j] = make_float2(a.x + b.w, a.y + b.z);
+        ui[j] = make_float2(a.z + b.y, a.w + b.x);
+        vr[j] = make_float2(a.x - b.w, a.y - b.z);
+        vi[j] = make_float2(a.z - b.y, a.w - b.x);
+    }
+    fft_from_uv<R>(ur, ui, vr, vi, dr, di);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        float2 re = dr[k], im = di[k];
+        if (k > 0) {
+            const float4 t = tw[k * (MC / 2)];
+            const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
+            re = __ffma2_rn(di[k], s, __fmul2_rn(dr[k], c));
+            im = __ffma2_rn(neg2(dr[k]), s, __fmul2_rn(di[k], c));
+        }
+        const float4 o = make_float4(re.x, re.y, im.x, im.y);
+        if (k < R / 2) x[k] = o;
+        else y[k - R / 2] = o;
+    }
+}
+
+template <int R, int MC>
+__device__ __forceinline__ void step_adjoint(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
+{
+    float2 dr[R], di[R], ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const float4 o = k < R / 2 ? x[k < R / 2 ? k : 0] : y[k < R / 2 ? 0 : k - R / 2];
+        const float2 re = make_float2(o.x, o.y), im = make_float2(o.z, o.w);
+        dr[k] = re;
+        di[k] = im;
+        if (k > 0) {
+            const float4 t = tw[k * (MC / 2)];
+            const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
+            dr[k] = __ffma2_rn(neg2(im), s, __fmul2_rn(re, c));
+            di[k] = __ffma2_rn(re, s, __fmul2_rn(im, c));
+        }
+    }
+    uv_from_fft<R>(di, dr, ui, ur, vi, vr);
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        x[j] = make_float4(ur[j].x + vr[j].x, ur[j].y + vr[j].y, ui[j].x + vi[j].x, ui[j].y + vi[j].y);
+        y[R / 2 - 1 - j] = make_float4(ui[j].y - vi[j].y, ui[j].x - vi[j].x, ur[j].y - vr[j].y, ur[j].x - vr[j].x);
+    }
+}
+
+// ---------------------------------------------------------------- last step
+// Columns c (units x, index m) and its partner C-c (units w): D_k's halves
+// become Z_{c + C k} and conj Z_{L - c - C k}.
+template <int R>
+__device__ __forceinline__ void last_forward(const float4 (&x)[R / 2], const float4 (&w)[R / 2], float2 (&dr)[R],
+                                             float2 (&di)[R])
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const float4 a = x[j], b = x[R / 2 - 1 - j], p = w[j], q = w[R / 2 - 1 - j];
+        ur[j] = make_float2(a.x + b.w, p.x + q.w);
+        ui[j] = make_float2(a.z + b.y, -p.z - q.y);
+        vr[j] = make_float2(a.x - b.w, p.x - q.w);
+        vi[j] = make_float2(a.z - b.y, q.y - p.z);
+    }
+    fft_from_uv<R>(ur, ui, vr, vi, dr, di);
+}
+
+template <int R>
+__device__ __forceinline__ void last_adjoint(float4 (&x)[R / 2], float4 (&w)[R / 2], const float2 (&dr)[R],
+                                             const float2 (&di)[R])
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+    uv_from_fft<R>(di, dr, ui, ur, vi, vr);
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const int m = R / 2 - 1 - j;
+        x[j].x = ur[j].x + vr[j].x;
+        x[m].w = ur[j].x - vr[j].x;
+        x[j].z = ui[j].x + vi[j].x;
+        x[m].y = ui[j].x - vi[j].x;
+        w[j].x = ur[j].y + vr[j].y;
+        w[m].w = ur[j].y - vr[j].y;
+        w[j].z = -ui[j].y - vi[j].y;
+        w[m].y = vi[j].y - ui[j].y;
+    }
+}
+
+// ---------------------------------------------------------------- the split
+// Four outputs from Z_k = (ar, ai) and conj Z_{L-k} = (br, bi): a = (y_k,
+// y_{L-k}), b = (y_{N-k}, y_{L+k}).  The table holds exp(-2 pi i k/N) = t.x -
+// i t.y and, times s_1 / 2, the pairs over (k, L-k) of Re W (t.z, t.w) and
+// -Im W (nwi).
+__device__ __forceinline__ void split_one(float ar, float ai, float br, float bi, const float4 t, const float2 nwi,
+                                          float2 &a, float2 &b)
+{
+    const float er = ar + br, ei = ai + bi, orr = ai - bi, oi = br - ar;
+    const float pr = fmaf(orr, t.x, oi * t.y), pi = fmaf(oi, t.x, -orr * t.y);
+    const float2 vr = make_float2(er + pr, er - pr), vi = make_float2(ei + pi, pi - ei);
+    const float2 wr = make_float2(t.z, t.w);
+    a = __ffma2_rn(vi, nwi, __fmul2_rn(vr, wr));
+    b = __ffma2_rn(neg2(vi), wr, __fmul2_rn(vr, nwi));
+}
+
+__device__ __forceinline__ void split_one_adjoint(float2 a, float2 b, const float4 t, const float2 nwi, float &ar,
+                                                  float &ai, float &br, float &bi)
+{
+    const float2 wr = make_float2(t.z, t.w);
+    const float2 vr = __ffma2_rn(b, nwi, __fmul2_rn(a, wr));
+    const float2 vi = __ffma2_rn(neg2(b), wr, __fmul2_rn(a, nwi));
+    const float er = vr.x + vr.y, pr = vr.x - vr.y, ei = vi.x - vi.y, pi = vi.x + vi.y;
+    const float orr = fmaf(pr, t.x, -pi * t.y), oi = fmaf(pr, t.y, pi * t.x);
+    ar = er - oi;
+    br = er + oi;
+    ai = ei + orr;
+    bi = ei - orr;
+}
+
+// The split's table by slot (k3 * (C/2) + c).
+struct SplitTable {
+    const float4 *ta;
+    const float2 *tb;
+    __device__ __forceinline__ float4 a(int i) const { return ta[i]; }
+    __device__ __forceinline__ float2 b(int i) const { return tb[i]; }
+};
+
+constexpr float kCos8 = 0.92387953251128675613f, kSin8 = 0.38268343236508977173f;  // of pi / 8
+constexpr float kRoot = 0.70710678118654752440f;
+
+// The outputs of couple c in slot order: slot k3 of c > 0 is k = c + C k3; of
+// c = 0, k = C k3 (k3 < R/2) and k = C/2 + C (k3 - R/2), with slot 0 holding
+// a = (y_0, y_L), b = (y_{L/2}, y_{3L/2}).  Column 0 pairs k3 with R - k3 in
+// its own half and column C/2 pairs k3 with R-1-k3, so each is one split.
+template <int R, int C>
+__device__ __forceinline__ void split_forward(int c, const float2 (&dr)[R], const float2 (&di)[R], SplitTable ts,
+                                              AxisScale s, float2 (&a)[R], float2 (&b)[R])
+{
+    if (c != 0) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            split_one(dr[k].x, di[k].x, dr[k].y, di[k].y, ts.a(k * (C / 2) + c), ts.b(k * (C / 2) + c), a[k], b[k]);
+    } else {
+        a[0] = make_float2((dr[0].x + di[0].x) * s.s0, (dr[0].x - di[0].x) * (kRoot * s.s1));
+        const float hr = dr[R / 2].x * s.s1, hi = di[R / 2].x * s.s1;
+        b[0] = make_float2(fmaf(hr, kCos8, -hi * kSin8), fmaf(hr, kSin8, hi * kCos8));
+#pragma unroll
+        for (int k = 1; k < R / 2; ++k)
+            split_one(dr[k].x, di[k].x, dr[R - k].x, -di[R - k].x, ts.a(k * (C / 2)), ts.b(k * (C / 2)), a[k], b[k]);
+#pragma unroll
+        for (int k = 0; k < R / 2; ++k)
+            split_one(dr[R - 1 - k].y, -di[R - 1 - k].y, dr[k].y, di[k].y, ts.a((R / 2 + k) * (C / 2)),
+                      ts.b((R / 2 + k) * (C / 2)), a[R / 2 + k], b[R / 2 + k]);
+    }
+}
+
+template <int R, int C>
+__device__ __forceinline__ void split_adjoint(int c, const float2 (&a)[R], const float2 (&b)[R], SplitTable ts,
+                                              AxisScale s, float2 (&dr)[R], float2 (&di)[R])
+{
+    if (c != 0) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            split_one_adjoint(a[k], b[k], ts.a(k * (C / 2) + c), ts.b(k * (C / 2) + c), dr[k].x, di[k].x, dr[k].y, di[k].y);
+    } else {
+        const float u = a[0].x * s.s0, v = a[0].y * (kRoot * s.s1);
+        dr[0].x = u + v;
+        di[0].x = u - v;
+        const float p = b[0].x * s.s1, q = b[0].y * s.s1;
+        dr[R / 2].x = fmaf(p, kCos8, q * kSin8);
+        di[R / 2].x = fmaf(q, kCos8, -p * kSin8);
+#pragma unroll
+        for (int k = 1; k < R / 2; ++k) {
+            float im;
+            split_one_adjoint(a[k], b[k], ts.a(k * (C / 2)), ts.b(k * (C / 2)), dr[k].x, di[k].x, dr[R - k].x, im);
+            di[R - k].x = -im;
+        }
+#pragma unroll
+        for (int k = 0; k < R / 2; ++k) {
+            float im;
+            split_one_adjoint(a[R / 2 + k], b[R / 2 + k], ts.a((R / 2 + k) * (C / 2)), ts.b((R / 2 + k) * (C / 2)), dr[R - 1 - k].y, im, dr[k].y,
+                              di[k].y);
+            di[R - 1 - k].y = -im;
+        }
+    }
+}
+
+// ------------------------------------------------------------ transposed side
+// visit(slot half, k): the output index of (a.x, a.y, b.x, b.y) of slot k3
+template <int N>
+struct SlotIndex {
+    using C = LineCfg<N>;
+    int lo, hi;   // first index of the lower and the upper half of the slots, minus C k3
+    bool zero;
+    __device__ __forceinline__ explicit SlotIndex(int c)
+        : lo(c), hi(c ? c : C::C / 2 - C::L / 2), zero(c == 0)
+    {
+    }
+    __device__ __forceinline__ int k(int k3) const { return C::C * k3 + (k3 < C::R3 / 2 ? lo : hi); }
+    __device__ __forceinline__ int ax(int k3) const { return k(k3); }
+    __device__ __forceinline__ int ay(int k3) const { return C::L - k(k3); }
+    __device__ __forceinline__ int bx(int k3) const { return (k3 == 0 && zero) ? C::L / 2 : N - k(k3); }
+    __device__ __forceinline__ int by(int k3) const { return (k3 == 0 && zero) ? 3 * C::L / 2 : C::L + k(k3); }
+};
+
+// Unit slot of first-step result k1: base and direction (k1 < R1/2 kept its
+// column's slots, the others the mirror's).
+template <int N>
+__device__ __forceinline__ int sub_base(int k1, int &sgn)
 {
     using C = LineCfg<N>;
-    extern __shared__ __align__(16) float lsm[];
-    float *panel = lsm;
-    float *scr_all = panel + C::PR * C::PP;  // per-line scratch (lines without the in-place steps)
-    float2 *ta = reinterpret_cast<float2 *>(scr_all + C::LPR * C::SCR);
-    const float4 *ts = reinterpret_cast<const float4 *>(ta + C::L);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int sub = lane / C::T, t = lane % C::T;
+    const bool e = k1 >= C::R1 / 2;
+    sgn = e ? -1 : 1;
+    return e ? C::M1 - 1 + C::M1 * (k1 - C::R1 / 2) : C::M1 * k1;
+}
 
-    pdl_launch_dependents();
-    pdl_wait_prerequisites();
-    // the plan's twiddle tables (FP64-generated): step A, then the split;
-    // forward and inverse fold s_1 / 2 into exp(-i pi k / (2N)) here
-    constexpr bool FOLD = DIR != DIR_RT;
-    const float fold = 0.5f * p.sc.s1;
-    for (int r = tid; r < C::TAB_F2; r += C::THREADS) {
-        float2 v = p.tw[r];
-        if (FOLD && r >= C::L && ((r - C::L) & 1)) v = make_float2(v.x * fold, v.y * fold);
-        ta[r] = v;
+template <int N, int MODE>
+__global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(const LinesParams p)
+{
+    using C = LineCfg<N>;
+    constexpr int R1 = C::R1, R2 = C::R2, R3 = C::R3, M1 = C::M1, CC = C::C, PR = C::PR, G = C::G;
+    constexpr bool ROWS_IN = MODE == MODE_F || MODE == MODE_RR;
+    constexpr bool ROWS_OUT = MODE == MODE_I || MODE == MODE_RR;
+    constexpr bool FWD = MODE != MODE_I, INV = MODE != MODE_F;
+    extern __shared__ __align__(128) float lsm[];
+    float4 *tab = reinterpret_cast<float4 *>(lsm + PR * C::PT);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(tab + C::TAB);
+    const float4 *t1 = tab, *t2 = tab + C::U1;
+    const SplitTable ts{t2 + C::U2, reinterpret_cast<const float2 *>(t2 + C::U2 + C::L / 2)};
+    const int tid = threadIdx.x, line = tid % PR, g = tid / PR;
+    float4 *row = reinterpret_cast<float4 *>(lsm + line * C::PT);
+
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
     }
+    pdl_launch_dependents();
+    // the tables are plan data, written before any transform was queued
+    for (int r = tid; r < C::TAB; r += C::THREADS) tab[r] = __ldg(p.tw + r);
+    pdl_wait_prerequisites();
     __syncthreads();
 
-    // The panel's 16-byte chunks, ITER per thread; for lines up to 2048 points
-    // the next panel's chunks are loaded into registers while the current
-    // panel is transformed, so the global-load latency overlaps the work.
-    constexpr int V4 = N / 4;
-    constexpr int ITER = C::PR * V4 / C::THREADS;
-    // (lines with a radix-3 stage hold 48 complex values through the split:
-    // only the 768-point forward keeps the prefetch, measured)
-    constexpr bool PREFETCH = N <= 2048 && (N % 3 != 0 || (N == 768 && DIR == DIR_FWD));
-    constexpr int NB = PREFETCH ? ITER : (ITER <= 8 ? ITER : (ITER % 8 == 0 ? 8 : (ITER % 6 == 0 ? 6 : 4)));
-    static_assert(ITER * C::THREADS == C::PR * V4 && ITER % NB == 0, "load batches");
-    auto panel_src = [&](int pn, long long &b, int &rr) -> const float4 * {
+    auto panel_at = [&](int pn, long long &b, int &r0) {
         if (p.reverse) pn = p.npanels - 1 - pn;
-        const long long r0 = (long long)pn * C::PR;  // first global row of the panel
-        b = r0 / p.rows;                             // its array (panels never straddle two)
-        rr = (int)(r0 - b * p.rows);
-        const float *srcb = p.src_off ? p.src + p.src_off[b] : p.src + b * (long long)N * p.rows;
-        return reinterpret_cast<const float4 *>(srcb + (long long)rr * N);
+        const long long r = (long long)pn * PR;
+        b = r / p.rows;  // panels never straddle two arrays
+        r0 = (int)(r - b * p.rows);
     };
-    // chunk u of this thread -> the panel row (Makhoul order for the forward)
-    auto put = [&](int i, const float4 v) {
-        const int l = i / V4, q = i - l * V4;
-        float2 *row = reinterpret_cast<float2 *>(panel + l * C::PP);
-        if constexpr (DIR == DIR_INV) {
-            row[2 * q] = make_float2(v.x, v.y);
-            row[2 * q + 1] = make_float2(v.z, v.w);
-        } else {
-            // Makhoul order: (v_{2q}, v_{2q+1}) = (x_{4q}, x_{4q+2}),
-            // (v_{N-2-2q}, v_{N-1-2q}) = (x_{4q+3}, x_{4q+1})
-            row[q] = make_float2(v.x, v.z);
-            row[N / 2 - 1 - q] = make_float2(v.w, v.y);
-        }
+    auto src_of = [&](long long b) { return p.src_off ? p.src + p.src_off[b] : p.src + b * (long long)N * p.rows; };
+    auto dst_of = [&](long long b) { return p.dst_off ? p.dst + p.dst_off[b] : p.dst + b * (long long)N * p.rows; };
+    // warp 0: one bulk copy per line of the panel
+    auto load_panel = [&](int pn) {
+        long long b;
+        int r0;
+        panel_at(pn, b, r0);
+        if (tid == 0) mbar_arrive_expect_tx(bar, PR * N * 4);
+        __syncwarp();
+        if (tid < PR) bulk_load(lsm + tid * C::PT, src_of(b) + (long long)(r0 + tid) * N, N * 4, bar);
     };
-    float4 pre[NB];
-    if constexpr (PREFETCH) {
-        if (blockIdx.x < (unsigned)p.npanels) {
-            long long b0;
-            int r00;
-            const float4 *src4 = panel_src(blockIdx.x, b0, r00);
-#pragma unroll
-            for (int u = 0; u < NB; ++u) pre[u] = __ldg(src4 + tid + u * C::THREADS);
-        }
-    }
+    if (ROWS_IN && tid < 32 && (int)blockIdx.x < p.npanels) load_panel(blockIdx.x);
 
+    uint32_t phase = 0;
     for (int pn = blockIdx.x; pn < p.npanels; pn += gridDim.x) {
         long long b;
-        int rr;
-        const float4 *src4 = panel_src(pn, b, rr);
-        // ---- the panel (rows of this array), coalesced 16-byte reads
-        if constexpr (PREFETCH) {
-#pragma unroll
-            for (int u = 0; u < NB; ++u) put(tid + u * C::THREADS, pre[u]);
-            __syncthreads();
-            const int nx = pn + (int)gridDim.x;
-            if (nx < p.npanels) {
-                long long b1;
-                int r1;
-                const float4 *n4 = panel_src(nx, b1, r1);
-#pragma unroll
-                for (int u = 0; u < NB; ++u) pre[u] = __ldg(n4 + tid + u * C::THREADS);
-            }
-        } else {
-#pragma unroll 1
-            for (int i0 = 0; i0 < ITER; i0 += NB) {
-#pragma unroll
-                for (int u = 0; u < NB; ++u) pre[u] = __ldg(src4 + tid + (i0 + u) * C::THREADS);
-#pragma unroll
-                for (int u = 0; u < NB; ++u) put(tid + (i0 + u) * C::THREADS, pre[u]);
-            }
-            __syncthreads();
+        int r0;
+        panel_at(pn, b, r0);
+        const int next = pn + (int)gridDim.x;
+        bool ok = true;
+        if constexpr (ROWS_IN) {
+            ok = mbar_wait_bounded(bar, phase);
+            phase ^= 1;
         }
-        // ---- transform every line of the panel
+        if constexpr (FWD) {
+            const float *src = MODE == MODE_CC ? src_of(b) + r0 + line : nullptr;
+            // ---- first step
 #pragma unroll 1
-        for (int rd = 0; rd < C::ROUNDS; ++rd) {
-            float *line = panel + line_row<N>(rd * C::NW + warp, sub) * C::PP;
-            float *scr = scr_all + (warp * C::LPW + sub) * C::SCR;
-            if constexpr (DIR == DIR_FWD) {
-                line_forward<N, true>(line, scr, ta, ts, t, lane, p.sc);
-            } else if constexpr (DIR == DIR_INV) {
-                line_inverse<N, true>(line, scr, ta, ts, t, p.sc);
+            for (int cc = g; cc < M1 / 2; cc += G) {
+                float4 x[R1 / 2], y[R1 / 2];
+#pragma unroll
+                for (int j = 0; j < R1 / 2; ++j) {
+                    if constexpr (MODE == MODE_CC) {
+                        const float *q = src + (long long)(4 * (cc + M1 * j)) * p.rows;
+                        x[j] = make_float4(q[0], q[p.rows], q[2 * p.rows], q[3 * p.rows]);
+                        q = src + (long long)(4 * (M1 - 1 - cc + M1 * j)) * p.rows;
+                        y[j] = make_float4(q[0], q[p.rows], q[2 * p.rows], q[3 * p.rows]);
+                    } else {
+                        x[j] = row[cc + M1 * j];
+                        y[j] = row[M1 - 1 - cc + M1 * j];
+                    }
+                }
+                step_forward<R1, M1>(x, y, t1 + cc);
+#pragma unroll
+                for (int j = 0; j < R1 / 2; ++j) {
+                    row[cc + M1 * j] = x[j];
+                    row[M1 - 1 - cc + M1 * j] = y[j];
+                }
+            }
+            if constexpr (ROWS_IN) {
+                if (!__syncthreads_and(ok)) {
+                    // the load did not land in time: record it, give the copies
+                    // one more bounded wait, and stop
+                    if (tid == 0) {
+                        record_timeout(p.status);
+                        mbar_wait_bounded(bar, phase ^ 1);
+                    }
+                    return;
+                }
             } else {
-                // round trip: forward core, E^2 correction, adjoint core
-                const AxisScale one = {1.0f, 1.0f};
-                line_forward<N>(line, scr, ta, ts, t, lane, p.sc);
-                line_inverse<N>(line, scr, ta, ts, t, one);
+                __syncthreads();
+            }
+            // ---- middle step
+            if constexpr (R2 > 1) {
+#pragma unroll 1
+                for (int q = g; q < R1 * R3 / 2; q += G) {
+                    int sgn;
+                    const int k1 = q / (R3 / 2), m3 = q % (R3 / 2);
+                    const int qb = sub_base<N>(k1, sgn);
+                    float4 *px = row + qb + sgn * m3, *py = row + qb + sgn * (R3 - 1 - m3);
+                    float4 x[R2 / 2], y[R2 / 2];
+#pragma unroll
+                    for (int j = 0; j < R2 / 2; ++j) {
+                        x[j] = px[sgn * R3 * j];
+                        y[j] = py[sgn * R3 * j];
+                    }
+                    step_forward<R2, R3>(x, y, t2 + m3);
+#pragma unroll
+                    for (int j = 0; j < R2 / 2; ++j) {
+                        px[sgn * R3 * j] = x[j];
+                        py[sgn * R3 * j] = y[j];
+                    }
+                }
+                __syncthreads();
             }
         }
-        __syncthreads();
-        // ---- transposed store: dst[b][k][r] with rows r0.. (same array b).
-        // A thread writes 4 consecutive rows of one column k as one 16-byte
-        // store; a warp instruction covers SEG rows x (128 / SEG) columns, and
-        // with a row pitch of 2 mod 32 floats its shared-memory reads touch
-        // all 32 banks.
+        // ---- last step, split, and the transposed side
         {
-            float *dstb = p.dst_off ? p.dst + p.dst_off[b] : p.dst + b * (long long)N * p.rows;
-            constexpr int SQ = C::SEG / 4;          // row quads per segment
-            constexpr int KPI = C::THREADS / SQ;    // columns per step
-            const int qd = tid % SQ, kk = tid / SQ;
-            const long long e0 = (long long)kk * p.rows + rr + 4 * qd;  // element offset in the array
-            float *g = dstb + e0;
-            const long long gstep = (long long)KPI * p.rows;
+            constexpr int ROUNDS = (CC / 2 + G - 1) / G;
+            const float *src = MODE == MODE_I ? src_of(b) + r0 + line : nullptr;
+            float *dst = MODE == MODE_F ? dst_of(b) + r0 + line : nullptr;
+            const float *lam = MODE == MODE_RR && p.lam ? p.lam + r0 + line : nullptr;
+            const long long ld = p.rows;
 #pragma unroll 1
-            for (int lb = 0; lb < C::PR; lb += C::SEG) {
-                const float *sp = panel + (lb + 4 * qd) * C::PP + kk;
-                float *gp = g + lb;
-                if (p.lam) {
-                    // the spectrum times the diagonal (Prop. 1), four rows of one column
-                    const float *lp = p.lam + e0 + lb;
-#pragma unroll 4
-                    for (int k = kk; k < N; k += KPI) {
-                        const float4 l = __ldg(reinterpret_cast<const float4 *>(lp));
-                        *reinterpret_cast<float4 *>(gp) =
-                            make_float4(sp[0] * l.x, sp[C::PP] * l.y, sp[2 * C::PP] * l.z, sp[3 * C::PP] * l.w);
-                        sp += KPI;
-                        gp += gstep;
-                        lp += gstep;
+            for (int rd = 0; rd < ROUNDS; ++rd) {
+                const int c = g + rd * G;
+                const bool active = (CC / 2) % G == 0 || c < CC / 2;
+                // the couple's columns: c and C-c (C/2 for c = 0)
+                float4 *px, *pw;
+                int sx = 1, sw = -1;
+                if constexpr (R2 == 1) {
+                    px = row + M1 * c;
+                    pw = row + M1 - 1 + M1 * ((c ? CC - c : CC / 2) - R1 / 2);
+                } else {
+                    const int k1 = c % R1, k2 = c / R1;
+                    px = row + sub_base<N>(k1, sx) + sx * (R3 * k2);
+                    const int k1p = k1 ? R1 - k1 : 0;
+                    const int k2p = k1 ? R2 - 1 - k2 : (c ? R2 - k2 : R2 / 2);
+                    pw = row + sub_base<N>(k1p, sw) + sw * (R3 - 1 + R3 * (k2p - R2 / 2));
+                    sw = -sw;
+                }
+                const SlotIndex<N> at(c);
+                float4 x[R3 / 2], w[R3 / 2];
+                float2 dr[R3], di[R3], a[R3], bb[R3];
+                if constexpr (FWD) {
+                    if (active) {
+#pragma unroll
+                        for (int m = 0; m < R3 / 2; ++m) {
+                            x[m] = px[sx * m];
+                            w[m] = pw[sw * m];
+                        }
+                    }
+                    if constexpr (MODE == MODE_F) {
+                        if (rd == ROUNDS - 1) {
+                            // every unit of the panel is in registers: the next panel may land
+                            fence_proxy_async_smem();
+                            __syncthreads();
+                            if (tid < 32 && next < p.npanels) load_panel(next);
+                        }
+                    }
+                    if (active) {
+                        last_forward<R3>(x, w, dr, di);
+                        split_forward<R3, CC>(c, dr, di, ts, p.sc, a, bb);
                     }
                 } else {
-#pragma unroll 4
-                    for (int k = kk; k < N; k += KPI) {
-                        *reinterpret_cast<float4 *>(gp) = make_float4(sp[0], sp[C::PP], sp[2 * C::PP], sp[3 * C::PP]);
-                        sp += KPI;
-                        gp += gstep;
+                    if (active) {
+#pragma unroll
+                        for (int k = 0; k < R3; ++k) {
+                            a[k].x = __ldg(src + at.ax(k) * ld);
+                            a[k].y = __ldg(src + at.ay(k) * ld);
+                            bb[k].x = __ldg(src + at.bx(k) * ld);
+                            bb[k].y = __ldg(src + at.by(k) * ld);
+                        }
+                    }
+                    if (rd == 0) {
+                        // the previous panel's stores must have read the buffer
+                        if (tid < PR) bulk_wait_read<0>();
+                        __syncthreads();
+                    }
+                }
+                if constexpr (MODE == MODE_F) {
+                    if (active) {
+#pragma unroll
+                        for (int k = 0; k < R3; ++k) {
+                            dst[at.ax(k) * ld] = a[k].x;
+                            dst[at.ay(k) * ld] = a[k].y;
+                            dst[at.bx(k) * ld] = bb[k].x;
+                            dst[at.by(k) * ld] = bb[k].y;
+                        }
+                    }
+                }
+                if constexpr (MODE == MODE_RR) {
+                    if (active && lam) {
+#pragma unroll
+                        for (int k = 0; k < R3; ++k) {
+                            a[k].x *= __ldg(lam + at.ax(k) * ld);
+                            a[k].y *= __ldg(lam + at.ay(k) * ld);
+                            bb[k].x *= __ldg(lam + at.bx(k) * ld);
+                            bb[k].y *= __ldg(lam + at.by(k) * ld);
+                        }
+                    }
+                }
+                if constexpr (INV) {
+                    if (active) {
+                        split_adjoint<R3, CC>(c, a, bb, ts, p.sc, dr, di);
+                        last_adjoint<R3>(x, w, dr, di);
+#pragma unroll
+                        for (int m = 0; m < R3 / 2; ++m) {
+                            px[sx * m] = x[m];
+                            pw[sw * m] = w[m];
+                        }
                     }
                 }
             }
         }
-        __syncthreads();
+        if constexpr (INV) {
+            __syncthreads();
+            if constexpr (R2 > 1) {
+#pragma unroll 1
+                for (int q = g; q < R1 * R3 / 2; q += G) {
+                    int sgn;
+                    const int k1 = q / (R3 / 2), m3 = q % (R3 / 2);
+                    const int qb = sub_base<N>(k1, sgn);
+                    float4 *px = row + qb + sgn * m3, *py = row + qb + sgn * (R3 - 1 - m3);
+                    float4 x[R2 / 2], y[R2 / 2];
+#pragma unroll
+                    for (int j = 0; j < R2 / 2; ++j) {
+                        x[j] = px[sgn * R3 * j];
+                        y[j] = py[sgn * R3 * j];
+                    }
+                    step_adjoint<R2, R3>(x, y, t2 + m3);
+#pragma unroll
+                    for (int j = 0; j < R2 / 2; ++j) {
+                        px[sgn * R3 * j] = x[j];
+                        py[sgn * R3 * j] = y[j];
+                    }
+                }
+                __syncthreads();
+            }
+            float *dst = MODE == MODE_CC ? dst_of(b) + r0 + line : nullptr;
+#pragma unroll 1
+            for (int cc = g; cc < M1 / 2; cc += G) {
+                float4 x[R1 / 2], y[R1 / 2];
+#pragma unroll
+                for (int j = 0; j < R1 / 2; ++j) {
+                    x[j] = row[cc + M1 * j];
+                    y[j] = row[M1 - 1 - cc + M1 * j];
+                }
+                step_adjoint<R1, M1>(x, y, t1 + cc);
+#pragma unroll
+                for (int j = 0; j < R1 / 2; ++j) {
+                    if constexpr (MODE == MODE_CC) {
+                        float *q = dst + (long long)(4 * (cc + M1 * j)) * p.rows;
+                        q[0] = x[j].x; q[p.rows] = x[j].y; q[2 * p.rows] = x[j].z; q[3 * p.rows] = x[j].w;
+                        q = dst + (long long)(4 * (M1 - 1 - cc + M1 * j)) * p.rows;
+                        q[0] = y[j].x; q[p.rows] = y[j].y; q[2 * p.rows] = y[j].z; q[3 * p.rows] = y[j].w;
+                    } else {
+                        row[cc + M1 * j] = x[j];
+                        row[M1 - 1 - cc + M1 * j] = y[j];
+                    }
+                }
+            }
+            if constexpr (ROWS_OUT) {
+                fence_proxy_async_smem();  // the stores read the panel through the async proxy
+                __syncthreads();
+                if (tid < PR) {
+                    bulk_store(dst_of(b) + (long long)(r0 + tid) * N, lsm + tid * C::PT, N * 4);
+                    bulk_commit();
+                }
+                if constexpr (MODE == MODE_RR) {
+                    if (tid < 32 && next < p.npanels) {
+                        if (tid < PR) bulk_wait_read<0>();
+                        __syncwarp();
+                        load_panel(next);
+                    }
+                }
+            }
+        }
+    }
+    if constexpr (ROWS_OUT) {
+        if (tid < PR) bulk_wait<0>();
     }
 }
 
-template <int N, int DIR>
-static cudaError_t lines_launch(const LinesParams &p0, cudaStream_t stream)
+template <int N, int MODE>
+cudaError_t lines_launch(const LinesParams &p0, long long nrows, cudaStream_t stream)
 {
     using C = LineCfg<N>;
-    auto kern = k_lines<N, DIR>;
+    auto kern = k_lines<N, MODE>;
     static DeviceLaunchCache cache;
     int dev = 0, blocks_per_sm = 0, num_sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -606,7 +697,7 @@ static cudaError_t lines_launch(const LinesParams &p0, cudaStream_t stream)
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
             if (r == cudaSuccess && bps < 1) r = cudaErrorInvalidConfiguration;
             if (r == cudaSuccess && debug_enabled())
-                fprintf(stderr, "[bdct] k_lines<%d,%d>: %d CTAs/SM x %d threads, panel %d rows, smem %zu B\n", N, DIR,
+                fprintf(stderr, "[bdct] k_lines<%d,%d>: %d CTAs/SM x %d threads, panel %d lines, smem %zu B\n", N, MODE,
                         bps, C::THREADS, C::PR, C::SMEM);
             return r;
         },
@@ -614,7 +705,7 @@ static cudaError_t lines_launch(const LinesParams &p0, cudaStream_t stream)
     if (e != cudaSuccess) return e;
     LinesParams p = p0;
     if (p.rows % C::PR != 0) return cudaErrorInvalidValue;  // panels never straddle two arrays
-    const long long np = p.nrows / C::PR;
+    const long long np = nrows / C::PR;
     if (np <= 0) return cudaSuccess;
     if (np > 0x7ff00000LL) return cudaErrorInvalidValue;
     p.npanels = (int)np;
@@ -634,102 +725,134 @@ static cudaError_t lines_launch(const LinesParams &p0, cudaStream_t stream)
 }
 
 template <int N>
-static cudaError_t lines_dir(Dir dir, const LinesParams &p, cudaStream_t s)
+cudaError_t lines_mode(LinesMode mode, const LinesParams &p, long long nrows, cudaStream_t s)
 {
-    switch (dir) {
-        case DIR_FWD: return lines_launch<N, DIR_FWD>(p, s);
-        case DIR_INV: return lines_launch<N, DIR_INV>(p, s);
-        default: return lines_launch<N, DIR_RT>(p, s);
+    switch (mode) {
+        case LINES_FORWARD: return lines_launch<N, MODE_F>(p, nrows, s);
+        case LINES_INVERSE: return lines_launch<N, MODE_I>(p, nrows, s);
+        case LINES_PAIR_ROWS: return lines_launch<N, MODE_RR>(p, nrows, s);
+        default: return lines_launch<N, MODE_CC>(p, nrows, s);
     }
 }
 
-// The line engine's tables for length n (L = n / 2 = L1 * L2), in FP64 with
-// the angle reduced exactly in integers:
-//  [0, L):   exp(-2 pi i m2 k1 / L) at index k1 * L2 + m2 (step A);
-//  [L, 3L):  for k < L the float4 (exp(-2 pi i k / n), exp(-i pi k / (2n)))
-//            (the split between the half-length FFT and the DCT).
-__global__ void k_gen_line_tw(float2 *t, int n, int l1)
+// The tables of length n = 2L, in FP64 with every angle reduced exactly in
+// integers; layout as LineCfg (first step, middle step, split).
+struct TableShape {
+    int n, r1, r2, r3;
+};
+
+__device__ void cos_sin_2pi(long long m, long long d, double &c, double &s)  // of 2 pi m / d
 {
-    const int L = n / 2, l2 = L / l1;
+    m %= d;
+    if (m < 0) m += d;
+    sincospi(2.0 * (double)m / (double)d, &s, &c);
+}
+
+__global__ void k_gen_line_tw(float4 *t, TableShape q, double s1)
+{
+    const int L = q.n / 2, m1 = L / q.r1, c3 = L / q.r3;
+    const int u1 = q.r1 * (m1 / 2), u2 = q.r2 > 1 ? q.r2 * (q.r3 / 2) : 0;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < L) {
-        const int k1 = r / l2, m2 = r % l2;
-        const long long m = ((long long)m2 * k1) % L;  // angle -2 pi m / L
-        double sn, cs;
-        sincospi(-2.0 * (double)m / (double)L, &sn, &cs);
-        t[r] = make_float2((float)cs, (float)sn);
-    } else if (r < 2 * L) {
-        const int k = r - L;
-        double s1, c1, s2, c2;
-        sincospi(-2.0 * (double)k / (double)n, &s1, &c1);
-        sincospi(-(double)k / (2.0 * (double)n), &s2, &c2);
-        float4 *q = reinterpret_cast<float4 *>(t + L);
-        q[k] = make_float4((float)c1, (float)s1, (float)c2, (float)s2);
+    double ca, sa, cb, sb;
+    if (r < u1 + u2) {
+        // entry (k, cc): exp(-2 pi i cc k / (R MC)) and exp(2 pi i (cc+1) k / (R MC)),
+        // k signed in the step before the last
+        const bool first = r < u1;
+        const int R = first ? q.r1 : q.r2, mc = first ? m1 : q.r3;
+        const int e = first ? r : r - u1;
+        int k = e / (mc / 2);
+        const int cc = e % (mc / 2);
+        if ((q.r2 == 1 || !first) && k >= R / 2) k -= R;
+        const long long d = (long long)R * mc;
+        cos_sin_2pi((long long)cc * k, d, ca, sa);
+        cos_sin_2pi((long long)(cc + 1) * k, d, cb, sb);
+        t[r] = make_float4((float)ca, (float)cb, (float)sa, (float)sb);
+    } else if (r < u1 + u2 + L / 2) {
+        const int e = r - u1 - u2;
+        const int k3 = e / (c3 / 2), c = e % (c3 / 2);
+        const int k = c3 * k3 + (c || k3 < q.r3 / 2 ? c : c3 / 2 - L / 2);
+        const double f = 0.5 * s1;
+        double cw, sw;
+        cos_sin_2pi(k, q.n, cw, sw);
+        cos_sin_2pi(k, 4ll * q.n, ca, sa);       // W_k = exp(-i pi k / (2n))
+        cos_sin_2pi(L - k, 4ll * q.n, cb, sb);   // W_{L-k}
+        float4 *o = t + u1 + u2;
+        o[e] = make_float4((float)cw, (float)sw, (float)(f * ca), (float)(f * cb));
+        reinterpret_cast<float2 *>(o + L / 2)[e] = make_float2((float)(f * sa), (float)(f * sb));
     }
 }
 
-static int line_l1(int n)
+template <int N>
+TableShape shape_of()
+{
+    return TableShape{N, LineCfg<N>::R1, LineCfg<N>::R2, LineCfg<N>::R3};
+}
+
+bool table_shape(int n, TableShape *q)
 {
     switch (n) {
-        case 64: return LineCfg<64>::L1;
-        case 128: return LineCfg<128>::L1;
-        case 256: return LineCfg<256>::L1;
-        case 512: return LineCfg<512>::L1;
-        case 1024: return LineCfg<1024>::L1;
-        case 2048: return LineCfg<2048>::L1;
-        case 4096: return LineCfg<4096>::L1;
-        case 192: return LineCfg<192>::L1;
-        case 384: return LineCfg<384>::L1;
-        case 768: return LineCfg<768>::L1;
-        case 1536: return LineCfg<1536>::L1;
-        default: return 0;
+        case 64: *q = shape_of<64>(); return true;
+        case 128: *q = shape_of<128>(); return true;
+        case 192: *q = shape_of<192>(); return true;
+        case 256: *q = shape_of<256>(); return true;
+        case 384: *q = shape_of<384>(); return true;
+        case 512: *q = shape_of<512>(); return true;
+        case 768: *q = shape_of<768>(); return true;
+        case 1024: *q = shape_of<1024>(); return true;
+        case 1536: *q = shape_of<1536>(); return true;
+        case 2048: *q = shape_of<2048>(); return true;
+        case 4096: *q = shape_of<4096>(); return true;
+        default: return false;
     }
 }
 
-cudaError_t lines_gen_table(float2 *dst, int n, cudaStream_t s)
+}  // namespace
+
+size_t lines_table_elems(int n)
 {
-    const int l1 = line_l1(n);
-    if (l1 == 0) return cudaErrorInvalidValue;
-    const int total = n;  // L step-A entries + L split entries (float4, two float2 each)
-    k_gen_line_tw<<<(total + 255) / 256, 256, 0, s>>>(dst, n, l1);
+    TableShape q;
+    if (!table_shape(n, &q)) return 0;
+    const int L = n / 2;
+    return (size_t)q.r1 * (L / q.r1 / 2) + (q.r2 > 1 ? (size_t)q.r2 * (q.r3 / 2) : 0) + L / 2 + L / 4;
+}
+
+cudaError_t lines_gen_table(float4 *dst, int n, double s1, cudaStream_t s)
+{
+    TableShape q;
+    if (!table_shape(n, &q)) return cudaErrorInvalidValue;
+    const int total = (int)lines_table_elems(n);
+    k_gen_line_tw<<<(total + 255) / 256, 256, 0, s>>>(dst, q, s1);
     return cudaGetLastError();
 }
 
-cudaError_t lines_pass(const float *src, float *dst, int rows, int n, long long count, Dir dir, AxisScale sc,
-                       const float2 *tw, unsigned int *status, cudaStream_t stream, const long long *src_off,
-                       const long long *dst_off, bool reverse)
+cudaError_t lines_pass(const float *src, float *dst, int rows, int n, long long count, LinesMode mode, AxisScale sc,
+                       const float4 *tw, const float *lam, unsigned int *status, cudaStream_t stream,
+                       const long long *src_off, const long long *dst_off, bool reverse)
 {
-    return lines_pass_lam(src, dst, rows, n, count, dir, sc, tw, status, stream, src_off, dst_off, reverse, nullptr);
-}
-
-cudaError_t lines_pass_lam(const float *src, float *dst, int rows, int n, long long count, Dir dir, AxisScale sc,
-                           const float2 *tw, unsigned int *status, cudaStream_t stream, const long long *src_off,
-                           const long long *dst_off, bool reverse, const float *lam)
-{
-    (void)status;
     LinesParams p{};
-    p.lam = lam;
-    p.reverse = reverse ? 1 : 0;
     p.src = src;
     p.dst = dst;
-    p.tw = tw;
+    p.rows = rows;
+    p.sc = sc;
     p.src_off = src_off;
     p.dst_off = dst_off;
-    p.rows = rows;
-    p.nrows = (long long)rows * count;
-    p.sc = sc;
+    p.tw = tw;
+    p.lam = lam;
+    p.status = status;
+    p.reverse = reverse ? 1 : 0;
+    const long long nrows = (long long)rows * count;
     switch (n) {
-        case 64: return lines_dir<64>(dir, p, stream);
-        case 128: return lines_dir<128>(dir, p, stream);
-        case 256: return lines_dir<256>(dir, p, stream);
-        case 512: return lines_dir<512>(dir, p, stream);
-        case 1024: return lines_dir<1024>(dir, p, stream);
-        case 2048: return lines_dir<2048>(dir, p, stream);
-        case 4096: return lines_dir<4096>(dir, p, stream);
-        case 192: return lines_dir<192>(dir, p, stream);
-        case 384: return lines_dir<384>(dir, p, stream);
-        case 768: return lines_dir<768>(dir, p, stream);
-        case 1536: return lines_dir<1536>(dir, p, stream);
+        case 64: return lines_mode<64>(mode, p, nrows, stream);
+        case 128: return lines_mode<128>(mode, p, nrows, stream);
+        case 192: return lines_mode<192>(mode, p, nrows, stream);
+        case 256: return lines_mode<256>(mode, p, nrows, stream);
+        case 384: return lines_mode<384>(mode, p, nrows, stream);
+        case 512: return lines_mode<512>(mode, p, nrows, stream);
+        case 768: return lines_mode<768>(mode, p, nrows, stream);
+        case 1024: return lines_mode<1024>(mode, p, nrows, stream);
+        case 1536: return lines_mode<1536>(mode, p, nrows, stream);
+        case 2048: return lines_mode<2048>(mode, p, nrows, stream);
+        case 4096: return lines_mode<4096>(mode, p, nrows, stream);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,4 +1,4 @@
-// Entry points of the line engine beyond lines_pass (fp32_lines.cu).
+// Entry points of the line engine (fp32_lines.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -7,14 +7,37 @@
 
 namespace bdct {
 
-// lines_pass with every output element (k, r) of an array (k < n the
-// transformed index, r < rows the line) multiplied by lam[k * rows + r] as
-// it is stored, or lines_pass itself for lam null: the second pass of a
-// forward transform times the diagonal, the first half of the spectral
-// composition of Prop. 1 (Eq. 4) on the line engine.  lam is 16-byte
-// aligned, rows a multiple of 4.
-cudaError_t lines_pass_lam(const float *src, float *dst, int rows, int n, long long count, Dir dir, AxisScale sc,
-                           const float2 *tw, unsigned int *status, cudaStream_t stream, const long long *src_off,
-                           const long long *dst_off, bool reverse, const float *lam);
+// What one separable pass does with arrays of `rows` lines of n points (r the
+// line, k or j the index along it):
+//   LINES_FORWARD    src[r][j] -> dst[k][r]   DCT-II, output scales
+//   LINES_INVERSE    src[k][r] -> dst[r][j]   DCT-III, input scales
+//   LINES_PAIR_ROWS  src[r][j] -> dst[r][j]   DCT-II, diagonal, DCT-III (Prop. 1)
+//   LINES_PAIR_COLS  src[j][r] -> dst[j][r]   the same along columns
+// A forward pass along w then one along h is the 2D forward transform in
+// natural layout (the intermediate is w x h), an inverse pass along h then one
+// along w the inverse, a row pair and a column pair the round trip.
+enum LinesMode { LINES_FORWARD, LINES_INVERSE, LINES_PAIR_ROWS, LINES_PAIR_COLS };
+
+// Copy the cosine tables (device buffers) into the line engine's constant
+// memory (called by fused_init_device).
+cudaError_t lines_init_table(const float *d_table);
+cudaError_t lines_init_table3(const float *d_table);
+// True if n has an FFT-based line engine: powers of two 64..4096, and 192,
+// 384, 768, 1536.
+bool lines_supported(int n);
+// The twiddle table of length n (lines_table_elems(n) float4 entries),
+// generated in FP64; s1 is the scale of every index above 0, folded in.
+size_t lines_table_elems(int n);
+cudaError_t lines_gen_table(float4 *dst, int n, double s1, cudaStream_t s);
+// One pass over `count` arrays.  sc holds the scales of the pass (sc.s1 the
+// table's s1; the pair modes apply them twice, so they take the orthonormal
+// ones); lam, if not null, is the diagonal of LINES_PAIR_ROWS: coefficient k
+// of line r is multiplied by lam[k * rows + r].  src_off / dst_off index the
+// arrays (element offsets) or are null for contiguous arrays.  src == dst is
+// allowed for LINES_PAIR_ROWS only, the other modes read what other CTAs
+// write.
+cudaError_t lines_pass(const float *src, float *dst, int rows, int n, long long count, LinesMode mode, AxisScale sc,
+                       const float4 *tw, const float *lam, unsigned int *status, cudaStream_t stream,
+                       const long long *src_off = nullptr, const long long *dst_off = nullptr, bool reverse = false);
 
 }  // namespace bdct
