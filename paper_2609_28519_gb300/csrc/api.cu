@@ -14,7 +14,7 @@
 #include "bdct_internal.h"
 #include "plan.h"
 #include "small_dense.h"
-#include "fp32_ring.h"
+#include "fp32_block.h"
 #include "fp32_lines.h"
 #include "dense_passes.h"
 
@@ -494,9 +494,7 @@ static DirScales ortho_scales(const bdct_plan *p, Dir dir)
 }
 
 // One direction of a fused or tensor-core plan over geometry g (contiguous,
-// indexed or tiled).  The spectral direction runs fused where a kernel has it
-// (sides 8-32, tensor cores) and otherwise as orthonormal forward (in -> out),
-// Lambda (in place), orthonormal inverse (out -> out, exact in place).
+// indexed or tiled), one launch.
 static int run_onchip(const bdct_plan *p, Dir dir, const ExecGeom &g0, cudaStream_t s)
 {
     ExecGeom g = g0;
@@ -511,30 +509,11 @@ static int run_onchip(const bdct_plan *p, Dir dir, const ExecGeom &g0, cudaStrea
         e = fused_launch(p->rows, p->cols, dir, p->scales[dir], g, p->status, s);
         return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
     }
-    if (!ring_supported(p->rows, p->cols)) {
-        g.lam = p->spec_fold;
-        e = fused_launch(p->rows, p->cols, DIR_SPEC, p->scales[DIR_RT], g, p->status, s);
-        return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
-    }
-    if (p->rows == 64 && p->cols == 64) {
-        // fused in the ring kernel: one read, one write
-        g.lam = p->spec_fold;
-        e = ring_launch(64, 64, DIR_SPEC, p->scales[DIR_RT], g, p->status, s);
-        return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
-    }
-    // the other ring shapes: the orthonormal forward multiplying its
-    // coefficients by Lambda as it stores them, then the orthonormal inverse
-    // in place
-    g.lam = p->spec_plain;
-    e = ring_forward_lam(p->rows, p->cols, ortho_scales(p, DIR_FWD), g, p->status, s);
-    g.lam = nullptr;
-    if (e == cudaSuccess) {
-        ExecGeom gi = g;
-        gi.in = g.out;
-        gi.in_off = g.out_off;
-        gi.ld_in = g.ld_out;
-        e = fused_launch(p->rows, p->cols, DIR_INV, ortho_scales(p, DIR_INV), gi, p->status, s);
-    }
+    // fused: one read, one write.  The kernels of sides 64 x 128, 128 x 64 and
+    // 128 x 128 apply Lambda between orthonormal passes, the others E Lambda E
+    // between unscaled ones.
+    g.lam = block_supported(p->rows, p->cols) && !ring_supported(p->rows, p->cols) ? p->spec_plain : p->spec_fold;
+    e = fused_launch(p->rows, p->cols, DIR_SPEC, p->scales[DIR_RT], g, p->status, s);
     return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
 }
 

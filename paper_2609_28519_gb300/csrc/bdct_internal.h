@@ -108,12 +108,11 @@ cudaError_t tma_map_2d(struct CUtensorMap_st *m, const float *base, unsigned lon
                        unsigned long long cols, unsigned long long ld, int box_rows);
 
 // ---- fp32_ring.cu
-// Warp-specialized ring kernels for sides 64 and 128 (all four combinations):
-// contiguous, indexed and tiled batches.
+// Warp-specialized ring kernel for 64 x 64 arrays: contiguous, indexed and
+// tiled batches.  The spectral direction takes the folded diagonal in g.lam.
 cudaError_t ring_init_table(const float *d_table);
 bool ring_supported(int rows, int cols);
-cudaError_t ring_launch(int rows, int cols, Dir dir, const DirScales &sc, const ExecGeom &g,
-                        unsigned int *status, cudaStream_t stream);
+cudaError_t ring_launch(Dir dir, const DirScales &sc, const ExecGeom &g, unsigned int *status, cudaStream_t stream);
 
 // ---- tc_split.cu
 // Split-BF16 tcgen05 route for square sides 16, 32, 64.

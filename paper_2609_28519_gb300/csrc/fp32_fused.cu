@@ -1,6 +1,7 @@
 // FP32 fused 2D DCT kernels for small power-of-two sides (8, 16, 32, in
-// every combination); sides 64 and 128 go to the ring kernels of
-// fp32_ring.cu through the same entry points.
+// every combination); 64 x 64 goes to the ring kernel of
+// fp32_ring.cu and the other shapes of sides 64 and 128 to fp32_block.cu,
+// through the same entry points.
 //
 // What is computed: Eq. 2 of the BRiDCT paper, C(X) = Q_h X Q_w^T (forward,
 // DCT-II), C^{-1}(Y) = Q_h^T Y Q_w (inverse, DCT-III) and the round trip,
@@ -21,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "bdct_internal.h"
+#include "fp32_block.h"
 #include "fp32_lines.h"
 #include "dct_cores.cuh"
 #include "ptx.cuh"
@@ -105,7 +107,7 @@ struct FusedCfg {
                   "lane mapping");
     static_assert((P % 8) == 4 && (SP % 8) == 4, "pitches must be 4 mod 8 floats");
     static_assert(LAYOUT == LAY_STRIP || G % 8 == 0, "slot-layout lanes span 8 arrays");
-    static_assert(H <= 32 && W <= 32, "sides 64 and 128 use the ring kernels");
+    static_assert(H <= 32 && W <= 32, "sides 64 and 128 have kernels of their own");
 };
 
 // Element (a, r, c) of a stage: array/tile a, row r, column c.
@@ -685,6 +687,7 @@ cudaError_t fused_init_device(int device)
     if (e == cudaSuccess) e = init_cos_table(tmp);
     if (e == cudaSuccess) e = lines_init_table(tmp);
     if (e == cudaSuccess) e = ring_init_table(tmp);
+    if (e == cudaSuccess) e = block_init_device(tmp);
     if (e == cudaSuccess) {
         k_gen_cos_table3<<<(769 + 255) / 256, 256>>>(tmp);
         e = cudaGetLastError();
@@ -700,7 +703,7 @@ cudaError_t fused_init_device(int device)
 bool fused_supported(int rows, int cols)
 {
     auto ok = [](int n) { return n == 8 || n == 16 || n == 32; };
-    return (ok(rows) && ok(cols)) || ring_supported(rows, cols);
+    return (ok(rows) && ok(cols)) || ring_supported(rows, cols) || block_supported(rows, cols);
 }
 
 template <int H, int W, int DIR, bool TILED>
@@ -833,10 +836,8 @@ static cudaError_t launch_h(int cols, Dir dir, const DirScales &sc, const ExecGe
 cudaError_t fused_launch(int rows, int cols, Dir dir, const DirScales &sc, const ExecGeom &g,
                          unsigned int *status, cudaStream_t stream)
 {
-    if (ring_supported(rows, cols)) {
-        if (dir == DIR_SPEC) return cudaErrorInvalidValue;  // composed by the caller from F, scale, I
-        return ring_launch(rows, cols, dir, sc, g, status, stream);
-    }
+    if (ring_supported(rows, cols)) return ring_launch(dir, sc, g, status, stream);
+    if (block_supported(rows, cols)) return block_launch(rows, cols, dir, sc, g, status, stream);
     switch (rows) {
         case 8: return launch_h<8>(cols, dir, sc, g, status, stream);
         case 16: return launch_h<16>(cols, dir, sc, g, status, stream);

@@ -1,4 +1,7 @@
-// FP32 ring kernels for sides 64 and 128: 64x64, 64x128, 128x64, 128x128.
+// FP32 ring kernel for 64x64 arrays (the other shapes of sides 64 and 128 run
+// in fp32_block.cu, which measured 0.77 / 0.77 / 0.44 / 0.40 of HBM on 64x64
+// against 0.90 / 0.91 / 0.76 / 0.60 here: forward, inverse, round trip,
+// spectral, 512 MiB).
 //
 // What is computed: Eq. 2 of the BRiDCT paper, C(X) = Q_h X Q_w^T (forward,
 // DCT-II), C^{-1}(Y) = Q_h^T Y Q_w (inverse, DCT-III) and the normalized
@@ -28,19 +31,7 @@
 // 16-byte accesses) and the column pass (one column per thread) are both
 // free of bank conflicts.
 //
-// 1D lines of 64 points run whole in one thread (dct_cores.cuh).  Lines of
-// 128 points are shared by two threads of different warps through the first
-// even/odd split of the DCT-II: role 0 evaluates the even outputs as a
-// 64-point DCT-II of the sums x_j + x_{127-j}, role 1 the odd outputs as a
-// 64-point DCT-IV of the differences.  The inverse runs the split backwards:
-// role 0 a 64-point DCT-III of the even inputs (a), role 1 a 64-point DCT-IV
-// of the odd inputs (b), then x_j = a_j + b_j and x_{127-j} = a_j - b_j.
-// After a 128-point row pass the row is left in a permuted order that the
-// column pass undoes when it writes back:
-//  * forward: Y_{2m} at position m, Y_{2m+1} at 64 + ((m + 16) mod 64);
-//  * inverse and round trip: x_j at j, x_{127-j} at 64 + j (j < 64);
-// either way the 32 columns a warp takes in the column pass occupy 32
-// distinct banks of every row.
+// Each line runs whole in one thread (dct_cores.cuh).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -49,7 +40,6 @@
 #include "bdct_internal.h"
 #include "dct_cores.cuh"
 #include "ptx.cuh"
-#include "fp32_ring.h"
 
 namespace bdct {
 
@@ -57,51 +47,42 @@ cudaError_t ring_init_table(const float *d_table) { return init_cos_table(d_tabl
 
 bool ring_supported(int rows, int cols)
 {
-    return (rows == 64 || rows == 128) && (cols == 64 || cols == 128);
+    return rows == 64 && cols == 64;
 }
 
 constexpr int kRingMaxSmem = 232448;  // 227 KiB, the opt-in limit per CTA
 
-// The group count depends on the direction (the kernels are instantiated per
-// direction); GT, the slot and box sizes do not, and the transform helpers
-// that use only those take the default.
-template <int H, int W, int DIR = DIR_FWD>
+// The group count depends on the direction; the group, slot and box sizes do
+// not, and the helpers that use only those take the default.
+template <int DIR = DIR_FWD>
 struct RingCfg {
-    static constexpr int TR = W / 64;   // threads per row line
-    static constexpr int TC = H / 64;   // threads per column line
-    static constexpr int GT = H * TR;   // threads per consumer group
+    static constexpr int H = 64, W = 64;
+    static constexpr int GT = 64;       // threads per consumer group (one line each)
     static constexpr int GW = GT / 32;  // warps per consumer group
     static constexpr int SLOT_BYTES = H * W * 4;
     static constexpr int SLOT_FLOATS = H * W;
     static constexpr int BOX_BYTES = H * 128;  // 32 columns x H rows
-    // spectral direction (64 x 64 only): the folded diagonal staged once per CTA
+    // spectral direction: the folded diagonal staged once per CTA
     static constexpr int LAM_BYTES = DIR == DIR_SPEC ? H * W * 4 : 0;
     static constexpr int S_MAX = (kRingMaxSmem - 2048 - LAM_BYTES) / SLOT_BYTES;
     // about three slots per group, so that a group's next arrays load while
     // it computes; the slot count is a multiple of the group count (a group
     // always reuses slots it consumed itself, which the slot barriers' parity
     // tracking relies on)
-    // (round trips, twice the arithmetic per array, run more groups over two
-    // slots each: 64 x 64 seven groups, 0.67 -> 0.76 of HBM, while forward
-    // and inverse measured 0.90 -> 0.81 that way; the rectangles three groups,
-    // 0.26 -> 0.30 / 0.33)
-    // (the spectral direction, four 1D cores per line pair like the round
-    // trip plus the diagonal, runs six groups over the thirteen slots left
-    // beside the diagonal, two each)
-    static constexpr int NG = (H == 64 && W == 64 && DIR == DIR_RT) ? 7
-                              : (H == 64 && W == 64 && DIR == DIR_SPEC) ? 6
-                              : (H != W && DIR == DIR_RT)             ? 3
-                                                                      : (S_MAX / 3 < 1 ? 1 : S_MAX / 3);
+    // (round trips, twice the arithmetic per array, run seven groups over two
+    // slots each: 0.67 -> 0.76 of HBM, while forward and inverse measured
+    // 0.90 -> 0.81 that way; the spectral direction, four 1D cores per line
+    // pair like the round trip plus the diagonal, six over the thirteen slots
+    // left beside the diagonal)
+    static constexpr int NG = DIR == DIR_RT ? 7 : DIR == DIR_SPEC ? 6 : S_MAX / 3;
     static constexpr int S = (S_MAX / NG) * NG;
     static constexpr int PROD_WARP = NG * GW;
     static constexpr int THREADS = (NG * GW + 1) * 32;
     // slots start 1024-byte aligned (128-byte swizzle atoms)
     static constexpr size_t SMEM = 1024 + (size_t)S * SLOT_BYTES + (size_t)2 * S * 8 + LAM_BYTES;
-    static_assert(H * TR == W * TC, "both passes use the whole group");
     static_assert(GT % 32 == 0 && S >= 2 && S % NG == 0, "ring shape");
     static_assert(SMEM <= (size_t)kRingMaxSmem, "shared memory");
     static_assert(BOX_BYTES % 1024 == 0, "swizzle atoms");
-    static_assert(DIR != DIR_SPEC || (H == 64 && W == 64), "the fused spectral direction is 64 x 64 only");
 };
 
 // Named barrier over the threads of one consumer group.
@@ -160,402 +141,61 @@ __device__ __forceinline__ T &at(char *base, uint32_t off)
     return *reinterpret_cast<T *>(base + off);
 }
 
-// Slot position of logical column c after the row pass (see the header).
-template <int W, int DIR>
-__device__ __forceinline__ int ring_colpos(int c)
-{
-    if constexpr (W == 64) return c;
-    else if constexpr (DIR == DIR_FWD) return (c & 1) ? 64 + (((c >> 1) + 16) & 63) : (c >> 1);
-    else return c < 64 ? c : 191 - c;
-}
-
-template <int N>
-__device__ __forceinline__ void scale_from(float (&x)[N], float first, float rest)
-{
-    x[0] *= first;
-#pragma unroll
-    for (int k = 1; k < N; ++k) x[k] *= rest;
-}
-
-// Role and line of a group thread when 128-point lines are shared by two
-// threads: warps alternate roles, so that each SM sub-partition (warps are
-// dealt to the four sub-partitions round robin) runs one role's code only,
-// and the 32 lanes of a warp take 32 consecutive lines.
-__device__ __forceinline__ int role_of(int gt) { return (gt >> 5) & 1; }
-__device__ __forceinline__ int line_of(int gt) { return ((gt >> 6) << 5) | (gt & 31); }
-
-// The 64-point core of one role of a 128-point line.  On entry v holds the
-// role's input (forward and round trip: sums or differences; inverse: the
-// even or odd coefficients, already scaled); on exit y holds the role's
-// output (forward: its coefficients, scaled; inverse and round trip: a or b).
-template <int DIR>
-__device__ __forceinline__ void role_core(int role, const float (&v)[64], float (&y)[64], AxisScale s)
-{
-    if constexpr (DIR == DIR_FWD) {
-        if (role == 0) DCT2<64>::run(v, y);
-        else DCT4<64>::run(v, y);
-        scale_from<64>(y, role ? s.s1 : s.s0, s.s1);
-    } else if constexpr (DIR == DIR_INV) {
-        if (role == 0) DCT3<64>::run(v, y);
-        else DCT4<64>::run(v, y);
-    } else {
-        float t[64];
-        if (role == 0) {
-            DCT2<64>::run(v, t);
-            scale_from<64>(t, s.s0, s.s1);
-            DCT3<64>::run(t, y);
-        } else {
-            DCT4<64>::run(v, t);
-            scale_from<64>(t, s.s1, s.s1);
-            DCT4<64>::run(t, y);
-        }
-    }
-}
-
-// ---------------------------------------------------------------- rectangles
-// 64 x 128 and 128 x 64: the 128 side's lines are shared by two threads
-// (roles), the 64 side's lines take one thread each; both passes (rows, then
-// columns) run in one loop body around a single call of role_core (role 0 is
-// the whole 64-point transform), so the 1D cores exist once in the code.
-// LAMF (forward only): the coefficients are multiplied by the diagonal lam
-// (H x W, row k = frequency along h) as the column pass stores them -- the
-// first half of the spectral composition of Prop. 1 for these shapes.
-template <int H, int W, int DIR, bool LAMF = false>
-__device__ __forceinline__ void ring_rect(char *slot, int gt, int bar, const DirScales &sc,
-                                          const float *lam = nullptr)
-{
-    using C = RingCfg<H, W>;
-    constexpr int BB = C::BOX_BYTES;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-        const AxisScale s = pass ? sc.h : sc.w;
-        const bool split = pass == 0 ? W == 128 : H == 128;  // this pass's lines have 128 points
-        const int role = split ? role_of(gt) : 0;
-        const int ln = split ? line_of(gt) : gt;  // row (pass 0) or logical column (pass 1)
-        float v[64];
-        if (pass == 0) {
-            const RowView rv(ln);
-            if (!split) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                    v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
-                }
-            } else if (DIR == DIR_INV) {
-                // role 0: even coefficients, role 1: odd coefficients
-                if (role == 0) {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                        v[2 * k] = t.x; v[2 * k + 1] = t.z;
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                        v[2 * k] = t.y; v[2 * k + 1] = t.w;
-                    }
-                }
-            } else {
-                // sums (role 0) or differences (role 1) of x_j and x_{127-j}
-                const float sg = role ? -1.0f : 1.0f;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const float4 a = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                    const float4 b = at<float4>(slot, ((31 - k) >> 3) * BB + rv.o[(31 - k) & 7]);
-                    v[4 * k] = fmaf(sg, b.w, a.x);
-                    v[4 * k + 1] = fmaf(sg, b.z, a.y);
-                    v[4 * k + 2] = fmaf(sg, b.y, a.z);
-                    v[4 * k + 3] = fmaf(sg, b.x, a.w);
-                }
-            }
-        } else {
-            const ColView<H> src(ring_colpos<W, DIR>(ln));
-            if (!split) {
-#pragma unroll
-                for (int i = 0; i < 64; ++i) v[i] = at<float>(slot, i * 128 + src.o[i & 7]);
-            } else if (DIR == DIR_INV) {
-                // even rows (role 0) or odd rows (role 1)
-                if (role == 0) {
-#pragma unroll
-                    for (int m = 0; m < 64; ++m) v[m] = at<float>(slot, 2 * m * 128 + src.o[(2 * m) & 7]);
-                } else {
-#pragma unroll
-                    for (int m = 0; m < 64; ++m) v[m] = at<float>(slot, (2 * m + 1) * 128 + src.o[(2 * m + 1) & 7]);
-                }
-            } else {
-                const float sg = role ? -1.0f : 1.0f;
-#pragma unroll
-                for (int i = 0; i < 64; ++i)
-                    v[i] = fmaf(sg, at<float>(slot, (127 - i) * 128 + src.o[(127 - i) & 7]),
-                                at<float>(slot, i * 128 + src.o[i & 7]));
-            }
-        }
-        if constexpr (DIR == DIR_INV) scale_from<64>(v, role ? s.s1 : s.s0, s.s1);
-        // every read of the pass done before anything is overwritten (the split
-        // lines' two threads share positions; the column pass of a 128-wide
-        // array writes natural positions over permuted ones)
-        if (split || (pass == 1 && W == 128)) group_sync(bar, C::GT);
-        float y[64];
-        role_core<DIR>(role, v, y, s);
-        if (pass == 0) {
-            const RowView rv(ln);
-            if (!split || role == 0) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]) = make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    // forward: Y_{2m+1} at 64 + ((m + 16) mod 64); inverse / round trip: b_j at 64 + j
-                    const int kk = 16 + (DIR == DIR_FWD ? ((k + 4) & 15) : k);
-                    at<float4>(slot, (kk >> 3) * BB + rv.o[kk & 7]) = make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
-                }
-            }
-            if (DIR != DIR_FWD && split) {
-                // x_j = a_j + b_j (position j), x_{127-j} = a_j - b_j (position 64 + j)
-                group_sync(bar, C::GT);
-                constexpr int TASKS = H * 16;  // (row, 4 consecutive j)
-#pragma unroll
-                for (int t = gt; t < TASKS; t += C::GT) {
-                    const int rr = t >> 4, k = t & 15;
-                    const uint32_t oa = sw_chunk<H>(rr, k), ob = sw_chunk<H>(rr, 16 + k);
-                    const float4 a = at<float4>(slot, oa), b = at<float4>(slot, ob);
-                    at<float4>(slot, oa) = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-                    at<float4>(slot, ob) = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-                }
-            }
-        } else {
-            const ColView<H> dst(ln);
-            if constexpr (LAMF) {
-                // coefficient row (2m + role for split lines, m otherwise) of column ln
-#pragma unroll
-                for (int m = 0; m < 64; ++m) y[m] *= __ldg(lam + (split ? 2 * m + role : m) * W + ln);
-            }
-            if (!split) {
-#pragma unroll
-                for (int i = 0; i < 64; ++i) at<float>(slot, i * 128 + dst.o[i & 7]) = y[i];
-            } else if (DIR == DIR_FWD) {
-                // rows 2m (role 0) or 2m + 1 (role 1)
-                if (role == 0) {
-#pragma unroll
-                    for (int m = 0; m < 64; ++m) at<float>(slot, 2 * m * 128 + dst.o[(2 * m) & 7]) = y[m];
-                } else {
-#pragma unroll
-                    for (int m = 0; m < 64; ++m) at<float>(slot, (2 * m + 1) * 128 + dst.o[(2 * m + 1) & 7]) = y[m];
-                }
-            } else {
-                if (role == 0) {
-#pragma unroll
-                    for (int j = 0; j < 64; ++j) at<float>(slot, j * 128 + dst.o[j & 7]) = y[j];  // a_j at row j
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 64; ++j)
-                        at<float>(slot, (127 - j) * 128 + dst.o[(127 - j) & 7]) = y[j];  // b_j at row 127 - j
-                }
-                group_sync(bar, C::GT);
-                // x_j = a_j + b_j, x_{127-j} = a_j - b_j; two threads per column, 32 pairs each
-                auto comb = [&](int j) {
-                    const uint32_t oa = j * 128 + dst.o[j & 7], ob = (127 - j) * 128 + dst.o[(127 - j) & 7];
-                    const float a = at<float>(slot, oa), b = at<float>(slot, ob);
-                    at<float>(slot, oa) = a + b;
-                    at<float>(slot, ob) = a - b;
-                };
-                if (role == 0) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) comb(j);
-                } else {
-#pragma unroll
-                    for (int j = 32; j < 64; ++j) comb(j);
-                }
-            }
-        }
-        group_sync(bar, C::GT);
-    }
-}
-
-// ---------------------------------------------------------------- square arrays
-// For h = w the two passes run in one loop, so that the 1D cores (the largest
-// part of the code) exist once: pass 0 takes rows, pass 1 columns.  Same
-// arithmetic, layouts and barriers as ring_rows / ring_cols.
+// ---------------------------------------------------------------- one array
+// The two passes run in one loop, so that the 1D cores (the largest part of
+// the code) exist once: pass 0 takes rows, pass 1 columns, in place.
 //
 // The spectral direction (64 x 64, Prop. 1 / Eq. 4 with a general diagonal)
 // takes three passes with the unscaled cores: rows forward; columns forward,
 // times the column's entries of the folded diagonal lam_s (E_h Lambda E_w
 // with every scale of both axes in it), adjoint; rows adjoint.
-template <int N, int DIR, bool LAMF = false>
-__device__ __forceinline__ void ring_square(char *slot, int gt, int bar, const DirScales &sc,
-                                            const float *lam_s = nullptr, const float *lam = nullptr)
+template <int DIR>
+__device__ __forceinline__ void ring_array(char *slot, int gt, int bar, const DirScales &sc, const float *lam_s)
 {
-    using C = RingCfg<N, N>;
+    using C = RingCfg<>;
     constexpr int BB = C::BOX_BYTES;
     constexpr int NPASS = DIR == DIR_SPEC ? 3 : 2;
 #pragma unroll 1
     for (int pass = 0; pass < NPASS; ++pass) {
         const AxisScale s = (pass & 1) ? sc.h : sc.w;
-        if constexpr (N == 64) {
-            // one thread per line; row r (passes 0 and 2) or column c (pass 1), in place
-            float x[64];
-            if ((pass & 1) == 0) {
-                const RowView rv(gt);
+        // one thread per line; row r (passes 0 and 2) or column c (pass 1)
+        float x[64];
+        if ((pass & 1) == 0) {
+            const RowView rv(gt);
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                    x[4 * k] = t.x; x[4 * k + 1] = t.y; x[4 * k + 2] = t.z; x[4 * k + 3] = t.w;
-                }
-            } else {
-                const ColView<N> cv(gt);
-#pragma unroll
-                for (int i = 0; i < 64; ++i) x[i] = at<float>(slot, i * 128 + cv.o[i & 7]);
-            }
-            if constexpr (DIR == DIR_SPEC) {
-                if (pass == 1) {
-                    line_op<64, CORE_FWD>(x, s);
-#pragma unroll
-                    for (int k = 0; k < 64; ++k) x[k] *= lam_s[k * 64 + gt];
-                    line_op<64, CORE_INV>(x, s);
-                } else if (pass == 0) {
-                    line_op<64, CORE_FWD>(x, s);
-                } else {
-                    line_op<64, CORE_INV>(x, s);
-                }
-            } else {
-                line_op<64, DIR>(x, s);
-            }
-            if ((pass & 1) == 0) {
-                const RowView rv(gt);
-#pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]) =
-                        make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
-            } else {
-                const ColView<N> cv(gt);
-#pragma unroll
-                for (int i = 0; i < 64; ++i) at<float>(slot, i * 128 + cv.o[i & 7]) = x[i];
+            for (int k = 0; k < 16; ++k) {
+                const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
+                x[4 * k] = t.x; x[4 * k + 1] = t.y; x[4 * k + 2] = t.z; x[4 * k + 3] = t.w;
             }
         } else {
-            // two threads (roles) per 128-point line
-            const int role = role_of(gt);
-            const int r = line_of(gt);  // row (pass 0) or logical column (pass 1)
-            float v[64];
-            if (pass == 0) {
-                const RowView rv(r);
-                if constexpr (DIR == DIR_INV) {
-                    if (role == 0) {
+            const ColView<64> cv(gt);
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) {
-                            const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                            v[2 * k] = t.x; v[2 * k + 1] = t.z;
-                        }
-                    } else {
+            for (int i = 0; i < 64; ++i) x[i] = at<float>(slot, i * 128 + cv.o[i & 7]);
+        }
+        if constexpr (DIR == DIR_SPEC) {
+            if (pass == 1) {
+                line_op<64, CORE_FWD>(x, s);
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) {
-                            const float4 t = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                            v[2 * k] = t.y; v[2 * k + 1] = t.w;
-                        }
-                    }
-                } else {
-                    const float sg = role ? -1.0f : 1.0f;
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float4 a = at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]);
-                        const float4 b = at<float4>(slot, ((31 - k) >> 3) * BB + rv.o[(31 - k) & 7]);
-                        v[4 * k] = fmaf(sg, b.w, a.x);
-                        v[4 * k + 1] = fmaf(sg, b.z, a.y);
-                        v[4 * k + 2] = fmaf(sg, b.y, a.z);
-                        v[4 * k + 3] = fmaf(sg, b.x, a.w);
-                    }
-                }
+                for (int k = 0; k < 64; ++k) x[k] *= lam_s[k * 64 + gt];
+                line_op<64, CORE_INV>(x, s);
+            } else if (pass == 0) {
+                line_op<64, CORE_FWD>(x, s);
             } else {
-                const ColView<N> src(ring_colpos<N, DIR>(r));
-                if constexpr (DIR == DIR_INV) {
-                    if (role == 0) {
-#pragma unroll
-                        for (int m = 0; m < 64; ++m) v[m] = at<float>(slot, 2 * m * 128 + src.o[(2 * m) & 7]);
-                    } else {
-#pragma unroll
-                        for (int m = 0; m < 64; ++m)
-                            v[m] = at<float>(slot, (2 * m + 1) * 128 + src.o[(2 * m + 1) & 7]);
-                    }
-                } else {
-                    const float sg = role ? -1.0f : 1.0f;
-#pragma unroll
-                    for (int i = 0; i < 64; ++i)
-                        v[i] = fmaf(sg, at<float>(slot, (127 - i) * 128 + src.o[(127 - i) & 7]),
-                                    at<float>(slot, i * 128 + src.o[i & 7]));
-                }
+                line_op<64, CORE_INV>(x, s);
             }
-            if constexpr (DIR == DIR_INV) scale_from<64>(v, role ? s.s1 : s.s0, s.s1);
-            group_sync(bar, C::GT);  // every read of the pass done before anything is overwritten
-            float y[64];
-            role_core<DIR>(role, v, y, s);
-            if (pass == 0) {
-                const RowView rv(r);
-                if (role == 0) {
+        } else {
+            line_op<64, DIR>(x, s);
+        }
+        if ((pass & 1) == 0) {
+            const RowView rv(gt);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]) =
-                            make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
-                } else {
+            for (int k = 0; k < 16; ++k)
+                at<float4>(slot, (k >> 3) * BB + rv.o[k & 7]) =
+                    make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+        } else {
+            const ColView<64> cv(gt);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const int kk = 16 + (DIR == DIR_FWD ? ((k + 4) & 15) : k);
-                        at<float4>(slot, (kk >> 3) * BB + rv.o[kk & 7]) =
-                            make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
-                    }
-                }
-                if constexpr (DIR != DIR_FWD) {
-                    group_sync(bar, C::GT);
-                    constexpr int TASKS = N * 16;
-#pragma unroll
-                    for (int t = gt; t < TASKS; t += C::GT) {
-                        const int rr = t >> 4, k = t & 15;
-                        const uint32_t oa = sw_chunk<N>(rr, k), ob = sw_chunk<N>(rr, 16 + k);
-                        const float4 a = at<float4>(slot, oa), b = at<float4>(slot, ob);
-                        at<float4>(slot, oa) = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-                        at<float4>(slot, ob) = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-                    }
-                }
-            } else {
-                const ColView<N> dst(r);
-                if constexpr (LAMF) {
-                    // coefficient rows 2m + role of column r, times the diagonal
-#pragma unroll
-                    for (int m = 0; m < 64; ++m) y[m] *= __ldg(lam + (2 * m + role) * N + r);
-                }
-                if constexpr (DIR == DIR_FWD) {
-                    if (role == 0) {
-#pragma unroll
-                        for (int m = 0; m < 64; ++m) at<float>(slot, 2 * m * 128 + dst.o[(2 * m) & 7]) = y[m];
-                    } else {
-#pragma unroll
-                        for (int m = 0; m < 64; ++m)
-                            at<float>(slot, (2 * m + 1) * 128 + dst.o[(2 * m + 1) & 7]) = y[m];
-                    }
-                } else {
-                    if (role == 0) {
-#pragma unroll
-                        for (int j = 0; j < 64; ++j) at<float>(slot, j * 128 + dst.o[j & 7]) = y[j];
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 64; ++j) at<float>(slot, (127 - j) * 128 + dst.o[(127 - j) & 7]) = y[j];
-                    }
-                    group_sync(bar, C::GT);
-                    auto comb = [&](int j) {
-                        const uint32_t oa = j * 128 + dst.o[j & 7], ob = (127 - j) * 128 + dst.o[(127 - j) & 7];
-                        const float a = at<float>(slot, oa), b = at<float>(slot, ob);
-                        at<float>(slot, oa) = a + b;
-                        at<float>(slot, ob) = a - b;
-                    };
-                    if (role == 0) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) comb(j);
-                    } else {
-#pragma unroll
-                        for (int j = 32; j < 64; ++j) comb(j);
-                    }
-                }
-            }
+            for (int i = 0; i < 64; ++i) at<float>(slot, i * 128 + cv.o[i & 7]) = x[i];
         }
         group_sync(bar, C::GT);
     }
@@ -591,10 +231,11 @@ __device__ __forceinline__ void ring_coords(const RingParams &p, long long a, in
     }
 }
 
-template <int H, int W, int DIR, bool LAMF = false>
-__global__ void __launch_bounds__(RingCfg<H, W, DIR>::THREADS, 1) k_ring(const __grid_constant__ RingParams p)
+template <int DIR>
+__global__ void __launch_bounds__(RingCfg<DIR>::THREADS, 1) k_ring(const __grid_constant__ RingParams p)
 {
-    using C = RingCfg<H, W, DIR>;
+    using C = RingCfg<DIR>;
+    constexpr int H = C::H, W = C::W;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned slots
     const uint32_t raw = smem_u32(smem_raw);
@@ -728,8 +369,7 @@ __global__ void __launch_bounds__(RingCfg<H, W, DIR>::THREADS, 1) k_ring(const _
             break;
         }
         char *slot = smem + s * C::SLOT_BYTES;
-        if constexpr (H == W) ring_square<H, DIR, LAMF>(slot, gt, bar, p.sc, lam_s, p.lam);  // both end with a group barrier
-        else ring_rect<H, W, DIR, LAMF>(slot, gt, bar, p.sc, p.lam);
+        ring_array<DIR>(slot, gt, bar, p.sc, lam_s);  // ends with a group barrier
         fence_proxy_async_smem();  // the TMA store reads the slot through the async proxy
         group_sync(bar, C::GT);
         if (gt == 0) mbar_arrive(&done[s]);
@@ -737,12 +377,13 @@ __global__ void __launch_bounds__(RingCfg<H, W, DIR>::THREADS, 1) k_ring(const _
 }
 
 // ---------------------------------------------------------------- host side
-template <int H, int W, int DIR, bool LAMF = false>
+template <int DIR>
 static cudaError_t ring_launch_one(const DirScales &sc, const ExecGeom &g, unsigned int *status,
                                    cudaStream_t stream)
 {
-    using C = RingCfg<H, W, DIR>;
-    auto kern = k_ring<H, W, DIR, LAMF>;
+    using C = RingCfg<DIR>;
+    constexpr int H = C::H, W = C::W;
+    auto kern = k_ring<DIR>;
     static DeviceLaunchCache cache;
     int dev = 0, bps_dev = 0, num_sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -755,8 +396,8 @@ static cudaError_t ring_launch_one(const DirScales &sc, const ExecGeom &g, unsig
             if (r == cudaSuccess && bps < 1) r = cudaErrorInvalidConfiguration;
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
             if (r == cudaSuccess && debug_enabled())
-                fprintf(stderr, "[bdct] k_ring<%d,%d,%d>: %d slots of %d B, %d groups x %d warps + producer, smem %zu B\n",
-                        H, W, DIR, C::S, C::SLOT_BYTES, C::NG, C::GW, C::SMEM);
+                fprintf(stderr, "[bdct] k_ring<%d>: %d slots of %d B, %d groups x %d warps + producer, smem %zu B\n", DIR,
+                        C::S, C::SLOT_BYTES, C::NG, C::GW, C::SMEM);
             return r;
         },
         &bps_dev, &num_sms);
@@ -776,7 +417,7 @@ static cudaError_t ring_launch_one(const DirScales &sc, const ExecGeom &g, unsig
     p.in_off = g.in_off;
     p.out_off = g.out_off;
     p.lam = g.lam;
-    if ((DIR == DIR_SPEC || LAMF) && !g.lam) return cudaErrorInvalidValue;
+    if (DIR == DIR_SPEC && !g.lam) return cudaErrorInvalidValue;
     p.indexed = (g.in_off != nullptr || g.out_off != nullptr) ? 1 : 0;
     if (p.indexed) {
         if (!g.in_off || !g.out_off) return cudaErrorInvalidValue;
@@ -808,36 +449,14 @@ static cudaError_t ring_launch_one(const DirScales &sc, const ExecGeom &g, unsig
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-template <int H, int W>
-static cudaError_t ring_dir(Dir dir, const DirScales &sc, const ExecGeom &g, unsigned int *st, cudaStream_t s)
+cudaError_t ring_launch(Dir dir, const DirScales &sc, const ExecGeom &g, unsigned int *status, cudaStream_t stream)
 {
     switch (dir) {
-        case DIR_FWD: return ring_launch_one<H, W, DIR_FWD>(sc, g, st, s);
-        case DIR_INV: return ring_launch_one<H, W, DIR_INV>(sc, g, st, s);
-        case DIR_SPEC:
-            if constexpr (H == 64 && W == 64) return ring_launch_one<H, W, DIR_SPEC>(sc, g, st, s);
-            else return cudaErrorInvalidValue;  // composed by the caller
-        default: return ring_launch_one<H, W, DIR_RT>(sc, g, st, s);
+        case DIR_FWD: return ring_launch_one<DIR_FWD>(sc, g, status, stream);
+        case DIR_INV: return ring_launch_one<DIR_INV>(sc, g, status, stream);
+        case DIR_SPEC: return ring_launch_one<DIR_SPEC>(sc, g, status, stream);
+        default: return ring_launch_one<DIR_RT>(sc, g, status, stream);
     }
-}
-
-cudaError_t ring_forward_lam(int rows, int cols, const DirScales &sc, const ExecGeom &g, unsigned int *status,
-                             cudaStream_t stream)
-{
-    if (rows == 64 && cols == 128) return ring_launch_one<64, 128, DIR_FWD, true>(sc, g, status, stream);
-    if (rows == 128 && cols == 64) return ring_launch_one<128, 64, DIR_FWD, true>(sc, g, status, stream);
-    if (rows == 128 && cols == 128) return ring_launch_one<128, 128, DIR_FWD, true>(sc, g, status, stream);
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t ring_launch(int rows, int cols, Dir dir, const DirScales &sc, const ExecGeom &g, unsigned int *status,
-                        cudaStream_t stream)
-{
-    if (rows == 64 && cols == 64) return ring_dir<64, 64>(dir, sc, g, status, stream);
-    if (rows == 64 && cols == 128) return ring_dir<64, 128>(dir, sc, g, status, stream);
-    if (rows == 128 && cols == 64) return ring_dir<128, 64>(dir, sc, g, status, stream);
-    if (rows == 128 && cols == 128) return ring_dir<128, 128>(dir, sc, g, status, stream);
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace bdct

@@ -1,0 +1,298 @@
+// Steps of the FFT evaluation of a DCT line on packed couples, shared by the
+// line engine (fp32_lines.cu) and the on-chip kernels of sides 64 and 128
+// (fp32_block.cu).  fp32_lines.cu's header derives the factorization and the
+// packed form; this file holds its short FFTs, twiddles and the split.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "dct_cores.cuh"
+
+namespace bdct {
+
+// Radices of a line of N points: L = N/2 = R1 R2 R3 (R2 = 1: two steps).
+template <int N>
+struct LineSplit {
+    static constexpr int L = N / 2;
+    static constexpr int R1 = N == 64 ? 4 : N == 128 ? 8 : N == 192 ? 8 : N == 256 ? 16 : N == 384 ? 16
+                            : N == 512 ? 16 : N == 2048 ? 16 : N == 4096 ? 16 : 8;
+    static constexpr int R3 = N == 64 ? 8 : N == 128 ? 8 : N == 192 ? 12 : N == 256 ? 8 : N == 384 ? 12
+                            : N == 512 ? 16 : N == 4096 ? 16 : 8;
+    static constexpr int R2 = L / (R1 * R3);
+    static constexpr int M1 = L / R1;  // columns of the first step
+    static constexpr int C = L / R3;   // columns of the last step
+    static constexpr int U1 = R1 * (M1 / 2);               // twiddle entries (float4) of the first step,
+    static constexpr int U2 = R2 > 1 ? R2 * (R3 / 2) : 0;  // of the middle step,
+    static constexpr int US = L / 2 + L / 4;               // and of the split (L/2 slots of 24 bytes)
+    static constexpr int TAB = U1 + U2 + US;
+    static_assert(R1 * R2 * R3 == L && R1 % 2 == 0 && R3 % 2 == 0 && M1 % 2 == 0 && C % 2 == 0, "split");
+    static_assert(R2 == 1 || R2 % 2 == 0, "split");
+};
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// (ar + i ai) exp(-2 pi i j / R) on both halves
+template <int R>
+__device__ __forceinline__ void rotr(float2 ar, float2 ai, int j, float2 &rr, float2 &ri)
+{
+    if constexpr (R % 3 == 0) rot3(ar, ai, j, R, rr, ri);
+    else rot(ar, ai, 2 * j, R, rr, ri);
+}
+
+// Second half of a decimation-in-frequency FFT of R points: u_j = a_j +
+// a_{j+R/2} and v_j = a_j - a_{j+R/2} give the even and odd outputs.
+template <int R>
+__device__ __forceinline__ void fft_from_uv(float2 (&ur)[R / 2], float2 (&ui)[R / 2], float2 (&vr)[R / 2],
+                                            float2 (&vi)[R / 2], float2 (&dr)[R], float2 (&di)[R])
+{
+#pragma unroll
+    for (int j = 1; j < R / 2; ++j) {
+        float2 a, b;
+        rotr<R>(vr[j], vi[j], j, a, b);
+        vr[j] = a;
+        vi[j] = b;
+    }
+    FFT<R / 2, float2>::run(ur, ui);
+    FFT<R / 2, float2>::run(vr, vi);
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+        dr[2 * k] = ur[k]; di[2 * k] = ui[k];
+        dr[2 * k + 1] = vr[k]; di[2 * k + 1] = vi[k];
+    }
+}
+
+// Its transpose up to the last sums and differences (called with the real and
+// imaginary arrays exchanged: the conjugate FFT).
+template <int R>
+__device__ __forceinline__ void uv_from_fft(const float2 (&dr)[R], const float2 (&di)[R], float2 (&ur)[R / 2],
+                                            float2 (&ui)[R / 2], float2 (&vr)[R / 2], float2 (&vi)[R / 2])
+{
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+        ur[k] = dr[2 * k]; ui[k] = di[2 * k];
+        vr[k] = dr[2 * k + 1]; vi[k] = di[2 * k + 1];
+    }
+    FFT<R / 2, float2>::run(ur, ui);
+    FFT<R / 2, float2>::run(vr, vi);
+#pragma unroll
+    for (int j = 1; j < R / 2; ++j) {
+        float2 a, b;
+        rotr<R>(vr[j], vi[j], j, a, b);
+        vr[j] = a;
+        vi[j] = b;
+    }
+}
+
+// ------------------------------------------------------- first and middle steps
+// The couple of columns cc and MC-1-cc: x holds units cc + MC j, y units
+// MC-1-cc + MC j (j < R/2).  Results k: into x (k < R/2) and y, the slots
+// they came from, times the twiddles tw[k * (MC/2)].
+template <int R, int MC>
+__device__ __forceinline__ void step_forward(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2], dr[R], di[R];
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const float4 a = x[j], b = y[R / 2 - 1 - j];
+        ur[j] = make_float2(a.x + b.w, a.y + b.z);
+        ui[j] = make_float2(a.z + b.y, a.w + b.x);
+        vr[j] = make_float2(a.x - b.w, a.y - b.z);
+        vi[j] = make_float2(a.z - b.y, a.w - b.x);
+    }
+    fft_from_uv<R>(ur, ui, vr, vi, dr, di);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        float2 re = dr[k], im = di[k];
+        if (k > 0) {
+            const float4 t = tw[k * (MC / 2)];
+            const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
+            re = __ffma2_rn(di[k], s, __fmul2_rn(dr[k], c));
+            im = __ffma2_rn(neg2(dr[k]), s, __fmul2_rn(di[k], c));
+        }
+        const float4 o = make_float4(re.x, re.y, im.x, im.y);
+        if (k < R / 2) x[k] = o;
+        else y[k - R / 2] = o;
+    }
+}
+
+template <int R, int MC>
+__device__ __forceinline__ void step_adjoint(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
+{
+    float2 dr[R], di[R], ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const float4 o = k < R / 2 ? x[k < R / 2 ? k : 0] : y[k < R / 2 ? 0 : k - R / 2];
+        const float2 re = make_float2(o.x, o.y), im = make_float2(o.z, o.w);
+        dr[k] = re;
+        di[k] = im;
+        if (k > 0) {
+            const float4 t = tw[k * (MC / 2)];
+            const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
+            dr[k] = __ffma2_rn(neg2(im), s, __fmul2_rn(re, c));
+            di[k] = __ffma2_rn(re, s, __fmul2_rn(im, c));
+        }
+    }
+    uv_from_fft<R>(di, dr, ui, ur, vi, vr);
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        x[j] = make_float4(ur[j].x + vr[j].x, ur[j].y + vr[j].y, ui[j].x + vi[j].x, ui[j].y + vi[j].y);
+        y[R / 2 - 1 - j] = make_float4(ui[j].y - vi[j].y, ui[j].x - vi[j].x, ur[j].y - vr[j].y, ur[j].x - vr[j].x);
+    }
+}
+
+// ---------------------------------------------------------------- last step
+// Columns c (units x, index m) and its partner C-c (units w): D_k's halves
+// become Z_{c + C k} and conj Z_{L - c - C k}.
+template <int R>
+__device__ __forceinline__ void last_forward(const float4 (&x)[R / 2], const float4 (&w)[R / 2], float2 (&dr)[R],
+                                             float2 (&di)[R])
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const float4 a = x[j], b = x[R / 2 - 1 - j], p = w[j], q = w[R / 2 - 1 - j];
+        ur[j] = make_float2(a.x + b.w, p.x + q.w);
+        ui[j] = make_float2(a.z + b.y, -p.z - q.y);
+        vr[j] = make_float2(a.x - b.w, p.x - q.w);
+        vi[j] = make_float2(a.z - b.y, q.y - p.z);
+    }
+    fft_from_uv<R>(ur, ui, vr, vi, dr, di);
+}
+
+template <int R>
+__device__ __forceinline__ void last_adjoint(float4 (&x)[R / 2], float4 (&w)[R / 2], const float2 (&dr)[R],
+                                             const float2 (&di)[R])
+{
+    float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
+    uv_from_fft<R>(di, dr, ui, ur, vi, vr);
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+        const int m = R / 2 - 1 - j;
+        x[j].x = ur[j].x + vr[j].x;
+        x[m].w = ur[j].x - vr[j].x;
+        x[j].z = ui[j].x + vi[j].x;
+        x[m].y = ui[j].x - vi[j].x;
+        w[j].x = ur[j].y + vr[j].y;
+        w[m].w = ur[j].y - vr[j].y;
+        w[j].z = -ui[j].y - vi[j].y;
+        w[m].y = vi[j].y - ui[j].y;
+    }
+}
+
+// ---------------------------------------------------------------- the split
+// Four outputs from Z_k = (ar, ai) and conj Z_{L-k} = (br, bi): a = (y_k,
+// y_{L-k}), b = (y_{N-k}, y_{L+k}).  The table holds exp(-2 pi i k/N) = t.x -
+// i t.y and, times s_1 / 2, the pairs over (k, L-k) of Re W (t.z, t.w) and
+// -Im W (nwi).
+__device__ __forceinline__ void split_one(float ar, float ai, float br, float bi, const float4 t, const float2 nwi,
+                                          float2 &a, float2 &b)
+{
+    const float er = ar + br, ei = ai + bi, orr = ai - bi, oi = br - ar;
+    const float pr = fmaf(orr, t.x, oi * t.y), pi = fmaf(oi, t.x, -orr * t.y);
+    const float2 vr = make_float2(er + pr, er - pr), vi = make_float2(ei + pi, pi - ei);
+    const float2 wr = make_float2(t.z, t.w);
+    a = __ffma2_rn(vi, nwi, __fmul2_rn(vr, wr));
+    b = __ffma2_rn(neg2(vi), wr, __fmul2_rn(vr, nwi));
+}
+
+__device__ __forceinline__ void split_one_adjoint(float2 a, float2 b, const float4 t, const float2 nwi, float &ar,
+                                                  float &ai, float &br, float &bi)
+{
+    const float2 wr = make_float2(t.z, t.w);
+    const float2 vr = __ffma2_rn(b, nwi, __fmul2_rn(a, wr));
+    const float2 vi = __ffma2_rn(neg2(b), wr, __fmul2_rn(a, nwi));
+    const float er = vr.x + vr.y, pr = vr.x - vr.y, ei = vi.x - vi.y, pi = vi.x + vi.y;
+    const float orr = fmaf(pr, t.x, -pi * t.y), oi = fmaf(pr, t.y, pi * t.x);
+    ar = er - oi;
+    br = er + oi;
+    ai = ei + orr;
+    bi = ei - orr;
+}
+
+// The split's table by slot (k3 * (C/2) + c).
+struct SplitTable {
+    const float4 *ta;
+    const float2 *tb;
+    __device__ __forceinline__ float4 a(int i) const { return ta[i]; }
+    __device__ __forceinline__ float2 b(int i) const { return tb[i]; }
+};
+
+constexpr float kCos8 = 0.92387953251128675613f, kSin8 = 0.38268343236508977173f;  // of pi / 8
+constexpr float kRoot = 0.70710678118654752440f;
+
+// The outputs of couple c in slot order: slot k3 of c > 0 is k = c + C k3; of
+// c = 0, k = C k3 (k3 < R/2) and k = C/2 + C (k3 - R/2), with slot 0 holding
+// a = (y_0, y_L), b = (y_{L/2}, y_{3L/2}).  Column 0 pairs k3 with R - k3 in
+// its own half and column C/2 pairs k3 with R-1-k3, so each is one split.
+template <int R, int C>
+__device__ __forceinline__ void split_forward(int c, const float2 (&dr)[R], const float2 (&di)[R], SplitTable ts,
+                                              AxisScale s, float2 (&a)[R], float2 (&b)[R])
+{
+    if (c != 0) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            split_one(dr[k].x, di[k].x, dr[k].y, di[k].y, ts.a(k * (C / 2) + c), ts.b(k * (C / 2) + c), a[k], b[k]);
+    } else {
+        a[0] = make_float2((dr[0].x + di[0].x) * s.s0, (dr[0].x - di[0].x) * (kRoot * s.s1));
+        const float hr = dr[R / 2].x * s.s1, hi = di[R / 2].x * s.s1;
+        b[0] = make_float2(fmaf(hr, kCos8, -hi * kSin8), fmaf(hr, kSin8, hi * kCos8));
+#pragma unroll
+        for (int k = 1; k < R / 2; ++k)
+            split_one(dr[k].x, di[k].x, dr[R - k].x, -di[R - k].x, ts.a(k * (C / 2)), ts.b(k * (C / 2)), a[k], b[k]);
+#pragma unroll
+        for (int k = 0; k < R / 2; ++k)
+            split_one(dr[R - 1 - k].y, -di[R - 1 - k].y, dr[k].y, di[k].y, ts.a((R / 2 + k) * (C / 2)),
+                      ts.b((R / 2 + k) * (C / 2)), a[R / 2 + k], b[R / 2 + k]);
+    }
+}
+
+template <int R, int C>
+__device__ __forceinline__ void split_adjoint(int c, const float2 (&a)[R], const float2 (&b)[R], SplitTable ts,
+                                              AxisScale s, float2 (&dr)[R], float2 (&di)[R])
+{
+    if (c != 0) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            split_one_adjoint(a[k], b[k], ts.a(k * (C / 2) + c), ts.b(k * (C / 2) + c), dr[k].x, di[k].x, dr[k].y, di[k].y);
+    } else {
+        const float u = a[0].x * s.s0, v = a[0].y * (kRoot * s.s1);
+        dr[0].x = u + v;
+        di[0].x = u - v;
+        const float p = b[0].x * s.s1, q = b[0].y * s.s1;
+        dr[R / 2].x = fmaf(p, kCos8, q * kSin8);
+        di[R / 2].x = fmaf(q, kCos8, -p * kSin8);
+#pragma unroll
+        for (int k = 1; k < R / 2; ++k) {
+            float im;
+            split_one_adjoint(a[k], b[k], ts.a(k * (C / 2)), ts.b(k * (C / 2)), dr[k].x, di[k].x, dr[R - k].x, im);
+            di[R - k].x = -im;
+        }
+#pragma unroll
+        for (int k = 0; k < R / 2; ++k) {
+            float im;
+            split_one_adjoint(a[R / 2 + k], b[R / 2 + k], ts.a((R / 2 + k) * (C / 2)), ts.b((R / 2 + k) * (C / 2)), dr[R - 1 - k].y, im, dr[k].y,
+                              di[k].y);
+            di[R - 1 - k].y = -im;
+        }
+    }
+}
+
+// ------------------------------------------------------------ transposed side
+// visit(slot half, k): the output index of (a.x, a.y, b.x, b.y) of slot k3
+template <int N>
+struct SlotIndex {
+    using C = LineSplit<N>;
+    int lo, hi;   // first index of the lower and the upper half of the slots, minus C k3
+    bool zero;
+    __device__ __forceinline__ explicit SlotIndex(int c)
+        : lo(c), hi(c ? c : C::C / 2 - C::L / 2), zero(c == 0)
+    {
+    }
+    __device__ __forceinline__ int k(int k3) const { return C::C * k3 + (k3 < C::R3 / 2 ? lo : hi); }
+    __device__ __forceinline__ int ax(int k3) const { return k(k3); }
+    __device__ __forceinline__ int ay(int k3) const { return C::L - k(k3); }
+    __device__ __forceinline__ int bx(int k3) const { return (k3 == 0 && zero) ? C::L / 2 : N - k(k3); }
+    __device__ __forceinline__ int by(int k3) const { return (k3 == 0 && zero) ? 3 * C::L / 2 : C::L + k(k3); }
+};
+
+}  // namespace bdct
