@@ -293,41 +293,39 @@ extern "C" int bdct_plan_create(bdct_plan **plan, int rows, int cols, unsigned k
         if (st != BDCT_OK) { plan_free(p); return st; }
     } else {
         p->variant = 2;
-        // operator matrices: forward and inverse in the plan's norm, and the
-        // orthonormal pair for the round trip (which is normalized for both)
-        size_t per_dir = (size_t)rows * rows + (size_t)cols * cols;
-        size_t total = 0;
+        // operators: forward and inverse in the plan's norm, and the
+        // orthonormal pair for the round trip (which is normalized for both);
+        // whole matrices for the on-chip route, half tables for the passes
+        p->small = small_dense_supported(rows, cols);
+        const size_t sh = p->small ? (size_t)rows * rows : dense_table_floats(rows);
+        const size_t sw = p->small ? (size_t)cols * cols : dense_table_floats(cols);
         const bool need[3] = {(kind & BDCT_FORWARD) != 0, (kind & BDCT_INVERSE) != 0,
                               (kind & (BDCT_ROUNDTRIP | BDCT_SPECTRAL)) != 0};
-        size_t nmats = (need[0] ? 1 : 0) + (need[1] ? 1 : 0) + (need[2] ? 2 : 0);
-        total = nmats * per_dir;
+        const size_t nmats = (need[0] ? 1 : 0) + (need[1] ? 1 : 0) + (need[2] ? 2 : 0);
+        p->op_pair = sh + sw;
+        const size_t total = nmats * p->op_pair;
         e = cudaMalloc(&p->ops, total * sizeof(float));
         if (e != cudaSuccess) { plan_free(p); t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
         p->table_bytes = total * sizeof(float);
         size_t off = 0;
         auto gen = [&](int direction, int nrm, size_t &oh, size_t &ow) -> cudaError_t {
-            oh = off; off += (size_t)rows * rows;
-            ow = off; off += (size_t)cols * cols;
-            cudaError_t r = dense_gen_operator(p->ops + oh, rows, direction, nrm, 0);
-            if (r == cudaSuccess) r = dense_gen_operator(p->ops + ow, cols, direction, nrm, 0);
+            oh = off; off += sh;
+            ow = off; off += sw;
+            auto one = p->small ? dense_gen_operator : dense_gen_table;
+            cudaError_t r = one(p->ops + oh, rows, direction, nrm, 0);
+            if (r == cudaSuccess) r = one(p->ops + ow, cols, direction, nrm, 0);
             return r;
         };
         if (need[0] && e == cudaSuccess) e = gen(1, norm, p->op_h_off[DIR_FWD], p->op_w_off[DIR_FWD]);
         if (need[1] && e == cudaSuccess) e = gen(2, norm, p->op_h_off[DIR_INV], p->op_w_off[DIR_INV]);
         if (need[2] && e == cudaSuccess) {
-            // RT forward half uses slot DIR_RT; its inverse half follows it
-            size_t fh, fw, ih, iw;
-            e = gen(1, BDCT_NORM_ORTHO, fh, fw);
+            // the forward half in slot DIR_RT; the inverse half follows it, op_pair later
+            size_t ih, iw;
+            e = gen(1, BDCT_NORM_ORTHO, p->op_h_off[DIR_RT], p->op_w_off[DIR_RT]);
             if (e == cudaSuccess) e = gen(2, BDCT_NORM_ORTHO, ih, iw);
-            p->op_h_off[DIR_RT] = fh;
-            p->op_w_off[DIR_RT] = fw;
-            (void)ih; (void)iw;  // located at fh + per_dir
         }
         if (e != cudaSuccess) { plan_free(p); return cuda_fail(e); }
-        if (small_dense_supported(rows, cols)) {
-            // every pass in shared memory (small_dense.cu): no workspace
-            p->small = true;
-        } else {
+        if (!p->small) {  // the on-chip route (small_dense.cu) keeps no workspace
             const size_t arr_bytes = (size_t)rows * cols * sizeof(float);
             long long chunk = (long long)(kChunkBytes / arr_bytes);
             if (chunk < 1) chunk = 1;
@@ -429,7 +427,7 @@ static int run_small(const bdct_plan *p, Dir dir, const ExecGeom &g, cudaStream_
     const Dir mdir = dir == DIR_SPEC ? DIR_RT : dir;  // the spectral direction uses the orthonormal pair
     const float *oph = p->ops + p->op_h_off[mdir];
     const float *opw = p->ops + p->op_w_off[mdir];
-    const size_t per_dir = (size_t)h * h + (size_t)w * w;
+    const size_t per_dir = p->op_pair;
     const bool pair = dir == DIR_RT || dir == DIR_SPEC;
     const int axis[4] = {0, 1, 1, 0};
     const float *ops[4] = {opw, oph, oph + per_dir, opw + per_dir};
@@ -449,36 +447,26 @@ static int run_separable(const bdct_plan *p, Dir dir, const float *in, const lon
     const Dir mdir = dir == DIR_SPEC ? DIR_RT : dir;  // the spectral direction uses the orthonormal pair
     const float *oph = p->ops + p->op_h_off[mdir];
     const float *opw = p->ops + p->op_w_off[mdir];
-    const size_t per_dir = (size_t)h * h + (size_t)w * w;
     float *w1 = p->work;
     float *w2 = p->work + (size_t)p->chunk_arrays * hw;
     for (long long b0 = 0; b0 < count; b0 += p->chunk_arrays) {
         const long long nb = (count - b0) < p->chunk_arrays ? (count - b0) : p->chunk_arrays;
-        const float *src = in + b0 * hw;
-        float *dst = out + b0 * hw;
+        const float *src = in_off ? in : in + b0 * hw;
+        float *dst = out_off ? out : out + b0 * hw;
         const long long *ioff = in_off ? in_off + b0 : nullptr;
         const long long *ooff = out_off ? out_off + b0 : nullptr;
-        cudaError_t e;
-        // first pass: rows of the input into w1
-        if (ioff) e = dense_pass_rows_indexed(in, ioff, w1, opw, h, w, nb, s);
-        else e = dense_pass_rows(src, w1, opw, (int)(nb * h), w, s);
-        if (dir != DIR_RT && dir != DIR_SPEC) {
-            if (e == cudaSuccess) {
-                if (ooff) e = dense_pass_cols_indexed(w1, out, ooff, oph, h, w, nb, s);
-                else e = dense_pass_cols(w1, dst, oph, h, w, nb, s);
-            }
+        const bool pair = dir == DIR_RT || dir == DIR_SPEC, inv = dir == DIR_INV;
+        cudaError_t e = dense_pass({src, w1, opw, h, w, nb, true, inv, ioff, nullptr}, s);
+        if (!pair) {
+            if (e == cudaSuccess) e = dense_pass({w1, dst, oph, h, w, nb, false, inv, nullptr, ooff}, s);
         } else {
-            // forward core, then the adjoint core (orthonormal pair)
-            const float *ioph = oph + per_dir, *iopw = opw + per_dir;
-            // the orthonormal spectrum of the chunk (times Lambda as it is
-            // stored, for the spectral direction: Eq. 4)
-            if (e == cudaSuccess)
-                e = dense_pass_cols_lam(w1, w2, oph, h, w, nb, dir == DIR_SPEC ? p->spec_plain : nullptr, s);
-            if (e == cudaSuccess) e = dense_pass_cols(w2, w1, ioph, h, w, nb, s);
-            if (e == cudaSuccess) {
-                if (ooff) e = dense_pass_rows_out_indexed(w1, out, ooff, iopw, h, w, nb, s);
-                else e = dense_pass_rows(w1, dst, iopw, (int)(nb * h), w, s);
-            }
+            // the orthonormal spectrum (times Lambda as it is stored, for the
+            // spectral direction: Eq. 4), then the adjoint pair
+            const float *ioph = oph + p->op_pair, *iopw = opw + p->op_pair;
+            const float *lam = dir == DIR_SPEC ? p->spec_plain : nullptr;
+            if (e == cudaSuccess) e = dense_pass({w1, w2, oph, h, w, nb, false, false, nullptr, nullptr, lam}, s);
+            if (e == cudaSuccess) e = dense_pass({w2, w1, ioph, h, w, nb, false, true}, s);
+            if (e == cudaSuccess) e = dense_pass({w1, dst, iopw, h, w, nb, true, true, nullptr, ooff}, s);
         }
         if (e != cudaSuccess) return cuda_fail(e);
     }

@@ -169,21 +169,4 @@ cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, cons
                     unsigned int *status, cudaStream_t stream);
 size_t tg_split_elems(long long rows, int K);
 
-// ---- dense_passes.cu
-// Separable dense passes through a workspace, any shape.  `op_h`, `op_w` are
-// the h x h and w x w FP32 operator matrices of one direction (scales folded
-// in); the result is op_h X op_w^T for every array.
-cudaError_t dense_gen_operator(float *op, int n, int direction, int norm, cudaStream_t stream);
-cudaError_t dense_pass_rows(const float *in, float *out, const float *op_w, int rows_total, int w,
-                            cudaStream_t stream);
-cudaError_t dense_pass_cols(const float *in, float *out, const float *op_h, int h, int w,
-                            long long count, cudaStream_t stream);
-// Indexed variants: array b of the batch at base + off[b] (element offsets).
-cudaError_t dense_pass_rows_indexed(const float *in, const long long *in_off, float *out, const float *op_w, int h,
-                                    int w, long long count, cudaStream_t stream);
-cudaError_t dense_pass_rows_out_indexed(const float *in, float *out, const long long *out_off, const float *op_w,
-                                        int h, int w, long long count, cudaStream_t stream);
-cudaError_t dense_pass_cols_indexed(const float *in, float *out, const long long *out_off, const float *op_h, int h,
-                                    int w, long long count, cudaStream_t stream);
-
 }  // namespace bdct

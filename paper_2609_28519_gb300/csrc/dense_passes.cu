@@ -3,18 +3,37 @@
 // Eq. 2 of the BRiDCT paper is the sandwich M_h X M_w^T, with M = Q_n for the
 // forward transform (Eq. 1) and M = Q_n^T for the inverse; Section 7.1 makes
 // h and w independent.  Here the two 1D operators are applied as two FP32
-// matrix products: every row first (T = X M_w^T), then every column
-// (Y = M_h T).  A direct length-n evaluation costs n multiply-adds per point
-// (Section 1.2), so this route serves shapes without a fused fast kernel --
-// non-power-of-two sides such as 768 (which Eq. 1 defines for any n) and
-// large whole arrays -- through a plan-owned workspace.
+// matrix products, one pass along each axis, through a plan-owned workspace:
+// the route of shapes without a fast kernel (sides above 64 with other
+// factors, which Eq. 1 defines for any n) and of the allocation-free entry
+// point.
 //
-// The operator tables are generated on the GPU in FP64 (cos with the
-// argument reduced exactly in integers) and rounded once to FP32.
+// Half products.  cos(pi (2j+1) k / (2n)) is even about the middle of the
+// line for even k and odd for odd k, so with s_j = x_j + x_{n-1-j} and d_j =
+// x_j - x_{n-1-j} (j < n/2) the even outputs are a product with s and the odd
+// ones a product with d, each half as long: n/2 multiply-adds per point
+// instead of n.  The inverse runs it backwards: a from the even coefficients,
+// b from the odd ones, x_j = a_j + b_j, x_{n-1-j} = a_j - b_j.
+//
+// Tiles.  The two products run in the halves of packed pairs: (s_j, d_j) of a
+// line times (M_even, M_odd) of an output pair is one instruction, and neither
+// operand has to be duplicated or moved to form its pair.  A CTA takes 64
+// lines and up to 64 output pairs, a thread 8 lines x 4 pairs.  Per contraction
+// index it reads six float4 for 64 multiply-adds; a warp's lanes are 8 lines
+// by 4 output quads, so each of those reads is two shared-memory wavefronts
+// and the multiply-adds, not the reads, bound the loop.  The outputs are dealt
+// to the tiles evenly in steps of 4, so a side of 100 fills 52 columns for its
+// 50 pairs.  Sums and differences are formed once, as a chunk of 16 indices
+// goes from global to shared memory; the next chunk's loads are in flight
+// during the current products.  Each chunk's products are summed on their own
+// and added to the running total, so the rounding error grows like 16 + n/32
+// rather than n/2.
+//
 #include <cuda_runtime.h>
 
 #include "bdct_internal.h"
 #include "dense_passes.h"
+#include "ptx.cuh"
 
 namespace bdct {
 
@@ -32,20 +51,25 @@ __device__ double cos_half_turns(long long m, long long n)
     return sign * cospi((double)r / (double)d);
 }
 
-// direction 1 = forward: op[k][j] = s_k cos(pi (2j+1) k / (2n))
-// direction 2 = inverse: op[j][k] = s_k cos(pi (2j+1) k / (2n))
+// s_k cos(pi (2j+1) k / (2n))
 // norm 0 (orthonormal): s_k = alpha_k of Eq. 1
-// norm 1 (REDFT pair):  forward s_k = 2, inverse s_0 = 1, s_k = 2
+// norm 1 (REDFT pair):  forward (direction 1) s_k = 2, inverse s_0 = 1, s_k = 2
+__device__ double operator_entry(int k, int j, int n, int direction, int norm)
+{
+    double s;
+    if (norm == 0) s = (k == 0) ? sqrt(1.0 / n) : sqrt(2.0 / n);
+    else if (direction == 1) s = 2.0;
+    else s = (k == 0) ? 1.0 : 2.0;
+    return s * cos_half_turns((2LL * j + 1) * k, n);
+}
+
+// direction 1 = forward: op[k][j], direction 2 = inverse: op[j][k]
 __global__ void k_gen_operator(float *op, int n, int direction, int norm)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)n * n) return;
     const int k = (int)(idx / n), j = (int)(idx % n);
-    double s;
-    if (norm == 0) s = (k == 0) ? sqrt(1.0 / n) : sqrt(2.0 / n);
-    else if (direction == 1) s = 2.0;
-    else s = (k == 0) ? 1.0 : 2.0;
-    const double v = s * cos_half_turns((2LL * j + 1) * k, n);
+    const double v = operator_entry(k, j, n, direction, norm);
     if (direction == 1) op[(size_t)k * n + j] = (float)v;
     else op[(size_t)j * n + k] = (float)v;
 }
@@ -57,151 +81,335 @@ cudaError_t dense_gen_operator(float *op, int n, int direction, int norm, cudaSt
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- GEMM tile
-// C[b][m][n] = sum_k A[b][m][k] B[b][k][n] with arbitrary element strides.
-// 64 x 64 output tile, K step 16, 256 threads, 4 x 4 outputs per thread.
-struct GemmArgs {
-    const float *A; long long sAb, sAm, sAk;
-    const float *B; long long sBb, sBk, sBn;
-    float *C; long long sCb, sCm, sCn;
-    int M, N, K;
-    // indexed batch: batch element b of A / B / C starts at off[b] (element offsets)
-    const long long *aoff = nullptr, *boff = nullptr, *coff = nullptr;
-    long long b0 = 0;  // index of this launch's first batch element in the offset arrays
-    const float *lam = nullptr;  // or null: C[b][m][n] *= lam[m * N + n] as it is stored
+namespace {
+
+constexpr int kThreads = 128;
+constexpr int kLines = 64;          // lines per CTA
+constexpr int kChunk = 16;          // contraction indices per stage
+constexpr int kPitch = kLines + 2;  // stage row pitch (pairs)
+constexpr int kMaxTile = 64;        // output pairs per CTA at most
+constexpr int kResident = 2;        // CTAs per SM: no spills (three, with 168 registers, measured slower)
+
+// Half operators of side n: pairs (even, odd) [kp][np], zero in the padding;
+// kp, np = n/2 rounded up to whole chunks and tiles.
+struct DenseShape {
+    int n, nh, tiles, tc, np, kp;
+    __host__ __device__ explicit DenseShape(int n_)
+        : n(n_), nh((n_ + 1) / 2), tiles((nh + kMaxTile - 1) / kMaxTile),
+          tc(((nh + tiles - 1) / tiles + 3) / 4), np(tiles * tc * 4), kp((nh + kChunk - 1) / kChunk * kChunk)
+    {
+    }
 };
 
-__global__ void __launch_bounds__(256) k_gemm_strided(GemmArgs g)
+// forward: t[j][o] = M[2o + e][j]; inverse: t[o][j] = M^T[j][2o + e], e the half
+__global__ void k_gen_half(float2 *t, DenseShape q, int direction, int norm)
 {
-    __shared__ float As[16][64 + 4];
-    __shared__ float Bs[16][64 + 4];
-    const int b = blockIdx.z;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const float *A = g.aoff ? g.A + g.aoff[g.b0 + b] : g.A + b * g.sAb;
-    const float *B = g.boff ? g.B + g.boff[g.b0 + b] : g.B + b * g.sBb;
-    float *C = g.coff ? g.C + g.coff[g.b0 + b] : g.C + b * g.sCb;
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)q.kp * q.np) return;
+    const int r = (int)(idx / q.np), c = (int)(idx % q.np);
+    const int k = 2 * (direction == 1 ? c : r), j = direction == 1 ? r : c;
+    float2 v = make_float2(0.f, 0.f);
+    if (j < q.nh) {
+        if (k < q.n) v.x = (float)operator_entry(k, j, q.n, direction, norm);
+        if (k + 1 < q.n) v.y = (float)operator_entry(k + 1, j, q.n, direction, norm);
+    }
+    t[idx] = v;
+}
+
+struct DenseParams {
+    const float *in;
+    float *out;
+    const float2 *table;
+    const long long *in_off, *out_off;  // indexed arrays (element offsets), or null
+    const float *lam;                   // columns, forward: output (k, l) times lam[k * w + l]; or null
+    long long lines;                    // rows or columns of all arrays
+    int h, w;
+};
+
+// ROWS: lines are rows (contiguous); else columns, four neighbours at a time.
+template <bool ROWS, bool INV>
+__global__ void __launch_bounds__(kThreads, kResident) k_dense(const DenseParams p)
+{
+    __shared__ __align__(16) float2 as[2][kChunk][kPitch];
+    __shared__ __align__(16) float2 bs[2][kChunk][kMaxTile];
+    const int n = ROWS ? p.w : p.h, w = p.w;
+    const DenseShape q(n);
     const int tid = threadIdx.x;
-    const int tm = (tid / 16) * 4, tn = (tid % 16) * 4;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < g.K; k0 += 16) {
-        for (int q = tid; q < 16 * 64; q += 256) {
-            // A tile: 64 (m) x 16 (k); B tile: 16 (k) x 64 (n)
-            const int am = q / 16, ak = q % 16;
-            const int gm = m0 + am, gk = k0 + ak;
-            As[ak][am] = (gm < g.M && gk < g.K) ? A[gm * g.sAm + gk * g.sAk] : 0.0f;
-            const int bk = q / 64, bn = q % 64;
-            const int gk2 = k0 + bk, gn = n0 + bn;
-            Bs[bk][bn] = (gk2 < g.K && gn < g.N) ? B[gk2 * g.sBk + gn * g.sBn] : 0.0f;
-        }
-        __syncthreads();
-        // two-level summation: each K tile of 16 products is summed on its own
-        // and then added to the running total, so the rounding error grows
-        // like 16 + K/16 rather than K for long dot products
-        float part[4][4] = {};
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float a[4], bb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = As[kk][tm + i]; bb[i] = Bs[kk][tn + i]; }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) part[i][j] = fmaf(a[i], bb[j], part[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
-        __syncthreads();
+    const long long per = ROWS ? p.h : p.w;  // lines per array
+    const int tile = blockIdx.x % q.tiles;
+    const long long line0 = (long long)(blockIdx.x / q.tiles) * kLines;
+
+    pdl_launch_dependents();
+    pdl_wait_prerequisites();
+
+    // where the CTA's lines begin (a column's first element), in the input and
+    // the output: the divisions are done once per line, not per use
+    __shared__ long long off_in[kLines], off_out[kLines];
+    if (tid < kLines && line0 + tid < p.lines) {
+        const long long b = (line0 + tid) / per, i = line0 + tid - b * per;
+        const long long in_array = ROWS ? i * w : i, packed = b * (long long)p.h * w;
+        off_in[tid] = (p.in_off ? p.in_off[b] : packed) + in_array;
+        off_out[tid] = (p.out_off ? p.out_off[b] : packed) + in_array;
     }
+    __syncthreads();
+
+    // ---- this thread's two tasks of a chunk: two float4 each
+    const float *pa[2], *pb[2];  // of the next chunk: moved on by each fetch
+    int kk[2], ln[2];
+    bool live[2];
+    const long long step_a = ROWS ? (INV ? 2 * kChunk : kChunk) : (INV ? 2 * kChunk : kChunk) * (long long)w;
+    const long long step_b = INV ? step_a : -step_a;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gm = m0 + tm + i, gn = n0 + tn + j;
-            if (gm < g.M && gn < g.N) C[gm * g.sCm + gn * g.sCn] = g.lam ? acc[i][j] * g.lam[gm * g.N + gn] : acc[i][j];
+    for (int u = 0; u < 2; ++u) {
+        if (ROWS) {
+            kk[u] = 4 * (tid % 4);  // four contraction indices of one line
+            ln[u] = tid / 4 + 32 * u;
+        } else {
+            kk[u] = tid / 16 + 8 * u;  // one contraction index of four columns
+            ln[u] = 4 * (tid % 16);
         }
-}
-
-static cudaError_t gemm(const GemmArgs &g, long long batch, cudaStream_t stream)
-{
-    if (batch <= 0 || g.M <= 0 || g.N <= 0) return cudaSuccess;
-    // grid.z is limited to 65535: split long batches
-    for (long long b0 = 0; b0 < batch; b0 += 65535) {
-        const long long nb = (batch - b0) < 65535 ? (batch - b0) : 65535;
-        GemmArgs s = g;
-        if (g.aoff || g.boff || g.coff) s.b0 = g.b0 + b0;
-        if (!g.aoff) s.A += b0 * g.sAb;
-        if (!g.boff) s.B += b0 * g.sBb;
-        if (!g.coff) s.C += b0 * g.sCb;
-        dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, (unsigned)nb);
-        if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-        k_gemm_strided<<<grid, 256, 0, stream>>>(s);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        live[u] = line0 + ln[u] < p.lines;
+        const float *base = live[u] ? p.in + off_in[ln[u]] : p.in;
+        // forward: index k and its mirror; inverse: coefficients 2k and 2k + 1 (rows: eight from 2k)
+        pa[u] = base + (INV ? 2 * kk[u] : kk[u]) * (ROWS ? 1ll : (long long)w);
+        pb[u] = base + (INV ? (ROWS ? 2 * kk[u] + 4 : 2 * kk[u] + 1) : (ROWS ? n - 4 - kk[u] : n - 1 - kk[u])) *
+                           (ROWS ? 1ll : (long long)w);
     }
-    return cudaSuccess;
-}
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 va[2], vb[2];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = k0 + kk[u];
+            const bool a = live[u] && (INV ? 2 * k < n : k < q.nh);
+            const bool b = live[u] && (INV ? (ROWS ? 2 * k + 4 : 2 * k + 1) < n : k < q.nh);
+            va[u] = a ? __ldcg(reinterpret_cast<const float4 *>(pa[u])) : zero;
+            vb[u] = b ? __ldcg(reinterpret_cast<const float4 *>(pb[u])) : zero;
+            pa[u] += step_a;
+            pb[u] += step_b;
+        }
+    };
+    auto put = [&](int st, int k0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float4 a = va[u], b = vb[u];
+            if (ROWS) {
+                float2 v[4];
+                if (!INV) {
+                    const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.w, b.z, b.y, b.x};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)  // past the middle: the mirrored pairs again, left out
+                        v[i] = k0 + kk[u] + i < q.nh ? make_float2(x[i] + y[i], x[i] - y[i]) : make_float2(0.f, 0.f);
+                } else {
+                    v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
+                    v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) as[st][kk[u] + i][ln[u]] = v[i];
+            } else {
+                float4 s = a, d = b;
+                if (!INV) {
+                    if (2 * (k0 + kk[u]) + 1 == n) {  // the middle of an odd length, its own mirror
+                        d = zero;
+                    } else {
+                        s = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+                        d = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+                    }
+                }
+                float4 *o = reinterpret_cast<float4 *>(&as[st][kk[u]][ln[u]]);
+                o[0] = make_float4(s.x, d.x, s.y, d.y);
+                o[1] = make_float4(s.z, d.z, s.w, d.w);
+            }
+        }
+    };
+    const float2 *tab = p.table + tile * (q.tc * 4);
+    auto fetch_op = [&](int st, int k0) {
+        // eight threads a row, 16 bytes at a time
+        const int r = tid / 8;
+        const float2 *g = tab + (long long)(k0 + r) * q.np;
+        for (int c = tid % 8; c < 2 * q.tc; c += 8) cp_async16(&bs[st][r][2 * c], g + 2 * c);
+        cp_async_commit();
+    };
+    static_assert(kThreads == 8 * kChunk, "operator rows");
 
-// Every row of a [rows_total x w] matrix times op_w^T: out[r][l] = sum_j in[r][j] op_w[l][j].
-cudaError_t dense_pass_rows(const float *in, float *out, const float *op_w, int rows_total, int w,
-                            cudaStream_t stream)
-{
-    // split the row count so that grid.y (tiles of 64 rows) stays within limits
-    const int max_rows = 65535 * 64;
-    for (long long r0 = 0; r0 < rows_total; r0 += max_rows) {
-        const int nr = (int)((rows_total - r0) < max_rows ? (rows_total - r0) : max_rows);
-        GemmArgs g{in + r0 * w, 0, w, 1, op_w, 0, 1, w, out + r0 * w, 0, w, 1, nr, w, w};
-        cudaError_t e = gemm(g, 1, stream);
-        if (e != cudaSuccess) return e;
+    // ---- compute role: lines 2 la + 16 i and the next (i < 4), output pairs 4 tc ..
+    // lanes: output quad from bits 0 and 2, lines from bits 1, 3 and 4, so that
+    // lanes i and i^1 read the same lines and lanes i and i^2 the same outputs
+    // (a 16-byte read then takes two wavefronts instead of four)
+    const int lane = tid % 32;
+    const int tc = tid / 32 * 4 + (lane & 1) + (lane >> 1 & 2), la = (lane >> 1 & 1) + (lane >> 2 & 6);
+    const bool active = tc < q.tc;
+    float2 acc[8][4];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[r][o] = make_float2(0.f, 0.f);
+    fetch_op(0, 0);
+    fetch(0);
+    put(0, 0);
+    cp_async_wait_group<0>();
+    __syncthreads();
+    for (int k0 = 0, st = 0; k0 < q.nh; k0 += kChunk, st ^= 1) {
+        const bool more = k0 + kChunk < q.nh;
+        if (more) {
+            fetch_op(st ^ 1, k0 + kChunk);
+            fetch(k0 + kChunk);
+        }
+        if (active) {
+            float2 part[8][4];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) part[r][o] = make_float2(0.f, 0.f);
+            auto step = [&](int k) {
+                float2 x[8], m[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(&as[st][k][2 * la + 16 * i]);
+                    x[2 * i] = make_float2(v.x, v.y);
+                    x[2 * i + 1] = make_float2(v.z, v.w);
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(&bs[st][k][4 * tc + 2 * i]);
+                    m[2 * i] = make_float2(v.x, v.y);
+                    m[2 * i + 1] = make_float2(v.z, v.w);
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) part[r][o] = __ffma2_rn(x[r], m[o], part[r][o]);
+            };
+            if (k0 + kChunk <= q.nh) {
+#pragma unroll
+                for (int k = 0; k < kChunk; ++k) step(k);
+            } else {
+                const int last = (q.nh - k0 + 1) / 2;  // the padding is zero
+#pragma unroll 1
+                for (int k = 0; k < last; ++k) {
+                    step(2 * k);
+                    step(2 * k + 1);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) acc[r][o] = __fadd2_rn(acc[r][o], part[r][o]);
+        }
+        if (more) {
+            put(st ^ 1, k0 + kChunk);
+            cp_async_wait_group<0>();
+            __syncthreads();
+        }
     }
-    return cudaSuccess;
+    if (!active) return;
+    const int o0 = 4 * (tile * q.tc + tc);  // first output pair of this thread
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const long long line = line0 + 2 * la + 16 * i;
+        if (line >= p.lines) continue;
+        if (!ROWS) {
+            // two neighbouring columns (w is a multiple of 4, so they share an array)
+            float *dst = p.out + off_out[2 * la + 16 * i];
+            const float *lam = !INV && p.lam ? p.lam + line % w : nullptr;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const float2 u = acc[2 * i][o], v = acc[2 * i + 1][o];
+                const int j = o0 + o;
+                if (j >= q.nh) continue;
+                float2 a, b;
+                int ka, kb;
+                if (!INV) {
+                    a = make_float2(u.x, v.x);
+                    b = make_float2(u.y, v.y);
+                    ka = 2 * j;
+                    kb = 2 * j + 1;
+                } else {
+                    a = make_float2(u.x + u.y, v.x + v.y);
+                    b = make_float2(u.x - u.y, v.x - v.y);
+                    ka = j;
+                    kb = n - 1 - j;
+                }
+                if (!INV && lam) {
+                    const float2 l = __ldg(reinterpret_cast<const float2 *>(lam + (long long)ka * w));
+                    a = make_float2(a.x * l.x, a.y * l.y);
+                    if (kb < n) {
+                        const float2 m = __ldg(reinterpret_cast<const float2 *>(lam + (long long)kb * w));
+                        b = make_float2(b.x * m.x, b.y * m.y);
+                    }
+                }
+                *reinterpret_cast<float2 *>(dst + (long long)ka * w) = a;
+                if (kb < n) *reinterpret_cast<float2 *>(dst + (long long)kb * w) = b;
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                if (line + r >= p.lines) continue;
+                float *dst = p.out + off_out[2 * la + 16 * i + r];
+                const float2 *v = acc[2 * i + r];
+                if (!INV) {
+                    // coefficients 2 o0 .. 2 o0 + 7
+                    if (2 * o0 < n) *reinterpret_cast<float4 *>(dst + 2 * o0) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+                    if (2 * o0 + 4 < n)
+                        *reinterpret_cast<float4 *>(dst + 2 * o0 + 4) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+                } else if (o0 + 4 <= q.nh) {
+                    *reinterpret_cast<float4 *>(dst + o0) =
+                        make_float4(v[0].x + v[0].y, v[1].x + v[1].y, v[2].x + v[2].y, v[3].x + v[3].y);
+                    *reinterpret_cast<float4 *>(dst + n - 4 - o0) =
+                        make_float4(v[3].x - v[3].y, v[2].x - v[2].y, v[1].x - v[1].y, v[0].x - v[0].y);
+                } else {
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+                        if (o0 + o < q.nh) {
+                            dst[o0 + o] = v[o].x + v[o].y;
+                            dst[n - 1 - o0 - o] = v[o].x - v[o].y;
+                        }
+                }
+            }
+        }
+    }
 }
 
-// Every column of `count` h x w arrays: out[b][k][l] = sum_i op_h[k][i] in[b][i][l].
-cudaError_t dense_pass_cols(const float *in, float *out, const float *op_h, int h, int w,
-                            long long count, cudaStream_t stream)
+template <bool ROWS, bool INV>
+cudaError_t launch(const DenseParams &p, cudaStream_t stream)
 {
-    return dense_pass_cols_lam(in, out, op_h, h, w, count, nullptr, stream);
+    const DenseShape q(ROWS ? p.w : p.h);
+    const long long blocks = (p.lines + kLines - 1) / kLines * q.tiles;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_dense<ROWS, INV>, p);
 }
 
-cudaError_t dense_pass_cols_lam(const float *in, float *out, const float *op_h, int h, int w, long long count,
-                                const float *lam, cudaStream_t stream)
+}  // namespace
+
+size_t dense_table_floats(int n)
 {
-    const long long hw = (long long)h * w;
-    GemmArgs g{op_h, 0, h, 1, in, hw, w, 1, out, hw, w, 1, h, w, h};
-    g.lam = lam;
-    return gemm(g, count, stream);
+    const DenseShape q(n);
+    return (size_t)2 * q.kp * q.np;
 }
 
-// Indexed batch: rows pass reads array b at in + in_off[b] and writes the
-// workspace contiguously; the columns pass reads the workspace and writes
-// array b at out + out_off[b].
-cudaError_t dense_pass_rows_indexed(const float *in, const long long *in_off, float *out, const float *op_w, int h,
-                                    int w, long long count, cudaStream_t stream)
+cudaError_t dense_gen_table(float *t, int n, int direction, int norm, cudaStream_t stream)
 {
-    const long long hw = (long long)h * w;
-    GemmArgs g{in, 0, w, 1, op_w, 0, 1, w, out, hw, w, 1, h, w, w};
-    g.aoff = in_off;
-    return gemm(g, count, stream);
+    const long long total = (long long)dense_table_floats(n) / 2;
+    k_gen_half<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(reinterpret_cast<float2 *>(t), DenseShape(n), direction,
+                                                                     norm);
+    return cudaGetLastError();
 }
 
-cudaError_t dense_pass_rows_out_indexed(const float *in, float *out, const long long *out_off, const float *op_w, int h,
-                                        int w, long long count, cudaStream_t stream)
+cudaError_t dense_pass(const DensePass &d, cudaStream_t stream)
 {
-    const long long hw = (long long)h * w;
-    GemmArgs g{in, hw, w, 1, op_w, 0, 1, w, out, 0, w, 1, h, w, w};
-    g.coff = out_off;
-    return gemm(g, count, stream);
-}
-
-cudaError_t dense_pass_cols_indexed(const float *in, float *out, const long long *out_off, const float *op_h, int h,
-                                    int w, long long count, cudaStream_t stream)
-{
-    const long long hw = (long long)h * w;
-    GemmArgs g{op_h, 0, h, 1, in, hw, w, 1, out, 0, w, 1, h, w, h};
-    g.coff = out_off;
-    return gemm(g, count, stream);
+    if (d.count <= 0) return cudaSuccess;
+    DenseParams p{d.in, d.out, reinterpret_cast<const float2 *>(d.table), d.in_off, d.out_off, d.lam, d.count * (d.rows ? d.h : d.w), d.h, d.w};
+    if (d.rows) return d.inverse ? launch<true, true>(p, stream) : launch<true, false>(p, stream);
+    return d.inverse ? launch<false, true>(p, stream) : launch<false, false>(p, stream);
 }
 
 }  // namespace bdct

@@ -9,7 +9,7 @@
 // For them this file offers one entry point that needs no plan and allocates
 // nothing: it runs the separable dense route (operator matrices, then a row
 // pass and a column pass through an intermediate buffer) with all of its
-// scratch -- the operator matrices and the intermediates -- in one
+// scratch -- the operator tables and the intermediates -- in one
 // file-scope device array of fixed size.
 //
 // Host code may not pass that array's name to a kernel: on the host the name
@@ -22,6 +22,7 @@
 #include <mutex>
 
 #include "bdct_internal.h"
+#include "dense_passes.h"
 
 namespace bdct {
 
@@ -79,30 +80,30 @@ extern "C" int bdct_execute_noalloc(int rows, int cols, unsigned kind, int norm,
     if (e != cudaSuccess) return BDCT_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
-    // scratch layout: operator matrices first, then the intermediates
-    const size_t per_dir = (size_t)rows * rows + (size_t)cols * cols;
+    // scratch layout: operator tables first, then the intermediates
+    const size_t th = dense_table_floats(rows), per_dir = th + dense_table_floats(cols);
     const bool rt = kind == BDCT_ROUNDTRIP;
     const size_t mats = rt ? 2 * per_dir : per_dir;
     const int nbuf = rt ? 2 : 1;
     const size_t room = kNoAllocScratchFloats - mats;
     const long long chunk = (long long)(room / (hw * nbuf));
     if (chunk < 1) return BDCT_ERR_UNSUPPORTED_SHAPE;
-    float *op_h = scratch, *op_w = scratch + (size_t)rows * rows;
+    float *op_h = scratch, *op_w = scratch + th;
     float *w1 = scratch + mats, *w2 = w1 + (size_t)chunk * hw;
 
-    // The matrices are regenerated by every call (FP64 cosines, rounded once
+    // The tables are regenerated by every call (FP64 cosines, rounded once
     // to FP32), so nothing left by an earlier call is ever read; no part of
     // the scratch needs to start at zero.
     if (!rt) {
         const int direction = kind == BDCT_FORWARD ? 1 : 2;
-        e = dense_gen_operator(op_h, rows, direction, norm, s);
-        if (e == cudaSuccess) e = dense_gen_operator(op_w, cols, direction, norm, s);
+        e = dense_gen_table(op_h, rows, direction, norm, s);
+        if (e == cudaSuccess) e = dense_gen_table(op_w, cols, direction, norm, s);
     } else {
         // the round trip is normalized: orthonormal forward core, then its adjoint
-        e = dense_gen_operator(op_h, rows, 1, BDCT_NORM_ORTHO, s);
-        if (e == cudaSuccess) e = dense_gen_operator(op_w, cols, 1, BDCT_NORM_ORTHO, s);
-        if (e == cudaSuccess) e = dense_gen_operator(op_h + per_dir, rows, 2, BDCT_NORM_ORTHO, s);
-        if (e == cudaSuccess) e = dense_gen_operator(op_w + per_dir, cols, 2, BDCT_NORM_ORTHO, s);
+        e = dense_gen_table(op_h, rows, 1, BDCT_NORM_ORTHO, s);
+        if (e == cudaSuccess) e = dense_gen_table(op_w, cols, 1, BDCT_NORM_ORTHO, s);
+        if (e == cudaSuccess) e = dense_gen_table(op_h + per_dir, rows, 2, BDCT_NORM_ORTHO, s);
+        if (e == cudaSuccess) e = dense_gen_table(op_w + per_dir, cols, 2, BDCT_NORM_ORTHO, s);
     }
     if (e != cudaSuccess) return BDCT_ERR_CUDA;
 
@@ -110,14 +111,14 @@ extern "C" int bdct_execute_noalloc(int rows, int cols, unsigned kind, int norm,
         const long long nb = ((long long)batch - b0) < chunk ? ((long long)batch - b0) : chunk;
         const float *src = in + b0 * (long long)hw;
         float *dst = out + b0 * (long long)hw;
+        const bool inv = kind == BDCT_INVERSE;
+        e = dense_pass({src, w1, op_w, rows, cols, nb, true, inv}, s);
         if (!rt) {
-            e = dense_pass_rows(src, w1, op_w, (int)(nb * rows), cols, s);
-            if (e == cudaSuccess) e = dense_pass_cols(w1, dst, op_h, rows, cols, nb, s);
+            if (e == cudaSuccess) e = dense_pass({w1, dst, op_h, rows, cols, nb, false, inv}, s);
         } else {
-            e = dense_pass_rows(src, w1, op_w, (int)(nb * rows), cols, s);
-            if (e == cudaSuccess) e = dense_pass_cols(w1, w2, op_h, rows, cols, nb, s);
-            if (e == cudaSuccess) e = dense_pass_cols(w2, w1, op_h + per_dir, rows, cols, nb, s);
-            if (e == cudaSuccess) e = dense_pass_rows(w1, dst, op_w + per_dir, (int)(nb * rows), cols, s);
+            if (e == cudaSuccess) e = dense_pass({w1, w2, op_h, rows, cols, nb, false, false}, s);
+            if (e == cudaSuccess) e = dense_pass({w2, w1, op_h + per_dir, rows, cols, nb, false, true}, s);
+            if (e == cudaSuccess) e = dense_pass({w1, dst, op_w + per_dir, rows, cols, nb, true, true}, s);
         }
         if (e != cudaSuccess) return BDCT_ERR_CUDA;
     }

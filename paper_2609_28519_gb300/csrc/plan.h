@@ -24,7 +24,8 @@ struct bdct_plan {
     int device = -1;
     bdct::DirScales scales[3];  // per Dir
     // separable route
-    float *ops = nullptr;  // dense route: operator matrices, see op_h_off / op_w_off
+    float *ops = nullptr;  // dense route: operators, see op_h_off / op_w_off
+    size_t op_pair = 0;    // floats of one direction's two operators
     size_t op_h_off[3] = {0, 0, 0}, op_w_off[3] = {0, 0, 0};
     float *work = nullptr;
     size_t work_bytes = 0;
