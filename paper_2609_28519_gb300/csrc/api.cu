@@ -294,11 +294,9 @@ extern "C" int bdct_plan_create(bdct_plan **plan, int rows, int cols, unsigned k
     } else {
         p->variant = 2;
         // operators: forward and inverse in the plan's norm, and the
-        // orthonormal pair for the round trip (which is normalized for both);
-        // whole matrices for the on-chip route, half tables for the passes
+        // orthonormal pair for the round trip (which is normalized for both)
         p->small = small_dense_supported(rows, cols);
-        const size_t sh = p->small ? (size_t)rows * rows : dense_table_floats(rows);
-        const size_t sw = p->small ? (size_t)cols * cols : dense_table_floats(cols);
+        const size_t sh = dense_table_floats(rows), sw = dense_table_floats(cols);
         const bool need[3] = {(kind & BDCT_FORWARD) != 0, (kind & BDCT_INVERSE) != 0,
                               (kind & (BDCT_ROUNDTRIP | BDCT_SPECTRAL)) != 0};
         const size_t nmats = (need[0] ? 1 : 0) + (need[1] ? 1 : 0) + (need[2] ? 2 : 0);
@@ -311,9 +309,8 @@ extern "C" int bdct_plan_create(bdct_plan **plan, int rows, int cols, unsigned k
         auto gen = [&](int direction, int nrm, size_t &oh, size_t &ow) -> cudaError_t {
             oh = off; off += sh;
             ow = off; off += sw;
-            auto one = p->small ? dense_gen_operator : dense_gen_table;
-            cudaError_t r = one(p->ops + oh, rows, direction, nrm, 0);
-            if (r == cudaSuccess) r = one(p->ops + ow, cols, direction, nrm, 0);
+            cudaError_t r = dense_gen_table(p->ops + oh, rows, direction, nrm, 0);
+            if (r == cudaSuccess) r = dense_gen_table(p->ops + ow, cols, direction, nrm, 0);
             return r;
         };
         if (need[0] && e == cudaSuccess) e = gen(1, norm, p->op_h_off[DIR_FWD], p->op_w_off[DIR_FWD]);
@@ -417,21 +414,17 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
     return BDCT_OK;
 }
 
-// The dense route in shared memory (both sides at most 64): rows then
-// columns (forward, inverse), and for the round trip and the spectral
-// direction the adjoint columns then rows after them, Lambda in between --
-// the passes of run_separable without the workspace.
+// The dense route in shared memory (both sides at most 64).
 static int run_small(const bdct_plan *p, Dir dir, const ExecGeom &g, cudaStream_t s)
 {
     const int h = p->rows, w = p->cols;
     const Dir mdir = dir == DIR_SPEC ? DIR_RT : dir;  // the spectral direction uses the orthonormal pair
     const float *oph = p->ops + p->op_h_off[mdir];
     const float *opw = p->ops + p->op_w_off[mdir];
-    const size_t per_dir = p->op_pair;
-    const bool pair = dir == DIR_RT || dir == DIR_SPEC;
-    const int axis[4] = {0, 1, 1, 0};
-    const float *ops[4] = {opw, oph, oph + per_dir, opw + per_dir};
-    cudaError_t e = small_dense_run(h, w, pair ? 4 : 2, axis, ops, dir == DIR_SPEC ? p->spec_plain : nullptr, g, s);
+    // a single direction's operators, or the adjoint's after the forward's
+    const size_t inv = dir == DIR_INV ? 0 : p->op_pair;
+    const SmallTables t{opw, oph, oph + inv, opw + inv};
+    cudaError_t e = small_dense_run(h, w, dir, t, dir == DIR_SPEC ? p->spec_plain : nullptr, g, s);
     return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
 }
 

@@ -63,24 +63,6 @@ __device__ double operator_entry(int k, int j, int n, int direction, int norm)
     return s * cos_half_turns((2LL * j + 1) * k, n);
 }
 
-// direction 1 = forward: op[k][j], direction 2 = inverse: op[j][k]
-__global__ void k_gen_operator(float *op, int n, int direction, int norm)
-{
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n * n) return;
-    const int k = (int)(idx / n), j = (int)(idx % n);
-    const double v = operator_entry(k, j, n, direction, norm);
-    if (direction == 1) op[(size_t)k * n + j] = (float)v;
-    else op[(size_t)j * n + k] = (float)v;
-}
-
-cudaError_t dense_gen_operator(float *op, int n, int direction, int norm, cudaStream_t stream)
-{
-    const long long total = (long long)n * n;
-    k_gen_operator<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(op, n, direction, norm);
-    return cudaGetLastError();
-}
-
 namespace {
 
 constexpr int kThreads = 128;

@@ -5,12 +5,9 @@
 
 namespace bdct {
 
-// The n x n operator matrix of one direction (1 forward, 2 inverse) and
-// normalization, row-major, y = M x; generated in FP64.
-cudaError_t dense_gen_operator(float *op, int n, int direction, int norm, cudaStream_t stream);
-
-// The same operator as the passes read it: its even and odd halves
-// (dense_table_floats(n) floats, 16-byte aligned).
+// The n x n operator of one direction (1 forward, 2 inverse) and
+// normalization, generated in FP64, as the passes read it: its even and odd
+// halves (dense_table_floats(n) floats, 16-byte aligned).
 size_t dense_table_floats(int n);
 cudaError_t dense_gen_table(float *t, int n, int direction, int norm, cudaStream_t stream);
 

@@ -2,32 +2,37 @@
 // kernels do not cover (non-power-of-two sides such as 24, 26, 40 or 48).
 //
 // What is computed: Eq. 2 of the BRiDCT paper as the sandwich M_h X M_w^T
-// with the FP32 operator tables of the dense route (M = Q_n forward, Q_n^T
-// inverse, Eq. 1; Section 7.1 makes h and w independent); the round trip is
-// the forward pair then the inverse pair of the orthonormal operators
-// (Prop. 1 with Lambda = I), and the spectral direction puts Lambda between
-// them (Eq. 4).  A direct evaluation costs n multiply-adds per point and
-// pass (Section 1.2); for n <= 64 that is arithmetic the GPU does at about
-// HBM speed, so the arrays are read once and written once and every pass
-// runs in shared memory -- the two-pass route through a workspace in HBM
-// moves twice the bytes per pass and launches two GEMMs per chunk.
+// (M = Q_n forward, Q_n^T inverse, Eq. 1; Section 7.1 makes h and w
+// independent); the round trip is the forward pair then the inverse pair of
+// the orthonormal operators (Prop. 1 with Lambda = I), and the spectral
+// direction puts Lambda between them (Eq. 4).  One read and one write of
+// every element; every pass runs in shared memory on the half products of
+// dense_passes.cu: n/2 multiply-adds per point, the even and the odd product
+// in the halves of packed pairs, operand pairs (s, d) = sums and differences
+// of mirrored elements (forward) or (y_2k, y_2k+1) (inverse).
 //
-// Organization: persistent CTAs of 256 threads; each iteration transforms
-// G arrays held in a shared buffer (rows padded to a multiple of 4 and a
-// pitch of 4 mod 32 floats, padding zero), running the passes between two
-// buffers and writing the last pass straight to global memory, while the
-// next G arrays arrive in a third buffer by 16-byte cp.async copies.  Each thread computes
-// 4 x 4 output tiles (four consecutive rows, four consecutive columns): a
-// step of four contraction indices reads four float4 of the input and four
-// of the operator (staged once per CTA, zero-padded; transposed for passes
-// along w so that the lanes of a warp read consecutive float4) for 64
-// fused multiply-adds, issued as 32 packed (two-column) instructions.  Sums of more than 16 terms are taken in blocks of
-// 16 added to the running total, as in the dense route.
+// Organization.  A CTA of four warps transforms G arrays at a time, G chosen
+// so that one tile of 8 lines x 4 output pairs per thread covers them
+// (about 8192 elements).  Every pass stores what the next one contracts,
+// already paired, from registers:
+//  * along w, forward: a thread's lines are mirrored rows (i, h-1-i), whose
+//    sum and difference is the pair the pass along h needs;
+//  * along h, forward: coefficient rows 2o and 2o + 1 come out as one pair,
+//    which the adjoint pass along h contracts (times Lambda), or go to global
+//    memory;
+//  * along h, inverse: a thread's lines are neighbouring columns (2q, 2q+1),
+//    the pair of the inverse along w;
+// so there is no conversion pass, and a pass costs one read and one write of
+// shared memory per element beyond the products' operands.  Lanes are laid
+// out as in dense_passes.cu (16-byte reads in two wavefronts); short sides
+// give the lanes to lines instead of outputs.  Sums of more than 16 terms are
+// taken in blocks of 16 added to the running total, as in the dense passes.
 #include <cuda_runtime.h>
 
 #include <cstdio>
 
 #include "bdct_internal.h"
+#include "dense_passes.h"
 #include "ptx.cuh"
 #include "small_dense.h"
 
@@ -35,312 +40,398 @@ namespace bdct {
 
 namespace {
 
-constexpr int kSmThreads = 256;
-constexpr int kSmMaxSide = 64;
-constexpr int kSmMaxPasses = 4;
+constexpr int kThreads = 128;
+constexpr int kMaxSide = 64;
+constexpr int kMaxArrays = 64;
+constexpr int kTarget = 8192;  // elements per CTA: one tile of 64 per thread
+constexpr int kSlack = 256;    // pairs past a buffer that an edge tile may read
+
+// Exact quotients of small unsigned values by a fixed divisor.
+struct FastDiv {
+    unsigned d, m;
+    __host__ FastDiv(unsigned d_ = 1) : d(d_), m((unsigned)(((1ull << 32) + d_ - 1) / d_)) {}
+    __device__ __forceinline__ unsigned div(unsigned x) const { return d == 1 ? x : __umulhi(x, m); }
+};
+
+// One axis of the products: half length (outputs pairs and contraction), lane
+// layout.
+struct Axis {
+    int nh, tc, np;   // pairs, output quads, table row (pairs)
+    int tcl;          // output quads per warp: 4, 2 or 1
+    __host__ __device__ explicit Axis(int n = 2)
+        : nh((n + 1) / 2), tc((nh + 3) / 4), np(4 * tc), tcl(tc > 2 ? 4 : tc)
+    {
+    }
+    __host__ __device__ int line_block() const { return 256 / tcl; }  // lines of a warp's tile
+};
 
 struct SmallParams {
     const float *in;
     float *out;
     const long long *in_off, *out_off;  // indexed arrays (element offsets), or null
     int tpr;                            // image tiles: tiles per image row (0: arrays)
-    long long ld_in, ld_out;            // image tiles: leading dimensions (floats)
+    long long ld_in, ld_out;            // row strides (floats)
     long long count;
     int h, w;
-    int hp, wp;      // sides padded to a multiple of 4
-    int pitch;       // buffer row pitch (floats): >= wp, 4 mod 32
-    int G;           // arrays per iteration
-    int npass;
-    int axis[kSmMaxPasses];          // 0: along w (every row), 1: along h (every column)
-    int op_at[kSmMaxPasses];         // offset (floats) of each pass's staged operator
-    const float *op[kSmMaxPasses];   // n x n row-major, y = M x, scales folded in
-    const float *lam;                // spectral: Lambda (h x w) after the second pass, or null
+    int G;                           // arrays per iteration
+    int buf0, buf1;                  // buffer sizes (pairs)
+    const float2 *fw, *fh, *ih, *iw;  // tables of the passes used (dense_gen_table)
+    const float *lam;                // spectral: Lambda (h x w), or null
+    FastDiv div_h, div_w4, div_hp, div_wq, div_kh;
+    long long groups;
 };
 
-__host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
+__host__ __device__ constexpr int even2(int n) { return (n + 3) / 4 * 4 + 2; }  // pitch: 2 mod 4 pairs
 
-// Row pitch of 4 mod 32 floats (>= n): the float4 rows read by the lanes of a
-// quarter-warp fall on distinct bank groups.
-__host__ __device__ inline int pitch4(int n)
-{
-    int p = pad4(n);
-    while (p % 32 != 4) p += 4;
-    return p;
-}
+// Pitches (pairs) of the operand buffers.
+__host__ __device__ inline int pitch_fw(int h, int G) { return even2(2 * ((h + 1) / 2) * G); }
+__host__ __device__ inline int pitch_h(int w, int G) { return even2(w * G); }
+__host__ __device__ inline int pitch_iw(int h, int G) { return even2(h * G); }
 
-// First element and row stride of array (or image tile) a.
-__device__ __forceinline__ const float *in_array(const SmallParams &p, long long a, long long &ld)
+// This lane's place in a warp tile of an axis: output quad and line group.
+__device__ __forceinline__ void lane_place(const Axis &x, int lane, int &tq, int &la)
 {
-    if (p.tpr) {
-        ld = p.ld_in;
-        return p.in + (a / p.tpr) * p.h * p.ld_in + (a % p.tpr) * p.w;
+    if (x.tcl == 4) {
+        tq = (lane & 1) + (lane >> 1 & 2);
+        la = (lane >> 1 & 1) + (lane >> 2 & 6);
+    } else if (x.tcl == 2) {
+        tq = lane & 1;
+        la = lane >> 1;
+    } else {
+        tq = 0;
+        la = lane;
     }
-    ld = p.w;
-    return p.in_off ? p.in + p.in_off[a] : p.in + a * (long long)p.h * p.w;
 }
-__device__ __forceinline__ float *out_array(const SmallParams &p, long long a, long long &ld)
+
+// Products of lines l0 + i * ls (+ 1) and output pairs 4 tc .. 4 tc + 3:
+// acc[2i + r][o] = (even, odd) sums over k < K of a[k][line] * t[k][o].
+template <bool LONG>
+__device__ __forceinline__ void products(const float2 *a, int pitch, int ls, const float2 *t, int np, int K,
+                                         float2 (&acc)[8][4])
 {
-    if (p.tpr) {
-        ld = p.ld_out;
-        return p.out + (a / p.tpr) * p.h * p.ld_out + (a % p.tpr) * p.w;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[r][o] = make_float2(0.f, 0.f);
+    auto step = [&](float2 (&sum)[8][4]) {
+        float2 x[8], m[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = *reinterpret_cast<const float4 *>(a + i * ls);
+            x[2 * i] = make_float2(v.x, v.y);
+            x[2 * i + 1] = make_float2(v.z, v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float4 v = *reinterpret_cast<const float4 *>(t + 2 * i);
+            m[2 * i] = make_float2(v.x, v.y);
+            m[2 * i + 1] = make_float2(v.z, v.w);
+        }
+        a += pitch;
+        t += np;
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) sum[r][o] = __ffma2_rn(x[r], m[o], sum[r][o]);
+    };
+    if constexpr (!LONG) {
+#pragma unroll 2
+        for (int k = 0; k < K; ++k) step(acc);
+    } else {
+        for (int k0 = 0; k0 < K; k0 += 16) {
+            const int kn = min(16, K - k0);
+            float2 part[8][4];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) part[r][o] = make_float2(0.f, 0.f);
+#pragma unroll 2
+            for (int k = 0; k < kn; ++k) step(part);
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) acc[r][o] = __fadd2_rn(acc[r][o], part[r][o]);
+        }
     }
-    ld = p.w;
-    return p.out_off ? p.out + p.out_off[a] : p.out + a * (long long)p.h * p.w;
 }
 
-// acc (two columns) += s * v, one packed instruction for both columns.
-__device__ __forceinline__ float2 fma2s(float s, float2 v, float2 acc)
+// DIR: DIR_FWD, DIR_INV, or DIR_RT for both pairs (Lambda between if set).
+template <int DIR, bool LONG>
+__global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallParams p)
 {
-    return __ffma2_rn(make_float2(s, s), v, acc);
-}
+    constexpr bool FWD = DIR != DIR_INV, INV = DIR != DIR_FWD;
+    extern __shared__ __align__(16) float2 ssm[];
+    float2 *buf[2] = {ssm, ssm + p.buf0};
+    const int h = p.h, w = p.w, G = p.G, tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    const Axis aw(w), ah(h);
+    const int kw = aw.nh, kh = ah.nh;
+    float2 *tab = ssm + p.buf0 + p.buf1;
+    float2 *t_fw = tab, *t_fh = t_fw + (FWD ? kw * aw.np : 0), *t_ih = t_fh + (FWD ? kh * ah.np : 0),
+           *t_iw = t_ih + (INV ? kh * ah.np : 0);
+    __shared__ long long base_in[kMaxArrays], base_out[kMaxArrays];
 
-// One pass from buffer `src` to buffer `dst` (or, for the last pass, to the
-// arrays in global memory).  Along w: dst[i][l] = sum_j src[i][j] Mt[j][l]
-// (Mt = M^T staged, n = w); along h: dst[k][l] = sum_i M[k][i] src[i][l]
-// (n = h).  Tiles: 4 rows x 4 columns, rt over the row tiles of all the
-// iteration's arrays, lt over the column tiles; the four columns of a tile
-// accumulate as two packed pairs.
-template <int AXIS, bool FINAL>
-__device__ __forceinline__ void small_pass(const SmallParams &p, const float *op_s, const float *src, float *dst,
-                                           long long a0, int na)
-{
-    const int hp = p.hp, wp = p.wp, pitch = p.pitch;
-    const int W4 = wp >> 2, H4 = hp >> 2;
-    const int n = AXIS == 0 ? wp : hp;  // padded contraction length (a multiple of 4)
-    const int tiles = na * H4 * W4;
-    // stride between consecutive contraction rows of the operand read per q
-    const int qstride = AXIS == 0 ? wp : pitch;
-    for (int t = threadIdx.x; t < tiles; t += kSmThreads) {
-        const int lt = t % W4, rt = t / W4;  // rt = a * H4 + row tile
-        const int a = rt / H4, r0 = (rt - a * H4) * 4;
-        const float *sa = src + (size_t)a * hp * pitch;
-        // rp: the four rows read along the contraction (input rows along w,
-        // operator rows along h); qp: the operand read four columns wide
-        const float *rp = AXIS == 0 ? sa + r0 * pitch : op_s + r0 * hp;
-        const int rstride = AXIS == 0 ? pitch : hp;
-        const float *qp = AXIS == 0 ? op_s + 4 * lt : sa + 4 * lt;
-        float2 acc[4][2];
+    pdl_launch_dependents();
+    // the tables are plan data, written before any transform was queued
+    auto stage = [&](float2 *t, const float2 *src, int n) {
+        for (int e = tid; e < n; e += kThreads) t[e] = __ldg(src + e);
+    };
+    if (FWD) {
+        stage(t_fw, p.fw, kw * aw.np);
+        stage(t_fh, p.fh, kh * ah.np);
+    }
+    if (INV) {
+        stage(t_ih, p.ih, kh * ah.np);
+        stage(t_iw, p.iw, kw * aw.np);
+    }
+    pdl_wait_prerequisites();
+
+    int tqw, law, tqh, lah;
+    lane_place(aw, lane, tqw, law);
+    lane_place(ah, lane, tqh, lah);
+    const int pfw = pitch_fw(h, G), ph = pitch_h(w, G), piw = pitch_iw(h, G);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+
+    for (long long grp = blockIdx.x; grp < p.groups; grp += gridDim.x) {
+        const long long a0 = grp * G;
+        const int na = (int)(p.count - a0 < G ? p.count - a0 : G);
+        __syncthreads();  // the last group's stores have taken their bases
+        if (tid < na) {
+            const long long a = a0 + tid;
+            if (p.tpr) {
+                const long long br = a / p.tpr, bc = a - br * p.tpr;
+                base_in[tid] = br * h * p.ld_in + bc * w;
+                base_out[tid] = br * h * p.ld_out + bc * w;
+            } else {
+                base_in[tid] = p.in_off ? p.in_off[a] : a * (long long)h * w;
+                base_out[tid] = p.out_off ? p.out_off[a] : a * (long long)h * w;
+            }
+        }
+        __syncthreads();
+
+        // ---- the arrays, paired for the first pass, four tasks in flight a thread
+        if constexpr (FWD) {
+            // four elements from the front of a row and their mirrors
+            const int Q = (w + 7) / 8, tasks = na * h * Q;
+            for (int e0 = tid; e0 < tasks; e0 += 4 * kThreads) {
+                float4 x[4], y[4];
+                int at[4], kq[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
-        for (int k0 = 0; k0 < n; k0 += 16) {
-            float2 part[4][2];
+                for (int u = 0; u < 4; ++u) {
+                    const int e = e0 + u * kThreads;
+                    x[u] = y[u] = zero;
+                    at[u] = -1;
+                    if (e < tasks) {
+                        const int row = p.div_wq.div(e), q = e - row * Q;
+                        const int a = p.div_h.div(row), r = row - a * h;
+                        const float *g = p.in + base_in[a] + r * p.ld_in;
+                        x[u] = __ldcg(reinterpret_cast<const float4 *>(g + 4 * q));
+                        y[u] = __ldcg(reinterpret_cast<const float4 *>(g + w - 4 - 4 * q));
+                        // mirrored rows side by side
+                        const int m = h - 1 - r;
+                        at[u] = 2 * (a * kh + min(r, m)) + (r > m);
+                        kq[u] = 4 * q;
+                    }
+                }
 #pragma unroll
-            for (int r = 0; r < 4; ++r) part[r][0] = part[r][1] = make_float2(0.0f, 0.0f);
+                for (int u = 0; u < 4; ++u) {
+                    if (at[u] < 0) continue;
+                    float2 *o = buf[0] + kq[u] * pfw + at[u];
+                    const float f[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, b[4] = {y[u].w, y[u].z, y[u].y, y[u].x};
 #pragma unroll
-            for (int s4 = 0; s4 < 16; s4 += 4) {
-                const int k = k0 + s4;
-                if (k < n) {
-                    float4 rv[4], qv[4];
+                    for (int i = 0; i < 4; ++i)
+                        if (kq[u] + i < kw) o[i * pfw] = make_float2(f[i] + b[i], f[i] - b[i]);
+                }
+            }
+        } else {
+            // coefficient rows 2k and 2k + 1, four columns
+            const int W4 = w / 4, tasks = na * kh * W4;
+            for (int e0 = tid; e0 < tasks; e0 += 4 * kThreads) {
+                float4 x[4], y[4];
+                int at[4];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) rv[r] = *reinterpret_cast<const float4 *>(rp + r * rstride + k);
+                for (int u = 0; u < 4; ++u) {
+                    const int e = e0 + u * kThreads;
+                    x[u] = y[u] = zero;
+                    at[u] = -1;
+                    if (e < tasks) {
+                        const int row = p.div_w4.div(e), c = 4 * (e - row * W4);
+                        const int a = p.div_kh.div(row), k = row - a * kh;
+                        const float *g = p.in + base_in[a] + 2 * k * p.ld_in + c;
+                        x[u] = __ldcg(reinterpret_cast<const float4 *>(g));
+                        if (2 * k + 1 < h) y[u] = __ldcg(reinterpret_cast<const float4 *>(g + p.ld_in));
+                        at[u] = k * ph + a * w + c;
+                    }
+                }
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) qv[q] = *reinterpret_cast<const float4 *>(qp + (k + q) * qstride);
+                for (int u = 0; u < 4; ++u) {
+                    if (at[u] < 0) continue;
+                    float4 *o = reinterpret_cast<float4 *>(buf[0] + at[u]);
+                    o[0] = make_float4(x[u].x, y[u].x, x[u].y, y[u].y);
+                    o[1] = make_float4(x[u].z, y[u].z, x[u].w, y[u].w);
+                }
+            }
+        }
+        __syncthreads();
+
+        float2 acc[8][4];
+        // tiles of a pass: line blocks x groups of tcl output quads, a warp each
+        auto for_tiles = [&](const Axis &x, int lines, int tq, int la, auto &&tile) {
+            const int lb = x.line_block(), nlb = (lines + lb - 1) / lb, nt = nlb * ((x.tc + x.tcl - 1) / x.tcl);
+            for (int t = warp; t < nt; t += kThreads / 32) {
+                const int tg = t / nlb;
+                const int q = tg * x.tcl + tq;
+                tile((t - tg * nlb) * lb + 2 * la, lb / 4, q < x.tc ? q : x.tc - 1, q < x.tc);
+            }
+        };
+
+        if constexpr (FWD) {
+            // ---- along w: rows (i, h-1-i) of an array
+            for_tiles(aw, 2 * kh * na, tqw, law, [&](int l0, int ls, int tc, bool live) {
+                products<LONG>(buf[0] + l0, pfw, ls, t_fw + 4 * tc, aw.np, kw, acc);
+                if (!live) return;
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float rs[4] = {rv[r].x, rv[r].y, rv[r].z, rv[r].w};
+                for (int i = 0; i < 4; ++i) {
+                    const int pr = (l0 + i * ls) / 2;
+                    const int a = p.div_hp.div(pr), r = pr - a * kh;
+                    if (a >= na) continue;
+                    const bool mid = 2 * r + 1 == h;  // an odd height's middle row, its own mirror
+                    float4 *o = reinterpret_cast<float4 *>(buf[1] + r * ph + a * w + 8 * tc);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            part[r][0] = fma2s(rs[q], make_float2(qv[q].x, qv[q].y), part[r][0]);
-                            part[r][1] = fma2s(rs[q], make_float2(qv[q].z, qv[q].w), part[r][1]);
+                    for (int c = 0; c < 4; ++c) {
+                        if (4 * tc + c >= kw) continue;
+                        const float2 u = acc[2 * i][c], v = acc[2 * i + 1][c];
+                        o[c] = mid ? make_float4(u.x, 0.f, u.y, 0.f)
+                                   : make_float4(u.x + v.x, u.x - v.x, u.y + v.y, u.y - v.y);
+                    }
+                }
+            });
+            __syncthreads();
+            // ---- along h: neighbouring columns; coefficient rows 2o, 2o + 1
+            for_tiles(ah, w * na, tqh, lah, [&](int l0, int ls, int tc, bool live) {
+                products<LONG>(buf[1] + l0, ph, ls, t_fh + 4 * tc, ah.np, kh, acc);
+                if (!live) return;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int l = l0 + i * ls;
+                    const int a = p.div_w4.div(l / 4), c = l - a * w;
+                    if (a >= na) continue;
+                    float *g = DIR == DIR_FWD ? p.out + base_out[a] + c : nullptr;
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) {
+                        const int k = 2 * (4 * tc + o);
+                        if (k >= h) continue;
+                        float2 u = acc[2 * i][o], v = acc[2 * i + 1][o];
+                        if constexpr (DIR == DIR_FWD) {
+                            *reinterpret_cast<float2 *>(g + k * p.ld_out) = make_float2(u.x, v.x);
+                            if (k + 1 < h)
+                                *reinterpret_cast<float2 *>(g + (k + 1) * p.ld_out) = make_float2(u.y, v.y);
+                        } else {
+                            if (p.lam) {
+                                const float2 l0v = __ldg(reinterpret_cast<const float2 *>(p.lam + k * w + c));
+                                u.x *= l0v.x;
+                                v.x *= l0v.y;
+                                if (k + 1 < h) {
+                                    const float2 l1v = __ldg(reinterpret_cast<const float2 *>(p.lam + (k + 1) * w + c));
+                                    u.y *= l1v.x;
+                                    v.y *= l1v.y;
+                                }
+                            }
+                            *reinterpret_cast<float4 *>(buf[0] + (k / 2) * ph + l) = make_float4(u.x, u.y, v.x, v.y);
                         }
                     }
                 }
-            }
+            });
+            if constexpr (DIR == DIR_RT) __syncthreads();
+        }
+        if constexpr (INV) {
+            // ---- along h, inverse: rows j and h-1-j of neighbouring columns
+            for_tiles(ah, w * na, tqh, lah, [&](int l0, int ls, int tc, bool live) {
+                products<LONG>(buf[0] + l0, ph, ls, t_ih + 4 * tc, ah.np, kh, acc);
+                if (!live) return;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                acc[r][0] = __fadd2_rn(acc[r][0], part[r][0]);
-                acc[r][1] = __fadd2_rn(acc[r][1], part[r][1]);
-            }
-        }
-        if constexpr (FINAL) {
-            // rows r0.. of array a0 + a, columns 4 lt.. (w is a multiple of 4)
-            long long ld;
-            float *g = out_array(p, a0 + a, ld);
+                for (int i = 0; i < 4; ++i) {
+                    const int l = l0 + i * ls;
+                    const int a = p.div_w4.div(l / 4), c = l - a * w;
+                    if (a >= na) continue;
+                    float2 *b = buf[1] + (c / 2) * piw + a * h;
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                if (r0 + r < p.h)
-                    *reinterpret_cast<float4 *>(g + (long long)(r0 + r) * ld + 4 * lt) =
-                        make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
-        } else {
-            // padding rows (h not a multiple of 4) are stored as zeros, not as
-            // their sums: a non-finite input would make those 0 * inf = NaN,
-            // and the buffer goes on to hold the CTA's later arrays, whose
-            // sums take the padding rows in with zero weights (0 * NaN)
-            float *da = dst + (size_t)a * hp * pitch;
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-                *reinterpret_cast<float4 *>(da + (r0 + r) * pitch + 4 * lt) =
-                    r0 + r < p.h ? make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y)
-                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-    }
-}
-
-// Issue the 16-byte asynchronous copies of arrays a0 .. a0 + na - 1 into
-// buffer `dst` (this thread's share).  Thread t copies chunk t mod q4 of the
-// group's rows t / q4, t / q4 + R, ... (R = 256 / q4 rows per sweep), its
-// array and row advanced incrementally rather than divided out per copy.
-__device__ __forceinline__ void small_fill(const SmallParams &p, float *dst, long long a0, int na)
-{
-    const int q4 = p.w >> 2, R = kSmThreads / q4;
-    const int c4 = threadIdx.x % q4, r_start = threadIdx.x / q4;
-    if (r_start < R) {
-        const int da = R / p.h, di = R - da * p.h;
-        int a = r_start / p.h, i = r_start - a * p.h;
-        for (int row = r_start; row < na * p.h; row += R) {
-            long long ld;
-            const float *g = in_array(p, a0 + a, ld);
-            cp_async16(dst + ((size_t)a * p.hp + i) * p.pitch + 4 * c4, g + (long long)i * ld + 4 * c4);
-            i += di;
-            a += da;
-            if (i >= p.h) {
-                i -= p.h;
-                ++a;
-            }
-        }
-    }
-    cp_async_commit();
-}
-
-template <int AXIS>
-__device__ __forceinline__ void small_pass_any(const SmallParams &p, bool final_pass, const float *op_s,
-                                               const float *src, float *dst, long long a0, int na)
-{
-    if (final_pass) small_pass<AXIS, true>(p, op_s, src, dst, a0, na);
-    else small_pass<AXIS, false>(p, op_s, src, dst, a0, na);
-}
-
-__global__ void __launch_bounds__(kSmThreads) k_small_dense(const SmallParams p)
-{
-    extern __shared__ __align__(16) float ssm[];
-    const int hp = p.hp, wp = p.wp, pitch = p.pitch;
-    const size_t buf = (size_t)p.G * hp * pitch;
-    // three buffers: the group being transformed alternates between two of
-    // them, the next group loads into the third
-    float *bufs[3] = {ssm, ssm + buf, ssm + 2 * buf};
-    float *ops = ssm + 3 * buf;
-    const int tid = threadIdx.x;
-
-    pdl_launch_dependents();
-    // the operators of every pass, zero-padded: along w transposed (Mt[j][l],
-    // wp x wp), along h as they are (M[k][i], hp x hp).  They are plan tables
-    // written before any transform, so reading them ahead of the wait on the
-    // previous kernel is safe.
-    for (int q = 0; q < p.npass; ++q) {
-        const int n = p.axis[q] == 0 ? p.w : p.h, np = p.axis[q] == 0 ? wp : hp;
-        float *o = ops + p.op_at[q];
-        for (int e = tid; e < np * np; e += kSmThreads) {
-            const int r = e / np, c = e % np;
-            float v = 0.0f;
-            if (r < n && c < n) v = p.axis[q] == 0 ? p.op[q][(size_t)c * n + r] : p.op[q][(size_t)r * n + c];
-            o[e] = v;
-        }
-    }
-    // zero the buffers once: padding rows stay zero (the copies write only
-    // the arrays' own rows, the passes zeros into the padding rows; the
-    // width is a multiple of 4, so there are no padding columns)
-    for (size_t e = tid; e < 3 * buf; e += kSmThreads) ssm[e] = 0.0f;
-    pdl_wait_prerequisites();
-    __syncthreads();
-
-    const long long step = (long long)gridDim.x * p.G;
-    long long a0 = (long long)blockIdx.x * p.G;
-    int cur = 0;  // buffer holding the current group
-    if (a0 < p.count) small_fill(p, bufs[cur], a0, (int)((p.count - a0) < p.G ? (p.count - a0) : p.G));
-    for (; a0 < p.count; a0 += step) {
-        const int na = (int)((p.count - a0) < p.G ? (p.count - a0) : p.G);
-        // the next group into the buffer that is neither the current one nor
-        // its partner (both free: the previous iteration ended on a barrier)
-        const int nxt = (cur + 2) % 3;
-        const long long an = a0 + step;
-        if (an < p.count) {
-            small_fill(p, bufs[nxt], an, (int)((p.count - an) < p.G ? (p.count - an) : p.G));
-            cp_async_wait_group<1>();  // this group's copies have landed, the next group's may not
-        } else {
-            cp_async_wait_group<0>();
-        }
-        __syncthreads();
-        float *src = bufs[cur], *dst = bufs[(cur + 1) % 3];
-        for (int q = 0; q < p.npass; ++q) {
-            const bool fin = q + 1 == p.npass;
-            if (p.axis[q] == 0) small_pass_any<0>(p, fin, ops + p.op_at[q], src, dst, a0, na);
-            else small_pass_any<1>(p, fin, ops + p.op_at[q], src, dst, a0, na);
-            __syncthreads();
-            if (fin) break;
-            if (q == 1 && p.lam) {
-                // the orthonormal spectrum times Lambda (Eq. 4)
-                const int hw = p.h * p.w;
-                for (int e = tid; e < na * hw; e += kSmThreads) {
-                    const int a = e / hw, rem = e - a * hw, k = rem / p.w, l = rem - k * p.w;
-                    dst[((size_t)a * hp + k) * pitch + l] *= p.lam[rem];
+                    for (int o = 0; o < 4; ++o) {
+                        const int j = 4 * tc + o;
+                        if (j >= kh) continue;
+                        const float2 u = acc[2 * i][o], v = acc[2 * i + 1][o];
+                        b[j] = make_float2(u.x + u.y, v.x + v.y);
+                        b[h - 1 - j] = make_float2(u.x - u.y, v.x - v.y);
+                    }
                 }
-                __syncthreads();
-            }
-            float *t = src;
-            src = dst;
-            dst = t;
+            });
+            __syncthreads();
+            // ---- along w, inverse: rows to global memory
+            for_tiles(aw, h * na, tqw, law, [&](int l0, int ls, int tc, bool live) {
+                products<LONG>(buf[1] + l0, piw, ls, t_iw + 4 * tc, aw.np, kw, acc);
+                if (!live) return;
+                const int o0 = 4 * tc;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const int l = l0 + i * ls + s;
+                        const int a = p.div_h.div(l), r = l - a * h;
+                        if (a >= na) continue;
+                        float *g = p.out + base_out[a] + r * p.ld_out;
+                        const float2 *v = acc[2 * i + s];
+                        if (o0 + 4 <= kw) {
+                            *reinterpret_cast<float4 *>(g + o0) =
+                                make_float4(v[0].x + v[0].y, v[1].x + v[1].y, v[2].x + v[2].y, v[3].x + v[3].y);
+                            *reinterpret_cast<float4 *>(g + w - 4 - o0) =
+                                make_float4(v[3].x - v[3].y, v[2].x - v[2].y, v[1].x - v[1].y, v[0].x - v[0].y);
+                        } else {
+                            // the two middle pairs (w a multiple of 4, w/2 not): one float4
+                            *reinterpret_cast<float4 *>(g + o0) =
+                                make_float4(v[0].x + v[0].y, v[1].x + v[1].y, v[1].x - v[1].y, v[0].x - v[0].y);
+                        }
+                    }
+            });
         }
-        cur = nxt;
     }
 }
 
-}  // namespace
-
-bool small_dense_supported(int h, int w)
+template <int DIR, bool LONG>
+cudaError_t launch(SmallParams p, cudaStream_t stream)
 {
-    return h >= 1 && w >= 4 && h <= kSmMaxSide && w <= kSmMaxSide && w % 4 == 0;
-}
-
-cudaError_t small_dense_run(int h, int w, int npass, const int *axis, const float *const *op, const float *lam,
-                            const ExecGeom &g, cudaStream_t stream)
-{
-    if (!small_dense_supported(h, w) || npass < 2 || npass > kSmMaxPasses) return cudaErrorInvalidValue;
-    if (g.count <= 0) return cudaSuccess;
-    SmallParams p{};
-    p.in = g.in;
-    p.out = g.out;
-    p.in_off = g.in_off;
-    p.out_off = g.out_off;
-    p.tpr = g.tiled ? g.tiles_per_row : 0;
-    p.ld_in = g.ld_in;
-    p.ld_out = g.ld_out;
-    p.count = g.count;
-    p.h = h;
-    p.w = w;
-    p.hp = pad4(h);
-    p.wp = pad4(w);
-    p.pitch = pitch4(w);
-    p.npass = npass;
-    p.lam = lam;
-    int at = 0;
-    for (int q = 0; q < npass; ++q) {
-        p.axis[q] = axis[q];
-        p.op[q] = op[q];
-        p.op_at[q] = at;
-        at += axis[q] == 0 ? p.wp * p.wp : p.hp * p.hp;
-    }
-    // arrays per iteration: the three buffers within 96 KiB, and among the
-    // counts that fit, the one whose output tiles fill the 256 threads best
-    // (a pass takes ceil(tiles / 256) tile times), the larger on a tie
-    const int tiles1 = (p.hp / 4) * (p.wp / 4);
-    const size_t arr_bytes = (size_t)p.hp * p.pitch * sizeof(float);
-    int gmax = (int)((96 * 1024) / (3 * arr_bytes));
+    const Axis aw(p.w), ah(p.h);
+    constexpr bool FWD = DIR != DIR_INV, INV = DIR != DIR_FWD;
+    // arrays per iteration: about kTarget elements, and among the counts near
+    // it the one whose warp tiles fill the four warps best (the larger on a tie)
+    auto tiles = [](const Axis &x, int lines) {
+        return (lines + x.line_block() - 1) / x.line_block() * ((x.tc + x.tcl - 1) / x.tcl);
+    };
+    int gmax = kTarget / (p.h * p.w);
     if (gmax < 1) gmax = 1;
-    if (gmax > 64) gmax = 64;
+    if (gmax > kMaxArrays) gmax = kMaxArrays;
     int G = 1;
     double best = 0.0;
-    for (int c = 1; c <= gmax; ++c) {
-        const int tiles = c * tiles1;
-        const double fill = (double)tiles / (kSmThreads * ((tiles + kSmThreads - 1) / kSmThreads));
-        if (fill >= best - 1e-9) {
-            best = fill;
-            G = c;
+    for (int g = gmax; g >= 1 && 2 * g >= gmax; --g) {
+        auto rounds = [&](int t) { return (t + 3) / 4; };
+        const int r = rounds(tiles(aw, FWD ? 2 * ah.nh * g : p.h * g)) + rounds(tiles(ah, p.w * g));
+        const double per = (double)g / r;
+        if (per > best * 1.02) {
+            best = per;
+            G = g;
         }
     }
     p.G = G;
-    const size_t smem = ((size_t)3 * G * p.hp * p.pitch + (size_t)at) * sizeof(float);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    const int fw = aw.nh * pitch_fw(p.h, G) + kSlack, hh = ah.nh * pitch_h(p.w, G) + kSlack,
+              iw = aw.nh * pitch_iw(p.h, G) + kSlack;
+    p.buf0 = FWD ? (INV && hh > fw ? hh : fw) : hh;
+    p.buf1 = FWD ? (INV && iw > hh ? iw : hh) : iw;
+    p.buf0 = (p.buf0 + 1) / 2 * 2;
+    p.buf1 = (p.buf1 + 1) / 2 * 2;
+    const int tabs = (FWD + INV) * (aw.nh * aw.np + ah.nh * ah.np);
+    const size_t smem = ((size_t)p.buf0 + p.buf1 + tabs) * sizeof(float2);
+    if (smem > 220 * 1024) return cudaErrorInvalidValue;
+    p.groups = (p.count + G - 1) / G;
 
+    auto kern = k_small<DIR, LONG>;
     static DeviceLaunchCache cache;
     int dev = 0, bps = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -348,8 +439,7 @@ cudaError_t small_dense_run(int h, int w, int npass, const int *axis, const floa
     e = cache.get(
         dev,
         [&](int d, int &b, int &n) {
-            cudaError_t r = cudaFuncSetAttribute(k_small_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 227 * 1024);
+            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
             b = 1;
             return r;
@@ -357,27 +447,26 @@ cudaError_t small_dense_run(int h, int w, int npass, const int *axis, const floa
         &bps, &sms);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_small_dense, kSmThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    const long long groups = (p.count + G - 1) / G;
     long long grid = (long long)per_sm * sms;
-    if (grid > groups) grid = groups;
+    if (grid > p.groups) grid = p.groups;
     if (debug_enabled()) {
         // once per configuration, not per launch
         static std::mutex mu;
         static long long last = -1;
-        const long long key = ((long long)h << 20) | ((long long)w << 8) | npass;
+        const long long key = ((long long)p.h << 20) | ((long long)p.w << 8) | DIR;
         std::lock_guard<std::mutex> lock(mu);
         if (key != last) {
             last = key;
-            fprintf(stderr, "[bdct] k_small_dense %dx%d: %d passes, %d arrays per iteration, %d CTAs/SM, smem %zu B\n",
-                    h, w, npass, G, per_sm, smem);
+            fprintf(stderr, "[bdct] k_small<%d,%d> %dx%d: %d arrays per iteration, %d CTAs/SM, smem %zu B\n", DIR,
+                    (int)LONG, p.h, p.w, G, per_sm, smem);
         }
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kSmThreads);
+    cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -385,7 +474,46 @@ cudaError_t small_dense_run(int h, int w, int npass, const int *axis, const floa
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_small_dense, p);
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+}  // namespace
+
+bool small_dense_supported(int h, int w)
+{
+    return h >= 1 && w >= 4 && h <= kMaxSide && w <= kMaxSide && w % 4 == 0;
+}
+
+cudaError_t small_dense_run(int h, int w, Dir dir, const SmallTables &t, const float *lam, const ExecGeom &g,
+                            cudaStream_t stream)
+{
+    if (!small_dense_supported(h, w)) return cudaErrorInvalidValue;
+    if (g.count <= 0) return cudaSuccess;
+    SmallParams p{};
+    p.in = g.in;
+    p.out = g.out;
+    p.in_off = g.in_off;
+    p.out_off = g.out_off;
+    p.tpr = g.tiled ? g.tiles_per_row : 0;
+    p.ld_in = g.tiled ? g.ld_in : w;
+    p.ld_out = g.tiled ? g.ld_out : w;
+    p.count = g.count;
+    p.h = h;
+    p.w = w;
+    p.fw = reinterpret_cast<const float2 *>(t.fw);
+    p.fh = reinterpret_cast<const float2 *>(t.fh);
+    p.ih = reinterpret_cast<const float2 *>(t.ih);
+    p.iw = reinterpret_cast<const float2 *>(t.iw);
+    p.lam = dir == DIR_SPEC ? lam : nullptr;
+    p.div_h = FastDiv(h);
+    p.div_w4 = FastDiv(w / 4);
+    p.div_hp = FastDiv((h + 1) / 2);
+    p.div_wq = FastDiv((w + 7) / 8);
+    p.div_kh = FastDiv((h + 1) / 2);
+    const bool is_long = h > 32 || w > 32;  // more than 16 pairs on an axis
+    if (dir == DIR_FWD) return is_long ? launch<DIR_FWD, true>(p, stream) : launch<DIR_FWD, false>(p, stream);
+    if (dir == DIR_INV) return is_long ? launch<DIR_INV, true>(p, stream) : launch<DIR_INV, false>(p, stream);
+    return is_long ? launch<DIR_RT, true>(p, stream) : launch<DIR_RT, false>(p, stream);
 }
 
 }  // namespace bdct
