@@ -144,25 +144,36 @@ static int tg_plan_tables(bdct_plan *p)
     return BDCT_OK;
 }
 
-// The line engine's tables: one per axis and scale (the forward and the
-// inverse of a normalization share their scale of the indices above 0).
+// The line engine's tables: per axis, for the forward passes and the others,
+// with the plan's scale (which its forward and inverse share at the indices
+// above 0) and the orthonormal one.
 static int lines_plan_tables(bdct_plan *p)
 {
-    const size_t ew = lines_table_elems(p->cols), eh = lines_table_elems(p->rows);
-    const bool plain = p->norm != BDCT_NORM_ORTHO && (p->kind & (BDCT_FORWARD | BDCT_INVERSE));
-    const size_t total = (plain ? 2 : 1) * (ew + eh);
+    const bool same = p->norm == BDCT_NORM_ORTHO;
+    size_t total = 0;
+    for (int other = 0; other < 2; ++other)
+        for (int ortho = 0; ortho < 2; ++ortho) {
+            if (ortho && same) {
+                p->line_w[other][1] = p->line_w[other][0];
+                p->line_h[other][1] = p->line_h[other][0];
+                continue;
+            }
+            p->line_w[other][ortho] = total;
+            total += lines_table_elems(p->cols, !other);
+            p->line_h[other][ortho] = total;
+            total += lines_table_elems(p->rows, !other);
+        }
     cudaError_t e = cudaMalloc(&p->line_tw, total * sizeof(float4));
     if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
-    p->line_w = p->line_w_ortho = 0;
-    p->line_h = p->line_h_ortho = ew;
-    e = lines_gen_table(p->line_tw, p->cols, std::sqrt(2.0 / p->cols), 0);
-    if (e == cudaSuccess) e = lines_gen_table(p->line_tw + ew, p->rows, std::sqrt(2.0 / p->rows), 0);
-    if (plain) {
-        p->line_w = ew + eh;
-        p->line_h = p->line_w + ew;
-        if (e == cudaSuccess) e = lines_gen_table(p->line_tw + p->line_w, p->cols, 2.0, 0);
-        if (e == cudaSuccess) e = lines_gen_table(p->line_tw + p->line_h, p->rows, 2.0, 0);
-    }
+    LineTable tables[8];
+    int n = 0;
+    for (int other = 0; other < 2; ++other)
+        for (int ortho = same ? 1 : 0; ortho < 2; ++ortho) {
+            auto scale = [&](int side) { return ortho ? std::sqrt(2.0 / side) : 2.0; };
+            tables[n++] = {p->line_tw + p->line_w[other][ortho], p->cols, !other, scale(p->cols)};
+            tables[n++] = {p->line_tw + p->line_h[other][ortho], p->rows, !other, scale(p->rows)};
+        }
+    e = lines_gen_tables(tables, n, 0);
     if (e != cudaSuccess) return cuda_fail(e);
     p->table_bytes = total * sizeof(float4);
     return BDCT_OK;
@@ -382,8 +393,8 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
     const long long hw = (long long)h * w;
     const bool ortho = dir == DIR_RT || dir == DIR_SPEC;
     const DirScales sc = ortho ? ortho_scales(p, DIR_FWD) : p->scales[dir];
-    const float4 *tw = p->line_tw + (ortho ? p->line_w_ortho : p->line_w);
-    const float4 *th = p->line_tw + (ortho ? p->line_h_ortho : p->line_h);
+    const float4 *fw = p->line_tw + p->line_w[0][ortho], *fh = p->line_tw + p->line_h[0][ortho];
+    const float4 *tw = p->line_tw + p->line_w[1][ortho], *th = p->line_tw + p->line_h[1][ortho];
     for (long long b0 = 0; b0 < count; b0 += p->chunk_arrays) {
         const long long nb = (count - b0) < p->chunk_arrays ? (count - b0) : p->chunk_arrays;
         const float *src = in_off ? in : in + b0 * hw;
@@ -399,9 +410,9 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
             if (e == cudaSuccess)
                 e = lines_pass(p->work, dst, w, h, nb, LINES_PAIR_COLS, sc.h, th, nullptr, p->status, s, nullptr, dof, true);
         } else {
-            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, tw, nullptr, p->status, s, so, nullptr);
+            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, fw, nullptr, p->status, s, so, nullptr);
             if (e == cudaSuccess && dir == DIR_FWD) {
-                e = lines_pass(p->work, dst, w, h, nb, LINES_FORWARD, sc.h, th, nullptr, p->status, s, nullptr, dof, true);
+                e = lines_pass(p->work, dst, w, h, nb, LINES_FORWARD, sc.h, fh, nullptr, p->status, s, nullptr, dof, true);
             } else if (e == cudaSuccess) {
                 e = lines_pass(p->work, p->work, w, h, nb, LINES_PAIR_ROWS, sc.h, th, p->spec_plain, p->status, s, nullptr,
                                nullptr, true);

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
                 float2 dr[8], di[8];
                 last_forward<8>(x, w, dr, di);
                 split_forward<8, AW::C>(gw, dr, di, sw, p.sc.w, a, b);
-                const SlotIndex<W> at(gw);
+                const SlotIndex<AW> at(gw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     bsm[at.ax(k) * C::PH + rw] = a[k].x;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
             last_forward<8>(x, w, dr, di);
             split_forward<8, AH::C>(gh, dr, di, sh, p.sc.h, a, b);
         }
-        const SlotIndex<H> at(gh);
+        const SlotIndex<AH> at(gh);
         if constexpr (DIR == DIR_FWD) {
             float *o = dst_of(ar) + rh;
 #pragma unroll
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
             first_step_adjoint<H, C::GH>(row_h, gh, th);
             __syncthreads();
             {
-                const SlotIndex<W> aw(gw);
+                const SlotIndex<AW> aw(gw);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     a[k].x = bsm[aw.ax(k) * C::PH + rw];
@@ -424,9 +424,9 @@ cudaError_t block_init_device(const float *d_table)
     void *t64 = nullptr, *t128 = nullptr;
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&t64, d_tab64);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&t128, d_tab128);
-    if (e == cudaSuccess) e = lines_gen_table((float4 *)t64, 64, 1.0, 0);
-    if (e == cudaSuccess) e = lines_gen_table((float4 *)t128, 128, 1.0, 0);
-    return e;
+    if (e != cudaSuccess) return e;
+    const LineTable tables[2] = {{(float4 *)t64, 64, false, 1.0}, {(float4 *)t128, 128, false, 1.0}};
+    return lines_gen_tables(tables, 2, 0);
 }
 
 bool block_supported(int rows, int cols)

@@ -65,29 +65,32 @@ bool lines_supported(int n)
 
 namespace {
 
-// Lines per panel and threads per line of length N.
-template <int N>
-struct LineCfg : LineSplit<N> {
-    static constexpr int G = N == 64 || N == 192 ? 2 : N <= 256 ? 4 : N <= 512 ? 8 : N == 768 ? 12
-                           : N == 1024 || N == 1536 ? 16 : N == 2048 ? 32 : 64;  // threads per line
-    static constexpr int PR = N <= 256 ? 32 : N <= 1536 ? 16 : 8;  // lines per panel
-    static constexpr int THREADS = PR * G;
-    // resident CTAs per SM the registers are held to: as many as shared memory
-    // and spill-free code allow (one more measured slower from 384 points on,
-    // 1024 points forward 0.378 -> 0.349 of HBM)
-    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? 5 : N == 384 ? 4 : N == 512 ? 4
-                            : N == 768 ? 3 : N == 1024 ? 2 : N == 1536 ? 2 : N == 2048 ? 2 : 1;
-    static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
-    // the tables are staged in shared memory (the split's read through L1
-    // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
-    static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N>::TAB * 16 + 16;
-    static_assert(THREADS % 32 == 0 && PR <= 32 && PR % 4 == 0, "lanes");
-    static_assert(SMEM <= 227 * 1024, "shared memory");
-};
-
 // rows -> transposed (forward), transposed -> rows (inverse), and forward,
 // diagonal, adjoint in one pass: rows -> rows or transposed -> transposed
 enum Mode { MODE_F = 0, MODE_I = 1, MODE_RR = 2, MODE_CC = 3 };
+
+// Lines per panel (PR), threads per line (G) and resident CTAs per SM that the
+// registers are held to (NB), by mode: the best of a sweep over radices and
+// these at 256 MiB, where one CTA more or half the lines per panel cost
+// 10-30%.  Panels of 8 lines (32-byte pieces on the transposed side) only
+// where shared memory holds no more.
+template <int N, int MODE>
+struct LineCfg : LineSplit<N, MODE == MODE_F> {
+    static constexpr bool F = MODE == MODE_F;
+    static constexpr int G = N == 64 || N == 192 ? 2 : N == 128 ? 4 : N == 256 ? (F ? 8 : 4) : N <= 512 ? 8
+                           : N == 768 ? 12 : N == 1024 ? 16 : N == 1536 ? (F ? 24 : 16) : N == 2048 ? 32 : 64;
+    static constexpr int PR = N <= 192 || (N == 256 && !F) ? 32 : N <= 1024 ? 16 : 8;
+    static constexpr int THREADS = PR * G;
+    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (F ? 6 : 5) : N == 384 ? (F ? 6 : 4)
+                            : N == 512 ? 4 : N == 768 ? (F ? 2 : 3) : N == 1024 ? 2 : N == 1536 ? (F ? 2 : 3)
+                            : N == 2048 ? 2 : 1;
+    static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
+    // the tables are staged in shared memory (the split's read through L1
+    // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
+    static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N, F>::TAB * 16 + 16;
+    static_assert(THREADS % 32 == 0 && PR <= 32 && PR % 4 == 0, "lanes");
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+};
 
 struct LinesParams {
     const float *src;
@@ -103,21 +106,47 @@ struct LinesParams {
                                          // what the previous pass wrote last, still in L2)
 };
 
+// Member m (0 .. 3: a.x, a.y, b.x, b.y) of slot k.
+template <int R>
+__device__ __forceinline__ float &member(float2 (&a)[R], float2 (&b)[R], int k, int m)
+{
+    return m == 0 ? a[k].x : m == 1 ? a[k].y : m == 2 ? b[k].x : b[k].y;
+}
+
+// Unit q = c + m j of a column (elements 4q .. 4q + 3, ld floats apart).
+__device__ __forceinline__ const char *unit_at(const float *p, int ld, int c, int m, int j, int i)
+{
+    const unsigned row = 4u * (unsigned)ld;
+    return mad_wide(4u * (unsigned)m * row, j, mad_wide(row, 4 * c + i, reinterpret_cast<const char *>(p)));
+}
+__device__ __forceinline__ float4 load_unit(const float *p, int ld, int c, int m, int j)
+{
+    auto at = [&](int i) { return __ldcg(reinterpret_cast<const float *>(unit_at(p, ld, c, m, j, i))); };
+    return make_float4(at(0), at(1), at(2), at(3));
+}
+__device__ __forceinline__ void store_unit(float *p, int ld, int c, int m, int j, float4 v)
+{
+    auto at = [&](int i) { return reinterpret_cast<float *>(const_cast<char *>(unit_at(p, ld, c, m, j, i))); };
+    __stcg(at(0), v.x);
+    __stcg(at(1), v.y);
+    __stcg(at(2), v.z);
+    __stcg(at(3), v.w);
+}
+
 // Unit slot of first-step result k1: base and direction (k1 < R1/2 kept its
 // column's slots, the others the mirror's).
-template <int N>
+template <typename C>
 __device__ __forceinline__ int sub_base(int k1, int &sgn)
 {
-    using C = LineCfg<N>;
     const bool e = k1 >= C::R1 / 2;
     sgn = e ? -1 : 1;
     return e ? C::M1 - 1 + C::M1 * (k1 - C::R1 / 2) : C::M1 * k1;
 }
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(const LinesParams p)
+__global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::NB) k_lines(const LinesParams p)
 {
-    using C = LineCfg<N>;
+    using C = LineCfg<N, MODE>;
     constexpr int R1 = C::R1, R2 = C::R2, R3 = C::R3, M1 = C::M1, CC = C::C, PR = C::PR, G = C::G;
     constexpr bool ROWS_IN = MODE == MODE_F || MODE == MODE_RR;
     constexpr bool ROWS_OUT = MODE == MODE_I || MODE == MODE_RR;
@@ -134,7 +163,6 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
         mbar_init(bar, 1);
         fence_mbar_init();
     }
-    pdl_launch_dependents();
     // the tables are plan data, written before any transform was queued
     for (int r = tid; r < C::TAB; r += C::THREADS) tab[r] = __ldg(p.tw + r);
     pdl_wait_prerequisites();
@@ -165,6 +193,10 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
         int r0;
         panel_at(pn, b, r0);
         const int next = pn + (int)gridDim.x;
+        // let the next kernel in only for the last panels: its CTAs, of another
+        // size, would hold registers and shared memory all along (128 x 512
+        // forward 434 -> 350 us, 256^2 spectral 725 -> 593 us)
+        if (next >= p.npanels) pdl_launch_dependents();
         bool ok = true;
         if constexpr (ROWS_IN) {
             ok = mbar_wait_bounded(bar, phase);
@@ -179,10 +211,8 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
                     if constexpr (MODE == MODE_CC) {
-                        const float *q = src + (long long)(4 * (cc + M1 * j)) * p.rows;
-                        x[j] = make_float4(__ldcg(q), __ldcg(q + p.rows), __ldcg(q + 2 * p.rows), __ldcg(q + 3 * p.rows));
-                        q = src + (long long)(4 * (M1 - 1 - cc + M1 * j)) * p.rows;
-                        y[j] = make_float4(__ldcg(q), __ldcg(q + p.rows), __ldcg(q + 2 * p.rows), __ldcg(q + 3 * p.rows));
+                        x[j] = load_unit(src, p.rows, cc, M1, j);
+                        y[j] = load_unit(src, p.rows, M1 - 1 - cc, M1, j);
                     } else {
                         x[j] = row[cc + M1 * j];
                         y[j] = row[M1 - 1 - cc + M1 * j];
@@ -214,7 +244,7 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
                 for (int q = g; q < R1 * R3 / 2; q += G) {
                     int sgn;
                     const int k1 = q / (R3 / 2), m3 = q % (R3 / 2);
-                    const int qb = sub_base<N>(k1, sgn);
+                    const int qb = sub_base<C>(k1, sgn);
                     float4 *px = row + qb + sgn * m3, *py = row + qb + sgn * (R3 - 1 - m3);
                     float4 x[R2 / 2], y[R2 / 2];
 #pragma unroll
@@ -238,7 +268,6 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
             const float *src = MODE == MODE_I ? src_of(b) + r0 + line : nullptr;
             float *dst = MODE == MODE_F ? dst_of(b) + r0 + line : nullptr;
             const float *lam = MODE == MODE_RR && p.lam ? p.lam + r0 + line : nullptr;
-            const long long ld = p.rows;
 #pragma unroll 1
             for (int rd = 0; rd < ROUNDS; ++rd) {
                 const int c = g + rd * G;
@@ -251,13 +280,12 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
                     pw = row + M1 - 1 + M1 * ((c ? CC - c : CC / 2) - R1 / 2);
                 } else {
                     const int k1 = c % R1, k2 = c / R1;
-                    px = row + sub_base<N>(k1, sx) + sx * (R3 * k2);
+                    px = row + sub_base<C>(k1, sx) + sx * (R3 * k2);
                     const int k1p = k1 ? R1 - k1 : 0;
                     const int k2p = k1 ? R2 - 1 - k2 : (c ? R2 - k2 : R2 / 2);
-                    pw = row + sub_base<N>(k1p, sw) + sw * (R3 - 1 + R3 * (k2p - R2 / 2));
+                    pw = row + sub_base<C>(k1p, sw) + sw * (R3 - 1 + R3 * (k2p - R2 / 2));
                     sw = -sw;
                 }
-                const SlotIndex<N> at(c);
                 float4 x[R3 / 2], w[R3 / 2];
                 float2 dr[R3], di[R3], a[R3], bb[R3];
                 if constexpr (FWD) {
@@ -282,13 +310,9 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
                     }
                 } else {
                     if (active) {
-#pragma unroll
-                        for (int k = 0; k < R3; ++k) {
-                            a[k].x = __ldcg(src + at.ax(k) * ld);
-                            a[k].y = __ldcg(src + at.ay(k) * ld);
-                            bb[k].x = __ldcg(src + at.bx(k) * ld);
-                            bb[k].y = __ldcg(src + at.by(k) * ld);
-                        }
+                        walk_slots<C>(src, c, p.rows, [&](const char *q, int k, int m) {
+                            member(a, bb, k, m) = __ldcg(reinterpret_cast<const float *>(q));
+                        });
                     }
                     if (rd == 0) {
                         // the previous panel's stores must have read the buffer
@@ -298,24 +322,16 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
                 }
                 if constexpr (MODE == MODE_F) {
                     if (active) {
-#pragma unroll
-                        for (int k = 0; k < R3; ++k) {
-                            dst[at.ax(k) * ld] = a[k].x;
-                            dst[at.ay(k) * ld] = a[k].y;
-                            dst[at.bx(k) * ld] = bb[k].x;
-                            dst[at.by(k) * ld] = bb[k].y;
-                        }
+                        walk_slots<C>(dst, c, p.rows, [&](const char *q, int k, int m) {
+                            __stcg(reinterpret_cast<float *>(const_cast<char *>(q)), member(a, bb, k, m));
+                        });
                     }
                 }
                 if constexpr (MODE == MODE_RR) {
                     if (active && lam) {
-#pragma unroll
-                        for (int k = 0; k < R3; ++k) {
-                            a[k].x *= __ldg(lam + at.ax(k) * ld);
-                            a[k].y *= __ldg(lam + at.ay(k) * ld);
-                            bb[k].x *= __ldg(lam + at.bx(k) * ld);
-                            bb[k].y *= __ldg(lam + at.by(k) * ld);
-                        }
+                        walk_slots<C>(lam, c, p.rows, [&](const char *q, int k, int m) {
+                            member(a, bb, k, m) *= __ldg(reinterpret_cast<const float *>(q));
+                        });
                     }
                 }
                 if constexpr (INV) {
@@ -338,7 +354,7 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
                 for (int q = g; q < R1 * R3 / 2; q += G) {
                     int sgn;
                     const int k1 = q / (R3 / 2), m3 = q % (R3 / 2);
-                    const int qb = sub_base<N>(k1, sgn);
+                    const int qb = sub_base<C>(k1, sgn);
                     float4 *px = row + qb + sgn * m3, *py = row + qb + sgn * (R3 - 1 - m3);
                     float4 x[R2 / 2], y[R2 / 2];
 #pragma unroll
@@ -368,10 +384,8 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
                     if constexpr (MODE == MODE_CC) {
-                        float *q = dst + (long long)(4 * (cc + M1 * j)) * p.rows;
-                        q[0] = x[j].x; q[p.rows] = x[j].y; q[2 * p.rows] = x[j].z; q[3 * p.rows] = x[j].w;
-                        q = dst + (long long)(4 * (M1 - 1 - cc + M1 * j)) * p.rows;
-                        q[0] = y[j].x; q[p.rows] = y[j].y; q[2 * p.rows] = y[j].z; q[3 * p.rows] = y[j].w;
+                        store_unit(dst, p.rows, cc, M1, j, x[j]);
+                        store_unit(dst, p.rows, M1 - 1 - cc, M1, j, y[j]);
                     } else {
                         row[cc + M1 * j] = x[j];
                         row[M1 - 1 - cc + M1 * j] = y[j];
@@ -403,7 +417,7 @@ __global__ void __launch_bounds__(LineCfg<N>::THREADS, LineCfg<N>::NB) k_lines(c
 template <int N, int MODE>
 cudaError_t lines_launch(const LinesParams &p0, long long nrows, cudaStream_t stream)
 {
-    using C = LineCfg<N>;
+    using C = LineCfg<N, MODE>;
     auto kern = k_lines<N, MODE>;
     static DeviceLaunchCache cache;
     int dev = 0, blocks_per_sm = 0, num_sms = 0;
@@ -468,8 +482,18 @@ __device__ void cos_sin_2pi(long long m, long long d, double &c, double &s)  // 
     sincospi(2.0 * (double)m / (double)d, &s, &c);
 }
 
-__global__ void k_gen_line_tw(float4 *t, TableShape q, double s1)
+// All tables of a plan in one launch, blockIdx.y the table.
+struct TableJobs {
+    float4 *dst[8];
+    TableShape shape[8];
+    double s1[8];
+};
+
+__global__ void k_gen_line_tw(const TableJobs jobs)
 {
+    float4 *t = jobs.dst[blockIdx.y];
+    const TableShape q = jobs.shape[blockIdx.y];
+    const double s1 = jobs.s1[blockIdx.y];
     const int L = q.n / 2, m1 = L / q.r1, c3 = L / q.r3;
     const int u1 = q.r1 * (m1 / 2), u2 = q.r2 > 1 ? q.r2 * (q.r3 / 2) : 0;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -503,45 +527,54 @@ __global__ void k_gen_line_tw(float4 *t, TableShape q, double s1)
 }
 
 template <int N>
-TableShape shape_of()
+TableShape shape_of(bool forward)
 {
-    return TableShape{N, LineCfg<N>::R1, LineCfg<N>::R2, LineCfg<N>::R3};
+    using A = LineSplit<N, true>;
+    using B = LineSplit<N, false>;
+    return forward ? TableShape{N, A::R1, A::R2, A::R3} : TableShape{N, B::R1, B::R2, B::R3};
 }
 
-bool table_shape(int n, TableShape *q)
+bool table_shape(int n, bool forward, TableShape *q)
 {
     switch (n) {
-        case 64: *q = shape_of<64>(); return true;
-        case 128: *q = shape_of<128>(); return true;
-        case 192: *q = shape_of<192>(); return true;
-        case 256: *q = shape_of<256>(); return true;
-        case 384: *q = shape_of<384>(); return true;
-        case 512: *q = shape_of<512>(); return true;
-        case 768: *q = shape_of<768>(); return true;
-        case 1024: *q = shape_of<1024>(); return true;
-        case 1536: *q = shape_of<1536>(); return true;
-        case 2048: *q = shape_of<2048>(); return true;
-        case 4096: *q = shape_of<4096>(); return true;
+        case 64: *q = shape_of<64>(forward); return true;
+        case 128: *q = shape_of<128>(forward); return true;
+        case 192: *q = shape_of<192>(forward); return true;
+        case 256: *q = shape_of<256>(forward); return true;
+        case 384: *q = shape_of<384>(forward); return true;
+        case 512: *q = shape_of<512>(forward); return true;
+        case 768: *q = shape_of<768>(forward); return true;
+        case 1024: *q = shape_of<1024>(forward); return true;
+        case 1536: *q = shape_of<1536>(forward); return true;
+        case 2048: *q = shape_of<2048>(forward); return true;
+        case 4096: *q = shape_of<4096>(forward); return true;
         default: return false;
     }
 }
 
 }  // namespace
 
-size_t lines_table_elems(int n)
+size_t lines_table_elems(int n, bool forward)
 {
     TableShape q;
-    if (!table_shape(n, &q)) return 0;
+    if (!table_shape(n, forward, &q)) return 0;
     const int L = n / 2;
     return (size_t)q.r1 * (L / q.r1 / 2) + (q.r2 > 1 ? (size_t)q.r2 * (q.r3 / 2) : 0) + L / 2 + L / 4;
 }
 
-cudaError_t lines_gen_table(float4 *dst, int n, double s1, cudaStream_t s)
+cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s)
 {
-    TableShape q;
-    if (!table_shape(n, &q)) return cudaErrorInvalidValue;
-    const int total = (int)lines_table_elems(n);
-    k_gen_line_tw<<<(total + 255) / 256, 256, 0, s>>>(dst, q, s1);
+    if (count < 1 || count > 8) return cudaErrorInvalidValue;
+    TableJobs jobs{};
+    int most = 0;
+    for (int i = 0; i < count; ++i) {
+        if (!table_shape(tables[i].n, tables[i].forward, &jobs.shape[i])) return cudaErrorInvalidValue;
+        jobs.dst[i] = tables[i].dst;
+        jobs.s1[i] = tables[i].s1;
+        const int e = (int)lines_table_elems(tables[i].n, tables[i].forward);
+        if (e > most) most = e;
+    }
+    k_gen_line_tw<<<dim3((most + 127) / 128, count), 128, 0, s>>>(jobs);
     return cudaGetLastError();
 }
 

@@ -25,10 +25,18 @@ cudaError_t lines_init_table3(const float *d_table);
 // True if n has an FFT-based line engine: powers of two 64..4096, and 192,
 // 384, 768, 1536.
 bool lines_supported(int n);
-// The twiddle table of length n (lines_table_elems(n) float4 entries),
-// generated in FP64; s1 is the scale of every index above 0, folded in.
-size_t lines_table_elems(int n);
-cudaError_t lines_gen_table(float4 *dst, int n, double s1, cudaStream_t s);
+// A twiddle table of length n (lines_table_elems float4 entries), for
+// LINES_FORWARD or for the other modes (they split the line differently); s1
+// is the scale of every index above 0, folded in.
+struct LineTable {
+    float4 *dst;
+    int n;
+    bool forward;
+    double s1;
+};
+size_t lines_table_elems(int n, bool forward);
+// Generate up to 8 tables in FP64, one launch.
+cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s);
 // One pass over `count` arrays.  sc holds the scales of the pass (sc.s1 the
 // table's s1; the pair modes apply them twice, so they take the orthonormal
 // ones); lam, if not null, is the diagonal of LINES_PAIR_ROWS: coefficient k

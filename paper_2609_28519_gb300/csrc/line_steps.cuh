@@ -10,14 +10,21 @@
 
 namespace bdct {
 
-// Radices of a line of N points: L = N/2 = R1 R2 R3 (R2 = 1: two steps).
-template <int N>
+// Radices of a line of N points: L = N/2 = R1 R2 R3 (R2 = 1: two steps), for
+// the line engine's forward passes (ROWS_FIRST) and for its others.  A forward
+// pass has its shared-memory traffic and its stores to hide and takes the
+// fewest, largest steps; the adjoint holds its loads in registers as well and
+// prefers smaller last steps (768 points: 24 x 16 runs 0.447 / 0.333 of HBM,
+// forward / inverse, 8 x 6 x 8 0.415 / 0.351).  Sides 64 and 128 split alike.
+template <int N, bool ROWS_FIRST = false>
 struct LineSplit {
     static constexpr int L = N / 2;
-    static constexpr int R1 = N == 64 ? 4 : N == 128 ? 8 : N == 192 ? 8 : N == 256 ? 16 : N == 384 ? 16
-                            : N == 512 ? 16 : N == 2048 ? 16 : N == 4096 ? 16 : 8;
-    static constexpr int R3 = N == 64 ? 8 : N == 128 ? 8 : N == 192 ? 12 : N == 256 ? 8 : N == 384 ? 12
-                            : N == 512 ? 16 : N == 4096 ? 16 : 8;
+    static constexpr int R1 = N == 64 ? 4 : N == 128 || N == 192 ? 8
+                            : ROWS_FIRST ? (N == 256 || N == 384 || N == 1536 ? 8 : N == 768 ? 24 : 16)
+                                         : (N == 768 || N == 1024 || N == 1536 ? 8 : 16);
+    static constexpr int R3 = N == 64 || N == 128 ? 8 : N == 192 ? 12
+                            : ROWS_FIRST ? (N == 256 || N == 512 ? 8 : N == 384 ? 6 : 16)
+                                         : (N == 384 ? 12 : N == 512 ? 16 : 8);
     static constexpr int R2 = L / (R1 * R3);
     static constexpr int M1 = L / R1;  // columns of the first step
     static constexpr int C = L / R3;   // columns of the last step
@@ -278,10 +285,13 @@ __device__ __forceinline__ void split_adjoint(int c, const float2 (&a)[R], const
 }
 
 // ------------------------------------------------------------ transposed side
-// visit(slot half, k): the output index of (a.x, a.y, b.x, b.y) of slot k3
-template <int N>
+// The coefficient index of every member of a couple's slots: slot k3 holds
+// k = C k3 + c (for c = 0 the upper half of the slots C/2 + C (k3 - R3/2)) in
+// a.x, L - k in a.y, N - k in b.x, L + k in b.y; slot 0 of c = 0 holds L/2 and
+// 3L/2 in b.
+template <typename C>
 struct SlotIndex {
-    using C = LineSplit<N>;
+    static constexpr int N = 2 * C::L;
     int lo, hi;   // first index of the lower and the upper half of the slots, minus C k3
     bool zero;
     __device__ __forceinline__ explicit SlotIndex(int c)
@@ -294,5 +304,49 @@ struct SlotIndex {
     __device__ __forceinline__ int bx(int k3) const { return (k3 == 0 && zero) ? C::L / 2 : N - k(k3); }
     __device__ __forceinline__ int by(int k3) const { return (k3 == 0 && zero) ? 3 * C::L / 2 : C::L + k(k3); }
 };
+
+// a + b * c, one instruction
+__device__ __forceinline__ const char *mad_wide(unsigned b, unsigned c, const char *a)
+{
+    unsigned long long r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(b), "r"(c), "l"(a));
+    return reinterpret_cast<const char *>(r);
+}
+
+// visit(address, member) for every slot of couple c in an array whose
+// consecutive coefficients lie ld floats apart from p on.  The four members of
+// a half of the slots step evenly (two up, two down), so an address is one
+// multiply-add from one of four bases (a 64-bit index times ld each took six
+// instructions per element, a quarter of a 256-point forward pass).
+// ld < 2^26 / C.
+template <typename C, typename F>
+__device__ __forceinline__ void walk_slots(const float *p, int c, int ld, F &&visit)
+{
+    constexpr int N = 2 * C::L;
+    constexpr int H = C::R3 / 2;
+    const unsigned step = 4u * C::C * (unsigned)ld;  // bytes per slot
+    const char *base = reinterpret_cast<const char *>(p);
+    const unsigned row = 4u * (unsigned)ld;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        const int k0 = half == 0 ? c : C::C * H + (c ? c : C::C / 2 - C::L / 2);  // of the half's first slot
+        const char *ax = mad_wide(row, k0, base), *by = mad_wide(row, C::L + k0, base);
+        // downward members from their lowest, the half's last slot
+        const char *ay = mad_wide(row, C::L - C::C * (H - 1) - k0, base), *bx = mad_wide(row, N - C::C * (H - 1) - k0, base);
+#pragma unroll
+        for (int t = 0; t < H; ++t) {
+            const int k3 = half * H + t;
+            visit(mad_wide(step, t, ax), k3, 0);
+            visit(mad_wide(step, H - 1 - t, ay), k3, 1);
+            const char *x = mad_wide(step, H - 1 - t, bx), *y = mad_wide(step, t, by);
+            if (k3 == 0 && c == 0) {
+                x = mad_wide(row, C::L / 2, base);
+                y = mad_wide(row, 3 * C::L / 2, base);
+            }
+            visit(x, k3, 2);
+            visit(y, k3, 3);
+        }
+    }
+}
 
 }  // namespace bdct
