@@ -518,12 +518,13 @@ static cudaError_t tg_direction(const bdct_plan *p, int slot, const float *src, 
                                 const long long *dst_off, long long nb, const float *lam, cudaStream_t s)
 {
     const int h = p->rows, w = p->cols;
+    const bool inv = slot & 1;
     if (p->tg_kron)
-        return tg_pass(src, dst, src_off, dst_off, nb, 1, 64, p->tg_ops + p->tg_h[slot], p->tc_terms, lam, p->tg_abuf, p->status, s);
-    cudaError_t e = tg_pass(src, p->work, src_off, nullptr, nb, h, w, p->tg_ops + p->tg_w[slot], p->tc_terms, nullptr,
+        return tg_pass(src, dst, src_off, dst_off, nb, 1, 64, inv, p->tg_ops + p->tg_h[slot], p->tc_terms, lam, p->tg_abuf, p->status, s);
+    cudaError_t e = tg_pass(src, p->work, src_off, nullptr, nb, h, w, inv, p->tg_ops + p->tg_w[slot], p->tc_terms, nullptr,
                             p->tg_abuf, p->status, s);
     if (e == cudaSuccess)
-        e = tg_pass(p->work, dst, nullptr, dst_off, nb, w, h, p->tg_ops + p->tg_h[slot], p->tc_terms, lam, p->tg_abuf, p->status, s);
+        e = tg_pass(p->work, dst, nullptr, dst_off, nb, w, h, inv, p->tg_ops + p->tg_h[slot], p->tc_terms, lam, p->tg_abuf, p->status, s);
     return e;
 }
 
@@ -543,7 +544,7 @@ static int run_tg(const bdct_plan *p, Dir dir, const float *in, const long long 
             const int slot = dir == DIR_FWD ? 0 : 1;
             if (p->tg_kron && inplace) {
                 // one pass cannot run in place: through the workspace
-                e = tg_pass(src, p->work, so, nullptr, nb, 1, 64, p->tg_ops + p->tg_h[slot], p->tc_terms, nullptr, p->tg_abuf,
+                e = tg_pass(src, p->work, so, nullptr, nb, 1, 64, slot & 1, p->tg_ops + p->tg_h[slot], p->tc_terms, nullptr, p->tg_abuf,
                             p->status, s);
                 ExecGeom g{p->work, dst, nb, 0, 0, 0, 0, nullptr, dof};
                 if (e == cudaSuccess) e = copy_arrays(p->work, g, p->rows, p->cols, s);
@@ -554,9 +555,9 @@ static int run_tg(const bdct_plan *p, Dir dir, const float *in, const long long 
             // round trip / spectral: orthonormal forward (times Lambda), then the inverse
             const float *lam = dir == DIR_SPEC ? p->spec_plain : nullptr;
             if (p->tg_kron) {
-                e = tg_pass(src, p->work, so, nullptr, nb, 1, 64, p->tg_ops + p->tg_h[2], p->tc_terms, lam, p->tg_abuf, p->status, s);
+                e = tg_pass(src, p->work, so, nullptr, nb, 1, 64, false, p->tg_ops + p->tg_h[2], p->tc_terms, lam, p->tg_abuf, p->status, s);
                 if (e == cudaSuccess)
-                    e = tg_pass(p->work, dst, nullptr, dof, nb, 1, 64, p->tg_ops + p->tg_h[3], p->tc_terms, nullptr,
+                    e = tg_pass(p->work, dst, nullptr, dof, nb, 1, 64, true, p->tg_ops + p->tg_h[3], p->tc_terms, nullptr,
                                 p->tg_abuf, p->status, s);
             } else {
                 e = tg_direction(p, 2, src, so, dst, dof, nb, lam, s);

@@ -163,10 +163,10 @@ cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, boo
 // Long contractions (K a multiple of 128) first split the input into
 // abuf (tg_split_elems(count * R, K) BF16 elements of plan workspace), then
 // run the warp-specialized kernel; shorter ones split in the kernel (abuf
-// unused, may be null).
+// unused, may be null).  `inverse` is the table's direction.
 cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, const long long *dst_off, long long count,
-                    int R, int K, const __nv_bfloat16 *ops, int terms, const float *lam, __nv_bfloat16 *abuf,
-                    unsigned int *status, cudaStream_t stream);
+                    int R, int K, bool inverse, const __nv_bfloat16 *ops, int terms, const float *lam,
+                    __nv_bfloat16 *abuf, unsigned int *status, cudaStream_t stream);
 size_t tg_split_elems(long long rows, int K);
 
 }  // namespace bdct

@@ -309,19 +309,37 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 //     mbarriers);
 //   warp 1, lane 0: issues the six products of a chunk into one of four TMEM
 //     partial accumulators and commits them twice (stage free, partial ready);
-//   warps 2-5: each reads its TMEM lane quadrant (warp % 4) of a finished
-//     partial, adds it to its row's running sums in registers (round to
-//     nearest, chunk order), releases the partial, and at the end of a tile
-//     stores the row transposed.
+//   warps 2-9: each reads its TMEM lane quadrant (warp % 4) and half of the
+//     columns of a finished partial, adds it to its row's running sums in
+//     registers (round to nearest, chunk order), releases the partial, and at
+//     the end of a tile stores its part of the row transposed (with four warps
+//     the reads of the partials held up the products).
 // Tiles are 128 rows by 128 outputs, K chunks of 64.
+
+//
+// Half products.  The operator's rows are even or odd about the middle of the
+// line, so for lengths that are multiples of 256 the forward contracts s_j =
+// x_j + x_{K-1-j} with the even operator and d_j = x_j - x_{K-1-j} with the odd
+// one (j < K/2), and the inverse the even and the odd coefficients with the
+// two halves of its operator, x_j = a_j + b_j, x_{K-1-j} = a_j - b_j: half the
+// products, half the input blocks each tile streams, half the partials.  An
+// item is then a row tile and 128 output pairs, its two products one after the
+// other, both sums of a thread's 64 pairs in registers until they meet.  16 arrays of 1024 x 1024, forward and inverse:
+// 761 -> 510 us.  (K/2 a multiple of 64 but not of 128 would leave half
+// tiles, so those lengths keep the whole operator.)
+
+enum SplitMode { SPLIT_WHOLE = 0, SPLIT_FWD = 1, SPLIT_INV = 2 };
 
 // Split src rows into the blocked BF16 terms: thread t of a group of eight
 // takes row (8 q + t % 8) of a core matrix, so that eight lanes write one
-// 128-byte core matrix and each lane reads one 32-byte sector.
-template <int TERMS>
+// 128-byte core matrix and each lane reads one 32-byte sector.  With half
+// products K is the half length, each unit makes eight pairs, and the blocks
+// of a row tile are the first operand's chunks, then the second's.
+template <int TERMS, int SPLIT>
 __global__ void k_tg_presplit(const float *src, const long long *src_off, long long rows_total, int R, int K, int KC,
                               long long m_tiles, __nv_bfloat16 *abuf)
 {
+    constexpr int SUB = SPLIT == SPLIT_WHOLE ? 1 : 2;
     const int nk = K / KC;
     const int groups = KC / 8;                       // 8-column groups per chunk row
     const long long per_tile = 128LL * K / 8;        // work units per row tile
@@ -338,36 +356,63 @@ __global__ void k_tg_presplit(const float *src, const long long *src_off, long l
         const int rq = (int)(rem / groups);          // core-matrix row block (0..15)
         const int row = rq * 8 + r8;                 // row within the tile
         const long long m = mt * 128 + row;
-        float v[8];
+        float v[SUB][8];
+#pragma unroll
+        for (int e = 0; e < 8 * SUB; ++e) v[e / 8][e % 8] = 0.0f;
         if (m < rows_total) {
             const long long b = m / R, r = m - b * R;
-            const float *q = src + (src_off ? src_off[b] : b * (long long)R * K) + r * K + (long long)kc * KC + 8 * g;
-            const float4 t0 = __ldg(reinterpret_cast<const float4 *>(q));
-            const float4 t1 = __ldg(reinterpret_cast<const float4 *>(q) + 1);
-            v[0] = t0.x; v[1] = t0.y; v[2] = t0.z; v[3] = t0.w;
-            v[4] = t1.x; v[5] = t1.y; v[6] = t1.z; v[7] = t1.w;
-        } else {
+            const int line = K * SUB, j0 = kc * KC + 8 * g;
+            const float *q = src + (src_off ? src_off[b] : b * (long long)R * line) + r * line;
+            auto load8 = [&](const float *f, float (&x)[8]) {
+                const float4 t0 = __ldg(reinterpret_cast<const float4 *>(f));
+                const float4 t1 = __ldg(reinterpret_cast<const float4 *>(f) + 1);
+                x[0] = t0.x; x[1] = t0.y; x[2] = t0.z; x[3] = t0.w;
+                x[4] = t1.x; x[5] = t1.y; x[6] = t1.z; x[7] = t1.w;
+            };
+            if constexpr (SPLIT == SPLIT_WHOLE) {
+                load8(q + j0, v[0]);
+            } else {
+                // the eight mirrored elements, or the next eight of sixteen
+                float x[8], y[8];
+                load8(SPLIT == SPLIT_FWD ? q + j0 : q + 2 * j0, x);
+                load8(SPLIT == SPLIT_FWD ? q + line - 8 - j0 : q + 2 * j0 + 8, y);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = 0.0f;
+                for (int e = 0; e < 8; ++e) {
+                    if (SPLIT == SPLIT_FWD) {
+                        v[0][e] = x[e] + y[7 - e];
+                        v[SUB - 1][e] = x[e] - y[7 - e];
+                    } else {
+                        v[0][e] = e < 4 ? x[2 * (e & 3)] : y[2 * (e & 3)];
+                        v[SUB - 1][e] = e < 4 ? x[2 * (e & 3) + 1] : y[2 * (e & 3) + 1];
+                    }
+                }
+            }
         }
-        __nv_bfloat16 t[TERMS][8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            __nv_bfloat16 sp[3];
-            split3<TERMS>(v[e], sp);
+        for (int sub = 0; sub < SUB; ++sub) {
+            __nv_bfloat16 t[TERMS][8];
 #pragma unroll
-            for (int tt = 0; tt < TERMS; ++tt) t[tt][e] = sp[tt];
+            for (int e = 0; e < 8; ++e) {
+                __nv_bfloat16 sp[3];
+                split3<TERMS>(v[sub][e], sp);
+#pragma unroll
+                for (int tt = 0; tt < TERMS; ++tt) t[tt][e] = sp[tt];
+            }
+            uint8_t *blk = reinterpret_cast<uint8_t *>(abuf) + ((mt * SUB + sub) * nk + kc) * (3LL * 128 * KC * 2);
+            const int off = kmaj_off_bytes(row, 8 * g, KC);
+#pragma unroll
+            for (int tt = 0; tt < TERMS; ++tt)
+                *reinterpret_cast<uint4 *>(blk + (long long)tt * 128 * KC * 2 + off) =
+                    *reinterpret_cast<const uint4 *>(t[tt]);
         }
-        uint8_t *blk = reinterpret_cast<uint8_t *>(abuf) + (mt * nk + kc) * (3LL * 128 * KC * 2);
-        const int off = kmaj_off_bytes(row, 8 * g, KC);
-#pragma unroll
-        for (int tt = 0; tt < TERMS; ++tt)
-            *reinterpret_cast<uint4 *>(blk + (long long)tt * 128 * KC * 2 + off) = *reinterpret_cast<const uint4 *>(t[tt]);
     }
 }
 
 constexpr int kTg2NT = 128;
 constexpr int kTg2Stages = 2;
+constexpr int kTg2Epi = 8;                            // epilogue warps: two per TMEM lane quadrant
+constexpr int kTg2Cols = kTg2NT / (kTg2Epi / 4);      // columns of each
+constexpr int kTg2Threads = 64 + 32 * kTg2Epi;
 // TMEM partial accumulators (kTg2Acc x 128 columns of the 512): the MMA lane
 // may run kTg2Acc - 1 chunks ahead of the epilogue warps' reads
 constexpr int kTg2Acc = 4;
@@ -378,19 +423,20 @@ constexpr int kTg2Stage = kTg2AStage + kTg2BStage;
 constexpr size_t kTg2Smem = (size_t)kTg2Stages * kTg2Stage + (2 * kTg2Stages + 2 * kTg2Acc) * 8 + 16;
 
 struct Tg2Params {
-    const __nv_bfloat16 *abuf;       // input terms, [row tile][chunk][term][128 x KC]
-    const __nv_bfloat16 *ops;        // operator terms, [n tile][chunk][term][128 x KC]
+    const __nv_bfloat16 *abuf;       // input terms, [row tile][product][chunk][term][128 x KC]
+    const __nv_bfloat16 *ops;        // operator terms, [product][n tile][chunk][term][128 x KC]
     float *dst;
     const long long *dst_off;
     long long rows_total;
-    int R, N, KC, nk, n_tiles;
+    int R, N, KC, nk, n_tiles;       // nk, n_tiles: of one product
+    int sub, inverse;                // products per item (2: half products), and which half form
     long long items;
     const float *lam;
     unsigned int *status;
 };
 
 template <int TERMS>
-__global__ void __launch_bounds__(192, 1) k_tcg2(const Tg2Params p)
+__global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
 {
     extern __shared__ __align__(1024) uint8_t t2s[];
     uint64_t *full = reinterpret_cast<uint64_t *>(t2s + kTg2Stages * kTg2Stage);
@@ -408,7 +454,7 @@ __global__ void __launch_bounds__(192, 1) k_tcg2(const Tg2Params p)
         }
         for (int a = 0; a < kTg2Acc; ++a) {
             mbar_init(&pfull[a], 1);
-            mbar_init(&pempty[a], 4);  // one arrival per epilogue warp
+            mbar_init(&pempty[a], kTg2Epi);  // one arrival per epilogue warp
         }
         *abort_flag = 0;
         fence_mbar_init();
@@ -438,16 +484,17 @@ __global__ void __launch_bounds__(192, 1) k_tcg2(const Tg2Params p)
             for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
                 const long long mt = item / p.n_tiles;
                 const int nt = (int)(item % p.n_tiles);
-                for (int kc = 0; kc < nk; ++kc, ++c) {
+                for (int ec = 0; ec < p.sub * nk; ++ec, ++c) {
                     const int s = (int)(c % kTg2Stages);
                     const uint32_t use = (uint32_t)(c / kTg2Stages);
                     if (c >= kTg2Stages && !mbar_wait_bounded(&empty[s], (use - 1) & 1u)) { ok = false; break; }
                     if (*abort_flag) { ok = false; break; }
                     uint8_t *st = t2s + s * kTg2Stage;
                     mbar_arrive_expect_tx(&full[s], (uint32_t)TERMS * (a_term + b_term));
-                    bulk_load(st, p.abuf + (mt * nk + kc) * blk_elems, (uint32_t)TERMS * a_term, &full[s]);
-                    bulk_load(st + kTg2AStage, p.ops + ((long long)nt * nk + kc) * blk_elems, (uint32_t)TERMS * b_term,
-                              &full[s]);
+                    const int e = ec >= nk, kc = ec - e * nk;
+                    bulk_load(st, p.abuf + (mt * p.sub * nk + ec) * blk_elems, (uint32_t)TERMS * a_term, &full[s]);
+                    bulk_load(st + kTg2AStage, p.ops + ((long long)(nt + e * p.n_tiles) * nk + kc) * blk_elems,
+                              (uint32_t)TERMS * b_term, &full[s]);
                     last_load = c;
                 }
             }
@@ -462,7 +509,7 @@ __global__ void __launch_bounds__(192, 1) k_tcg2(const Tg2Params p)
             constexpr int first = TERMS == 3 ? 0 : (TERMS == 2 ? 3 : 5);
             long long c = 0;
             for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-                for (int kc = 0; kc < nk; ++kc, ++c) {
+                for (int ec = 0; ec < p.sub * nk; ++ec, ++c) {
                     const int s = (int)(c % kTg2Stages), a = (int)(c % kTg2Acc);
                     if (!mbar_wait_bounded(&full[s], (uint32_t)(c / kTg2Stages) & 1u)) { ok = false; break; }
                     if (c >= kTg2Acc && !mbar_wait_bounded(&pempty[a], (uint32_t)(c / kTg2Acc - 1) & 1u)) {
@@ -486,47 +533,67 @@ __global__ void __launch_bounds__(192, 1) k_tcg2(const Tg2Params p)
             }
         }
     } else {
-        // ---- epilogue: TMEM lane quadrant q of every partial
+        // ---- epilogue: TMEM lane quadrant q, half of the columns of every partial
         const int q = warp & 3;
         const int row = 32 * q + lane;
+        const int col0 = (warp - 2) / 4 * kTg2Cols;
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-        float sum[kTg2NT];
-#pragma unroll
-        for (int j = 0; j < kTg2NT; ++j) sum[j] = 0.0f;
+        float sum[2][kTg2Cols];  // of the item's one or two products
         long long c = 0;
-        for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
+        auto product = [&](float (&acc)[kTg2Cols]) {
+#pragma unroll
+            for (int j = 0; j < kTg2Cols; ++j) acc[j] = 0.0f;
             for (int kc = 0; kc < nk; ++kc, ++c) {
                 const int a = (int)(c % kTg2Acc);
                 bool w = mbar_wait_bounded(&pfull[a], (uint32_t)(c / kTg2Acc) & 1u);
                 w = __all_sync(0xffffffffu, w);
-                if (!w) { ok = false; break; }
+                if (!w) return false;
                 tc_fence_after();
 #pragma unroll
-                for (int cc = 0; cc < kTg2NT / 16; ++cc) {
+                for (int cc = 0; cc < kTg2Cols / 16; ++cc) {
                     float y[16];
-                    tmem_ld16(tmem + (uint32_t)(a * kTg2NT) + lane_off + 16 * cc, y);
+                    tmem_ld16(tmem + (uint32_t)(a * kTg2NT + col0) + lane_off + 16 * cc, y);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) sum[16 * cc + j] += y[j];
+                    for (int j = 0; j < 16; ++j) acc[16 * cc + j] += y[j];
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&pempty[a]);
             }
+            return true;
+        };
+        for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
+            ok = product(sum[0]);
+            if (ok && p.sub == 2) ok = product(sum[1]);
             if (!ok) break;
             const long long m = (item / p.n_tiles) * 128 + row;
-            if (m < p.rows_total) {
-                const long long b = m / p.R, r = m - b * p.R;
-                float *dbase = p.dst + (p.dst_off ? p.dst_off[b] : b * (long long)p.N * p.R);
-                const int n0 = (int)(item % p.n_tiles) * kTg2NT;
-                if (p.lam) {
+            if (m >= p.rows_total) continue;
+            const long long b = m / p.R, r = m - b * p.R;
+            float *dbase = p.dst + (p.dst_off ? p.dst_off[b] : b * (long long)p.N * p.R) + r;
+            const long long n0 = (item % p.n_tiles) * kTg2NT + col0, ld = p.R;
+            if (p.sub == 1) {
+                const float *l = p.lam ? p.lam + n0 * ld + r : nullptr;
 #pragma unroll
-                    for (int j = 0; j < kTg2NT; ++j) sum[j] *= __ldg(p.lam + (long long)(n0 + j) * p.R + r);
+                for (int j = 0; j < kTg2Cols; ++j)
+                    dbase[(n0 + j) * ld] = l ? sum[0][j] * __ldg(l + j * ld) : sum[0][j];
+            } else if (!p.inverse) {
+                // coefficients 2 (n0 + j) and the next
+                float *d = dbase + 2 * n0 * ld;
+                const float *l = p.lam ? p.lam + 2 * n0 * ld + r : nullptr;
+#pragma unroll
+                for (int j = 0; j < kTg2Cols; ++j) {
+                    d[2 * j * ld] = l ? sum[0][j] * __ldg(l + 2 * j * ld) : sum[0][j];
+                    d[(2 * j + 1) * ld] = l ? sum[1][j] * __ldg(l + (2 * j + 1) * ld) : sum[1][j];
                 }
+            } else {
+                // samples n0 + j and their mirrors
+                float *d = dbase + n0 * ld, *u = dbase + (p.N - 1 - n0) * ld;
 #pragma unroll
-                for (int j = 0; j < kTg2NT; ++j) dbase[(long long)(n0 + j) * p.R + r] = sum[j];
+                for (int j = 0; j < kTg2Cols; ++j) {
+                    d[j * ld] = sum[0][j] + sum[1][j];
+                    u[-j * ld] = sum[0][j] - sum[1][j];
+                }
             }
-#pragma unroll
-            for (int j = 0; j < kTg2NT; ++j) sum[j] = 0.0f;
         }
     }
     if (!ok) {
@@ -820,12 +887,18 @@ __device__ double tg_op_value(int row, int col, int n, int direction, int norm)
     return s * c;
 }
 
-__global__ void k_gen_tg_op(__nv_bfloat16 *dst, int N, int K, int direction, int norm, int NT, int KC, int kron)
+// half: N outputs of contraction length K = N/2 -- N/2 of the even product, then
+// of the odd one.
+__global__ void k_gen_tg_op(__nv_bfloat16 *dst, int N, int K, int direction, int norm, int NT, int KC, int kron, int half)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)N * K) return;
     const int nn = (int)(idx / K), kk = (int)(idx % K);
     double val;
+    if (half) {
+        const int e = nn >= N / 2, i = nn - e * (N / 2);
+        val = direction == 1 ? tg_op_value(2 * i + e, kk, N, 1, norm) : tg_op_value(i, 2 * kk + e, N, 2, norm);
+    } else
     if (kron) {
         // (Q (x) Q)[(f1, f2)][(i, j)] = M8[f1][i] * M8[f2][j] for the row-major 8 x 8 array
         val = tg_op_value(nn >> 3, kk >> 3, 8, direction, norm) * tg_op_value(nn & 7, kk & 7, 8, direction, norm);
@@ -867,15 +940,20 @@ static int tg_kc(int k) { return k % 64 == 0 ? 64 : ((k == 16 || k == 32) ? k : 
 
 bool tg_axis_ok(int n) { return n == 16 || n == 32 || (n % 64 == 0 && n >= 64 && n <= 8192); }
 
-size_t tg_table_elems(int n) { return (size_t)3 * n * n; }
+// Half products: both halves of the outputs in whole tiles.
+static bool tg_half(int n) { return n % 256 == 0; }
+
+size_t tg_table_elems(int n) { return (size_t)3 * n * (tg_half(n) ? n / 2 : n); }
 
 cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, bool kron, cudaStream_t s)
 {
     const int N = kron ? 64 : n;
     const int NT = tg_nt(N), KC = tg_kc(N);
     if (!NT || !KC) return cudaErrorInvalidValue;
-    const long long total = (long long)N * N;
-    k_gen_tg_op<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(dst, N, N, direction, norm, NT, KC, kron ? 1 : 0);
+    const int K = tg_half(N) ? N / 2 : N;
+    const long long total = (long long)N * K;
+    k_gen_tg_op<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(dst, N, K, direction, norm, NT, KC, kron ? 1 : 0,
+                                                               tg_half(N) ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -962,8 +1040,8 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
             b = 1;
             if (r == cudaSuccess && debug_enabled())
-                fprintf(stderr, "[bdct] k_tcg2<%d>: 1 CTA/SM x 192 threads, smem %zu B, TMEM %d cols\n", TERMS,
-                        kTg2Smem, kTg2Acc * kTg2NT);
+                fprintf(stderr, "[bdct] k_tcg2<%d>: 1 CTA/SM x %d threads, smem %zu B, TMEM %d cols\n", TERMS,
+                        kTg2Threads, kTg2Smem, kTg2Acc * kTg2NT);
             return r;
         },
         &bps, &sms);
@@ -975,8 +1053,9 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
         const long long work = m_tiles * 128LL * K / 8;
         long long blocks = (work + 255) / 256;
         if (blocks > (long long)sms * 16) blocks = (long long)sms * 16;
-        k_tg_presplit<TERMS><<<(unsigned)blocks, 256, 0, stream>>>(src, src_off, p.rows_total, p.R, K, p.KC, m_tiles,
-                                                                    abuf);
+        auto split = p.sub == 1 ? k_tg_presplit<TERMS, SPLIT_WHOLE>
+                     : p.inverse ? k_tg_presplit<TERMS, SPLIT_INV> : k_tg_presplit<TERMS, SPLIT_FWD>;
+        split<<<(unsigned)blocks, 256, 0, stream>>>(src, src_off, p.rows_total, p.R, K, p.KC, m_tiles, abuf);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -986,7 +1065,7 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
     if (grid > p.items) grid = p.items;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(192);
+    cfg.blockDim = dim3(kTg2Threads);
     cfg.dynamicSmemBytes = kTg2Smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -998,8 +1077,8 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
 }
 
 cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, const long long *dst_off, long long count,
-                    int R, int K, const __nv_bfloat16 *ops, int terms, const float *lam, __nv_bfloat16 *abuf,
-                    unsigned int *status, cudaStream_t stream)
+                    int R, int K, bool inverse, const __nv_bfloat16 *ops, int terms, const float *lam,
+                    __nv_bfloat16 *abuf, unsigned int *status, cudaStream_t stream)
 {
     if (count <= 0) return cudaSuccess;
     const int N = K;  // square 1D operators (the Kronecker one included)
@@ -1028,15 +1107,18 @@ cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, cons
         p.R = R;
         p.N = N;
         p.KC = KC;
-        p.nk = K / KC;
-        p.n_tiles = N / kTg2NT;
+        p.sub = tg_half(K) ? 2 : 1;
+        p.inverse = inverse ? 1 : 0;
+        const int KH = K / p.sub;
+        p.nk = KH / KC;
+        p.n_tiles = N / p.sub / kTg2NT;
         p.items = ((p.rows_total + 127) / 128) * p.n_tiles;
         p.lam = lam;
         p.status = status;
         switch (terms) {
-            case 3: return tg2_launch<3>(src, src_off, p, K, abuf, stream);
-            case 2: return tg2_launch<2>(src, src_off, p, K, abuf, stream);
-            default: return tg2_launch<1>(src, src_off, p, K, abuf, stream);
+            case 3: return tg2_launch<3>(src, src_off, p, KH, abuf, stream);
+            case 2: return tg2_launch<2>(src, src_off, p, KH, abuf, stream);
+            default: return tg2_launch<1>(src, src_off, p, KH, abuf, stream);
         }
     }
     TgParams p{};
