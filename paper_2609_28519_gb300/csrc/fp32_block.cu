@@ -41,17 +41,13 @@ namespace bdct {
 
 namespace {
 
-// Tables of 64 and 128 points with s_1 = 1; a CTA folds the scale in as it
-// stages them.
-__device__ float4 d_tab64[LineSplit<64>::TAB];
-__device__ float4 d_tab128[LineSplit<128>::TAB];
-
-template <int N>
-__device__ __forceinline__ const float4 *line_table()
-{
-    if constexpr (N == 64) return d_tab64;
-    else return d_tab128;
-}
+// Tables of 64 and 128 points, for the orthonormal scale and the unnormalized
+// pair's.  A warp's 32 lanes take 32 lines of one couple, so every entry is
+// uniform over the warp and comes through the constant cache: in shared memory
+// the tables took a quarter of its wavefronts (128 x 128 forward 242 -> 220 us,
+// round trip 437 -> 375, 8192 arrays).
+constexpr int kTabMax = LineSplit<128>::TAB;
+__constant__ float4 c_line[4 * kTabMax];  // [plain][64 or 128]
 
 template <int H, int W>
 struct BlockCfg {
@@ -62,7 +58,7 @@ struct BlockCfg {
     static constexpr int NB = 1024 / THREADS;  // CTAs per SM: 64 registers a thread
     static constexpr int PW = W + 4, PH = H + 4;  // row pitch before and after the transposition (floats)
     static constexpr int BUF = H * PW > W * PH ? H * PW : W * PH;
-    static constexpr size_t SMEM = (size_t)BUF * 4 + (size_t)(AW::TAB + AH::TAB) * 16 + 16;
+    static constexpr size_t SMEM = (size_t)BUF * 4 + 16;
     static_assert(GH == AH::C / 2 && GW == AW::C / 2, "one couple each");
     static_assert(THREADS >= H && H % 32 == 0 && W % 32 == 0, "lanes");
     static_assert(AW::R2 == 1 && AH::R2 == 1, "two steps");
@@ -78,6 +74,7 @@ struct BlockParams {
     DirScales sc;
     const float *lam;         // spectral: Lambda (H x W), else null
     unsigned int *status;
+    int plain;                // the unnormalized pair's scales
 };
 
 // First step of this thread's couples of line `row` (in place), and its transpose.
@@ -140,11 +137,11 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
     using AH = LineSplit<H>;
     constexpr bool FWD = DIR != DIR_INV, INV = DIR != DIR_FWD;
     extern __shared__ __align__(128) float bsm[];
-    float4 *tw = reinterpret_cast<float4 *>(bsm + C::BUF), *th = tw + AW::TAB;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(th + AH::TAB);
+    const float4 *tw = c_line + (2 * p.plain + (W == 128)) * kTabMax, *th = c_line + (2 * p.plain + (H == 128)) * kTabMax;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(bsm + C::BUF);
     const int tid = threadIdx.x;
     // row pass: row rw, couple gw; column pass: column rh, couple gh
-    const int rw = tid % H, gw = tid / H, rh = tid % W, gh = tid / W;
+    const int rw = tid % H, gw = __shfl_sync(0xffffffffu, tid / H, 0), rh = tid % W, gh = __shfl_sync(0xffffffffu, tid / W, 0);
     float4 *row_w = reinterpret_cast<float4 *>(bsm + rw * C::PW);
     float4 *row_h = reinterpret_cast<float4 *>(bsm + rh * C::PH);
     const SplitTable sw{tw + AW::U1, reinterpret_cast<const float2 *>(tw + AW::U1 + AW::L / 2)};
@@ -155,23 +152,6 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
         fence_mbar_init();
     }
     pdl_launch_dependents();
-    // the tables (device constants), the split's entries times s_1
-    auto stage = [&](float4 *t, const float4 *src, int u1, int l2, int n, float s1) {
-        for (int e = tid; e < n; e += C::THREADS) {
-            float4 v = src[e];
-            if (e >= u1) {
-                v.z *= s1;
-                v.w *= s1;
-                if (e >= u1 + l2) {
-                    v.x *= s1;
-                    v.y *= s1;
-                }
-            }
-            t[e] = v;
-        }
-    };
-    stage(tw, line_table<W>(), AW::U1, AW::L / 2, AW::TAB, p.sc.w.s1);
-    stage(th, line_table<H>(), AH::U1, AH::L / 2, AH::TAB, p.sc.h.s1);
     pdl_wait_prerequisites();
     __syncthreads();
 
@@ -198,6 +178,9 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
     for (long long ar = blockIdx.x; ar < p.count; ar += gridDim.x) {
         const long long next = ar + gridDim.x;
         float2 a[8], b[8];  // the couple's coefficients (R3 = 8 for both lengths)
+        // the inverse's next array into L2: its loads go straight to registers
+        // (128 x 128 251 -> 243 us; the other directions gain nothing)
+        if (DIR == DIR_INV && !TILED && tid == 0 && next < p.count) bulk_prefetch_l2(src_of(next), H * W * 4);
         if constexpr (FWD) {
             const bool ok = mbar_wait_bounded(bar, phase);
             phase ^= 1;
@@ -382,6 +365,7 @@ cudaError_t block_launch_one(const DirScales &sc, const ExecGeom &g, unsigned in
         p.sc = DirScales{ortho(H), ortho(W)};
     }
     p.lam = g.lam;
+    p.plain = p.sc.w.s1 == 2.0f;
     p.status = status;
     if (DIR == DIR_SPEC && !g.lam) return cudaErrorInvalidValue;
     long long grid = (long long)bps_dev * num_sms;
@@ -421,12 +405,20 @@ cudaError_t block_dir(Dir dir, const DirScales &sc, const ExecGeom &g, unsigned 
 cudaError_t block_init_device(const float *d_table)
 {
     cudaError_t e = init_cos_table(d_table);
-    void *t64 = nullptr, *t128 = nullptr;
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&t64, d_tab64);
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&t128, d_tab128);
+    float4 *tmp = nullptr;
+    const size_t bytes = sizeof(float4) * 4 * kTabMax;
+    if (e == cudaSuccess) e = cudaMalloc(&tmp, bytes);
     if (e != cudaSuccess) return e;
-    const LineTable tables[2] = {{(float4 *)t64, 64, false, 1.0}, {(float4 *)t128, 128, false, 1.0}};
-    return lines_gen_tables(tables, 2, 0);
+    LineTable tables[4];
+    for (int i = 0; i < 4; ++i) {
+        const int n = i % 2 ? 128 : 64;
+        tables[i] = {tmp + i * kTabMax, n, false, i / 2 ? 2.0 : std::sqrt(2.0 / n)};
+    }
+    e = cudaMemset(tmp, 0, bytes);
+    if (e == cudaSuccess) e = lines_gen_tables(tables, 4, 0);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_line, tmp, bytes, 0, cudaMemcpyDeviceToDevice);
+    cudaFree(tmp);
+    return e;
 }
 
 bool block_supported(int rows, int cols)

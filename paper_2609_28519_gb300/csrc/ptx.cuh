@@ -117,6 +117,12 @@ __device__ __forceinline__ void bulk_store(void *gdst, const void *smem_src, uin
                  : "memory");
 }
 
+// Ask for `bytes` (a multiple of 16) of global memory in L2.
+__device__ __forceinline__ void bulk_prefetch_l2(const void *gsrc, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gsrc), "r"(bytes) : "memory");
+}
+
 // 2D tensor tile global -> shared (box defined by the tensor map).
 __device__ __forceinline__ void tensor_load_2d(void *smem_dst, const CUtensorMap *map, int x, int y,
                                                uint64_t *bar)
