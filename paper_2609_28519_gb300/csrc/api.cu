@@ -144,35 +144,44 @@ static int tg_plan_tables(bdct_plan *p)
     return BDCT_OK;
 }
 
-// The line engine's tables: per axis, for the forward passes and the others,
-// with the plan's scale (which its forward and inverse share at the indices
-// above 0) and the orthonormal one.
+// The line engine's tables: per axis, for each set of modes that the plan's
+// directions run, with the plan's scale (which its forward and inverse share
+// at the indices above 0) or the orthonormal one (round trip and spectral).
 static int lines_plan_tables(bdct_plan *p)
 {
     const bool same = p->norm == BDCT_NORM_ORTHO;
+    const unsigned k = p->kind;
+    // needed by set and scale: the forward, the inverse and the round trip, the spectral direction's
+    const bool need[3][2] = {{(k & BDCT_FORWARD) != 0, (k & BDCT_SPECTRAL) != 0},
+                             {(k & BDCT_INVERSE) != 0, (k & BDCT_ROUNDTRIP) != 0},
+                             {false, (k & BDCT_SPECTRAL) != 0}};
+    LineTable tables[12];
+    int n = 0;
     size_t total = 0;
-    for (int other = 0; other < 2; ++other)
+    for (int set = 0; set < 3; ++set)
         for (int ortho = 0; ortho < 2; ++ortho) {
-            if (ortho && same) {
-                p->line_w[other][1] = p->line_w[other][0];
-                p->line_h[other][1] = p->line_h[other][0];
+            if (!need[set][ortho]) continue;
+            if (ortho && same && need[set][0]) {
+                p->line_w[set][1] = p->line_w[set][0];
+                p->line_h[set][1] = p->line_h[set][0];
                 continue;
             }
-            p->line_w[other][ortho] = total;
-            total += lines_table_elems(p->cols, !other);
-            p->line_h[other][ortho] = total;
-            total += lines_table_elems(p->rows, !other);
+            auto scale = [&](int side) { return ortho || same ? std::sqrt(2.0 / side) : 2.0; };
+            auto add = [&](size_t &at, int side) {
+                at = total;
+                tables[n++] = LineTable{nullptr, side, set, scale(side)};
+                total += lines_table_elems(side, set);
+            };
+            add(p->line_w[set][ortho], p->cols);
+            add(p->line_h[set][ortho], p->rows);
         }
     cudaError_t e = cudaMalloc(&p->line_tw, total * sizeof(float4));
     if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
-    LineTable tables[8];
-    int n = 0;
-    for (int other = 0; other < 2; ++other)
-        for (int ortho = same ? 1 : 0; ortho < 2; ++ortho) {
-            auto scale = [&](int side) { return ortho ? std::sqrt(2.0 / side) : 2.0; };
-            tables[n++] = {p->line_tw + p->line_w[other][ortho], p->cols, !other, scale(p->cols)};
-            tables[n++] = {p->line_tw + p->line_h[other][ortho], p->rows, !other, scale(p->rows)};
-        }
+    size_t at = 0;
+    for (int i = 0; i < n; ++i) {
+        tables[i].dst = p->line_tw + at;
+        at += lines_table_elems(tables[i].n, tables[i].set);
+    }
     e = lines_gen_tables(tables, n, 0);
     if (e != cudaSuccess) return cuda_fail(e);
     p->table_bytes = total * sizeof(float4);
@@ -382,10 +391,9 @@ static bool ranges_partially_overlap(const void *a, const void *b, size_t bytes)
 
 static DirScales ortho_scales(const bdct_plan *p, Dir dir);
 
-// The line engine, chunk by chunk through the workspace.  Forward: along w,
-// then along h; inverse: along h, then along w; round trip: a row pair, then a
-// column pair; spectral: the forward along w, the pair along h with Lambda
-// between (in place in the workspace), the inverse along w.
+// The line engine, chunk by chunk through the workspace: along w, then along
+// h, each pass transposing; spectral: the forward along w, the pair along h
+// with Lambda between (in place in the workspace), the inverse along w.
 static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long long *in_off, float *out,
                      const long long *out_off, long long count, cudaStream_t s)
 {
@@ -393,32 +401,27 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
     const long long hw = (long long)h * w;
     const bool ortho = dir == DIR_RT || dir == DIR_SPEC;
     const DirScales sc = ortho ? ortho_scales(p, DIR_FWD) : p->scales[dir];
-    const float4 *fw = p->line_tw + p->line_w[0][ortho], *fh = p->line_tw + p->line_h[0][ortho];
-    const float4 *tw = p->line_tw + p->line_w[1][ortho], *th = p->line_tw + p->line_h[1][ortho];
+    auto tab_w = [&](int set) { return p->line_tw + p->line_w[set][ortho]; };
+    auto tab_h = [&](int set) { return p->line_tw + p->line_h[set][ortho]; };
     for (long long b0 = 0; b0 < count; b0 += p->chunk_arrays) {
         const long long nb = (count - b0) < p->chunk_arrays ? (count - b0) : p->chunk_arrays;
         const float *src = in_off ? in : in + b0 * hw;
         float *dst = out_off ? out : out + b0 * hw;
         const long long *so = in_off ? in_off + b0 : nullptr, *dof = out_off ? out_off + b0 : nullptr;
         cudaError_t e;
-        if (dir == DIR_INV) {
-            e = lines_pass(src, p->work, w, h, nb, LINES_INVERSE, sc.h, th, nullptr, p->status, s, so, nullptr);
+        if (dir == DIR_SPEC) {
+            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, tab_w(0), nullptr, p->status, s, so, nullptr);
             if (e == cudaSuccess)
-                e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE, sc.w, tw, nullptr, p->status, s, nullptr, dof, true);
-        } else if (dir == DIR_RT) {
-            e = lines_pass(src, p->work, h, w, nb, LINES_PAIR_ROWS, sc.w, tw, nullptr, p->status, s, so, nullptr);
-            if (e == cudaSuccess)
-                e = lines_pass(p->work, dst, w, h, nb, LINES_PAIR_COLS, sc.h, th, nullptr, p->status, s, nullptr, dof, true);
-        } else {
-            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, fw, nullptr, p->status, s, so, nullptr);
-            if (e == cudaSuccess && dir == DIR_FWD) {
-                e = lines_pass(p->work, dst, w, h, nb, LINES_FORWARD, sc.h, fh, nullptr, p->status, s, nullptr, dof, true);
-            } else if (e == cudaSuccess) {
-                e = lines_pass(p->work, p->work, w, h, nb, LINES_PAIR_ROWS, sc.h, th, p->spec_plain, p->status, s, nullptr,
+                e = lines_pass(p->work, p->work, w, h, nb, LINES_PAIR_ROWS, sc.h, tab_h(2), p->spec_plain, p->status, s, nullptr,
                                nullptr, true);
-                if (e == cudaSuccess)
-                    e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE, sc.w, tw, nullptr, p->status, s, nullptr, dof);
-            }
+            if (e == cudaSuccess)
+                e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE_ROWS, sc.w, tab_w(2), nullptr, p->status, s, nullptr, dof);
+        } else {
+            const LinesMode mode = dir == DIR_FWD ? LINES_FORWARD : dir == DIR_INV ? LINES_INVERSE : LINES_PAIR;
+            const int set = dir == DIR_FWD ? 0 : 1;
+            e = lines_pass(src, p->work, h, w, nb, mode, sc.w, tab_w(set), nullptr, p->status, s, so, nullptr);
+            if (e == cudaSuccess)
+                e = lines_pass(p->work, dst, w, h, nb, mode, sc.h, tab_h(set), nullptr, p->status, s, nullptr, dof, true);
         }
         if (e != cudaSuccess) return cuda_fail(e);
     }

@@ -412,7 +412,7 @@ cudaError_t block_init_device(const float *d_table)
     LineTable tables[4];
     for (int i = 0; i < 4; ++i) {
         const int n = i % 2 ? 128 : 64;
-        tables[i] = {tmp + i * kTabMax, n, false, i / 2 ? 2.0 : std::sqrt(2.0 / n)};
+        tables[i] = {tmp + i * kTabMax, n, 1, i / 2 ? 2.0 : std::sqrt(2.0 / n)};
     }
     e = cudaMemset(tmp, 0, bytes);
     if (e == cudaSuccess) e = lines_gen_tables(tables, 4, 0);

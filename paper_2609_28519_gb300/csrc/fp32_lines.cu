@@ -65,29 +65,33 @@ bool lines_supported(int n)
 
 namespace {
 
-// rows -> transposed (forward), transposed -> rows (inverse), and forward,
-// diagonal, adjoint in one pass: rows -> rows or transposed -> transposed
-enum Mode { MODE_F = 0, MODE_I = 1, MODE_RR = 2, MODE_CC = 3 };
+// LinesMode as the kernel's parameter: forward and inverse, rows ->
+// transposed; forward and adjoint in one pass, rows -> transposed or (with the
+// diagonal) rows -> rows; inverse, transposed -> rows
+enum Mode { MODE_F = 0, MODE_J = 1, MODE_P = 2, MODE_RR = 3, MODE_I = 4 };
 
 // Lines per panel (PR), threads per line (G) and resident CTAs per SM that the
 // registers are held to (NB), by mode: the best of a sweep over radices and
 // these at 256 MiB, where one CTA more or half the lines per panel cost
 // 10-30%.  Panels of 8 lines (32-byte pieces on the transposed side) only
 // where shared memory holds no more.
+constexpr int set_of(int mode) { return mode == MODE_F ? 0 : mode == MODE_J || mode == MODE_P ? 1 : 2; }
+
 template <int N, int MODE>
-struct LineCfg : LineSplit<N, MODE == MODE_F> {
-    static constexpr bool F = MODE == MODE_F;
-    static constexpr int G = N == 64 || N == 192 ? 2 : N == 128 ? 4 : N == 256 ? (F ? 8 : 4) : N <= 512 ? 8
-                           : N == 768 ? 12 : N == 1024 ? 16 : N == 1536 ? (F ? 24 : 16) : N == 2048 ? 32 : 64;
-    static constexpr int PR = N <= 192 || (N == 256 && !F) ? 32 : N <= 1024 ? 16 : 8;
+struct LineCfg : LineSplit<N, set_of(MODE)> {
+    static constexpr int SET = set_of(MODE);
+    static constexpr int G = N <= 192 ? (N == 128 ? 4 : 2) : N == 256 ? (SET ? 4 : 8) : N == 384 ? (SET == 1 ? 4 : 8)
+                           : N == 512 ? 8 : N == 768 ? (SET == 1 ? 8 : 12) : N == 1024 ? (SET == 1 ? 8 : 16)
+                           : N == 1536 ? (SET ? 16 : 24) : N == 2048 ? 32 : 64;
+    static constexpr int PR = N <= 192 || (N == 256 && SET) || (N == 384 && SET == 1) ? 32 : N <= 1024 ? 16 : 8;
     static constexpr int THREADS = PR * G;
-    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (F ? 6 : 5) : N == 384 ? (F ? 6 : 4)
-                            : N == 512 ? 4 : N == 768 ? (F ? 2 : 3) : N == 1024 ? 2 : N == 1536 ? (F ? 2 : 3)
-                            : N == 2048 ? 2 : 1;
+    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET == 0 ? 6 : SET == 1 ? 4 : 5)
+                            : N == 384 ? (SET == 0 ? 6 : SET == 1 ? 3 : 4) : N == 512 ? 4 : N == 768 ? (SET ? 3 : 2)
+                            : N == 1024 ? (SET == 1 ? 3 : 2) : N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
     static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
     // the tables are staged in shared memory (the split's read through L1
     // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
-    static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N, F>::TAB * 16 + 16;
+    static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N, SET>::TAB * 16 + 16;
     static_assert(THREADS % 32 == 0 && PR <= 32 && PR % 4 == 0, "lanes");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
@@ -119,11 +123,6 @@ __device__ __forceinline__ const char *unit_at(const float *p, int ld, int c, in
     const unsigned row = 4u * (unsigned)ld;
     return mad_wide(4u * (unsigned)m * row, j, mad_wide(row, 4 * c + i, reinterpret_cast<const char *>(p)));
 }
-__device__ __forceinline__ float4 load_unit(const float *p, int ld, int c, int m, int j)
-{
-    auto at = [&](int i) { return __ldcg(reinterpret_cast<const float *>(unit_at(p, ld, c, m, j, i))); };
-    return make_float4(at(0), at(1), at(2), at(3));
-}
 __device__ __forceinline__ void store_unit(float *p, int ld, int c, int m, int j, float4 v)
 {
     auto at = [&](int i) { return reinterpret_cast<float *>(const_cast<char *>(unit_at(p, ld, c, m, j, i))); };
@@ -148,9 +147,9 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
 {
     using C = LineCfg<N, MODE>;
     constexpr int R1 = C::R1, R2 = C::R2, R3 = C::R3, M1 = C::M1, CC = C::C, PR = C::PR, G = C::G;
-    constexpr bool ROWS_IN = MODE == MODE_F || MODE == MODE_RR;
+    constexpr bool ROWS_IN = MODE != MODE_I;
     constexpr bool ROWS_OUT = MODE == MODE_I || MODE == MODE_RR;
-    constexpr bool FWD = MODE != MODE_I, INV = MODE != MODE_F;
+    constexpr bool FWD = MODE != MODE_I && MODE != MODE_J, INV = MODE != MODE_F;
     extern __shared__ __align__(128) float lsm[];
     float4 *tab = reinterpret_cast<float4 *>(lsm + PR * C::PT);
     uint64_t *bar = reinterpret_cast<uint64_t *>(tab + C::TAB);
@@ -202,21 +201,27 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
             ok = mbar_wait_bounded(bar, phase);
             phase ^= 1;
         }
+        constexpr int ROUNDS = (CC / 2 + G - 1) / G;  // couples of the last step per thread
+        float2 ya[MODE == MODE_J ? ROUNDS : 1][R3], yb[MODE == MODE_J ? ROUNDS : 1][R3];
+        if constexpr (MODE == MODE_J) {
+            // ---- every coefficient of this thread's couples, before units go over the rows
+#pragma unroll
+            for (int rd = 0; rd < ROUNDS; ++rd) {
+                const int c = g + rd * G;
+                if ((CC / 2) % G == 0 || c < CC / 2)
+                    walk_row<C>(reinterpret_cast<const float *>(row), c,
+                                [&](const float *q, int k, int m) { member(ya[rd], yb[rd], k, m) = *q; });
+            }
+        }
         if constexpr (FWD) {
-            const float *src = MODE == MODE_CC ? src_of(b) + r0 + line : nullptr;
             // ---- first step
 #pragma unroll 1
             for (int cc = g; cc < M1 / 2; cc += G) {
                 float4 x[R1 / 2], y[R1 / 2];
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
-                    if constexpr (MODE == MODE_CC) {
-                        x[j] = load_unit(src, p.rows, cc, M1, j);
-                        y[j] = load_unit(src, p.rows, M1 - 1 - cc, M1, j);
-                    } else {
-                        x[j] = row[cc + M1 * j];
-                        y[j] = row[M1 - 1 - cc + M1 * j];
-                    }
+                    x[j] = row[cc + M1 * j];
+                    y[j] = row[M1 - 1 - cc + M1 * j];
                 }
                 step_forward<R1, M1>(x, y, t1 + cc);
 #pragma unroll
@@ -225,19 +230,19 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
                     row[M1 - 1 - cc + M1 * j] = y[j];
                 }
             }
-            if constexpr (ROWS_IN) {
-                if (!__syncthreads_and(ok)) {
-                    // the load did not land in time: record it, give the copies
-                    // one more bounded wait, and stop
-                    if (tid == 0) {
-                        record_timeout(p.status);
-                        mbar_wait_bounded(bar, phase ^ 1);
-                    }
-                    return;
+        }
+        if constexpr (ROWS_IN) {
+            if (!__syncthreads_and(ok)) {
+                // the load did not land in time: record it, give the copies
+                // one more bounded wait, and stop
+                if (tid == 0) {
+                    record_timeout(p.status);
+                    mbar_wait_bounded(bar, phase ^ 1);
                 }
-            } else {
-                __syncthreads();
+                return;
             }
+        }
+        if constexpr (FWD) {
             // ---- middle step
             if constexpr (R2 > 1) {
 #pragma unroll 1
@@ -264,11 +269,10 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
         }
         // ---- last step, split, and the transposed side
         {
-            constexpr int ROUNDS = (CC / 2 + G - 1) / G;
             const float *src = MODE == MODE_I ? src_of(b) + r0 + line : nullptr;
             float *dst = MODE == MODE_F ? dst_of(b) + r0 + line : nullptr;
             const float *lam = MODE == MODE_RR && p.lam ? p.lam + r0 + line : nullptr;
-#pragma unroll 1
+#pragma unroll(MODE == MODE_J ? ROUNDS : 1)
             for (int rd = 0; rd < ROUNDS; ++rd) {
                 const int c = g + rd * G;
                 const bool active = (CC / 2) % G == 0 || c < CC / 2;
@@ -307,6 +311,12 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
                     if (active) {
                         last_forward<R3>(x, w, dr, di);
                         split_forward<R3, CC>(c, dr, di, ts, p.sc, a, bb);
+                    }
+                } else if constexpr (MODE == MODE_J) {
+#pragma unroll
+                    for (int k = 0; k < R3; ++k) {
+                        a[k] = ya[rd][k];
+                        bb[k] = yb[rd][k];
                     }
                 } else {
                     if (active) {
@@ -371,24 +381,37 @@ __global__ void __launch_bounds__(LineCfg<N, MODE>::THREADS, LineCfg<N, MODE>::N
                 }
                 __syncthreads();
             }
-            float *dst = MODE == MODE_CC ? dst_of(b) + r0 + line : nullptr;
+            // ---- first step: rows in place, or the transposed side
+            constexpr int ROUNDS1 = (M1 / 2 + G - 1) / G;
+            float *dst = ROWS_OUT ? nullptr : dst_of(b) + r0 + line;
 #pragma unroll 1
-            for (int cc = g; cc < M1 / 2; cc += G) {
+            for (int rd = 0; rd < ROUNDS1; ++rd) {
+                const int cc = g + rd * G;
+                const bool active = (M1 / 2) % G == 0 || cc < M1 / 2;
                 float4 x[R1 / 2], y[R1 / 2];
+                if (active) {
 #pragma unroll
-                for (int j = 0; j < R1 / 2; ++j) {
-                    x[j] = row[cc + M1 * j];
-                    y[j] = row[M1 - 1 - cc + M1 * j];
+                    for (int j = 0; j < R1 / 2; ++j) {
+                        x[j] = row[cc + M1 * j];
+                        y[j] = row[M1 - 1 - cc + M1 * j];
+                    }
                 }
+                if (!ROWS_OUT && rd == ROUNDS1 - 1) {
+                    // every unit of the panel is in registers: the next panel may land
+                    fence_proxy_async_smem();
+                    __syncthreads();
+                    if (tid < 32 && next < p.npanels) load_panel(next);
+                }
+                if (!active) continue;
                 step_adjoint<R1, M1>(x, y, t1 + cc);
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
-                    if constexpr (MODE == MODE_CC) {
-                        store_unit(dst, p.rows, cc, M1, j, x[j]);
-                        store_unit(dst, p.rows, M1 - 1 - cc, M1, j, y[j]);
-                    } else {
+                    if constexpr (ROWS_OUT) {
                         row[cc + M1 * j] = x[j];
                         row[M1 - 1 - cc + M1 * j] = y[j];
+                    } else {
+                        store_unit(dst, p.rows, cc, M1, j, x[j]);
+                        store_unit(dst, p.rows, M1 - 1 - cc, M1, j, y[j]);
                     }
                 }
             }
@@ -463,9 +486,10 @@ cudaError_t lines_mode(LinesMode mode, const LinesParams &p, long long nrows, cu
 {
     switch (mode) {
         case LINES_FORWARD: return lines_launch<N, MODE_F>(p, nrows, s);
-        case LINES_INVERSE: return lines_launch<N, MODE_I>(p, nrows, s);
+        case LINES_INVERSE: return lines_launch<N, MODE_J>(p, nrows, s);
+        case LINES_PAIR: return lines_launch<N, MODE_P>(p, nrows, s);
         case LINES_PAIR_ROWS: return lines_launch<N, MODE_RR>(p, nrows, s);
-        default: return lines_launch<N, MODE_CC>(p, nrows, s);
+        default: return lines_launch<N, MODE_I>(p, nrows, s);
     }
 }
 
@@ -483,10 +507,11 @@ __device__ void cos_sin_2pi(long long m, long long d, double &c, double &s)  // 
 }
 
 // All tables of a plan in one launch, blockIdx.y the table.
+constexpr int kMaxTables = 12;
 struct TableJobs {
-    float4 *dst[8];
-    TableShape shape[8];
-    double s1[8];
+    float4 *dst[kMaxTables];
+    TableShape shape[kMaxTables];
+    double s1[kMaxTables];
 };
 
 __global__ void k_gen_line_tw(const TableJobs jobs)
@@ -526,52 +551,58 @@ __global__ void k_gen_line_tw(const TableJobs jobs)
     }
 }
 
-template <int N>
-TableShape shape_of(bool forward)
+template <int N, int SET>
+TableShape shape_of()
 {
-    using A = LineSplit<N, true>;
-    using B = LineSplit<N, false>;
-    return forward ? TableShape{N, A::R1, A::R2, A::R3} : TableShape{N, B::R1, B::R2, B::R3};
+    using S = LineSplit<N, SET>;
+    return TableShape{N, S::R1, S::R2, S::R3};
 }
 
-bool table_shape(int n, bool forward, TableShape *q)
+template <int N>
+bool shape_of_set(int set, TableShape *q)
+{
+    *q = set == 0 ? shape_of<N, 0>() : set == 1 ? shape_of<N, 1>() : shape_of<N, 2>();
+    return true;
+}
+
+bool table_shape(int n, int set, TableShape *q)
 {
     switch (n) {
-        case 64: *q = shape_of<64>(forward); return true;
-        case 128: *q = shape_of<128>(forward); return true;
-        case 192: *q = shape_of<192>(forward); return true;
-        case 256: *q = shape_of<256>(forward); return true;
-        case 384: *q = shape_of<384>(forward); return true;
-        case 512: *q = shape_of<512>(forward); return true;
-        case 768: *q = shape_of<768>(forward); return true;
-        case 1024: *q = shape_of<1024>(forward); return true;
-        case 1536: *q = shape_of<1536>(forward); return true;
-        case 2048: *q = shape_of<2048>(forward); return true;
-        case 4096: *q = shape_of<4096>(forward); return true;
+        case 64: return shape_of_set<64>(set, q);
+        case 128: return shape_of_set<128>(set, q);
+        case 192: return shape_of_set<192>(set, q);
+        case 256: return shape_of_set<256>(set, q);
+        case 384: return shape_of_set<384>(set, q);
+        case 512: return shape_of_set<512>(set, q);
+        case 768: return shape_of_set<768>(set, q);
+        case 1024: return shape_of_set<1024>(set, q);
+        case 1536: return shape_of_set<1536>(set, q);
+        case 2048: return shape_of_set<2048>(set, q);
+        case 4096: return shape_of_set<4096>(set, q);
         default: return false;
     }
 }
 
 }  // namespace
 
-size_t lines_table_elems(int n, bool forward)
+size_t lines_table_elems(int n, int set)
 {
     TableShape q;
-    if (!table_shape(n, forward, &q)) return 0;
+    if (!table_shape(n, set, &q)) return 0;
     const int L = n / 2;
     return (size_t)q.r1 * (L / q.r1 / 2) + (q.r2 > 1 ? (size_t)q.r2 * (q.r3 / 2) : 0) + L / 2 + L / 4;
 }
 
 cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s)
 {
-    if (count < 1 || count > 8) return cudaErrorInvalidValue;
+    if (count < 1 || count > kMaxTables) return cudaErrorInvalidValue;
     TableJobs jobs{};
     int most = 0;
     for (int i = 0; i < count; ++i) {
-        if (!table_shape(tables[i].n, tables[i].forward, &jobs.shape[i])) return cudaErrorInvalidValue;
+        if (!table_shape(tables[i].n, tables[i].set, &jobs.shape[i])) return cudaErrorInvalidValue;
         jobs.dst[i] = tables[i].dst;
         jobs.s1[i] = tables[i].s1;
-        const int e = (int)lines_table_elems(tables[i].n, tables[i].forward);
+        const int e = (int)lines_table_elems(tables[i].n, tables[i].set);
         if (e > most) most = e;
     }
     k_gen_line_tw<<<dim3((most + 127) / 128, count), 128, 0, s>>>(jobs);

@@ -9,14 +9,15 @@ namespace bdct {
 
 // What one separable pass does with arrays of `rows` lines of n points (r the
 // line, k or j the index along it):
-//   LINES_FORWARD    src[r][j] -> dst[k][r]   DCT-II, output scales
-//   LINES_INVERSE    src[k][r] -> dst[r][j]   DCT-III, input scales
-//   LINES_PAIR_ROWS  src[r][j] -> dst[r][j]   DCT-II, diagonal, DCT-III (Prop. 1)
-//   LINES_PAIR_COLS  src[j][r] -> dst[j][r]   the same along columns
-// A forward pass along w then one along h is the 2D forward transform in
-// natural layout (the intermediate is w x h), an inverse pass along h then one
-// along w the inverse, a row pair and a column pair the round trip.
-enum LinesMode { LINES_FORWARD, LINES_INVERSE, LINES_PAIR_ROWS, LINES_PAIR_COLS };
+//   LINES_FORWARD       src[r][j] -> dst[k][r]   DCT-II, output scales
+//   LINES_INVERSE       src[r][k] -> dst[j][r]   DCT-III, input scales
+//   LINES_PAIR          src[r][j] -> dst[j][r]   DCT-II, DCT-III (round trip)
+//   LINES_PAIR_ROWS     src[r][j] -> dst[r][j]   DCT-II, diagonal, DCT-III (Prop. 1)
+//   LINES_INVERSE_ROWS  src[k][r] -> dst[r][j]   DCT-III, input scales
+// Two transposing passes, along w and then along h (the intermediate is w x
+// h), give the 2D transform in natural layout; the spectral composition is a
+// forward along w, the pair along h in place, an inverse to rows along w.
+enum LinesMode { LINES_FORWARD, LINES_INVERSE, LINES_PAIR, LINES_PAIR_ROWS, LINES_INVERSE_ROWS };
 
 // Copy the cosine tables (device buffers) into the line engine's constant
 // memory (called by fused_init_device).
@@ -25,17 +26,17 @@ cudaError_t lines_init_table3(const float *d_table);
 // True if n has an FFT-based line engine: powers of two 64..4096, and 192,
 // 384, 768, 1536.
 bool lines_supported(int n);
-// A twiddle table of length n (lines_table_elems float4 entries), for
-// LINES_FORWARD or for the other modes (they split the line differently); s1
-// is the scale of every index above 0, folded in.
+// A twiddle table of length n (lines_table_elems float4 entries) for a set of
+// modes that split the line alike: 0 LINES_FORWARD, 1 LINES_INVERSE and
+// LINES_PAIR, 2 LINES_PAIR_ROWS and LINES_INVERSE_ROWS; s1 is the scale of
+// every index above 0, folded in.
 struct LineTable {
     float4 *dst;
-    int n;
-    bool forward;
+    int n, set;
     double s1;
 };
-size_t lines_table_elems(int n, bool forward);
-// Generate up to 8 tables in FP64, one launch.
+size_t lines_table_elems(int n, int set);
+// Generate up to 12 tables in FP64, one launch.
 cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s);
 // One pass over `count` arrays.  sc holds the scales of the pass (sc.s1 the
 // table's s1; the pair modes apply them twice, so they take the orthonormal

@@ -11,20 +11,23 @@
 namespace bdct {
 
 // Radices of a line of N points: L = N/2 = R1 R2 R3 (R2 = 1: two steps), for
-// the line engine's forward passes (ROWS_FIRST) and for its others.  A forward
-// pass has its shared-memory traffic and its stores to hide and takes the
-// fewest, largest steps; the adjoint holds its loads in registers as well and
-// prefers smaller last steps (768 points: 24 x 16 runs 0.447 / 0.333 of HBM,
-// forward / inverse, 8 x 6 x 8 0.415 / 0.351).  Sides 64 and 128 split alike.
-template <int N, bool ROWS_FIRST = false>
+// the line engine's forward passes (set 0), its inverse and pair passes (1) and
+// the two that the spectral composition adds (2).  The best of a sweep: fewer,
+// larger steps move less through shared memory, but the adjoint also holds its
+// coefficients in registers (1024 points: 32 x 16 runs 0.398 of HBM inverse
+// where 8 x 8 x 8 runs 0.356, but 0.303 against 0.336 from the transposed
+// side).  Sides 64, 128 and 192 split alike in all.
+template <int N, int SET = 1>
 struct LineSplit {
     static constexpr int L = N / 2;
     static constexpr int R1 = N == 64 ? 4 : N == 128 || N == 192 ? 8
-                            : ROWS_FIRST ? (N == 256 || N == 384 || N == 1536 ? 8 : N == 768 ? 24 : 16)
-                                         : (N == 768 || N == 1024 || N == 1536 ? 8 : 16);
+                            : SET == 0 ? (N == 256 || N == 384 || N == 1536 ? 8 : N == 768 ? 24 : 16)
+                            : SET == 1 ? (N == 384 || N == 768 ? 24 : N == 1024 ? 32 : N == 1536 ? 12 : 16)
+                                       : (N == 768 || N == 1024 || N == 1536 ? 8 : 16);
     static constexpr int R3 = N == 64 || N == 128 ? 8 : N == 192 ? 12
-                            : ROWS_FIRST ? (N == 256 || N == 512 ? 8 : N == 384 ? 6 : 16)
-                                         : (N == 384 ? 12 : N == 512 ? 16 : 8);
+                            : SET == 0 ? (N == 256 || N == 512 ? 8 : N == 384 ? 6 : 16)
+                            : SET == 1 ? (N == 512 || N == 1024 ? 16 : 8)
+                                       : (N == 384 ? 12 : N == 512 ? 16 : 8);
     static constexpr int R2 = L / (R1 * R3);
     static constexpr int M1 = L / R1;  // columns of the first step
     static constexpr int C = L / R3;   // columns of the last step
@@ -304,6 +307,28 @@ struct SlotIndex {
     __device__ __forceinline__ int bx(int k3) const { return (k3 == 0 && zero) ? C::L / 2 : N - k(k3); }
     __device__ __forceinline__ int by(int k3) const { return (k3 == 0 && zero) ? 3 * C::L / 2 : C::L + k(k3); }
 };
+
+// visit(address, slot, member) for every slot of couple c of a line in shared
+// memory (consecutive coefficients): constant steps from four bases.
+template <typename C, typename F>
+__device__ __forceinline__ void walk_row(const float *p, int c, F &&visit)
+{
+    constexpr int N = 2 * C::L, H = C::R3 / 2;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        const int k0 = half == 0 ? c : C::C * H + (c ? c : C::C / 2 - C::L / 2);
+        const float *ax = p + k0, *ay = p + C::L - k0, *bx = p + N - k0, *by = p + C::L + k0;
+#pragma unroll
+        for (int t = 0; t < H; ++t) {
+            const int k3 = half * H + t;
+            const bool zero = k3 == 0 && c == 0;
+            visit(ax + C::C * t, k3, 0);
+            visit(ay - C::C * t, k3, 1);
+            visit(zero ? p + C::L / 2 : bx - C::C * t, k3, 2);
+            visit(zero ? p + 3 * C::L / 2 : by + C::C * t, k3, 3);
+        }
+    }
+}
 
 // a + b * c, one instruction
 __device__ __forceinline__ const char *mad_wide(unsigned b, unsigned c, const char *a)

@@ -17,10 +17,10 @@ struct bdct_plan {
     int variant = 0;  // 1 fused register tile, 2 separable passes, 3 tensor core, 4 tensor-core passes
     bool lines = false;  // separable passes through the FFT line engine (else dense GEMM passes)
     bool small = false;  // dense route on chip (both sides at most 64): no workspace
-    // line engine tables: [forward or other modes][the plan's scale or the
-    // orthonormal one] per axis (the same table where the scales agree)
+    // line engine tables per axis: [set of modes][the plan's scale or the
+    // orthonormal one] (the same table where the scales agree)
     float4 *line_tw = nullptr;
-    size_t line_w[2][2] = {}, line_h[2][2] = {};
+    size_t line_w[3][2] = {}, line_h[3][2] = {};
     int device = -1;
     bdct::DirScales scales[3];  // per Dir
     // separable route
