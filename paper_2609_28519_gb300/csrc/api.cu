@@ -151,10 +151,10 @@ static int lines_plan_tables(bdct_plan *p)
 {
     const bool same = p->norm == BDCT_NORM_ORTHO;
     const unsigned k = p->kind;
-    // needed by set and scale: the forward, the inverse and the round trip, the spectral direction's
-    const bool need[3][2] = {{(k & BDCT_FORWARD) != 0, (k & BDCT_SPECTRAL) != 0},
-                             {(k & BDCT_INVERSE) != 0, (k & BDCT_ROUNDTRIP) != 0},
-                             {false, (k & BDCT_SPECTRAL) != 0}};
+    // needed by set and scale: the forward, the inverse and the round trip, the
+    // spectral direction's, which is also every direction's for few lines
+    const bool f = k & BDCT_FORWARD, i = k & BDCT_INVERSE, r = k & BDCT_ROUNDTRIP, sp = k & BDCT_SPECTRAL;
+    const bool need[3][2] = {{f, sp}, {i, r}, {f || i, r || sp}};
     LineTable tables[12];
     int n = 0;
     size_t total = 0;
@@ -178,9 +178,9 @@ static int lines_plan_tables(bdct_plan *p)
     cudaError_t e = cudaMalloc(&p->line_tw, total * sizeof(float4));
     if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
     size_t at = 0;
-    for (int i = 0; i < n; ++i) {
-        tables[i].dst = p->line_tw + at;
-        at += lines_table_elems(tables[i].n, tables[i].set);
+    for (int t = 0; t < n; ++t) {
+        tables[t].dst = p->line_tw + at;
+        at += lines_table_elems(tables[t].n, tables[t].set);
     }
     e = lines_gen_tables(tables, n, 0);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -408,20 +408,24 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
         const float *src = in_off ? in : in + b0 * hw;
         float *dst = out_off ? out : out + b0 * hw;
         const long long *so = in_off ? in_off + b0 : nullptr, *dof = out_off ? out_off + b0 : nullptr;
+        const int set = dir == DIR_INV || dir == DIR_RT ? 1 : 0;
+        // along w: rows of the arrays to the workspace; along h: its rows to the output
+        LinesCall cw{src, p->work, h, nb, sc.w, tab_w(set), tab_w(2), p->status, so, nullptr};
+        LinesCall ch{p->work, dst, w, nb, sc.h, tab_h(set), tab_h(2), p->status, nullptr, dof, true};
         cudaError_t e;
         if (dir == DIR_SPEC) {
-            e = lines_pass(src, p->work, h, w, nb, LINES_FORWARD, sc.w, tab_w(0), nullptr, p->status, s, so, nullptr);
-            if (e == cudaSuccess)
-                e = lines_pass(p->work, p->work, w, h, nb, LINES_PAIR_ROWS, sc.h, tab_h(2), p->spec_plain, p->status, s, nullptr,
-                               nullptr, true);
-            if (e == cudaSuccess)
-                e = lines_pass(p->work, dst, h, w, nb, LINES_INVERSE_ROWS, sc.w, tab_w(2), nullptr, p->status, s, nullptr, dof);
+            e = lines_pass(cw, w, LINES_FORWARD, s);
+            ch.dst = p->work;
+            ch.dst_off = nullptr;
+            ch.tw = tab_h(2);
+            ch.lam = p->spec_plain;
+            if (e == cudaSuccess) e = lines_pass(ch, h, LINES_PAIR_ROWS, s);
+            LinesCall ci{p->work, dst, h, nb, sc.w, tab_w(2), tab_w(2), p->status, nullptr, dof};
+            if (e == cudaSuccess) e = lines_pass(ci, w, LINES_INVERSE_ROWS, s);
         } else {
             const LinesMode mode = dir == DIR_FWD ? LINES_FORWARD : dir == DIR_INV ? LINES_INVERSE : LINES_PAIR;
-            const int set = dir == DIR_FWD ? 0 : 1;
-            e = lines_pass(src, p->work, h, w, nb, mode, sc.w, tab_w(set), nullptr, p->status, s, so, nullptr);
-            if (e == cudaSuccess)
-                e = lines_pass(p->work, dst, w, h, nb, mode, sc.h, tab_h(set), nullptr, p->status, s, nullptr, dof, true);
+            e = lines_pass(cw, w, mode, s);
+            if (e == cudaSuccess) e = lines_pass(ch, h, mode, s);
         }
         if (e != cudaSuccess) return cuda_fail(e);
     }

@@ -38,15 +38,27 @@ struct LineTable {
 size_t lines_table_elems(int n, int set);
 // Generate up to 12 tables in FP64, one launch.
 cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s);
-// One pass over `count` arrays.  sc holds the scales of the pass (sc.s1 the
-// table's s1; the pair modes apply them twice, so they take the orthonormal
-// ones); lam, if not null, is the diagonal of LINES_PAIR_ROWS: coefficient k
-// of line r is multiplied by lam[k * rows + r].  src_off / dst_off index the
-// arrays (element offsets) or are null for contiguous arrays.  src == dst is
-// allowed for LINES_PAIR_ROWS only, the other modes read what other CTAs
-// write.
-cudaError_t lines_pass(const float *src, float *dst, int rows, int n, long long count, LinesMode mode, AxisScale sc,
-                       const float4 *tw, const float *lam, unsigned int *status, cudaStream_t stream,
-                       const long long *src_off = nullptr, const long long *dst_off = nullptr, bool reverse = false);
+// One pass over `count` arrays of `rows` lines.  sc holds the scales of the
+// pass (sc.s1 the tables' s1; the pair modes apply them twice, so they take the
+// orthonormal ones); tw is the table of the mode's set, tw_few the one of set 2
+// with the same scale, which a call with few lines uses; lam, if not null, is
+// the diagonal of LINES_PAIR_ROWS: coefficient k of line r is multiplied by
+// lam[k * rows + r].  src_off / dst_off index the arrays (element offsets) or
+// are null for contiguous arrays; reverse takes the lines last to first.
+// src == dst is allowed for LINES_PAIR_ROWS only, the other modes read what
+// other CTAs write.
+struct LinesCall {
+    const float *src;
+    float *dst;
+    int rows;
+    long long count;
+    AxisScale sc;
+    const float4 *tw, *tw_few;
+    unsigned int *status;
+    const long long *src_off = nullptr, *dst_off = nullptr;
+    bool reverse = false;
+    const float *lam = nullptr;
+};
+cudaError_t lines_pass(const LinesCall &c, int n, LinesMode mode, cudaStream_t stream);
 
 }  // namespace bdct

@@ -1,6 +1,6 @@
 // Steps of the FFT evaluation of a DCT line on packed couples, shared by the
-// line engine (fp32_lines.cu) and the on-chip kernels of sides 64 and 128
-// (fp32_block.cu).  fp32_lines.cu's header derives the factorization and the
+// line engine (fp32_lines_kernel.cuh) and the on-chip kernels of sides 64 and 128
+// (fp32_block.cu).  fp32_lines_kernel.cuh's header derives the factorization and the
 // packed form; this file holds its short FFTs, twiddles and the split.
 #pragma once
 
