@@ -74,7 +74,7 @@ struct SmallParams {
     long long count;
     int h, w;
     int G;                           // arrays per iteration
-    int buf0, buf1;                  // buffer sizes (pairs)
+    int buf0, buf1, tabs;            // buffer and table sizes (pairs)
     const float2 *fw, *fh, *ih, *iw;  // tables of the passes used (dense_gen_table)
     const float *lam;                // spectral: Lambda (h x w), or null
     FastDiv div_h, div_w4, div_hp, div_wq, div_kh;
@@ -169,6 +169,17 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
     float2 *t_fw = tab, *t_fh = t_fw + (FWD ? kw * aw.np : 0), *t_ih = t_fh + (FWD ? kh * ah.np : 0),
            *t_iw = t_ih + (INV ? kh * ah.np : 0);
     __shared__ long long base_in[kMaxArrays], base_out[kMaxArrays];
+    // offsets of every row of the group: in global memory (the input's for the
+    // first forward pass, the output's for the last inverse one) and, fixed, the
+    // place of a row beside its mirror
+    long long *row_off = reinterpret_cast<long long *>(tab + p.tabs);
+    int *row_at = reinterpret_cast<int *>(row_off + G * h);
+    if (FWD) {
+        for (int l = tid; l < G * h; l += kThreads) {
+            const int a = p.div_h.div(l), r = l - a * h, m = h - 1 - r;
+            row_at[l] = 2 * (a * kh + min(r, m)) + (r > m);
+        }
+    }
 
     pdl_launch_dependents();
     // the tables are plan data, written before any transform was queued
@@ -207,6 +218,11 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
             }
         }
         __syncthreads();
+        for (int l = tid; l < na * h; l += kThreads) {
+            const int a = p.div_h.div(l), r = l - a * h;
+            row_off[l] = FWD ? base_in[a] + r * p.ld_in : base_out[a] + r * p.ld_out;
+        }
+        __syncthreads();
 
         // ---- the arrays, paired for the first pass, four tasks in flight a thread
         if constexpr (FWD) {
@@ -222,13 +238,10 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     at[u] = -1;
                     if (e < tasks) {
                         const int row = p.div_wq.div(e), q = e - row * Q;
-                        const int a = p.div_h.div(row), r = row - a * h;
-                        const float *g = p.in + base_in[a] + r * p.ld_in;
+                        const float *g = p.in + row_off[row];
                         x[u] = __ldcg(reinterpret_cast<const float4 *>(g + 4 * q));
                         y[u] = __ldcg(reinterpret_cast<const float4 *>(g + w - 4 - 4 * q));
-                        // mirrored rows side by side
-                        const int m = h - 1 - r;
-                        at[u] = 2 * (a * kh + min(r, m)) + (r > m);
+                        at[u] = row_at[row];
                         kq[u] = 4 * q;
                     }
                 }
@@ -237,9 +250,10 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     if (at[u] < 0) continue;
                     float2 *o = buf[0] + kq[u] * pfw + at[u];
                     const float f[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, b[4] = {y[u].w, y[u].z, y[u].y, y[u].x};
+                    // w/2 is even: all four pairs, or the middle two
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (kq[u] + i < kw) o[i * pfw] = make_float2(f[i] + b[i], f[i] - b[i]);
+                        if (i < 2 || kq[u] + 4 <= kw) o[i * pfw] = make_float2(f[i] + b[i], f[i] - b[i]);
                 }
             }
         } else {
@@ -298,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     float4 *o = reinterpret_cast<float4 *>(buf[1] + r * ph + a * w + 8 * tc);
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        if (4 * tc + c >= kw) continue;
+                        if (c >= 2 && 4 * tc + 4 > kw) continue;  // w/2 is even
                         const float2 u = acc[2 * i][c], v = acc[2 * i + 1][c];
                         o[c] = mid ? make_float4(u.x, 0.f, u.y, 0.f)
                                    : make_float4(u.x + v.x, u.x - v.x, u.y + v.y, u.y - v.y);
@@ -315,17 +329,22 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     const int l = l0 + i * ls;
                     const int a = p.div_w4.div(l / 4), c = l - a * w;
                     if (a >= na) continue;
-                    float *g = DIR == DIR_FWD ? p.out + base_out[a] + c : nullptr;
+                    if constexpr (DIR == DIR_FWD) {
+                        // up to eight coefficient rows, one after the other
+                        float *g = p.out + base_out[a] + c + 8 * tc * p.ld_out;
+                        const int rows = h - 8 * tc;
 #pragma unroll
-                    for (int o = 0; o < 4; ++o) {
-                        const int k = 2 * (4 * tc + o);
-                        if (k >= h) continue;
-                        float2 u = acc[2 * i][o], v = acc[2 * i + 1][o];
-                        if constexpr (DIR == DIR_FWD) {
-                            *reinterpret_cast<float2 *>(g + k * p.ld_out) = make_float2(u.x, v.x);
-                            if (k + 1 < h)
-                                *reinterpret_cast<float2 *>(g + (k + 1) * p.ld_out) = make_float2(u.y, v.y);
-                        } else {
+                        for (int q = 0; q < 8; ++q) {
+                            const float2 u = acc[2 * i][q / 2], v = acc[2 * i + 1][q / 2];
+                            if (q < rows) *reinterpret_cast<float2 *>(g) = q % 2 ? make_float2(u.y, v.y) : make_float2(u.x, v.x);
+                            g += p.ld_out;
+                        }
+                    } else {
+#pragma unroll
+                        for (int o = 0; o < 4; ++o) {
+                            const int k = 2 * (4 * tc + o);
+                            if (k >= h) continue;
+                            float2 u = acc[2 * i][o], v = acc[2 * i + 1][o];
                             if (p.lam) {
                                 const float2 l0v = __ldg(reinterpret_cast<const float2 *>(p.lam + k * w + c));
                                 u.x *= l0v.x;
@@ -364,6 +383,12 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     }
                 }
             });
+            if constexpr (DIR == DIR_RT) {
+                for (int l = tid; l < na * h; l += kThreads) {
+                    const int a = p.div_h.div(l), r = l - a * h;
+                    row_off[l] = base_out[a] + r * p.ld_out;
+                }
+            }
             __syncthreads();
             // ---- along w, inverse: rows to global memory
             for_tiles(aw, h * na, tqw, law, [&](int l0, int ls, int tc, bool live) {
@@ -375,9 +400,8 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
                         const int l = l0 + i * ls + s;
-                        const int a = p.div_h.div(l), r = l - a * h;
-                        if (a >= na) continue;
-                        float *g = p.out + base_out[a] + r * p.ld_out;
+                        if (l >= na * h) continue;
+                        float *g = p.out + row_off[l];
                         const float2 *v = acc[2 * i + s];
                         if (o0 + 4 <= kw) {
                             *reinterpret_cast<float4 *>(g + o0) =
@@ -427,7 +451,8 @@ cudaError_t launch(SmallParams p, cudaStream_t stream)
     p.buf0 = (p.buf0 + 1) / 2 * 2;
     p.buf1 = (p.buf1 + 1) / 2 * 2;
     const int tabs = (FWD + INV) * (aw.nh * aw.np + ah.nh * ah.np);
-    const size_t smem = ((size_t)p.buf0 + p.buf1 + tabs) * sizeof(float2);
+    p.tabs = tabs;
+    const size_t smem = ((size_t)p.buf0 + p.buf1 + tabs) * sizeof(float2) + (size_t)G * p.h * 12;
     if (smem > 220 * 1024) return cudaErrorInvalidValue;
     p.groups = (p.count + G - 1) / G;
 
