@@ -151,10 +151,9 @@ static int lines_plan_tables(bdct_plan *p)
 {
     const bool same = p->norm == BDCT_NORM_ORTHO;
     const unsigned k = p->kind;
-    // needed by set and scale: the forward, the inverse and the round trip, the
-    // spectral direction's, which is also every direction's for few lines
+    // needed by set and scale: the forward's, the others', every direction's for few lines
     const bool f = k & BDCT_FORWARD, i = k & BDCT_INVERSE, r = k & BDCT_ROUNDTRIP, sp = k & BDCT_SPECTRAL;
-    const bool need[3][2] = {{f, sp}, {i, r}, {f || i, r || sp}};
+    const bool need[3][2] = {{f, sp}, {i, r || sp}, {f || i, r || sp}};
     LineTable tables[12];
     int n = 0;
     size_t total = 0;
@@ -393,7 +392,7 @@ static DirScales ortho_scales(const bdct_plan *p, Dir dir);
 
 // The line engine, chunk by chunk through the workspace: along w, then along
 // h, each pass transposing; spectral: the forward along w, the pair along h
-// with Lambda between (in place in the workspace), the inverse along w.
+// with Lambda between, the inverse of the rows along w in place.
 static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long long *in_off, float *out,
                      const long long *out_off, long long count, cudaStream_t s)
 {
@@ -415,12 +414,10 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
         cudaError_t e;
         if (dir == DIR_SPEC) {
             e = lines_pass(cw, w, LINES_FORWARD, s);
-            ch.dst = p->work;
-            ch.dst_off = nullptr;
-            ch.tw = tab_h(2);
+            ch.tw = tab_h(1);
             ch.lam = p->spec_plain;
-            if (e == cudaSuccess) e = lines_pass(ch, h, LINES_PAIR_ROWS, s);
-            LinesCall ci{p->work, dst, h, nb, sc.w, tab_w(2), tab_w(2), p->status, nullptr, dof};
+            if (e == cudaSuccess) e = lines_pass(ch, h, LINES_PAIR_DIAGONAL, s);
+            const LinesCall ci{dst, dst, h, nb, sc.w, tab_w(1), tab_w(2), p->status, dof, dof};
             if (e == cudaSuccess) e = lines_pass(ci, w, LINES_INVERSE_ROWS, s);
         } else {
             const LinesMode mode = dir == DIR_FWD ? LINES_FORWARD : dir == DIR_INV ? LINES_INVERSE : LINES_PAIR;

@@ -6,9 +6,9 @@
 // line of a batch of arrays -- y_k = s_k sum_j x_j cos(pi (2j+1) k / (2N))
 // (forward), its adjoint x_j = sum_k s_k y_k cos(...) (inverse), or the
 // forward, a diagonal and the adjoint in one pass (round trip and spectral
-// composition, Prop. 1).  The forward reads rows and writes its result
-// transposed, the inverse reads transposed and writes rows, so two passes
-// give the 2D transform in natural layout.
+// composition, Prop. 1).  A pass reads rows and writes its result
+// transposed, so two of them give the 2D transform in natural layout; only the
+// last of the spectral composition's three passes writes rows.
 //
 // The length-N DCT-II of a real line is evaluated exactly through a complex
 // FFT of L = N/2 points (Makhoul's reordering): z_m = (x_{4m}, x_{4m+2}) and
@@ -58,17 +58,18 @@ namespace bdct {
 
 namespace {
 
-// LinesMode as the kernel's parameter: forward and inverse, rows ->
-// transposed; forward and adjoint in one pass, rows -> transposed or (with the
-// diagonal) rows -> rows; inverse, transposed -> rows
-enum Mode { MODE_F = 0, MODE_J = 1, MODE_P = 2, MODE_RR = 3, MODE_I = 4 };
+// LinesMode as the kernel's parameter: forward, inverse, forward and adjoint in
+// one pass, the same with a diagonal between (its own mode: a test of a null
+// diagonal in MODE_P cost 1024^2 round trips 577 -> 592 us), each rows ->
+// transposed; inverse, rows -> rows
+enum Mode { MODE_F = 0, MODE_I = 1, MODE_P = 2, MODE_D = 3, MODE_R = 4 };
 
 // Lines per panel (PR), threads per line (G) and resident CTAs per SM that the
 // registers are held to (NB), by mode: the best of a sweep over radices and
 // these at 256 MiB, where one CTA more or half the lines per panel cost
 // 10-30%.  Panels of 8 lines (32-byte pieces on the transposed side) only
 // where shared memory holds no more.
-constexpr int set_of(int mode) { return mode == MODE_F ? 0 : mode == MODE_J || mode == MODE_P ? 1 : 2; }
+constexpr int set_of(int mode) { return mode == MODE_F ? 0 : 1; }
 
 // FEW: a call with less than one panel per SM lasts as long as one panel's
 // chain of steps, so its panels are 8 lines and a step is one couple per
@@ -90,14 +91,13 @@ struct LineCfg<N, MODE, true> : LineSplit<N, 2> {
 template <int N, int MODE>
 struct LineCfg<N, MODE, false> : LineSplit<N, set_of(MODE)> {
     static constexpr int SET = set_of(MODE);
-    static constexpr int G = N <= 192 ? (N == 128 ? 4 : 2) : N == 256 ? (SET ? 4 : 8) : N == 384 ? (SET == 1 ? 4 : 8)
-                           : N == 512 ? 8 : N == 768 ? (SET == 1 ? 8 : 12) : N == 1024 ? (SET == 1 ? 8 : 16)
-                           : N == 1536 ? (SET ? 16 : 24) : N == 2048 ? 32 : 64;
-    static constexpr int PR = N <= 192 || (N == 256 && SET) || (N == 384 && SET == 1) ? 32 : N <= 1024 ? 16 : 8;
+    static constexpr int G = N <= 192 ? (N == 128 ? 4 : 2) : N == 256 || N == 384 ? (SET ? 4 : 8) : N == 512 ? 8
+                           : N == 768 ? (SET ? 8 : 12) : N == 1024 ? (SET ? 8 : 16) : N == 1536 ? (SET ? 16 : 24)
+                           : N == 2048 ? 32 : 64;
+    static constexpr int PR = N <= 192 || (N <= 384 && SET) ? 32 : N <= 1024 ? 16 : 8;
     static constexpr int THREADS = PR * G;
-    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET == 0 ? 6 : SET == 1 ? 4 : 5)
-                            : N == 384 ? (SET == 0 ? 6 : SET == 1 ? 3 : 4) : N == 512 ? 4 : N == 768 ? (SET ? 3 : 2)
-                            : N == 1024 ? (SET == 1 ? 3 : 2) : N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
+    static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET ? 4 : 6) : N == 384 ? (SET ? 3 : 6)
+                            : N == 512 ? 4 : N == 768 || N == 1024 || N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
     static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
     // the tables are staged in shared memory (the split's read through L1
     // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
@@ -115,7 +115,7 @@ struct LinesParams {
     const long long *src_off, *dst_off;  // indexed arrays (element offsets), or null
     const float4 *tw;                    // the plan's table for N and the modes' set
     const float4 *tw_few;                // and of set 2
-    const float *lam;                    // MODE_RR, or null: output k of line r times lam[k * rows + r]
+    const float *lam;                    // MODE_D: coefficient k of line r times lam[k * rows + r]
     unsigned int *status;
     int reverse;                         // take panels last to first (the pass then starts with
                                          // what the previous pass wrote last, still in L2)
@@ -158,9 +158,8 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
 {
     using C = LineCfg<N, MODE, FEW>;
     constexpr int R1 = C::R1, R2 = C::R2, R3 = C::R3, M1 = C::M1, CC = C::C, PR = C::PR, G = C::G;
-    constexpr bool ROWS_IN = MODE != MODE_I;
-    constexpr bool ROWS_OUT = MODE == MODE_I || MODE == MODE_RR;
-    constexpr bool FWD = MODE != MODE_I && MODE != MODE_J, INV = MODE != MODE_F;
+    constexpr bool ROWS_OUT = MODE == MODE_R;
+    constexpr bool FWD = MODE == MODE_F || MODE == MODE_P || MODE == MODE_D, INV = MODE != MODE_F;
     extern __shared__ __align__(128) float lsm[];
     float4 *tab = reinterpret_cast<float4 *>(lsm + PR * C::PT);
     uint64_t *bar = reinterpret_cast<uint64_t *>(tab + C::TAB);
@@ -195,7 +194,7 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
         __syncwarp();
         if (tid < PR) bulk_load(lsm + tid * C::PT, src_of(b) + (long long)(r0 + tid) * N, N * 4, bar);
     };
-    if (ROWS_IN && tid < 32 && (int)blockIdx.x < p.npanels) load_panel(blockIdx.x);
+    if (tid < 32 && (int)blockIdx.x < p.npanels) load_panel(blockIdx.x);
 
     uint32_t phase = 0;
     for (int pn = blockIdx.x; pn < p.npanels; pn += gridDim.x) {
@@ -207,14 +206,11 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
         // size, would hold registers and shared memory all along (128 x 512
         // forward 434 -> 350 us, 256^2 spectral 725 -> 593 us)
         if (next >= p.npanels) pdl_launch_dependents();
-        bool ok = true;
-        if constexpr (ROWS_IN) {
-            ok = mbar_wait_bounded(bar, phase);
-            phase ^= 1;
-        }
+        const bool ok = mbar_wait_bounded(bar, phase);
+        phase ^= 1;
         constexpr int ROUNDS = (CC / 2 + G - 1) / G;  // couples of the last step per thread
-        float2 ya[MODE == MODE_J ? ROUNDS : 1][R3], yb[MODE == MODE_J ? ROUNDS : 1][R3];
-        if constexpr (MODE == MODE_J) {
+        float2 ya[!FWD ? ROUNDS : 1][R3], yb[!FWD ? ROUNDS : 1][R3];
+        if constexpr (!FWD) {
             // ---- every coefficient of this thread's couples, before units go over the rows
 #pragma unroll
             for (int rd = 0; rd < ROUNDS; ++rd) {
@@ -242,16 +238,14 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
                 }
             }
         }
-        if constexpr (ROWS_IN) {
-            if (!__syncthreads_and(ok)) {
-                // the load did not land in time: record it, give the copies
-                // one more bounded wait, and stop
-                if (tid == 0) {
-                    record_timeout(p.status);
-                    mbar_wait_bounded(bar, phase ^ 1);
-                }
-                return;
+        if (!__syncthreads_and(ok)) {
+            // the load did not land in time: record it, give the copies one
+            // more bounded wait, and stop
+            if (tid == 0) {
+                record_timeout(p.status);
+                mbar_wait_bounded(bar, phase ^ 1);
             }
+            return;
         }
         if constexpr (FWD) {
             // ---- middle step
@@ -280,10 +274,9 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
         }
         // ---- last step, split, and the transposed side
         {
-            const float *src = MODE == MODE_I ? src_of(b) + r0 + line : nullptr;
             float *dst = MODE == MODE_F ? dst_of(b) + r0 + line : nullptr;
-            const float *lam = MODE == MODE_RR && p.lam ? p.lam + r0 + line : nullptr;
-#pragma unroll(MODE == MODE_J ? ROUNDS : 1)
+            const float *lam = MODE == MODE_D ? p.lam + r0 + line : nullptr;
+#pragma unroll(!FWD ? ROUNDS : 1)
             for (int rd = 0; rd < ROUNDS; ++rd) {
                 const int c = g + rd * G;
                 const bool active = (CC / 2) % G == 0 || c < CC / 2;
@@ -323,22 +316,11 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
                         last_forward<R3>(x, w, dr, di);
                         split_forward<R3, CC>(c, dr, di, ts, p.sc, a, bb);
                     }
-                } else if constexpr (MODE == MODE_J) {
+                } else {
 #pragma unroll
                     for (int k = 0; k < R3; ++k) {
                         a[k] = ya[rd][k];
                         bb[k] = yb[rd][k];
-                    }
-                } else {
-                    if (active) {
-                        walk_slots<C>(src, c, p.rows, [&](const char *q, int k, int m) {
-                            member(a, bb, k, m) = __ldcg(reinterpret_cast<const float *>(q));
-                        });
-                    }
-                    if (rd == 0) {
-                        // the previous panel's stores must have read the buffer
-                        if (tid < PR) bulk_wait_read<0>();
-                        __syncthreads();
                     }
                 }
                 if constexpr (MODE == MODE_F) {
@@ -348,8 +330,8 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
                         });
                     }
                 }
-                if constexpr (MODE == MODE_RR) {
-                    if (active && lam) {
+                if constexpr (MODE == MODE_D) {
+                    if (active) {
                         walk_slots<C>(lam, c, p.rows, [&](const char *q, int k, int m) {
                             member(a, bb, k, m) *= __ldg(reinterpret_cast<const float *>(q));
                         });
@@ -433,12 +415,10 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
                     bulk_store(dst_of(b) + (long long)(r0 + tid) * N, lsm + tid * C::PT, N * 4);
                     bulk_commit();
                 }
-                if constexpr (MODE == MODE_RR) {
-                    if (tid < 32 && next < p.npanels) {
-                        if (tid < PR) bulk_wait_read<0>();
-                        __syncwarp();
-                        load_panel(next);
-                    }
+                if (tid < 32 && next < p.npanels) {
+                    if (tid < PR) bulk_wait_read<0>();
+                    __syncwarp();
+                    load_panel(next);
                 }
             }
         }
@@ -518,10 +498,10 @@ cudaError_t lines_run(LinesMode mode, const LinesCall &c, cudaStream_t s)
     const long long nrows = (long long)c.rows * c.count;
     switch (mode) {
         case LINES_FORWARD: return lines_launch<N, MODE_F>(p, nrows, s);
-        case LINES_INVERSE: return lines_launch<N, MODE_J>(p, nrows, s);
+        case LINES_INVERSE: return lines_launch<N, MODE_I>(p, nrows, s);
         case LINES_PAIR: return lines_launch<N, MODE_P>(p, nrows, s);
-        case LINES_PAIR_ROWS: return lines_launch<N, MODE_RR>(p, nrows, s);
-        default: return lines_launch<N, MODE_I>(p, nrows, s);
+        case LINES_PAIR_DIAGONAL: return lines_launch<N, MODE_D>(p, nrows, s);
+        default: return lines_launch<N, MODE_R>(p, nrows, s);
     }
 }
 

@@ -11,12 +11,11 @@
 namespace bdct {
 
 // Radices of a line of N points: L = N/2 = R1 R2 R3 (R2 = 1: two steps), for
-// the line engine's forward passes (set 0), its inverse and pair passes (1) and
-// the two that the spectral composition adds (2).  The best of a sweep: fewer,
-// larger steps move less through shared memory, but the adjoint also holds its
-// coefficients in registers (1024 points: 32 x 16 runs 0.398 of HBM inverse
-// where 8 x 8 x 8 runs 0.356, but 0.303 against 0.336 from the transposed
-// side).  Sides 64, 128 and 192 split alike in all.
+// the line engine's forward passes (set 0), its others (1) and every pass over
+// few lines (2).  The best of a sweep: fewer, larger steps move less through
+// shared memory (1024 points inverse: 32 x 16 runs 0.398 of HBM where 8 x 8 x 8
+// runs 0.356), but the adjoint also holds its coefficients in registers; few
+// lines want the shortest chain.  Sides 64, 128 and 192 split alike in all.
 template <int N, int SET = 1>
 struct LineSplit {
     static constexpr int L = N / 2;
