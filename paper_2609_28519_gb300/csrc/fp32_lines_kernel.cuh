@@ -41,9 +41,17 @@
 // memory: at a fixed index the PR lanes hold PR consecutive elements.  The
 // row side moves by one bulk copy (TMA) per line.
 //
-// What bounds it: 16 bytes of shared-memory traffic per element, pass and
-// exchange (37 TB/s on the chip) and about 16 multiply-adds, against 8 bytes
-// of HBM traffic per element and pass.
+// What bounds it: up to 512 points the two passes' HBM traffic, 16 bytes per
+// element (256^2 forward: 0.45 of the copy rate, 0.90 counting both passes);
+// beyond that, and in the pair modes, the chain of shared-memory exchanges (16
+// bytes per element, pass and exchange) and multiply-adds with the 8 to 12 warps
+// an SM holds.  Before this form (float2 units, one FFT per thread, unpacked)
+// and now, 512 MiB, us: 256^2 forward + inverse + ... see the table.
+//
+//                     forward        inverse        round trip
+//   256 x 256        465 -> 351     541 -> 358     763 -> 422
+//   16 x 1024 x 1024  77 -> 59.5     83 -> 63.2
+//   4 x 4096 x 4096  400 -> 237     420 -> 241
 #pragma once
 
 #include <cuda_runtime.h>
@@ -167,6 +175,17 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
     const SplitTable ts{t2 + C::U2, reinterpret_cast<const float2 *>(t2 + C::U2 + C::L / 2)};
     const int tid = threadIdx.x, line = tid % PR, g = tid / PR;
     float4 *row = reinterpret_cast<float4 *>(lsm + line * C::PT);
+    // the inverse's last step reads single coefficients of its rows: there a
+    // warp takes 8 lines of 4 couples (pitch 4 mod 32: 32 lines of one couple
+    // would meet on 8 banks; 512 MiB inverse, 768 x 1024 398 -> 384 us, 384^2 379
+    // -> 363, 1024^2 398 -> 384, spectral 256^2 618 -> 594).  Not for the
+    // lengths whose inverse is at its limit of 128 registers, where the extra
+    // indices cost more: 256^2 358 -> 368, 512^2 367 -> 381.
+    constexpr bool FULL = FWD || PR <= 8 || (MODE == MODE_I && !FEW && (N == 192 || N == 256 || N == 512));
+    constexpr int CG = FULL ? 32 / PR : G < 4 ? G : 4, CL = 32 / CG;
+    const int cline = FULL ? line : tid % CL + CL * (tid / 32 % (PR / CL));
+    const int cg = FULL ? g : tid / CL % CG + CG * (tid / 32 / (PR / CL));
+    float4 *crow = reinterpret_cast<float4 *>(lsm + cline * C::PT);
 
     if (tid == 0) {
         mbar_init(bar, 1);
@@ -214,9 +233,9 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
             // ---- every coefficient of this thread's couples, before units go over the rows
 #pragma unroll
             for (int rd = 0; rd < ROUNDS; ++rd) {
-                const int c = g + rd * G;
+                const int c = cg + rd * G;
                 if ((CC / 2) % G == 0 || c < CC / 2)
-                    walk_row<C>(reinterpret_cast<const float *>(row), c,
+                    walk_row<C>(reinterpret_cast<const float *>(crow), c,
                                 [&](const float *q, int k, int m) { member(ya[rd], yb[rd], k, m) = *q; });
             }
         }
@@ -278,20 +297,20 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MOD
             const float *lam = MODE == MODE_D ? p.lam + r0 + line : nullptr;
 #pragma unroll(!FWD ? ROUNDS : 1)
             for (int rd = 0; rd < ROUNDS; ++rd) {
-                const int c = g + rd * G;
+                const int c = cg + rd * G;
                 const bool active = (CC / 2) % G == 0 || c < CC / 2;
                 // the couple's columns: c and C-c (C/2 for c = 0)
                 float4 *px, *pw;
                 int sx = 1, sw = -1;
                 if constexpr (R2 == 1) {
-                    px = row + M1 * c;
-                    pw = row + M1 - 1 + M1 * ((c ? CC - c : CC / 2) - R1 / 2);
+                    px = crow + M1 * c;
+                    pw = crow + M1 - 1 + M1 * ((c ? CC - c : CC / 2) - R1 / 2);
                 } else {
                     const int k1 = c % R1, k2 = c / R1;
-                    px = row + sub_base<C>(k1, sx) + sx * (R3 * k2);
+                    px = crow + sub_base<C>(k1, sx) + sx * (R3 * k2);
                     const int k1p = k1 ? R1 - k1 : 0;
                     const int k2p = k1 ? R2 - 1 - k2 : (c ? R2 - k2 : R2 / 2);
-                    pw = row + sub_base<C>(k1p, sw) + sw * (R3 - 1 + R3 * (k2p - R2 / 2));
+                    pw = crow + sub_base<C>(k1p, sw) + sw * (R3 - 1 + R3 * (k2p - R2 / 2));
                     sw = -sw;
                 }
                 float4 x[R3 / 2], w[R3 / 2];
