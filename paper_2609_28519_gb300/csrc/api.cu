@@ -172,7 +172,8 @@ static int lines_plan_tables(bdct_plan *p)
                 total += lines_table_elems(side, set);
             };
             add(p->line_w[set][ortho], p->cols);
-            add(p->line_h[set][ortho], p->rows);
+            if (p->rows == p->cols) p->line_h[set][ortho] = p->line_w[set][ortho];
+            else add(p->line_h[set][ortho], p->rows);
         }
     cudaError_t e = cudaMalloc(&p->line_tw, total * sizeof(float4));
     if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }

@@ -143,7 +143,8 @@ cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s)
         const int e = (int)lines_table_elems(tables[i].n, tables[i].set);
         if (e > most) most = e;
     }
-    k_gen_line_tw<<<dim3((most + 127) / 128, count), 128, 0, s>>>(jobs);
+    // one warp per block: FP64 runs at two lanes a cycle, so the warps are spread over the SMs
+    k_gen_line_tw<<<dim3((most + 31) / 32, count), 32, 0, s>>>(jobs);
     return cudaGetLastError();
 }
 
