@@ -68,8 +68,9 @@ extern "C" {
 #define BDCT_NORM_NONE  1
 
 /* ------------------------------------------------------------------ paths
- * FP32       : CUDA-core FP32 fast factorization (even/odd DCT-II recursion,
- *              DCT-IV through a half-length complex FFT), passes fused on chip.
+ * FP32       : CUDA-core FP32 fast factorization (even/odd DCT-II recursion with
+ *              DCT-IV through a half-length complex FFT, or the whole line
+ *              through one), passes fused on chip where the array fits.
  * SPLIT_TC   : dense C X C^T on tcgen05 tensor cores, every operand split
  *              into three BF16 terms, six products accumulated in FP32.
  * SPLIT_HILO : the same with two BF16 terms and three products; its error is
@@ -90,9 +91,9 @@ typedef struct bdct_plan bdct_plan;
  *       only for those).
  * norm: BDCT_NORM_ORTHO or BDCT_NORM_NONE.   path: one of BDCT_PATH_*.
  * Supported shapes: FP32 path, any 1 <= rows, cols <= 8192 with cols a
- * multiple of 4; power-of-two sides 8..256 run fused on chip, other shapes
- * take separable passes through a plan-owned workspace.  Tensor-core paths:
- * rows and cols powers of two in 8..256.
+ * multiple of 4; sides of 8, 16 and 32, sides of 64 and 128, and any two sides
+ * up to 64 run on chip, other shapes take separable passes through a plan-owned
+ * workspace.  Tensor-core paths: sides 16, 32 or multiples of 64, and 8 x 8.
  * The plan owns its device tables and workspace (Section 3.2: no allocation
  * or planning inside a transform).  Plan creation synchronizes the device.
  * On success *plan is set; on failure *plan is NULL and nothing leaks.      */

@@ -42,16 +42,18 @@
 // row side moves by one bulk copy (TMA) per line.
 //
 // What bounds it: up to 512 points the two passes' HBM traffic, 16 bytes per
-// element (256^2 forward: 0.45 of the copy rate, 0.90 counting both passes);
+// element (256^2 forward: 0.90 of the copy rate over the bytes it moves);
 // beyond that, and in the pair modes, the chain of shared-memory exchanges (16
-// bytes per element, pass and exchange) and multiply-adds with the 8 to 12 warps
-// an SM holds.  Before this form (float2 units, one FFT per thread, unpacked)
-// and now, 512 MiB, us: 256^2 forward + inverse + ... see the table.
-//
-//                     forward        inverse        round trip
-//   256 x 256        465 -> 351     541 -> 358     763 -> 422
-//   16 x 1024 x 1024  77 -> 59.5     83 -> 63.2
-//   4 x 4096 x 4096  400 -> 237     420 -> 241
+// bytes per element, pass and exchange) and the multiply-adds, with 12 to 16
+// warps per SM at full registers.  The form before this one ran four-step FFTs
+// with one sub-FFT per thread, unpacked, 33 instructions per element and pass
+// where this takes 19 to 26 one way.  512 MiB, before -> now, us:
+//                 forward      inverse      round trip   spectral
+//   256^2         469 -> 351   542 -> 357   758 -> 421   1052 -> 592
+//   768 x 1024    557 -> 363   654 -> 383   983 -> 583   1304 -> 707
+//   1024^2        526 -> 375   574 -> 384   872 -> 571   1197 -> 726
+//   2048^2        640 -> 428   671 -> 442   994 -> 657   1452 -> 834
+//   4 x 4096^2    397 -> 237   416 -> 242   642 -> 359    924 -> 514
 #pragma once
 
 #include <cuda_runtime.h>

@@ -315,7 +315,6 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 //     the end of a tile stores its part of the row transposed (with four warps
 //     the reads of the partials held up the products).
 // Tiles are 128 rows by 128 outputs, K chunks of 64.
-
 //
 // Half products.  The operator's rows are even or odd about the middle of the
 // line, so for lengths that are multiples of 256 the forward contracts s_j =
@@ -324,8 +323,10 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 // two halves of its operator, x_j = a_j + b_j, x_{K-1-j} = a_j - b_j: half the
 // products, half the input blocks each tile streams, half the partials.  An
 // item is then a row tile and 128 output pairs, its two products one after the
-// other, both sums of a thread's 64 pairs in registers until they meet.  16 arrays of 1024 x 1024, forward and inverse:
-// 761 -> 510 us.  (K/2 a multiple of 64 but not of 128 would leave half
+// other, both sums of a thread's 64 pairs in registers until they meet.  16
+// arrays of 1024 x 1024, forward and inverse: 761 -> 505 us; what bounds it then
+// is shared memory, 96 KB loaded and 192 KB read by the products per chunk
+// (tensor pipe 51%).  (K/2 a multiple of 64 but not of 128 would leave half
 // tiles, so those lengths keep the whole operator.)
 
 enum SplitMode { SPLIT_WHOLE = 0, SPLIT_FWD = 1, SPLIT_INV = 2 };

@@ -198,8 +198,7 @@ class Plan:
     # The execution calls are the hot path of small batches, where the host
     # side is most of a call: plain integers go to ctypes (the prototypes
     # convert them), torch is looked up once, and the current stream comes as
-    # its raw handle (8.5 -> 4.0 us a call for
-    # 1024 arrays of 8 x 8).
+    # its raw handle (8.5 -> 4.0 us a call for 1024 arrays of 8 x 8).
     def execute(self, kind: int, x, out=None, stream=None):
         k = KINDS[kind] if isinstance(kind, str) else int(kind)
         b = self._batch(x)
