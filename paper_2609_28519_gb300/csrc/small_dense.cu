@@ -31,7 +31,7 @@
 // What bounds it: multiply-adds and the reads of their operands with 12 warps
 // per SM (FMA pipe 41-44%).  Against 4 x 4 tiles over the whole operators, 256
 // MiB, us, forward / round trip: 12 x 12 344 / 585 -> 165 / 266, 26 x 32 382 /
-// 704 -> 197 / 341, 48 x 48 573 / 1080 -> 408 / 731, 60 x 60 749 / 1413 -> 331 /
+// 704 -> 197 / 341, 48 x 48 573 / 1080 -> 399 / 717, 60 x 60 749 / 1413 -> 331 /
 // 577.
 #include <cuda_runtime.h>
 
@@ -63,9 +63,12 @@ struct FastDiv {
 // layout.
 struct Axis {
     int nh, tc, np;   // pairs, output quads, table row (pairs)
-    int tcl;          // output quads per warp: 4, 2 or 1
+    int tcl;          // output quads per warp: 4, 2 or 1; 2 where 4 would idle two more of
+                      // them (5 and 6 quads: 40 x 40 forward 368 -> 360 us, 48 x 48 408 -> 400,
+                      // 36 x 36 393 -> 383, 256 MiB), but not 1 for 3 quads (24 x 24 inverse
+                      // 194 -> 206: every lane then reads its own lines)
     __host__ __device__ explicit Axis(int n = 2)
-        : nh((n + 1) / 2), tc((nh + 3) / 4), np(4 * tc), tcl(tc > 2 ? 4 : tc)
+        : nh((n + 1) / 2), tc((nh + 3) / 4), np(4 * tc), tcl(tc <= 2 ? tc : tc == 5 || tc == 6 ? 2 : 4)
     {
     }
     __host__ __device__ int line_block() const { return 256 / tcl; }  // lines of a warp's tile
