@@ -3,6 +3,9 @@
 // fp32_lines_long.cu).
 #include <cuda_runtime.h>
 
+#include <cmath>
+#include <mutex>
+
 #include "fp32_lines_kernel.cuh"
 
 namespace bdct {
@@ -89,6 +92,59 @@ __global__ void k_gen_line_tw(const TableJobs jobs)
     }
 }
 
+// |w| - 1 of w = exp(2 pi i m / d) with both parts rounded to FP32.
+double root_error(long long m, long long d)
+{
+    const double a = 2.0 * 3.14159265358979323846 * (double)(m % d) / (double)d;
+    const double c = (float)std::cos(a), s = (float)std::sin(a);
+    return 0.5 * (c * c + s * s - 1.0);
+}
+
+// Mean gain error of an R-point FFT's rounded roots over its inputs and
+// outputs (radix 2 and 3, decimation in time: one or two thirds of the terms
+// of a stage are multiplied).
+double fft_error(int R)
+{
+    double g = 0.0;
+    if (R % 3 == 0) {
+        const int M = R / 3;
+        for (int k = 0; k < M; ++k) g += (root_error(k, R) + root_error(2 * k, R)) / (3.0 * M);
+        const double h = 0.5 * std::sqrt(3.0);
+        g += ((float)h / h - 1.0) / 3.0;  // the imaginary parts of the 3-point DFT: a third of its energy
+        R = M;
+    }
+    for (; R > 1; R /= 2)
+        for (int k = 0; k < R / 2; ++k) g += root_error(k, R) / R;
+    return g;
+}
+
+// Mean gain error of a step's twiddles: column cc and its mirror, k signed in
+// the step before the last (as k_gen_line_tw).
+double step_error(int R, int mc, bool signed_k)
+{
+    double g = 0.0;
+    for (int k = 0; k < R; ++k)
+        for (int cc = 0; cc < mc / 2; ++cc) {
+            const long long kk = signed_k && k >= R / 2 ? k - R : k, d = (long long)R * mc;
+            g += root_error(cc * kk, d) + root_error((cc + 1) * kk, d);
+        }
+    return g / ((double)R * mc);
+}
+
+// Mean gain error of the whole line but for the split's last factor.  Rounded
+// roots are shorter than 1 on average (1/sqrt 2, in every short FFT, by 1.7e-8),
+// so it is -1.5e-8 to -4e-8, the same for every input, and a fifth to a third
+// of the squared error of a round trip; the last factor takes it back.
+double line_error(const TableShape &q)
+{
+    const int L = q.n / 2;
+    double g = fft_error(q.r1) + fft_error(q.r2) + fft_error(q.r3) + step_error(q.r1, L / q.r1, q.r2 == 1);
+    if (q.r2 > 1) g += step_error(q.r2, q.r3, true);
+    double p = 0.0;
+    for (int k = 0; k < L; ++k) p += root_error(k, q.n) / L;
+    return g + 0.5 * p;
+}
+
 template <int N, int SET>
 TableShape shape_of()
 {
@@ -134,12 +190,24 @@ size_t lines_table_elems(int n, int set)
 cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s)
 {
     if (count < 1 || count > kMaxTables) return cudaErrorInvalidValue;
+    // by log2 of the length, or of its third, and set; once per process
+    static std::mutex mu;
+    static double known[2][16][3];
     TableJobs jobs{};
     int most = 0;
     for (int i = 0; i < count; ++i) {
+        const TableShape &q = jobs.shape[i];
         if (!table_shape(tables[i].n, tables[i].set, &jobs.shape[i])) return cudaErrorInvalidValue;
         jobs.dst[i] = tables[i].dst;
-        jobs.s1[i] = tables[i].s1;
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            const bool three = q.n % 3 == 0;
+            int e = 0;
+            while ((three ? 3 : 1) << e < q.n) ++e;
+            double &g = known[three][e][tables[i].set];
+            if (g == 0.0) g = line_error(q);
+            jobs.s1[i] = tables[i].s1 / (1.0 + g);
+        }
         const int e = (int)lines_table_elems(tables[i].n, tables[i].set);
         if (e > most) most = e;
     }

@@ -94,6 +94,10 @@ struct LineCfg<N, MODE, true> : LineSplit<N, 2> {
     static constexpr int PR = 8;
     static constexpr int THREADS = PR * G;
     static constexpr int NB = THREADS >= 384 ? 1 : 2;
+    // registers as for 256 threads: at 128 a panel of the next pass, of another
+    // length, fits beside one of this pass and starts under it (1 x 1024 x 768
+    // round trip 13.0 us with 136 registers at 768 points, 10.1 with 128)
+    static constexpr int BOUND = THREADS == 192 ? 256 : THREADS;
     static constexpr int PT = N + 4;  // line pitch (floats)
     static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N, 2>::TAB * 16 + 16;
 };
@@ -105,7 +109,7 @@ struct LineCfg<N, MODE, false> : LineSplit<N, set_of(MODE)> {
                            : N == 768 ? (SET ? 8 : 12) : N == 1024 ? (SET ? 8 : 16) : N == 1536 ? (SET ? 16 : 24)
                            : N == 2048 ? 32 : 64;
     static constexpr int PR = N <= 192 || (N <= 384 && SET) ? 32 : N <= 1024 ? 16 : 8;
-    static constexpr int THREADS = PR * G;
+    static constexpr int THREADS = PR * G, BOUND = THREADS;
     static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET ? 4 : 6) : N == 384 ? (SET ? 3 : 6)
                             : N == 512 ? 4 : N == 768 || N == 1024 || N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
     static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
@@ -164,7 +168,7 @@ __device__ __forceinline__ int sub_base(int k1, int &sgn)
 }
 
 template <int N, int MODE, bool FEW>
-__global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::THREADS, LineCfg<N, MODE, FEW>::NB) k_lines(const LinesParams p)
+__global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::BOUND, LineCfg<N, MODE, FEW>::NB) k_lines(const LinesParams p)
 {
     using C = LineCfg<N, MODE, FEW>;
     constexpr int R1 = C::R1, R2 = C::R2, R3 = C::R3, M1 = C::M1, CC = C::C, PR = C::PR, G = C::G;
