@@ -9,10 +9,10 @@
 // point.
 //
 // Half products.  cos(pi (2j+1) k / (2n)) is even about the middle of the
-// line for even k and odd for odd k, so with s_j = x_j + x_{n-1-j} and d_j =
-// x_j - x_{n-1-j} (j < n/2) the even outputs are a product with s and the odd
-// ones a product with d, each half as long: n/2 multiply-adds per point
-// instead of n.  The inverse runs it backwards: a from the even coefficients,
+// line for even k and odd for odd k, so with s_j = (x_j + x_{n-1-j}) / 2 and
+// d_j = (x_j - x_{n-1-j}) / 2 (j < n/2; half_pair, ptx.cuh) the even outputs are
+// a product with s and the odd ones a product with d, each half as long: n/2
+// multiply-adds per point instead of n.  The inverse runs it backwards: a from the even coefficients,
 // b from the odd ones, x_j = a_j + b_j, x_{n-1-j} = a_j - b_j.
 //
 // Tiles.  The two products run in the halves of packed pairs: (s_j, d_j) of a
@@ -88,7 +88,7 @@ struct DenseShape {
     }
 };
 
-// forward: t[j][o] = M[2o + e][j]; inverse: t[o][j] = M^T[j][2o + e], e the half.
+// forward: t[j][o] = 2 M[2o + e][j]; inverse: t[o][j] = M^T[j][2o + e], e the half.
 // One warp per block and one entry per thread: FP64 runs at two lanes a cycle,
 // so the warps are spread over the SMs.
 __global__ void k_gen_half(float *t, DenseShape q, int direction, int norm)
@@ -97,7 +97,8 @@ __global__ void k_gen_half(float *t, DenseShape q, int direction, int norm)
     if (idx >= 2ll * q.kp * q.np) return;
     const int r = (int)(idx / 2 / q.np), c = (int)(idx / 2 % q.np), e = (int)(idx & 1);
     const int k = 2 * (direction == 1 ? c : r) + e, j = direction == 1 ? r : c;
-    t[idx] = j < q.nh && k < q.n ? (float)operator_entry(k, j, q.n, direction, norm) : 0.f;
+    const double f = direction == 1 ? 2.0 : 1.0;
+    t[idx] = j < q.nh && k < q.n ? (float)(f * operator_entry(k, j, q.n, direction, norm)) : 0.f;
 }
 
 struct DenseParams {
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, kResident) k_dense(const DenseParams
                     const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.w, b.z, b.y, b.x};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)  // past the middle: the mirrored pairs again, left out
-                        v[i] = k0 + kk[u] + i < q.nh ? make_float2(x[i] + y[i], x[i] - y[i]) : make_float2(0.f, 0.f);
+                        v[i] = k0 + kk[u] + i < q.nh ? half_pair(x[i], y[i]) : make_float2(0.f, 0.f);
                 } else {
                     v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
                     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
@@ -191,18 +192,24 @@ __global__ void __launch_bounds__(kThreads, kResident) k_dense(const DenseParams
 #pragma unroll
                 for (int i = 0; i < 4; ++i) as[st][kk[u] + i][ln[u]] = v[i];
             } else {
-                float4 s = a, d = b;
+                float2 v0 = make_float2(a.x, b.x), v1 = make_float2(a.y, b.y), v2 = make_float2(a.z, b.z),
+                       v3 = make_float2(a.w, b.w);
                 if (!INV) {
                     if (2 * (k0 + kk[u]) + 1 == n) {  // the middle of an odd length, its own mirror
-                        d = zero;
+                        v0 = make_float2(0.5f * a.x, 0.f);
+                        v1 = make_float2(0.5f * a.y, 0.f);
+                        v2 = make_float2(0.5f * a.z, 0.f);
+                        v3 = make_float2(0.5f * a.w, 0.f);
                     } else {
-                        s = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-                        d = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+                        v0 = half_pair(a.x, b.x);
+                        v1 = half_pair(a.y, b.y);
+                        v2 = half_pair(a.z, b.z);
+                        v3 = half_pair(a.w, b.w);
                     }
                 }
                 float4 *o = reinterpret_cast<float4 *>(&as[st][kk[u]][ln[u]]);
-                o[0] = make_float4(s.x, d.x, s.y, d.y);
-                o[1] = make_float4(s.z, d.z, s.w, d.w);
+                o[0] = make_float4(v0.x, v0.y, v1.x, v1.y);
+                o[1] = make_float4(v2.x, v2.y, v3.x, v3.y);
             }
         }
     };

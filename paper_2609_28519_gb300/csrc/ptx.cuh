@@ -197,4 +197,17 @@ __device__ __forceinline__ void bulk_wait()
     asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// (x + y) / 2 and (x - y) / 2, the operand pair of a half product: the full sum
+// of two mirrored values can exceed FLT_MAX where no output does (2^127.5 twice,
+// 12 x 12), so the forward's tables hold the factor 2.  Exact but for subnormals.
+__device__ __forceinline__ float2 half_pair(float x, float y)
+{
+    // opaque: the compiler otherwise moves the products up to the loads of x and
+    // y, where they wait ahead of the work those were to overlap (116508 arrays
+    // of 12 x 12 44 -> 64 us; so 45)
+    asm("" : "+f"(x), "+f"(y));
+    const float h = 0.5f * y;
+    return make_float2(fmaf(0.5f, x, h), fmaf(0.5f, x, -h));
+}
+
 }  // namespace bdct

@@ -8,8 +8,9 @@
 // direction puts Lambda between them (Eq. 4).  One read and one write of
 // every element; every pass runs in shared memory on the half products of
 // dense_passes.cu: n/2 multiply-adds per point, the even and the odd product
-// in the halves of packed pairs, operand pairs (s, d) = sums and differences
-// of mirrored elements (forward) or (y_2k, y_2k+1) (inverse).
+// in the halves of packed pairs, operand pairs (s, d) = half the sums and
+// differences of mirrored elements (forward; half_pair, ptx.cuh) or (y_2k,
+// y_2k+1) (inverse).
 //
 // Organization.  A CTA of four warps transforms G arrays at a time, G chosen
 // so that one tile of 8 lines x 4 output pairs per thread covers them
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     // w/2 is even: all four pairs, or the middle two
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (i < 2 || kq[u] + 4 <= kw) o[i * pfw] = make_float2(f[i] + b[i], f[i] - b[i]);
+                        if (i < 2 || kq[u] + 4 <= kw) o[i * pfw] = half_pair(f[i], b[i]);
                 }
             }
         } else {
@@ -323,8 +324,8 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
                     for (int c = 0; c < 4; ++c) {
                         if (c >= 2 && 4 * tc + 4 > kw) continue;  // w/2 is even
                         const float2 u = acc[2 * i][c], v = acc[2 * i + 1][c];
-                        o[c] = mid ? make_float4(u.x, 0.f, u.y, 0.f)
-                                   : make_float4(u.x + v.x, u.x - v.x, u.y + v.y, u.y - v.y);
+                        const float2 e = half_pair(u.x, v.x), d = half_pair(u.y, v.y);
+                        o[c] = mid ? make_float4(0.5f * u.x, 0.f, 0.5f * u.y, 0.f) : make_float4(e.x, e.y, d.x, d.y);
                     }
                 }
             });

@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 //
 // Half products.  The operator's rows are even or odd about the middle of the
 // line, so for lengths that are multiples of 256 the forward contracts s_j =
-// x_j + x_{K-1-j} with the even operator and d_j = x_j - x_{K-1-j} with the odd
-// one (j < K/2), and the inverse the even and the odd coefficients with the
+// (x_j + x_{K-1-j}) / 2 (half_pair, ptx.cuh) with twice the even operator and d_j =
+// (x_j - x_{K-1-j}) / 2 with twice the odd one (j < K/2), and the inverse the even and the odd coefficients with the
 // two halves of its operator, x_j = a_j + b_j, x_{K-1-j} = a_j - b_j: half the
 // products, half the input blocks each tile streams, half the partials.  An
 // item is then a row tile and 128 output pairs, its two products one after the
@@ -380,8 +380,9 @@ __global__ void k_tg_presplit(const float *src, const long long *src_off, long l
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     if (SPLIT == SPLIT_FWD) {
-                        v[0][e] = x[e] + y[7 - e];
-                        v[SUB - 1][e] = x[e] - y[7 - e];
+                        const float2 p = half_pair(x[e], y[7 - e]);
+                        v[0][e] = p.x;
+                        v[SUB - 1][e] = p.y;
                     } else {
                         v[0][e] = e < 4 ? x[2 * (e & 3)] : y[2 * (e & 3)];
                         v[SUB - 1][e] = e < 4 ? x[2 * (e & 3) + 1] : y[2 * (e & 3) + 1];
@@ -889,7 +890,7 @@ __device__ double tg_op_value(int row, int col, int n, int direction, int norm)
 }
 
 // half: N outputs of contraction length K = N/2 -- N/2 of the even product, then
-// of the odd one.
+// of the odd one, the forward's doubled.
 __global__ void k_gen_tg_op(__nv_bfloat16 *dst, int N, int K, int direction, int norm, int NT, int KC, int kron, int half)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -898,9 +899,8 @@ __global__ void k_gen_tg_op(__nv_bfloat16 *dst, int N, int K, int direction, int
     double val;
     if (half) {
         const int e = nn >= N / 2, i = nn - e * (N / 2);
-        val = direction == 1 ? tg_op_value(2 * i + e, kk, N, 1, norm) : tg_op_value(i, 2 * kk + e, N, 2, norm);
-    } else
-    if (kron) {
+        val = direction == 1 ? 2.0 * tg_op_value(2 * i + e, kk, N, 1, norm) : tg_op_value(i, 2 * kk + e, N, 2, norm);
+    } else if (kron) {
         // (Q (x) Q)[(f1, f2)][(i, j)] = M8[f1][i] * M8[f2][j] for the row-major 8 x 8 array
         val = tg_op_value(nn >> 3, kk >> 3, 8, direction, norm) * tg_op_value(nn & 7, kk & 7, 8, direction, norm);
     } else {
