@@ -12,10 +12,13 @@
 // runs on those rows the same way and stores its outputs straight to global
 // memory, a warp writing 32 consecutive coefficients of one row.  The inverse
 // runs the transposed steps: coefficients straight into registers, the column
-// pass, the row pass, and one bulk store per row.  The round trip and the
-// spectral direction join the two in the middle: the column pass's
-// coefficients stay in registers, take the diagonal, and go back through the
-// adjoint steps in place.
+// pass, the row pass, and one bulk store per row.  The spectral direction joins
+// the two in the middle: the column pass's coefficients stay in registers, take
+// the diagonal, and go back through the adjoint steps in place.  The round trip
+// runs forward and back along the rows, is transposed, and the same along the
+// columns: one transposition, and the range of one axis (joined in the middle
+// as the spectral direction is, a constant 128 x 128 array overflowed from
+// 2^118, this way from 2^121).
 //
 // Every thread has exactly one couple of the last step (two short FFTs of 8
 // points in packed halves, 32 values), so the transposed write needs no
@@ -76,7 +79,7 @@ struct BlockParams {
     int tiles_per_row;        // tiled only
     long long ld_in, ld_out;  // tiled only (floats)
     const long long *in_off, *out_off;
-    DirScales sc;
+    DirScales sc;             // twice the scales of the forward's outputs or the inverse's inputs
     const float *lam;         // spectral: Lambda (H x W), else null
     unsigned int *status;
     int plain;                // the unnormalized pair's scales
@@ -95,7 +98,7 @@ __device__ __forceinline__ void first_step(float4 *row, int g, const float4 *t1)
             x[j] = row[cc + S::M1 * j];
             y[j] = row[S::M1 - 1 - cc + S::M1 * j];
         }
-        step_forward<S::R1, S::M1>(x, y, t1 + cc);
+        step_forward<S::R1, S::M1, true>(x, y, t1 + cc);
 #pragma unroll
         for (int j = 0; j < S::R1 / 2; ++j) {
             row[cc + S::M1 * j] = x[j];
@@ -116,11 +119,40 @@ __device__ __forceinline__ void first_step_adjoint(float4 *row, int g, const flo
             x[j] = row[cc + S::M1 * j];
             y[j] = row[S::M1 - 1 - cc + S::M1 * j];
         }
-        step_adjoint<S::R1, S::M1>(x, y, t1 + cc);
+        step_adjoint<S::R1, S::M1, true>(x, y, t1 + cc);
 #pragma unroll
         for (int j = 0; j < S::R1 / 2; ++j) {
             row[cc + S::M1 * j] = x[j];
             row[S::M1 - 1 - cc + S::M1 * j] = y[j];
+        }
+    }
+}
+
+// The line's first-step adjoint with its results handed on instead: read() once
+// every unit of this thread's couples is in registers, put(i, v) for element i.
+template <int N, int G, typename R, typename P>
+__device__ __forceinline__ void first_step_adjoint_out(const float4 *row, int g, const float4 *t1, R &&read, P &&put)
+{
+    using S = LineSplit<N>;
+    constexpr int NC = S::M1 / 2 / G;
+    static_assert(NC * G == S::M1 / 2, "couples");
+    float4 x[NC][S::R1 / 2], y[NC][S::R1 / 2];
+#pragma unroll
+    for (int i = 0; i < NC; ++i)
+#pragma unroll
+        for (int j = 0; j < S::R1 / 2; ++j) {
+            x[i][j] = row[g + G * i + S::M1 * j];
+            y[i][j] = row[S::M1 - 1 - g - G * i + S::M1 * j];
+        }
+    read();
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        step_adjoint<S::R1, S::M1, true>(x[i], y[i], t1 + g + G * i);
+#pragma unroll
+        for (int j = 0; j < S::R1 / 2; ++j) {
+            const int p = 4 * (g + G * i + S::M1 * j), q = 4 * (S::M1 - 1 - g - G * i + S::M1 * j);
+            put(p, x[i][j].x); put(p + 1, x[i][j].y); put(p + 2, x[i][j].z); put(p + 3, x[i][j].w);
+            put(q, y[i][j].x); put(q + 1, y[i][j].y); put(q + 2, y[i][j].z); put(q + 3, y[i][j].w);
         }
     }
 }
@@ -132,6 +164,30 @@ __device__ __forceinline__ void couple_units(float4 *row, int c, float4 *&px, fl
     using S = LineSplit<N>;
     px = row + S::M1 * c;
     pw = row + S::M1 - 1 + S::M1 * ((c ? S::C - c : S::C / 2) - S::R1 / 2);
+}
+
+// The couple's coefficients and back, in place: the middle of a line's round trip.
+template <int N>
+__device__ __forceinline__ void couple_round_trip(float4 *row, int c, SplitTable ts, AxisScale sc)
+{
+    using S = LineSplit<N>;
+    float4 x[4], w[4], *px, *pw;
+    couple_units<N>(row, c, px, pw);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        x[m] = px[m];
+        w[m] = pw[-m];
+    }
+    float2 dr[8], di[8], a[8], b[8];
+    last_forward<8>(x, w, dr, di);
+    split_forward<8, S::C>(c, dr, di, ts, sc, a, b);
+    split_adjoint<8, S::C>(c, a, b, ts, sc, dr, di);
+    last_adjoint<8>(x, w, dr, di);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        px[m] = x[m];
+        pw[-m] = w[m];
+    }
 }
 
 template <int H, int W, int DIR, bool TILED>
@@ -198,6 +254,29 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
                     mbar_wait_bounded(bar, phase ^ 1);
                 }
                 return;
+            }
+            if constexpr (DIR == DIR_RT) {
+                // each axis forward and back in turn, so that no coefficient is
+                // larger than its own axis makes it
+                couple_round_trip<W>(row_w, gw, sw, p.sc.w);
+                __syncthreads();
+                first_step_adjoint_out<W, C::GW>(
+                    row_w, gw, tw, [] { __syncthreads(); }, [&](int i, float v) { bsm[i * C::PH + rw] = v; });
+                __syncthreads();
+                first_step<H, C::GH>(row_h, gh, th);
+                __syncthreads();
+                couple_round_trip<H>(row_h, gh, sh, p.sc.h);
+                __syncthreads();
+                float *o = dst_of(ar) + rh;
+                first_step_adjoint_out<H, C::GH>(
+                    row_h, gh, th,
+                    [&] {  // the next array may land
+                        fence_proxy_async_smem();
+                        __syncthreads();
+                        if (next < p.count) load(next);
+                    },
+                    [&](int i, float v) { o[i * ldo] = v; });
+                continue;
             }
             {
                 float4 x[4], w[4], *px, *pw;
@@ -327,7 +406,7 @@ __global__ void __launch_bounds__(BlockCfg<H, W>::THREADS, BlockCfg<H, W>::NB) k
             }
         }
     }
-    if (INV && tid < H) bulk_wait<0>();
+    if ((DIR == DIR_INV || DIR == DIR_SPEC) && tid < H) bulk_wait<0>();
 }
 
 template <int H, int W, int DIR, bool TILED>
@@ -371,6 +450,7 @@ cudaError_t block_launch_one(const DirScales &sc, const ExecGeom &g, unsigned in
     }
     p.lam = g.lam;
     p.plain = p.sc.w.s1 == 2.0f;
+    for (AxisScale *a : {&p.sc.h, &p.sc.w}) *a = AxisScale{2.0f * a->s0, 2.0f * a->s1};  // the first steps halve
     p.status = status;
     if (DIR == DIR_SPEC && !g.lam) return cudaErrorInvalidValue;
     long long grid = (long long)bps_dev * num_sms;

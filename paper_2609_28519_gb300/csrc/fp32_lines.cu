@@ -76,19 +76,19 @@ __global__ void k_gen_line_tw(const TableJobs jobs)
         const long long d = (long long)R * mc;
         cos_sin_2pi((long long)cc * k, d, ca, sa);
         cos_sin_2pi((long long)(cc + 1) * k, d, cb, sb);
-        t[r] = make_float4((float)ca, (float)cb, (float)sa, (float)sb);
+        const double h = first ? 0.5 : 1.0;  // step_forward's HALF
+        t[r] = make_float4((float)(h * ca), (float)(h * cb), (float)(h * sa), (float)(h * sb));
     } else if (r < u1 + u2 + L / 2) {
         const int e = r - u1 - u2;
         const int k3 = e / (c3 / 2), c = e % (c3 / 2);
         const int k = c3 * k3 + (c || k3 < q.r3 / 2 ? c : c3 / 2 - L / 2);
-        const double f = 0.5 * s1;
         double cw, sw;
         cos_sin_2pi(k, q.n, cw, sw);
         cos_sin_2pi(k, 4ll * q.n, ca, sa);       // W_k = exp(-i pi k / (2n))
         cos_sin_2pi(L - k, 4ll * q.n, cb, sb);   // W_{L-k}
         float4 *o = t + u1 + u2;
-        o[e] = make_float4((float)cw, (float)sw, (float)(f * ca), (float)(f * cb));
-        reinterpret_cast<float2 *>(o + L / 2)[e] = make_float2((float)(f * sa), (float)(f * sb));
+        o[e] = make_float4((float)cw, (float)sw, (float)(s1 * ca), (float)(s1 * cb));
+        reinterpret_cast<float2 *>(o + L / 2)[e] = make_float2((float)(s1 * sa), (float)(s1 * sb));
     }
 }
 

@@ -17,6 +17,7 @@
 // V = E + P, V' = conj(E - P) and W_k = exp(-i pi k / (2N)) / 2:
 //   y_k = Re(W_k V),  y_{N-k} = -Im(W_k V),
 //   y_{L-k} = Re(W_{L-k} V'),  y_{L+k} = -Im(W_{L-k} V').
+// (The factor 1/2 of W_k is in the first step's twiddles, ahead of the sums.)
 // The FFT takes two or three steps, L = R1 R2 R3 (R2 = 1 for two), each a set
 // of short FFTs in registers with one exchange through shared memory between
 // steps.  The DCT-III is the exact transpose of those steps in reverse order.
@@ -125,7 +126,7 @@ struct LinesParams {
     float *dst;
     int rows;                            // lines per array
     int npanels;
-    AxisScale sc;                        // forward: output scales, inverse: input scales (both when both run)
+    AxisScale sc;                        // twice the forward's output scales or the inverse's input scales (both when both run)
     const long long *src_off, *dst_off;  // indexed arrays (element offsets), or null
     const float4 *tw;                    // the plan's table for N and the modes' set
     const float4 *tw_few;                // and of set 2
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::BOUND, LineCfg<N, MODE,
                     x[j] = row[cc + M1 * j];
                     y[j] = row[M1 - 1 - cc + M1 * j];
                 }
-                step_forward<R1, M1>(x, y, t1 + cc);
+                step_forward<R1, M1, true>(x, y, t1 + cc);
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
                     row[cc + M1 * j] = x[j];
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::BOUND, LineCfg<N, MODE,
                         x[j] = px[sgn * R3 * j];
                         y[j] = py[sgn * R3 * j];
                     }
-                    step_forward<R2, R3>(x, y, t2 + m3);
+                    step_forward<R2, R3, false>(x, y, t2 + m3);
 #pragma unroll
                     for (int j = 0; j < R2 / 2; ++j) {
                         px[sgn * R3 * j] = x[j];
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::BOUND, LineCfg<N, MODE,
                         x[j] = px[sgn * R3 * j];
                         y[j] = py[sgn * R3 * j];
                     }
-                    step_adjoint<R2, R3>(x, y, t2 + m3);
+                    step_adjoint<R2, R3, false>(x, y, t2 + m3);
 #pragma unroll
                     for (int j = 0; j < R2 / 2; ++j) {
                         px[sgn * R3 * j] = x[j];
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(LineCfg<N, MODE, FEW>::BOUND, LineCfg<N, MODE,
                     if (tid < 32 && next < p.npanels) load_panel(next);
                 }
                 if (!active) continue;
-                step_adjoint<R1, M1>(x, y, t1 + cc);
+                step_adjoint<R1, M1, true>(x, y, t1 + cc);
 #pragma unroll
                 for (int j = 0; j < R1 / 2; ++j) {
                     if constexpr (ROWS_OUT) {
@@ -512,7 +513,7 @@ cudaError_t lines_run(LinesMode mode, const LinesCall &c, cudaStream_t s)
     p.src = c.src;
     p.dst = c.dst;
     p.rows = c.rows;
-    p.sc = c.sc;
+    p.sc = AxisScale{2.0f * c.sc.s0, 2.0f * c.sc.s1};  // the first step halves
     p.src_off = c.src_off;
     p.dst_off = c.dst_off;
     p.tw = c.tw;

@@ -237,7 +237,11 @@ __device__ __forceinline__ void adjoint_out(float2 ur, float2 ui, float2 vr, flo
 // MC-1-cc + MC j (j < R/2).  Results k: into x (k < R/2) and y, the slots
 // they came from, times the twiddles tw[k * (MC/2)].  The sine goes first: most
 // angles are small.
-template <int R, int MC>
+// HALF (the first step): the twiddles hold a factor 1/2, which the last factor
+// would carry otherwise, so that the split's sums are no larger than their
+// results (without it a forward's range ends a binade earlier, and the
+// inverse's products lose a bit of subnormal values).
+template <int R, int MC, bool HALF>
 __device__ __forceinline__ void step_forward(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
 {
     float2 ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2], dr[R], di[R];
@@ -253,6 +257,10 @@ __device__ __forceinline__ void step_forward(float4 (&x)[R / 2], float4 (&y)[R /
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         float2 re = dr[k], im = di[k];
+        if (HALF && k == 0) {
+            re = VOps<float2>::mul(re, 0.5f);
+            im = VOps<float2>::mul(im, 0.5f);
+        }
         if (k > 0) {
             const float4 t = tw[k * (MC / 2)];
             const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
@@ -265,7 +273,7 @@ __device__ __forceinline__ void step_forward(float4 (&x)[R / 2], float4 (&y)[R /
     }
 }
 
-template <int R, int MC>
+template <int R, int MC, bool HALF>
 __device__ __forceinline__ void step_adjoint(float4 (&x)[R / 2], float4 (&y)[R / 2], const float4 *tw)
 {
     float2 dr[R], di[R], ur[R / 2], ui[R / 2], vr[R / 2], vi[R / 2];
@@ -273,8 +281,8 @@ __device__ __forceinline__ void step_adjoint(float4 (&x)[R / 2], float4 (&y)[R /
     for (int k = 0; k < R; ++k) {
         const float4 o = k < R / 2 ? x[k < R / 2 ? k : 0] : y[k < R / 2 ? 0 : k - R / 2];
         const float2 re = make_float2(o.x, o.y), im = make_float2(o.z, o.w);
-        dr[k] = re;
-        di[k] = im;
+        dr[k] = HALF ? VOps<float2>::mul(re, 0.5f) : re;
+        di[k] = HALF ? VOps<float2>::mul(im, 0.5f) : im;
         if (k > 0) {
             const float4 t = tw[k * (MC / 2)];
             const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
@@ -336,7 +344,7 @@ __device__ __forceinline__ void last_adjoint(float4 (&x)[R / 2], float4 (&w)[R /
 // ---------------------------------------------------------------- the split
 // Four outputs from Z_k = (ar, ai) and conj Z_{L-k} = (br, bi): a = (y_k,
 // y_{L-k}), b = (y_{N-k}, y_{L+k}).  The table holds exp(-2 pi i k/N) = t.x -
-// i t.y and, times s_1 / 2, the pairs over (k, L-k) of Re W (t.z, t.w) and
+// i t.y and, times s_1, the pairs over (k, L-k) of Re W (t.z, t.w) and
 // -Im W (nwi).
 // Whether |cos| is the smaller of the split's angle pi (k + x) / R, 0 <= x < 1/2 (of slot k).
 template <int R>

@@ -1,6 +1,9 @@
 """Values near the ends of the FP32 range without range protection: where the
-exact result is representable and the direct sums reached it, half products,
-which add mirrored values before any weight, reach it too.
+exact result is representable and the direct sums (or the transforms that the
+kernels replaced) reached it, the kernels reach it too.
+
+Half products add mirrored values before any weight, FFT steps add a whole line
+before the scale: both are checked with the arrays that meet their limit first.
 """
 import numpy as np
 import pytest
@@ -48,3 +51,24 @@ def test_half_products_of_mirrored_large_values(cuda_dev, h, w, path, sign):
     for kind in ("roundtrip", "spectral"):
         got = plan.execute(kind, xd).cpu().numpy().astype(np.float64)
         assert np.linalg.norm(got / 2.0 ** 120 - x / 2.0 ** 120) <= 1e-6 * np.linalg.norm(x / 2.0 ** 120), kind
+
+
+# log2 of the amplitude that the kernels replaced took to finite results, halves of a binade: constant
+# arrays and the middle cosine, round trip; +-1 signs, forward and spectral
+LIMITS = [(128, 128, 121.0, 122.0, 122.5), (64, 128, 121.0, 122.0, 122.5), (128, 64, 121.0, 122.0, 122.5),
+          (192, 192, 118.5, 121.0, 121.5), (256, 256, 118.0, 121.0, 121.5), (384, 384, 117.5, 120.0, 121.0),
+          (512, 512, 117.0, 120.0, 121.0), (768, 768, 116.5, 119.0, 120.5), (1024, 1024, 116.0, 119.0, 120.0)]
+
+
+@pytest.mark.parametrize("h,w,const,cos,sign", LIMITS)
+def test_lines_reach_the_range_of_the_kernels_replaced(cuda_dev, h, w, const, cos, sign):
+    import torch
+    plan = _plan(h, w, "fp32")
+    wave = lambda n: np.cos(np.pi * (2 * np.arange(n) + 1) * (n // 3) / (2 * n))
+    signs = np.random.default_rng(h + w).integers(0, 2, (h, w)) * 2.0 - 1.0
+    for name, x, e, kinds in (("const", np.ones((h, w)), const, ("roundtrip",)),
+                              ("cos", np.outer(wave(h), wave(w)), cos, ("roundtrip",)),
+                              ("signs", signs, sign, ("forward", "roundtrip", "spectral"))):
+        xd = torch.from_numpy((x * 0.99 * 2.0 ** e).astype(np.float32)[None]).to(cuda_dev)
+        for kind in kinds:
+            assert torch.isfinite(plan.execute(kind, xd)).all(), (name, kind)
