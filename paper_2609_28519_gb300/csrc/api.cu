@@ -113,7 +113,7 @@ static int tg_plan_tables(bdct_plan *p)
     if (k & BDCT_FORWARD) add(0, 1, p->norm);
     if (k & BDCT_INVERSE) add(1, 2, p->norm);
     if (pair) { add(2, 1, BDCT_NORM_ORTHO); add(3, 2, BDCT_NORM_ORTHO); }
-    // distinct tables, each 3 n^2 BF16 elements (64 x 64 for the Kronecker operator)
+    // distinct tables, each tg_table_elems BF16 elements (64 x 64 for the Kronecker operator)
     int uniq[8][3];
     size_t uoff[8];
     int nu = 0;
@@ -126,7 +126,7 @@ static int tg_plan_tables(bdct_plan *p)
         if (j == nu) {
             uniq[nu][0] = want[i].n; uniq[nu][1] = want[i].direction; uniq[nu][2] = want[i].norm;
             uoff[nu] = total;
-            total += tg_table_elems(p->tg_kron ? 64 : want[i].n);
+            total += tg_table_elems(p->tg_kron ? 64 : want[i].n, p->tc_terms);
             ++nu;
         }
         off_of[i] = uoff[j];
@@ -135,7 +135,7 @@ static int tg_plan_tables(bdct_plan *p)
     if (e != cudaSuccess) { t_last_cuda_error = (int)e; return BDCT_ERR_NO_MEMORY; }
     p->table_bytes = total * sizeof(__nv_bfloat16);
     for (int j = 0; j < nu && e == cudaSuccess; ++j)
-        e = tg_gen_table(p->tg_ops + uoff[j], uniq[j][0], uniq[j][1], uniq[j][2], p->tg_kron, 0);
+        e = tg_gen_table(p->tg_ops + uoff[j], uniq[j][0], uniq[j][1], uniq[j][2], p->tg_kron, p->tc_terms, 0);
     if (e != cudaSuccess) return cuda_fail(e);
     for (int i = 0; i < nw; ++i) {
         if (want[i].axis == 0) p->tg_h[want[i].slot] = off_of[i];

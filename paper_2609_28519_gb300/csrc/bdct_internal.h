@@ -150,11 +150,13 @@ cudaError_t range_postscale(const ExecGeom &g, int h, int w, const unsigned int 
 // Split-BF16 tensor-core separable passes: any side 16, 32 or a multiple of
 // 64 up to 8192 per axis, and 8 x 8 arrays as one 64 x 64 Kronecker product.
 bool tg_axis_ok(int n);
-// BF16 elements of one blocked operator table of side n (64 for Kronecker).
-size_t tg_table_elems(int n);
+// BF16 elements of one blocked operator table of side n (64 for Kronecker), for
+// passes of `terms` terms.
+size_t tg_table_elems(int n, int terms);
 // Split the FP64 operator of (direction 1 fwd / 2 inv, norm) of side n (or
 // the 8 x 8 Kronecker operator) into three BF16 terms, blocked for tg_pass.
-cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, bool kron, cudaStream_t s);
+cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, bool kron, int terms,
+                         cudaStream_t s);
 // One pass over `count` arrays of R rows of length K: every row gets the 1D
 // operator (K x K) and the result is written transposed, dst[b][n][r]
 // (arrays of K x R; R = 1 writes dst[b][n]).  src_off / dst_off index the

@@ -309,25 +309,26 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 //     mbarriers);
 //   warp 1, lane 0: issues the six products of a chunk into one of four TMEM
 //     partial accumulators and commits them twice (stage free, partial ready);
-//   warps 2-9: each reads its TMEM lane quadrant (warp % 4) and half of the
-//     columns of a finished partial, adds it to its row's running sums in
+//   the other warps (Tg2Cfg): each reads its TMEM lane quadrant (warp % 4) and
+//     its columns of a finished partial, adds them to its row's running sums in
 //     registers (round to nearest, chunk order), releases the partial, and at
-//     the end of a tile stores its part of the row transposed (with four warps
-//     the reads of the partials held up the products).
+//     the end of a tile stores its part of the row transposed (with one warp per
+//     quadrant at three terms the reads of the partials held up the products).
 // Tiles are 128 rows by 128 outputs, K chunks of 64.
 //
 // Half products.  The operator's rows are even or odd about the middle of the
-// line, so for lengths that are multiples of 256 the forward contracts s_j =
-// (x_j + x_{K-1-j}) / 2 (half_pair, ptx.cuh) with twice the even operator and d_j =
-// (x_j - x_{K-1-j}) / 2 with twice the odd one (j < K/2), and the inverse the even and the odd coefficients with the
-// two halves of its operator, x_j = a_j + b_j, x_{K-1-j} = a_j - b_j: half the
-// products, half the input blocks each tile streams, half the partials.  An
-// item is then a row tile and 128 output pairs, its two products one after the
-// other, both sums of a thread's 64 pairs in registers until they meet.  16
-// arrays of 1024 x 1024, forward and inverse: 761 -> 505 us; what bounds it then
-// is shared memory, 96 KB loaded and 192 KB read by the products per chunk
-// (tensor pipe 51%).  (K/2 a multiple of 64 but not of 128 would leave half
-// tiles, so those lengths keep the whole operator.)
+// line, so for lengths that are multiples of 256 (and three terms: tg_half) the
+// forward contracts s_j = (x_j + x_{K-1-j}) / 2 (half_pair, ptx.cuh) with twice
+// the even operator and d_j = (x_j - x_{K-1-j}) / 2 with twice the odd one (j <
+// K/2), and the inverse the even and the odd coefficients with the two halves
+// of its operator, x_j = a_j + b_j, x_{K-1-j} = a_j - b_j: half the products,
+// half the input blocks each tile streams, half the partials.  An item is then a
+// row tile and 128 output pairs, its two products one after the other, both
+// sums of a thread's 64 pairs in registers until they meet.  16 arrays of 1024 x
+// 1024, forward and inverse: 761 -> 505 us; what bounds it then is shared
+// memory, 96 KB loaded and 192 KB read by the products per chunk (tensor pipe
+// 51%).  (K/2 a multiple of 64 but not of 128 would leave half tiles, so those
+// lengths keep the whole operator.)
 
 enum SplitMode { SPLIT_WHOLE = 0, SPLIT_FWD = 1, SPLIT_INV = 2 };
 
@@ -412,9 +413,6 @@ __global__ void k_tg_presplit(const float *src, const long long *src_off, long l
 
 constexpr int kTg2NT = 128;
 constexpr int kTg2Stages = 2;
-constexpr int kTg2Epi = 8;                            // epilogue warps: two per TMEM lane quadrant
-constexpr int kTg2Cols = kTg2NT / (kTg2Epi / 4);      // columns of each
-constexpr int kTg2Threads = 64 + 32 * kTg2Epi;
 // TMEM partial accumulators (kTg2Acc x 128 columns of the 512): the MMA lane
 // may run kTg2Acc - 1 chunks ahead of the epilogue warps' reads
 constexpr int kTg2Acc = 4;
@@ -424,22 +422,36 @@ constexpr int kTg2BStage = 3 * kTg2NT * kTgKC * 2;    // bytes of the operator t
 constexpr int kTg2Stage = kTg2AStage + kTg2BStage;
 constexpr size_t kTg2Smem = (size_t)kTg2Stages * kTg2Stage + (2 * kTg2Stages + 2 * kTg2Acc) * 8 + 16;
 
+// Epilogue warps: two per TMEM lane quadrant, each half of an item's NT columns;
+// one per quadrant below three terms, whose products are fewer (16 arrays of 1024
+// x 1024, one term, 196 us with two, 193 with one).
+template <int TERMS, int NT>
+struct Tg2Cfg {
+    static constexpr int EPI = TERMS == 3 ? 8 : 4;
+    static constexpr int COLS = NT / (EPI / 4);  // columns of each
+    static constexpr int THREADS = 64 + 32 * EPI;
+};
+
 struct Tg2Params {
     const __nv_bfloat16 *abuf;       // input terms, [row tile][product][chunk][term][128 x KC]
     const __nv_bfloat16 *ops;        // operator terms, [product][n tile][chunk][term][128 x KC]
     float *dst;
     const long long *dst_off;
     long long rows_total;
-    int R, N, KC, nk, n_tiles;       // nk, n_tiles: of one product
-    int sub, inverse;                // products per item (2: half products), and which half form
+    int R, N, KC, nk, n_tiles;       // nk, n_tiles (of 128 outputs): of one product
+    int sub, inverse;                // products per item (2: half products, three terms only), and which half form
     long long items;
     const float *lam;
     unsigned int *status;
 };
 
-template <int TERMS>
-__global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
+// NT: outputs (or output pairs) per item.
+template <int TERMS, int NT>
+__global__ void __launch_bounds__(Tg2Cfg<TERMS, NT>::THREADS, 1) k_tcg2(const Tg2Params p)
 {
+    constexpr int EPI = Tg2Cfg<TERMS, NT>::EPI, COLS = Tg2Cfg<TERMS, NT>::COLS;
+    constexpr int PARTS = kTg2NT / NT;  // items of one tile of the operator
+    const int sub = TERMS == 3 ? p.sub : 1;
     extern __shared__ __align__(1024) uint8_t t2s[];
     uint64_t *full = reinterpret_cast<uint64_t *>(t2s + kTg2Stages * kTg2Stage);
     uint64_t *empty = full + kTg2Stages;
@@ -456,7 +468,7 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
         }
         for (int a = 0; a < kTg2Acc; ++a) {
             mbar_init(&pfull[a], 1);
-            mbar_init(&pempty[a], kTg2Epi);  // one arrival per epilogue warp
+            mbar_init(&pempty[a], EPI);  // one arrival per epilogue warp
         }
         *abort_flag = 0;
         fence_mbar_init();
@@ -474,19 +486,20 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const int KC = p.KC, nk = p.nk;
-    const uint32_t a_term = 128u * KC * 2, b_term = (uint32_t)kTg2NT * KC * 2;
-    const long long blk_elems = 3LL * 128 * KC;  // input and operator blocks alike (NT = 128)
+    const uint32_t a_term = 128u * KC * 2, b_term = (uint32_t)NT * KC * 2;
+    const long long blk_elems = 3LL * 128 * KC;  // input and operator blocks alike
     long long last_load = -1, last_commit = -1;  // error path: the last copy and commit issued
     bool ok = true;
+    const int n_items = p.n_tiles * PARTS;       // per row tile
 
     if (warp == 0) {
         // ---- producer
         if (lane == 0) {
             long long c = 0;
             for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-                const long long mt = item / p.n_tiles;
-                const int nt = (int)(item % p.n_tiles);
-                for (int ec = 0; ec < p.sub * nk; ++ec, ++c) {
+                const long long mt = item / n_items;
+                const int nt = (int)(item % n_items) / PARTS, part = (int)(item % n_items) % PARTS;
+                for (int ec = 0; ec < sub * nk; ++ec, ++c) {
                     const int s = (int)(c % kTg2Stages);
                     const uint32_t use = (uint32_t)(c / kTg2Stages);
                     if (c >= kTg2Stages && !mbar_wait_bounded(&empty[s], (use - 1) & 1u)) { ok = false; break; }
@@ -494,9 +507,16 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
                     uint8_t *st = t2s + s * kTg2Stage;
                     mbar_arrive_expect_tx(&full[s], (uint32_t)TERMS * (a_term + b_term));
                     const int e = ec >= nk, kc = ec - e * nk;
-                    bulk_load(st, p.abuf + (mt * p.sub * nk + ec) * blk_elems, (uint32_t)TERMS * a_term, &full[s]);
-                    bulk_load(st + kTg2AStage, p.ops + ((long long)(nt + e * p.n_tiles) * nk + kc) * blk_elems,
-                              (uint32_t)TERMS * b_term, &full[s]);
+                    bulk_load(st, p.abuf + (mt * sub * nk + ec) * blk_elems, (uint32_t)TERMS * a_term, &full[s]);
+                    const __nv_bfloat16 *b = p.ops + ((long long)(nt + e * p.n_tiles) * nk + kc) * blk_elems;
+                    if constexpr (PARTS == 1) {
+                        bulk_load(st + kTg2AStage, b, (uint32_t)TERMS * b_term, &full[s]);
+                    } else {
+                        // NT of every term's 128 outputs (eight rows of the layout are contiguous)
+#pragma unroll
+                        for (int t = 0; t < TERMS; ++t)
+                            bulk_load(st + kTg2AStage + t * b_term, b + (t * 128 + part * NT) * KC, b_term, &full[s]);
+                    }
                     last_load = c;
                 }
             }
@@ -504,14 +524,14 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
     } else if (warp == 1) {
         // ---- MMA issue
         if (lane == 0) {
-            constexpr uint32_t idesc = tc_idesc(kTg2NT, false);
+            constexpr uint32_t idesc = tc_idesc(NT, false);
             const uint32_t sbo = (uint32_t)(KC / 8) * 128u;
             constexpr int pa[6] = {2, 1, 0, 1, 0, 0};
             constexpr int pb[6] = {0, 1, 2, 0, 1, 0};
             constexpr int first = TERMS == 3 ? 0 : (TERMS == 2 ? 3 : 5);
             long long c = 0;
             for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-                for (int ec = 0; ec < p.sub * nk; ++ec, ++c) {
+                for (int ec = 0; ec < sub * nk; ++ec, ++c) {
                     const int s = (int)(c % kTg2Stages), a = (int)(c % kTg2Acc);
                     if (!mbar_wait_bounded(&full[s], (uint32_t)(c / kTg2Stages) & 1u)) { ok = false; break; }
                     if (c >= kTg2Acc && !mbar_wait_bounded(&pempty[a], (uint32_t)(c / kTg2Acc - 1) & 1u)) {
@@ -535,16 +555,16 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
             }
         }
     } else {
-        // ---- epilogue: TMEM lane quadrant q, half of the columns of every partial
+        // ---- epilogue: TMEM lane quadrant q, this warp's columns of every partial
         const int q = warp & 3;
         const int row = 32 * q + lane;
-        const int col0 = (warp - 2) / 4 * kTg2Cols;
+        const int col0 = (warp - 2) / 4 * COLS;
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-        float sum[2][kTg2Cols];  // of the item's one or two products
+        float sum[TERMS == 3 ? 2 : 1][COLS];  // of the item's one or two products
         long long c = 0;
-        auto product = [&](float (&acc)[kTg2Cols]) {
+        auto product = [&](float (&acc)[COLS]) {
 #pragma unroll
-            for (int j = 0; j < kTg2Cols; ++j) acc[j] = 0.0f;
+            for (int j = 0; j < COLS; ++j) acc[j] = 0.0f;
             for (int kc = 0; kc < nk; ++kc, ++c) {
                 const int a = (int)(c % kTg2Acc);
                 bool w = mbar_wait_bounded(&pfull[a], (uint32_t)(c / kTg2Acc) & 1u);
@@ -552,7 +572,7 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
                 if (!w) return false;
                 tc_fence_after();
 #pragma unroll
-                for (int cc = 0; cc < kTg2Cols / 16; ++cc) {
+                for (int cc = 0; cc < COLS / 16; ++cc) {
                     float y[16];
                     tmem_ld16(tmem + (uint32_t)(a * kTg2NT + col0) + lane_off + 16 * cc, y);
 #pragma unroll
@@ -566,34 +586,37 @@ __global__ void __launch_bounds__(kTg2Threads, 1) k_tcg2(const Tg2Params p)
         };
         for (long long item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
             ok = product(sum[0]);
-            if (ok && p.sub == 2) ok = product(sum[1]);
+            if constexpr (TERMS == 3)
+                if (ok && sub == 2) ok = product(sum[1]);
             if (!ok) break;
-            const long long m = (item / p.n_tiles) * 128 + row;
+            const long long m = (item / n_items) * 128 + row;
             if (m >= p.rows_total) continue;
             const long long b = m / p.R, r = m - b * p.R;
             float *dbase = p.dst + (p.dst_off ? p.dst_off[b] : b * (long long)p.N * p.R) + r;
-            const long long n0 = (item % p.n_tiles) * kTg2NT + col0, ld = p.R;
-            if (p.sub == 1) {
+            const long long n0 = (item % n_items) * NT + col0, ld = p.R;
+            if (sub == 1) {
                 const float *l = p.lam ? p.lam + n0 * ld + r : nullptr;
 #pragma unroll
-                for (int j = 0; j < kTg2Cols; ++j)
+                for (int j = 0; j < COLS; ++j)
                     dbase[(n0 + j) * ld] = l ? sum[0][j] * __ldg(l + j * ld) : sum[0][j];
-            } else if (!p.inverse) {
-                // coefficients 2 (n0 + j) and the next
-                float *d = dbase + 2 * n0 * ld;
-                const float *l = p.lam ? p.lam + 2 * n0 * ld + r : nullptr;
+            } else if constexpr (TERMS == 3) {
+                if (!p.inverse) {
+                    // coefficients 2 (n0 + j) and the next
+                    float *d = dbase + 2 * n0 * ld;
+                    const float *l = p.lam ? p.lam + 2 * n0 * ld + r : nullptr;
 #pragma unroll
-                for (int j = 0; j < kTg2Cols; ++j) {
-                    d[2 * j * ld] = l ? sum[0][j] * __ldg(l + 2 * j * ld) : sum[0][j];
-                    d[(2 * j + 1) * ld] = l ? sum[1][j] * __ldg(l + (2 * j + 1) * ld) : sum[1][j];
-                }
-            } else {
-                // samples n0 + j and their mirrors
-                float *d = dbase + n0 * ld, *u = dbase + (p.N - 1 - n0) * ld;
+                    for (int j = 0; j < COLS; ++j) {
+                        d[2 * j * ld] = l ? sum[0][j] * __ldg(l + 2 * j * ld) : sum[0][j];
+                        d[(2 * j + 1) * ld] = l ? sum[1][j] * __ldg(l + (2 * j + 1) * ld) : sum[1][j];
+                    }
+                } else {
+                    // samples n0 + j and their mirrors
+                    float *d = dbase + n0 * ld, *u = dbase + (p.N - 1 - n0) * ld;
 #pragma unroll
-                for (int j = 0; j < kTg2Cols; ++j) {
-                    d[j * ld] = sum[0][j] + sum[1][j];
-                    u[-j * ld] = sum[0][j] - sum[1][j];
+                    for (int j = 0; j < COLS; ++j) {
+                        d[j * ld] = sum[0][j] + sum[1][j];
+                        u[-j * ld] = sum[0][j] - sum[1][j];
+                    }
                 }
             }
         }
@@ -941,20 +964,27 @@ static int tg_kc(int k) { return k % 64 == 0 ? 64 : ((k == 16 || k == 32) ? k : 
 
 bool tg_axis_ok(int n) { return n == 16 || n == 32 || (n % 64 == 0 && n >= 64 && n <= 8192); }
 
-// Half products: both halves of the outputs in whole tiles.
-static bool tg_half(int n) { return n % 256 == 0; }
+// Half products: both halves of the outputs in whole tiles, and three terms.
+// A sum of two values that fit one or two terms takes a bit more than they
+// hold, so below three terms the whole operator, which meets the values as they
+// are, is more exact (256 x 256 forward, uniform values: one term 3.28e-3 against
+// 3.34e-3, two 6.22e-6 against 6.38e-6; whole numbers that the terms hold, 15%
+// less); half products would take 138 us where it takes 190 (16 arrays of 1024
+// x 1024, one term).
+static bool tg_half(int n, int terms) { return n % 256 == 0 && terms == 3; }
 
-size_t tg_table_elems(int n) { return (size_t)3 * n * (tg_half(n) ? n / 2 : n); }
+size_t tg_table_elems(int n, int terms) { return (size_t)3 * n * (tg_half(n, terms) ? n / 2 : n); }
 
-cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, bool kron, cudaStream_t s)
+cudaError_t tg_gen_table(__nv_bfloat16 *dst, int n, int direction, int norm, bool kron, int terms, cudaStream_t s)
 {
     const int N = kron ? 64 : n;
     const int NT = tg_nt(N), KC = tg_kc(N);
     if (!NT || !KC) return cudaErrorInvalidValue;
-    const int K = tg_half(N) ? N / 2 : N;
+    const bool half = tg_half(N, terms);
+    const int K = half ? N / 2 : N;
     const long long total = (long long)N * K;
     k_gen_tg_op<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(dst, N, K, direction, norm, NT, KC, kron ? 1 : 0,
-                                                               tg_half(N) ? 1 : 0);
+                                                               half ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1025,6 +1055,43 @@ size_t tg_split_elems(long long rows, int K)
     return (size_t)m_tiles * 128 * (size_t)K * 3;
 }
 
+// Step 2 of tg2_launch: the products, persistent CTAs over the items.
+template <int TERMS, int NT>
+static cudaError_t tg2_products(Tg2Params p, int sms, cudaStream_t stream)
+{
+    static DeviceLaunchCache cache;
+    int dev = 0, bps = 0, unused = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    auto kern = k_tcg2<TERMS, NT>;
+    e = cache.get(
+        dev,
+        [&](int, int &b, int &n) {
+            b = n = 1;
+            const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTg2Smem);
+            if (r == cudaSuccess && debug_enabled())
+                fprintf(stderr, "[bdct] k_tcg2<%d,%d>: 1 CTA/SM x %d threads, smem %zu B, TMEM %d cols\n", TERMS, NT,
+                        Tg2Cfg<TERMS, NT>::THREADS, kTg2Smem, kTg2Acc * kTg2NT);
+            return r;
+        },
+        &bps, &unused);
+    if (e != cudaSuccess) return e;
+    p.items *= kTg2NT / NT;
+    long long grid = (long long)sms;
+    if (grid > p.items) grid = p.items;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(Tg2Cfg<TERMS, NT>::THREADS);
+    cfg.dynamicSmemBytes = kTg2Smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
 template <int TERMS>
 static cudaError_t tg2_launch(const float *src, const long long *src_off, const Tg2Params &p0, int K,
                               __nv_bfloat16 *abuf, cudaStream_t stream)
@@ -1033,17 +1100,11 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
     int dev = 0, bps = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    auto kern = k_tcg2<TERMS>;
     e = cache.get(
         dev,
         [&](int d, int &b, int &n) {
-            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTg2Smem);
-            if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
             b = 1;
-            if (r == cudaSuccess && debug_enabled())
-                fprintf(stderr, "[bdct] k_tcg2<%d>: 1 CTA/SM x %d threads, smem %zu B, TMEM %d cols\n", TERMS,
-                        kTg2Threads, kTg2Smem, kTg2Acc * kTg2NT);
-            return r;
+            return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
         },
         &bps, &sms);
     if (e != cudaSuccess) return e;
@@ -1054,27 +1115,16 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
         const long long work = m_tiles * 128LL * K / 8;
         long long blocks = (work + 255) / 256;
         if (blocks > (long long)sms * 16) blocks = (long long)sms * 16;
-        auto split = p.sub == 1 ? k_tg_presplit<TERMS, SPLIT_WHOLE>
-                     : p.inverse ? k_tg_presplit<TERMS, SPLIT_INV> : k_tg_presplit<TERMS, SPLIT_FWD>;
+        auto split = k_tg_presplit<TERMS, SPLIT_WHOLE>;
+        if constexpr (TERMS == 3)
+            if (p.sub == 2) split = p.inverse ? k_tg_presplit<TERMS, SPLIT_INV> : k_tg_presplit<TERMS, SPLIT_FWD>;
         split<<<(unsigned)blocks, 256, 0, stream>>>(src, src_off, p.rows_total, p.R, K, p.KC, m_tiles, abuf);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    // 2. the products, persistent CTAs over the tiles
+    // 2. the products
     p.abuf = abuf;
-    long long grid = (long long)sms;
-    if (grid > p.items) grid = p.items;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kTg2Threads);
-    cfg.dynamicSmemBytes = kTg2Smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p);
+    return tg2_products<TERMS, kTg2NT>(p, sms, stream);
 }
 
 cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, const long long *dst_off, long long count,
@@ -1108,7 +1158,7 @@ cudaError_t tg_pass(const float *src, float *dst, const long long *src_off, cons
         p.R = R;
         p.N = N;
         p.KC = KC;
-        p.sub = tg_half(K) ? 2 : 1;
+        p.sub = tg_half(K, terms) ? 2 : 1;
         p.inverse = inverse ? 1 : 0;
         const int KH = K / p.sub;
         p.nk = KH / KC;
