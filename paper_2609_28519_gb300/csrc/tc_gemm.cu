@@ -445,7 +445,8 @@ struct Tg2Params {
     unsigned int *status;
 };
 
-// NT: outputs (or output pairs) per item.
+// NT: outputs (or output pairs) per item, 128 or, for calls that leave SMs
+// without an item, 64 (tg2_launch).
 template <int TERMS, int NT>
 __global__ void __launch_bounds__(Tg2Cfg<TERMS, NT>::THREADS, 1) k_tcg2(const Tg2Params p)
 {
@@ -1092,6 +1093,11 @@ static cudaError_t tg2_products(Tg2Params p, int sms, cudaStream_t stream)
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
+// Items of 64 output pairs while that many fit the chip at once: an item's
+// stores alone (256 outputs of 128 rows) take as long as its products on a few
+// chunks (256 x 256 forward, one array 28.3 -> 25.0 us, 32 arrays 34.9 -> 32.5;
+// 1024 x 1024, two arrays 68.4 -> 65.0).  With more, an SM would take two narrow
+// items one after the other, and stream the input's terms twice.
 template <int TERMS>
 static cudaError_t tg2_launch(const float *src, const long long *src_off, const Tg2Params &p0, int K,
                               __nv_bfloat16 *abuf, cudaStream_t stream)
@@ -1124,6 +1130,8 @@ static cudaError_t tg2_launch(const float *src, const long long *src_off, const 
     }
     // 2. the products
     p.abuf = abuf;
+    if constexpr (TERMS == 3)
+        if (p.sub == 2 && 2 * p.items <= sms) return tg2_products<3, 64>(p, sms, stream);
     return tg2_products<TERMS, kTg2NT>(p, sms, stream);
 }
 

@@ -71,3 +71,21 @@ def test_three_terms_in_place(cuda_dev, h, w):
         y, z = plan.execute(kind, x), x.clone()
         plan.execute(kind, z, z)
         assert torch.equal(y, z), kind
+
+
+@pytest.mark.parametrize("h,w", [(256, 256), (256, 384), (768, 512), (1024, 1024)])
+def test_narrow_items_equal_the_wide_ones(cuda_dev, h, w):
+    """A call of few row tiles takes items of half the width, the same sums: one
+    array alone is bit for bit what it is in a batch that fills the chip."""
+    import torch
+    from paper_2609_28519_gb300 import Plan
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    plan = Plan(h, w, kind=15, path="split_tc")
+    plan.set_spectral(inputs.random_diagonal(9, h, w))
+    x = torch.from_numpy(inputs.uniform(h + 2 * w, 2, h, w)).to(cuda_dev)
+    many = x.repeat(-(-128 * sms // min(h, w)), 1, 1)
+    for kind in ("forward", "inverse", "roundtrip", "spectral"):
+        y = plan.execute(kind, many)
+        assert torch.equal(y, plan.execute(kind, x).repeat(len(many) // 2, 1, 1)), kind
+        assert torch.equal(y[1], plan.execute(kind, x[1:].contiguous())[0]), kind
+    assert plan.device_status() == 0
