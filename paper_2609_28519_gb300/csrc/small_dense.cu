@@ -14,7 +14,8 @@
 //
 // Organization.  A CTA of four warps transforms G arrays at a time, G chosen
 // so that one tile of 8 lines x 4 output pairs per thread covers them
-// (about 8192 elements).  Every pass stores what the next one contracts,
+// (about 8192 elements), or, in a call of few arrays, of eight warps with tiles
+// of 2 lines.  Every pass stores what the next one contracts,
 // already paired, from registers:
 //  * along w, forward: a thread's lines are mirrored rows (i, h-1-i), whose
 //    sum and difference is the pair the pass along h needs;
@@ -37,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdio>
+#include <type_traits>
 
 #include "bdct_internal.h"
 #include "dense_passes.h"
@@ -47,11 +49,27 @@ namespace bdct {
 
 namespace {
 
-constexpr int kThreads = 128;
+// Threads per CTA, by the line pairs I per thread and tile: 4, or 1 for calls
+// of few arrays (small_dense_run).
+template <int I>
+constexpr int kThreadsOf = I == 1 ? 256 : 128;
 constexpr int kMaxSide = 64;
 constexpr int kMaxArrays = 64;
-constexpr int kTarget = 8192;  // elements per CTA: one tile of 64 per thread
 constexpr int kSlack = 256;    // pairs past a buffer that an edge tile may read
+
+// Calls of at most this many elements per SM take tiles of 2 lines and eight
+// warps: such a call lasts as long as one CTA's chain of passes, which large
+// tiles and arrays packed into few CTAs only lengthen, and the short code of
+// small tiles is fetched sooner (333 arrays of 12 x 12 forward 4.7 -> 2.9 us,
+// round trip 7.7 -> 4.1; one 60 x 60 array 6.6 -> 4.9; 1000 of 20 x 20 6.0 ->
+// 4.6).  From about 7000 the large tiles' fewer operand reads win (1000 arrays
+// of 40 x 40, 10526 an SM, 14.3 us with small tiles, 13.1 with large; 2000 of
+// 24 x 24, 7579 an SM, 8.9 and 8.2).
+constexpr long long kFew = 6144;
+
+// Elements per CTA: one tile of 2 I lines x 8 outputs per thread.
+template <int I>
+constexpr int kTarget = kThreadsOf<I> * 16 * I;
 
 // Exact quotients of small unsigned values by a fixed divisor.
 struct FastDiv {
@@ -72,7 +90,7 @@ struct Axis {
         : nh((n + 1) / 2), tc((nh + 3) / 4), np(4 * tc), tcl(tc <= 2 ? tc : tc == 5 || tc == 6 ? 2 : 4)
     {
     }
-    __host__ __device__ int line_block() const { return 256 / tcl; }  // lines of a warp's tile
+    __host__ __device__ int line_block(int I) const { return 64 * I / tcl; }  // lines of a warp's tile
 };
 
 struct SmallParams {
@@ -113,20 +131,20 @@ __device__ __forceinline__ void lane_place(const Axis &x, int lane, int &tq, int
     }
 }
 
-// Products of lines l0 + i * ls (+ 1) and output pairs 4 tc .. 4 tc + 3:
+// Products of lines l0 + i * ls (+ 1), i < I, and output pairs 4 tc .. 4 tc + 3:
 // acc[2i + r][o] = (even, odd) sums over k < K of a[k][line] * t[k][o].
-template <bool LONG>
+template <bool LONG, int I>
 __device__ __forceinline__ void products(const float2 *a, int pitch, int ls, const float2 *t, int np, int K,
-                                         float2 (&acc)[8][4])
+                                         float2 (&acc)[2 * I][4])
 {
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 2 * I; ++r)
 #pragma unroll
         for (int o = 0; o < 4; ++o) acc[r][o] = make_float2(0.f, 0.f);
-    auto step = [&](float2 (&sum)[8][4]) {
-        float2 x[8], m[4];
+    auto step = [&](float2 (&sum)[2 * I][4]) {
+        float2 x[2 * I], m[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < I; ++i) {
             const float4 v = *reinterpret_cast<const float4 *>(a + i * ls);
             x[2 * i] = make_float2(v.x, v.y);
             x[2 * i + 1] = make_float2(v.z, v.w);
@@ -140,7 +158,7 @@ __device__ __forceinline__ void products(const float2 *a, int pitch, int ls, con
         a += pitch;
         t += np;
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
+        for (int r = 0; r < 2 * I; ++r)
 #pragma unroll
             for (int o = 0; o < 4; ++o) sum[r][o] = __ffma2_rn(x[r], m[o], sum[r][o]);
     };
@@ -150,15 +168,15 @@ __device__ __forceinline__ void products(const float2 *a, int pitch, int ls, con
     } else {
         for (int k0 = 0; k0 < K; k0 += 16) {
             const int kn = min(16, K - k0);
-            float2 part[8][4];
+            float2 part[2 * I][4];
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
+            for (int r = 0; r < 2 * I; ++r)
 #pragma unroll
                 for (int o = 0; o < 4; ++o) part[r][o] = make_float2(0.f, 0.f);
 #pragma unroll 2
             for (int k = 0; k < kn; ++k) step(part);
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
+            for (int r = 0; r < 2 * I; ++r)
 #pragma unroll
                 for (int o = 0; o < 4; ++o) acc[r][o] = __fadd2_rn(acc[r][o], part[r][o]);
         }
@@ -166,9 +184,10 @@ __device__ __forceinline__ void products(const float2 *a, int pitch, int ls, con
 }
 
 // DIR: DIR_FWD, DIR_INV, or DIR_RT for both pairs (Lambda between if set).
-template <int DIR, bool LONG>
-__global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallParams p)
+template <int DIR, bool LONG, int I>
+__global__ void __launch_bounds__(kThreadsOf<I>, I == 1 ? 2 : LONG ? 2 : 3) k_small(const SmallParams p)
 {
+    constexpr int kThreads = kThreadsOf<I>;
     constexpr bool FWD = DIR != DIR_INV, INV = DIR != DIR_FWD;
     extern __shared__ __align__(16) float2 ssm[];
     float2 *buf[2] = {ssm, ssm + p.buf0};
@@ -297,24 +316,24 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
         }
         __syncthreads();
 
-        float2 acc[8][4];
+        float2 acc[2 * I][4];
         // tiles of a pass: line blocks x groups of tcl output quads, a warp each
         auto for_tiles = [&](const Axis &x, int lines, int tq, int la, auto &&tile) {
-            const int lb = x.line_block(), nlb = (lines + lb - 1) / lb, nt = nlb * ((x.tc + x.tcl - 1) / x.tcl);
+            const int lb = x.line_block(I), nlb = (lines + lb - 1) / lb, nt = nlb * ((x.tc + x.tcl - 1) / x.tcl);
             for (int t = warp; t < nt; t += kThreads / 32) {
                 const int tg = t / nlb;
                 const int q = tg * x.tcl + tq;
-                tile((t - tg * nlb) * lb + 2 * la, lb / 4, q < x.tc ? q : x.tc - 1, q < x.tc);
+                tile((t - tg * nlb) * lb + 2 * la, lb / I, q < x.tc ? q : x.tc - 1, q < x.tc);
             }
         };
 
         if constexpr (FWD) {
             // ---- along w: rows (i, h-1-i) of an array
             for_tiles(aw, 2 * kh * na, tqw, law, [&](int l0, int ls, int tc, bool live) {
-                products<LONG>(buf[0] + l0, pfw, ls, t_fw + 4 * tc, aw.np, kw, acc);
+                products<LONG, I>(buf[0] + l0, pfw, ls, t_fw + 4 * tc, aw.np, kw, acc);
                 if (!live) return;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < I; ++i) {
                     const int pr = (l0 + i * ls) / 2;
                     const int a = p.div_hp.div(pr), r = pr - a * kh;
                     if (a >= na) continue;
@@ -332,10 +351,10 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
             __syncthreads();
             // ---- along h: neighbouring columns; coefficient rows 2o, 2o + 1
             for_tiles(ah, w * na, tqh, lah, [&](int l0, int ls, int tc, bool live) {
-                products<LONG>(buf[1] + l0, ph, ls, t_fh + 4 * tc, ah.np, kh, acc);
+                products<LONG, I>(buf[1] + l0, ph, ls, t_fh + 4 * tc, ah.np, kh, acc);
                 if (!live) return;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < I; ++i) {
                     const int l = l0 + i * ls;
                     const int a = p.div_w4.div(l / 4), c = l - a * w;
                     if (a >= na) continue;
@@ -375,10 +394,10 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
         if constexpr (INV) {
             // ---- along h, inverse: rows j and h-1-j of neighbouring columns
             for_tiles(ah, w * na, tqh, lah, [&](int l0, int ls, int tc, bool live) {
-                products<LONG>(buf[0] + l0, ph, ls, t_ih + 4 * tc, ah.np, kh, acc);
+                products<LONG, I>(buf[0] + l0, ph, ls, t_ih + 4 * tc, ah.np, kh, acc);
                 if (!live) return;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < I; ++i) {
                     const int l = l0 + i * ls;
                     const int a = p.div_w4.div(l / 4), c = l - a * w;
                     if (a >= na) continue;
@@ -402,11 +421,11 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
             __syncthreads();
             // ---- along w, inverse: rows to global memory
             for_tiles(aw, h * na, tqw, law, [&](int l0, int ls, int tc, bool live) {
-                products<LONG>(buf[1] + l0, piw, ls, t_iw + 4 * tc, aw.np, kw, acc);
+                products<LONG, I>(buf[1] + l0, piw, ls, t_iw + 4 * tc, aw.np, kw, acc);
                 if (!live) return;
                 const int o0 = 4 * tc;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < I; ++i)
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
                         const int l = l0 + i * ls + s;
@@ -429,23 +448,26 @@ __global__ void __launch_bounds__(kThreads, LONG ? 2 : 3) k_small(const SmallPar
     }
 }
 
-template <int DIR, bool LONG>
-cudaError_t launch(SmallParams p, cudaStream_t stream)
+template <int DIR, bool LONG, int I>
+cudaError_t launch(SmallParams p, int sms, cudaStream_t stream)
 {
+    constexpr int kThreads = kThreadsOf<I>;
     const Axis aw(p.w), ah(p.h);
     constexpr bool FWD = DIR != DIR_INV, INV = DIR != DIR_FWD;
-    // arrays per iteration: about kTarget elements, and among the counts near
-    // it the one whose warp tiles fill the four warps best (the larger on a tie)
+    // arrays per iteration: about kTarget elements but no more than spread the
+    // call over the SMs, and among the counts near it the one whose warp tiles
+    // fill the four warps best (the larger on a tie)
     auto tiles = [](const Axis &x, int lines) {
-        return (lines + x.line_block() - 1) / x.line_block() * ((x.tc + x.tcl - 1) / x.tcl);
+        return (lines + x.line_block(I) - 1) / x.line_block(I) * ((x.tc + x.tcl - 1) / x.tcl);
     };
-    int gmax = kTarget / (p.h * p.w);
+    long long gmax = kTarget<I> / (p.h * p.w);
+    if (gmax > (p.count + sms - 1) / sms) gmax = (p.count + sms - 1) / sms;
     if (gmax < 1) gmax = 1;
     if (gmax > kMaxArrays) gmax = kMaxArrays;
     int G = 1;
     double best = 0.0;
-    for (int g = gmax; g >= 1 && 2 * g >= gmax; --g) {
-        auto rounds = [&](int t) { return (t + 3) / 4; };
+    for (int g = (int)gmax; g >= 1 && 2 * g >= gmax; --g) {
+        auto rounds = [&](int t) { return (t + kThreads / 32 - 1) / (kThreads / 32); };
         const int r = rounds(tiles(aw, FWD ? 2 * ah.nh * g : p.h * g)) + rounds(tiles(ah, p.w * g));
         const double per = (double)g / r;
         if (per > best * 1.02) {
@@ -466,20 +488,18 @@ cudaError_t launch(SmallParams p, cudaStream_t stream)
     if (smem > 220 * 1024) return cudaErrorInvalidValue;
     p.groups = (p.count + G - 1) / G;
 
-    auto kern = k_small<DIR, LONG>;
+    auto kern = k_small<DIR, LONG, I>;
     static DeviceLaunchCache cache;
-    int dev = 0, bps = 0, sms = 0;
+    int dev = 0, bps = 0, unused = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cache.get(
         dev,
-        [&](int d, int &b, int &n) {
-            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-            if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
-            b = 1;
-            return r;
+        [&](int, int &b, int &n) {
+            b = n = 1;
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         },
-        &bps, &sms);
+        &bps, &unused);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
@@ -491,12 +511,12 @@ cudaError_t launch(SmallParams p, cudaStream_t stream)
         // once per configuration, not per launch
         static std::mutex mu;
         static long long last = -1;
-        const long long key = ((long long)p.h << 20) | ((long long)p.w << 8) | DIR;
+        const long long key = ((long long)p.h << 20) | ((long long)p.w << 8) | (DIR * 8 + I);
         std::lock_guard<std::mutex> lock(mu);
         if (key != last) {
             last = key;
-            fprintf(stderr, "[bdct] k_small<%d,%d> %dx%d: %d arrays per iteration, %d CTAs/SM, smem %zu B\n", DIR,
-                    (int)LONG, p.h, p.w, G, per_sm, smem);
+            fprintf(stderr, "[bdct] k_small<%d,%d,%d> %dx%d: %d arrays per iteration, %d CTAs/SM, smem %zu B\n", DIR,
+                    (int)LONG, I, p.h, p.w, G, per_sm, smem);
         }
     }
     cudaLaunchConfig_t cfg = {};
@@ -545,10 +565,28 @@ cudaError_t small_dense_run(int h, int w, Dir dir, const SmallTables &t, const f
     p.div_hp = FastDiv((h + 1) / 2);
     p.div_wq = FastDiv((w + 7) / 8);
     p.div_kh = FastDiv((h + 1) / 2);
+    static DeviceLaunchCache cache;
+    int dev = 0, bps = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = cache.get(
+        dev,
+        [&](int d, int &b, int &n) {
+            b = 1;
+            return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d);
+        },
+        &bps, &sms);
+    if (e != cudaSuccess) return e;
     const bool is_long = h > 32 || w > 32;  // more than 16 pairs on an axis
-    if (dir == DIR_FWD) return is_long ? launch<DIR_FWD, true>(p, stream) : launch<DIR_FWD, false>(p, stream);
-    if (dir == DIR_INV) return is_long ? launch<DIR_INV, true>(p, stream) : launch<DIR_INV, false>(p, stream);
-    return is_long ? launch<DIR_RT, true>(p, stream) : launch<DIR_RT, false>(p, stream);
+    const bool few = g.count * (long long)(h * w) <= kFew * sms;
+    auto run = [&](auto dir_c) {
+        constexpr int D = decltype(dir_c)::value;
+        if (few) return is_long ? launch<D, true, 1>(p, sms, stream) : launch<D, false, 1>(p, sms, stream);
+        return is_long ? launch<D, true, 4>(p, sms, stream) : launch<D, false, 4>(p, sms, stream);
+    };
+    if (dir == DIR_FWD) return run(std::integral_constant<int, DIR_FWD>{});
+    if (dir == DIR_INV) return run(std::integral_constant<int, DIR_INV>{});
+    return run(std::integral_constant<int, DIR_RT>{});
 }
 
 }  // namespace bdct
