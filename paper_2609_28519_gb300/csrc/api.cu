@@ -414,14 +414,18 @@ static int run_lines(const bdct_plan *p, Dir dir, const float *in, const long lo
         LinesCall ch{p->work, dst, w, nb, sc.h, tab_h(set), tab_h(2), p->status, nullptr, dof, true};
         cudaError_t e;
         if (dir == DIR_SPEC) {
+            cw.beside = LINES_PAIR_DIAGONAL;
+            ch.beside = LINES_INVERSE_ROWS;
             e = lines_pass(cw, w, LINES_FORWARD, s);
             ch.tw = tab_h(1);
             ch.lam = p->spec_plain;
             if (e == cudaSuccess) e = lines_pass(ch, h, LINES_PAIR_DIAGONAL, s);
-            const LinesCall ci{dst, dst, h, nb, sc.w, tab_w(1), tab_w(2), p->status, dof, dof};
+            LinesCall ci{dst, dst, h, nb, sc.w, tab_w(1), tab_w(2), p->status, dof, dof};
+            ci.beside = LINES_PAIR_DIAGONAL;
             if (e == cudaSuccess) e = lines_pass(ci, w, LINES_INVERSE_ROWS, s);
         } else {
             const LinesMode mode = dir == DIR_FWD ? LINES_FORWARD : dir == DIR_INV ? LINES_INVERSE : LINES_PAIR;
+            cw.beside = ch.beside = mode;
             e = lines_pass(cw, w, mode, s);
             if (e == cudaSuccess) e = lines_pass(ch, h, mode, s);
         }

@@ -60,6 +60,7 @@ struct LinesCall {
     unsigned int *status;
     const long long *src_off = nullptr, *dst_off = nullptr;
     bool reverse = false;
+    LinesMode beside = LINES_FORWARD;  // what the call's pass along the other axis does
     const float *lam = nullptr;
 };
 cudaError_t lines_pass(const LinesCall &c, int n, LinesMode mode, cudaStream_t stream);

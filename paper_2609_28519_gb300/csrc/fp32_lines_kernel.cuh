@@ -82,10 +82,12 @@ enum Mode { MODE_F = 0, MODE_I = 1, MODE_P = 2, MODE_D = 3, MODE_R = 4 };
 // where shared memory holds no more.
 constexpr int set_of(int mode) { return mode == MODE_F ? 0 : 1; }
 
-// FEW: a call with less than one panel per SM lasts as long as one panel's
-// chain of steps, so its panels are 8 lines and a step is one couple per
-// thread, with the short radices of set 2 (a single 1024 x 768 array, forward
-// and inverse: 24.9 -> 15.2 us).
+// FEW: a call with few panels lasts as long as one panel's chain of steps, so its
+// panels are 8 lines and a step is one couple per thread, with the short radices
+// of set 2 (a single 1024 x 768 array, forward and inverse: 24.9 -> 15.2 us).
+constexpr bool has_few(int n) { return n >= 192 && n < 4096; }
+// Lines per panel of the ordinary form.
+constexpr int panel_lines(int n, int set) { return n <= 192 || (n <= 384 && set) ? 32 : n <= 1024 ? 16 : 8; }
 template <int N, int MODE, bool FEW>
 struct LineCfg;
 
@@ -109,7 +111,7 @@ struct LineCfg<N, MODE, false> : LineSplit<N, set_of(MODE)> {
     static constexpr int G = N <= 192 ? (N == 128 ? 4 : 2) : N == 256 || N == 384 ? (SET ? 4 : 8) : N == 512 ? 8
                            : N == 768 ? (SET ? 8 : 12) : N == 1024 ? (SET ? 8 : 16) : N == 1536 ? (SET ? 16 : 24)
                            : N == 2048 ? 32 : 64;
-    static constexpr int PR = N <= 192 || (N <= 384 && SET) ? 32 : N <= 1024 ? 16 : 8;
+    static constexpr int PR = panel_lines(N, SET);
     static constexpr int THREADS = PR * G, BOUND = THREADS;
     static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET ? 4 : 6) : N == 384 ? (SET ? 3 : 6)
                             : N == 512 ? 4 : N == 768 || N == 1024 || N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
@@ -120,6 +122,9 @@ struct LineCfg<N, MODE, false> : LineSplit<N, set_of(MODE)> {
     static_assert(THREADS % 32 == 0 && PR <= 32 && PR % 4 == 0, "lanes");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
+
+// Shared memory of an SM, of that a CTA's own share, and the most a CTA can ask for.
+constexpr long long kSmemPerSm = 228 * 1024, kSmemReserved = 1024, kSmemMax = kSmemPerSm - kSmemReserved;
 
 struct LinesParams {
     const float *src;
@@ -132,6 +137,7 @@ struct LinesParams {
     const float4 *tw_few;                // and of set 2
     const float *lam;                    // MODE_D: coefficient k of line r times lam[k * rows + r]
     unsigned int *status;
+    int beside_set;                      // table set of the pass along the other axis
     int reverse;                         // take panels last to first (the pass then starts with
                                          // what the previous pass wrote last, still in L2)
 };
@@ -466,7 +472,7 @@ cudaError_t lines_launch(const LinesParams &p0, long long nrows, cudaStream_t st
     e = cache.get(
         dev,
         [&](int d, int &bps, int &sms) {
-            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
             if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, C::THREADS, C::SMEM);
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
             if (r == cudaSuccess && bps < 1) r = cudaErrorInvalidConfiguration;
@@ -481,8 +487,15 @@ cudaError_t lines_launch(const LinesParams &p0, long long nrows, cudaStream_t st
     if (p.rows % C::PR != 0) return cudaErrorInvalidValue;  // panels never straddle two arrays
     const long long np = nrows / C::PR;
     if (np <= 0) return cudaSuccess;
-    // fewer panels than SMs: the short chain (4096 points have the same form)
-    if constexpr (!FEW && N >= 256 && N < 4096) {
+    // fewer panels than SMs: the short chain.  At half the line and at the line
+    // (2048 lines of 512 points) 512 x 512 x 2 takes 6.6 us with it and 7.4 with the
+    // ordinary form inverse, 11.1 and 11.0 round trip, 512 x 512 x 4 8.0 and 8.2,
+    // 12.8 and 12.3; 192 x 64 x 24 (48 panels) forward 6.0 and 9.9.  At 2048 points
+    // the pair modes spill in this form (220 to 300 bytes): up to 16 panels the
+    // ordinary one is the faster (2048 x 64 round trip 12.7 us, 11.3), from 32 on
+    // this one (13.2, 16.6).  4096 points have one form; at 64 and 128 the forms
+    // differ by less than 10% of calls of 6 us.
+    if constexpr (has_few(N) && !FEW) {
         if (np < num_sms) {
             LinesParams few = p;
             few.tw = p.tw_few;
@@ -497,6 +510,20 @@ cudaError_t lines_launch(const LinesParams &p0, long long nrows, cudaStream_t st
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(C::THREADS);
     cfg.dynamicSmemBytes = C::SMEM;
+    // More panels than SMs but fewer than fit at once: the CTAs ask for so much
+    // shared memory that an SM holds no more than its share.  They start while the
+    // pass before them still drains and would otherwise pile up on the SMs it has
+    // left (192 x 128 x 48 inverse 13.0 -> 9.9 us, 512 x 256 x 16 forward 14.1 ->
+    // 10.7, 192 x 1024 x 12 14.9 -> 11.2).  Not beside a pass of fewer than 3/4 panels
+    // per SM, whose small CTAs fit in anywhere and would wait (1024 x 64 x 8 round
+    // trip 8.8 us, 11.1), but for 192 points, whose own chain is the longer (192 x
+    // 1024 x 8 inverse 16.4 -> 11.6).
+    const bool beside_few =  // of the pass along the other axis
+        N != 192 && has_few(p.rows) && 4 * (nrows / p.rows * N / panel_lines(p.rows, p.beside_set)) < 3 * num_sms;
+    if (!FEW && !beside_few && np > num_sms && np < (long long)blocks_per_sm * num_sms) {
+        const long long share = kSmemPerSm / ((np + num_sms - 1) / num_sms) - kSmemReserved;
+        if (share > (long long)C::SMEM) cfg.dynamicSmemBytes = (size_t)share / 128 * 128;
+    }
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -520,6 +547,7 @@ cudaError_t lines_run(LinesMode mode, const LinesCall &c, cudaStream_t s)
     p.tw_few = c.tw_few;
     p.lam = c.lam;
     p.status = c.status;
+    p.beside_set = c.beside == LINES_FORWARD ? 0 : 1;
     p.reverse = c.reverse ? 1 : 0;
     const long long nrows = (long long)c.rows * c.count;
     switch (mode) {
