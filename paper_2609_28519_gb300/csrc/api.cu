@@ -168,6 +168,7 @@ static int lines_plan_tables(bdct_plan *p)
             auto scale = [&](int side) { return ortho || same ? std::sqrt(2.0 / side) : 2.0; };
             auto add = [&](size_t &at, int side) {
                 at = total;
+                if (lines_table_elems(side, set) == 0) return;
                 tables[n++] = LineTable{nullptr, side, set, scale(side)};
                 total += lines_table_elems(side, set);
             };
@@ -513,7 +514,7 @@ static int run_onchip(const bdct_plan *p, Dir dir, const ExecGeom &g0, cudaStrea
     // fused: one read, one write.  The kernels of sides 64 x 128, 128 x 64 and
     // 128 x 128 apply Lambda between orthonormal passes, the others E Lambda E
     // between unscaled ones.
-    g.lam = block_supported(p->rows, p->cols) && !ring_supported(p->rows, p->cols) ? p->spec_plain : p->spec_fold;
+    g.lam = block_supported(p->rows, p->cols) ? p->spec_plain : p->spec_fold;
     e = fused_launch(p->rows, p->cols, DIR_SPEC, p->scales[DIR_RT], g, p->status, s);
     return e == cudaSuccess ? BDCT_OK : cuda_fail(e);
 }

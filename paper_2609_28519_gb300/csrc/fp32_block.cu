@@ -1,5 +1,5 @@
-// On-chip FP32 kernels for sides 64 and 128: 128 x 128, 64 x 128, 128 x 64 and
-// 64 x 64 arrays, one read and one write of every element.
+// On-chip FP32 kernels for sides 64 and 128: 128 x 128, 64 x 128 and 128 x 64
+// arrays, one read and one write of every element.
 //
 // What is computed: Eq. 2 of the BRiDCT paper, C(X) = Q_h X Q_w^T (forward,
 // DCT-II), C^{-1}(Y) = Q_h^T Y Q_w (inverse, DCT-III), the normalized round
@@ -508,13 +508,12 @@ cudaError_t block_init_device(const float *d_table)
 
 bool block_supported(int rows, int cols)
 {
-    return (rows == 64 || rows == 128) && (cols == 64 || cols == 128);
+    return (rows == 64 || rows == 128) && (cols == 64 || cols == 128) && !(rows == 64 && cols == 64);
 }
 
 cudaError_t block_launch(int rows, int cols, Dir dir, const DirScales &sc, const ExecGeom &g, unsigned int *status,
                          cudaStream_t stream)
 {
-    if (rows == 64 && cols == 64) return block_dir<64, 64>(dir, sc, g, status, stream);
     if (rows == 64 && cols == 128) return block_dir<64, 128>(dir, sc, g, status, stream);
     if (rows == 128 && cols == 64) return block_dir<128, 64>(dir, sc, g, status, stream);
     if (rows == 128 && cols == 128) return block_dir<128, 128>(dir, sc, g, status, stream);

@@ -155,8 +155,10 @@ TableShape shape_of()
 template <int N>
 bool shape_of_set(int set, TableShape *q)
 {
-    *q = set == 0 ? shape_of<N, 0>() : set == 1 ? shape_of<N, 1>() : shape_of<N, 2>();
-    return true;
+    if constexpr (has_few(N))
+        if (set == 2) *q = shape_of<N, 2>();
+    if (set != 2) *q = set == 0 ? shape_of<N, 0>() : shape_of<N, 1>();
+    return set != 2 || has_few(N);
 }
 
 bool table_shape(int n, int set, TableShape *q)

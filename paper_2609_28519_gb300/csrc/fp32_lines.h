@@ -38,6 +38,7 @@ struct LineTable {
     int n, set;
     double s1;
 };
+// Entries of a table: 0 for set 2 of a length without a few-panel form.
 size_t lines_table_elems(int n, int set);
 // Generate up to 12 tables in FP64, one launch.
 cudaError_t lines_gen_tables(const LineTable *tables, int count, cudaStream_t s);

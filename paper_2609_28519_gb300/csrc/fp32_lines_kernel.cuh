@@ -115,7 +115,7 @@ struct LineCfg<N, MODE, false> : LineSplit<N, set_of(MODE)> {
     static constexpr int THREADS = PR * G, BOUND = THREADS;
     static constexpr int NB = N == 64 ? 12 : N == 128 ? 6 : N == 192 ? 8 : N == 256 ? (SET ? 4 : 6) : N == 384 ? (SET ? 3 : 6)
                             : N == 512 ? 4 : N == 768 || N == 1024 || N == 1536 ? (SET ? 3 : 2) : N == 2048 ? 2 : 1;
-    static constexpr int PT = N + (PR >= 8 ? 4 : 32 / PR);  // line pitch (floats)
+    static constexpr int PT = N + 4;  // line pitch (floats)
     // the tables are staged in shared memory (the split's read through L1
     // instead: 1024 points inverse 0.328 -> 0.275 of HBM)
     static constexpr size_t SMEM = (size_t)PR * PT * 4 + (size_t)LineSplit<N, SET>::TAB * 16 + 16;
