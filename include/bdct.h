@@ -123,7 +123,10 @@ int bdct_plan_set_spectral(bdct_plan *plan, const double *lambda);
  * normal): the cores then never see magnitudes near FLT_MAX, and subnormal
  * inputs are transformed as normal numbers.  Costs two extra passes over the
  * output and one over the input; results equal the unprotected ones
- * wherever those stay within range.  Arrays whose largest magnitude is 0,
+ * wherever those stay within range.  Without it the butterfly kernels overflow
+ * where a line's unscaled sum does (constant arrays of side n from about
+ * FLT_MAX / n^1.5); the dense and tensor-core routes weight values before they
+ * add them.  Arrays whose largest magnitude is 0,
  * infinite or NaN are left unscaled.  The plan allocates 4 MiB of exponent
  * words (chunks of up to 2^20 arrays; a tiled call may hold at most 2^20
  * blocks, else BDCT_ERR_UNSUPPORTED_SHAPE).  on == 0 turns it off and frees
@@ -144,10 +147,12 @@ int bdct_inverse(const bdct_plan *plan, const float *in, float *out, size_t batc
 int bdct_roundtrip(const bdct_plan *plan, const float *in, float *out, size_t batch, void *stream);
 
 /* Same as above with the direction as an argument (one of the kind bits).
- * BDCT_SPECTRAL runs in one read and one write of every element on the fused
- * kernels of sides 8..32 and on the tensor-core route; the other shapes
- * compose it from the orthonormal forward, the diagonal and the inverse
- * (three passes over the output).                                          */
+ * BDCT_SPECTRAL (Prop. 1: orthonormal forward, diagonal, inverse) runs in one
+ * read and one write of every element where the array stays on chip: sides of
+ * 8 to 32, 64 and 128, any two sides up to 64, and 16 x 16 on the tensor cores.
+ * Longer powers of two and 3 * 2^k run it in three passes, through the
+ * workspace and the output; the dense passes and the other tensor-core shapes
+ * as a forward and an inverse.                                              */
 int bdct_execute(const bdct_plan *plan, unsigned kind, const float *in, float *out,
                  size_t batch, void *stream);
 

@@ -32,9 +32,11 @@ int cuda_fail(cudaError_t e)
 
 // Workspace of the separable routes: arrays per chunk are chosen so that a
 // chunk holds at least one array and about 256 MiB.  Every chunk costs two
-// pass launches with their ramp-up and drain: measured on 256^2 batches
-// 0.30 / 0.34 / 0.35 of HBM with 64 / 128 / 256 MiB chunks, 768 x 1024
-// batches 0.23 / 0.26 / 0.28 (bdct_plan_set_chunk_bytes changes it per plan).
+// pass launches with their ramp-up and drain, which is more than an
+// intermediate kept in L2 saves: 512 MiB forward, us, with 16 / 32 / 64 / 128 /
+// 256 / 512 MiB chunks: 256^2 586 / 446 / 391 / 362 / 345 / 339, 768 x 1024 675 /
+// 522 / 464 / 398 / 362 / 351, 100 x 100 1404 / 1193 / 1148 / 1094 / 1072 / 1061
+// (bdct_plan_set_chunk_bytes changes it per plan).
 constexpr size_t kChunkBytes = 256ull << 20;
 
 }  // namespace

@@ -29,10 +29,10 @@
 // and added to the running total, so the rounding error grows like 16 + n/32
 // rather than n/2.
 //
-// What bounds it: multiply-adds, with eight warps per SM (FMA pipe 47-49%).
-// Against whole operators in 64 x 64 tiles, us: 100 x 100, 256 MiB, forward 1715
-// -> 526, inverse 1715 -> 512, round trip 3430 -> 1036; 16 arrays of 1000 x
-// 1000, forward 2431 -> 725.  Three CTAs per SM (168 registers, spills), the
+// What bounds it: multiply-adds, with eight warps per SM (FMA pipe 46-49%).
+// Against whole operators in 64 x 64 tiles, us: 100 x 100, 256 MiB, forward 1696
+// -> 528, inverse 1696 -> 510, round trip 3392 -> 1037; 16 arrays of 1000 x
+// 1000, forward 2431 -> 728.  Three CTAs per SM (168 registers, spills), the
 // products split by warps and a persistent form were 7-23% slower.
 #include <cuda_runtime.h>
 

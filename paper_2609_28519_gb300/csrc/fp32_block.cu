@@ -28,11 +28,11 @@
 //
 // What bounds it: 40 bytes of shared-memory traffic and about 30
 // multiply-adds per element, against 8 bytes of HBM traffic, and the latency
-// between the barriers of one array (shared wavefronts 39-51%, FMA pipe 40-51%).
+// between the barriers of one array (shared wavefronts 40-50%, FMA pipe 39-57%).
 // Against the form before it (one CTA of eight warps per SM over a ring of
-// arrays), 512 MiB, us: 128 x 128 forward 426 -> 220, inverse 504 -> 245, round
-// trip 870 -> 376, spectral 972 -> 436; 64 x 128 272 -> 209, 342 -> 206, 537 ->
-// 341, 642 -> 356.  64 x 64 is faster in fp32_ring.cu.
+// arrays), 512 MiB, us: 128 x 128 forward 424 -> 215, inverse 506 -> 245, round
+// trip 868 -> 324, spectral 974 -> 386; 64 x 128 272 -> 207, 340 -> 206, 536 ->
+// 309, 642 -> 347.  64 x 64 is faster in fp32_ring.cu.
 #include <cuda_runtime.h>
 
 #include <cmath>

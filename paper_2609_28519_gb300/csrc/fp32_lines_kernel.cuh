@@ -43,18 +43,18 @@
 // row side moves by one bulk copy (TMA) per line.
 //
 // What bounds it: up to 512 points the two passes' HBM traffic, 16 bytes per
-// element (256^2 forward: 0.90 of the copy rate over the bytes it moves);
+// element (256^2 forward: 0.92 of the copy rate over the bytes it moves);
 // beyond that, and in the pair modes, the chain of shared-memory exchanges (16
 // bytes per element, pass and exchange) and the multiply-adds, with 12 to 16
 // warps per SM at full registers.  The form before this one ran four-step FFTs
 // with one sub-FFT per thread, unpacked, 33 instructions per element and pass
-// where this takes 19 to 26 one way.  512 MiB, before -> now, us:
+// where this takes 18 to 26 one way.  512 MiB, before -> now, us:
 //                 forward      inverse      round trip   spectral
-//   256^2         469 -> 351   542 -> 357   758 -> 421   1052 -> 592
-//   768 x 1024    557 -> 363   654 -> 383   983 -> 583   1304 -> 707
-//   1024^2        526 -> 375   574 -> 384   872 -> 571   1197 -> 726
-//   2048^2        640 -> 428   671 -> 442   994 -> 657   1452 -> 834
-//   4 x 4096^2    397 -> 237   416 -> 242   642 -> 359    924 -> 514
+//   256^2         469 -> 345   543 -> 355   758 -> 411   1053 -> 583
+//   768 x 1024    556 -> 361   652 -> 376   979 -> 569   1303 -> 699
+//   1024^2        525 -> 369   575 -> 362   872 -> 553   1185 -> 706
+//   2048^2        638 -> 422   671 -> 439   992 -> 651   1445 -> 820
+//   4 x 4096^2    395 -> 232   414 -> 243   639 -> 361    917 -> 510
 #pragma once
 
 #include <cuda_runtime.h>

@@ -145,9 +145,9 @@ static int time_plan(bdct_plan *plan, unsigned kind_mask, float *d_in, float *d_
 // and the on-chip split-BF16 tensor-core route where it exists), and for a
 // separable route the workspace chunk (64, 128 or 256 MiB: every chunk
 // costs two launches with their ramp-up and drain, which measured more than
-// keeping the intermediate in L2 -- 256^2 batches ran at 0.19 / 0.31 / 0.34
-// of HBM with 8 / 64 / 128 MiB chunks), each timed on scratch arrays of the
-// class's shape.
+// keeping the intermediate in L2 -- 256^2 batches run at 0.27 / 0.41 / 0.44 /
+// 0.46 of HBM with 16 / 64 / 128 / 256 MiB chunks), each timed on scratch arrays
+// of the class's shape.
 static int class_plan(RaggedClass &c, unsigned kind, int norm, int path)
 {
     const bool tc_ok = tc_supported(c.rows, c.cols);

@@ -32,9 +32,9 @@
 //
 // What bounds it: multiply-adds and the reads of their operands with 12 warps
 // per SM (FMA pipe 41-44%).  Against 4 x 4 tiles over the whole operators, 256
-// MiB, us, forward / round trip: 12 x 12 344 / 585 -> 165 / 266, 26 x 32 382 /
-// 704 -> 197 / 341, 48 x 48 573 / 1080 -> 399 / 717, 60 x 60 749 / 1413 -> 331 /
-// 577.
+// MiB, us, forward / round trip: 12 x 12 343 / 585 -> 167 / 267, 26 x 32 382 /
+// 704 -> 197 / 339, 48 x 48 573 / 1081 -> 396 / 718, 60 x 60 750 / 1414 -> 329 /
+// 575.
 #include <cuda_runtime.h>
 
 #include <cstdio>

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(128) k_tcg(const TgParams p)
 // half the input blocks each tile streams, half the partials.  An item is then a
 // row tile and 128 output pairs, its two products one after the other, both
 // sums of a thread's 64 pairs in registers until they meet.  16 arrays of 1024 x
-// 1024, forward and inverse: 761 -> 505 us; what bounds it then is shared
+// 1024, forward and inverse: 761 -> 507 us; what bounds it then is shared
 // memory, 96 KB loaded and 192 KB read by the products per chunk (tensor pipe
 // 51%).  (K/2 a multiple of 64 but not of 128 would leave half tiles, so those
 // lengths keep the whole operator.)
